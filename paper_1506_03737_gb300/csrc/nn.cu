@@ -7,23 +7,28 @@
 // fine-mesh, many-step run from the same seed; plain COLA stays the fallback.
 //
 // Layout
-//   activations  bf16 [z][y][x][16] (32 B per voxel; unused channels are zero)
+//   activations  bf16 [n + 2][n + 2][n + 2][16] ([z][y][x], 32 B per voxel) with the periodic images around
+//                the box stored, so that the halo of any tile is one box of the array: voxel x sits at
+//                x + 1, its image at n + 1 (x = 0) or 0 (x = n - 1), likewise y and z; whoever writes a
+//                voxel writes its images. Channels 0..7 and 8..15 are two 16-byte halves, which swap
+//                places where (stored x >> 2) & 1, so that rows copied as they are into shared memory are
+//                read by ldmatrix without bank conflicts (8 consecutive voxels, one half)
+//   3 channels   the same with 8 channels (16 B per voxel, the rest zero): the packed input and the
+//                gradient at the network output
 //   weights      bf16 [tap][c_out 16][c_in 16], tap = (dz+1) 9 + (dy+1) 3 + (dx+1)
 //   master       fp32 [layer][28][16][16]: taps 0..26 = W[tap][o][i], slot 27 holds the bias in i = 0
 //
 // Every convolution (forward of each layer, backward-data of layers 2..4) is one implicit GEMM:
-// with mma.sync (k_conv, the default) over a 16 x 8 x 8 voxel tile, or on the tcgen05 tensor cores
-// (k_conv_tc, engine 1, grid side a multiple of 128). With 16 channels each tcgen05.mma (M = 128
-// voxels, N = 16, K = 16) reads a 4 KB operand from shared memory for 65,536 FLOP, which bounds it
-// by shared-memory bandwidth; measured at 128^3 it is slower than the mma.sync kernel. mma.sync: M = 16 consecutive x voxels per mma, N = output channels,
-// K = 16 input channels per tap, 27 taps. The 18 x 10 x 10 halo tile of the input is staged in
-// shared memory with cp.async; each voxel's two 16-byte halves swap places on every other
-// group of four voxels so that ldmatrix reads are free of bank conflicts.
+// with mma.sync (k_conv, the default), or on the tcgen05 tensor cores (k_conv_tc, engine 1, grid side
+// a multiple of 128). With 16 channels each tcgen05.mma (M = 128 voxels, N = 16, K = 16) reads a 4 KB
+// operand from shared memory for 65,536 FLOP, which bounds it by shared-memory bandwidth; measured at
+// 128^3 it is slower than the mma.sync kernel.
 //
 //   forward        out[v][o]  = b[o] + sum_tap sum_i W[tap][o][i] a[v + d_tap][i]
 //   backward-data  da[u][i]   = sum_tap sum_o W[tap][o][i] dz[u - d_tap][o]
 //                             = forward with W'[tap][i][o] = W[26 - tap][o][i], no bias
 //   weight grad    dW[tap][o][i] = sum_v dz[v][o] a[v + d_tap][i];  db[o] = sum_v dz[v][o]
+#include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -36,36 +41,31 @@
 #include "../../include/colapm.h"
 #include "../../include/colapm_nn.h"
 #include "colapm_internal.h"
+#include "launch_cache.h"
 
 namespace colapm {
 namespace nn {
 namespace {
 
 constexpr int C = 16;                          // padded channel count
-constexpr int TX = 16, TY = 8, TZ = 8;         // output tile
-constexpr int HX = TX + 2, HY = TY + 2, HZ = TZ + 2;
-constexpr int HALO = HX * HY * HZ;             // 1800 voxels
-constexpr int TILE = TX * TY * TZ;             // 1024 voxels
-constexpr int NTHREADS = 256;                  // 8 warps: warp w owns output plane z = w of the tile
+constexpr int TX = 16, TY = 8;                 // output tile 16 x 8 x TZ voxels (TZ = 8, or 2 on small grids)
+constexpr int HX = TX + 2, HY = TY + 2;
+constexpr int CONV_TZ = 8;                      // planes of a k_conv tile
 constexpr int SLOTS = 28;                      // 27 taps + bias
 constexpr int LAYERS = 4;
 constexpr int LSIZE = SLOTS * C * C;           // 7168 master slots per layer
 constexpr int CIN[LAYERS] = {3, 16, 16, 16};
 constexpr int COUT[LAYERS] = {16, 16, 16, 3};
-
-constexpr size_t SMEM_HALO = (size_t)HALO * 32;   // 57600
-constexpr size_t SMEM_W = 27 * C * 32;            // 13824
-constexpr size_t SMEM_CONV = SMEM_HALO + SMEM_W;
-constexpr size_t SMEM_WGRAD = SMEM_HALO + (size_t)TILE * 32;
+constexpr long long SPIN_LIMIT = 1ll << 24;    // polls of a bounded wait
 
 enum Epi { EPI_RELU = 0, EPI_OUT = 1, EPI_MASK = 2 };
 
 struct ConvArgs {
-    const __nv_bfloat16* in;     // [n^3][16]
+    const __nv_bfloat16* in;     // input voxels (k_conv_tc; k_conv takes them through its tensor map)
     const __nv_bfloat16* w;      // [27][16][16]
     const float* bias;           // [16] or null
     int n;
-    __nv_bfloat16* out;          // EPI_RELU / EPI_MASK: [n^3][16]; EPI_OUT with target: dz [n^3][16]
+    __nv_bfloat16* out;          // EPI_RELU / EPI_MASK: 16 channels; EPI_OUT with target: dz, 8 channels
     const __nv_bfloat16* mask;   // EPI_MASK: the layer input whose ReLU gates the gradient
     float* y;                    // EPI_OUT: [n^3][3] = base + oscale * net
     const float* base;           // EPI_OUT: optional [n^3][3]
@@ -73,31 +73,50 @@ struct ConvArgs {
     const float* target;         // EPI_OUT training: [n^3][3] physical; normalised by tscale
     float tscale, gscale;        // gscale = 2 / (3 n^3)
     double* loss;                // sum of squared normalised errors
-    int* err;                    // bit 4: a bounded wait for the tensor cores gave up
+    int* err;                    // bit 4: a bounded wait gave up
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
+__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t* r) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
 }
-
-__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
+__device__ __forceinline__ void ldsm_x2(uint32_t addr, uint32_t& r0, uint32_t& r1) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(addr));
+}
+__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t* r) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void ldsm_x2_t(uint32_t addr, uint32_t& r0, uint32_t& r1) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(addr));
 }
 
-__device__ __forceinline__ void mma_bf16(float* d, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                         uint32_t b1) {
+__device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
                  "{%0,%1,%2,%3};\n"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Byte offset of half `k` (0: channels 0..7, 1: channels 8..15) of staged voxel `h`.
-__device__ __forceinline__ uint32_t vox_off(int h, int k) { return (uint32_t)(h * 32 + ((k ^ ((h >> 2) & 1)) << 4)); }
+// Place of half `k` (0: channels 0..7, 1: channels 8..15) of a voxel stored at x: its 16-byte slot.
+__host__ __device__ __forceinline__ int half_slot(int x, int k) { return k ^ ((x >> 2) & 1); }
+
+// Index of voxel (x, y, z) in the stored array, and a call f(index) for each of its periodic images there.
+__device__ __forceinline__ size_t voxel(int n, int x, int y, int z) {
+    return ((size_t)(z + 1) * (n + 2) + (y + 1)) * (n + 2) + (x + 1);
+}
+template <class F>
+__device__ __forceinline__ void at_images(int n, int x, int y, int z, F f) {
+    const int ox = x == 0 ? n : (x == n - 1 ? -n : 0), oy = y == 0 ? n : (y == n - 1 ? -n : 0),
+              oz = z == 0 ? n : (z == n - 1 ? -n : 0);
+#pragma unroll 1
+    for (int k = 1; k < 8; ++k) {
+        if (((k & 1) && !ox) || ((k & 2) && !oy) || ((k & 4) && !oz)) continue;
+        f(voxel(n, x + (k & 1 ? ox : 0), y + (k & 2 ? oy : 0), z + (k & 4 ? oz : 0)));
+    }
+}
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src));
@@ -107,6 +126,42 @@ __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.wait_group 0;\n" ::);
 }
 
+__device__ __forceinline__ void mbar_init(uint32_t bar) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+}
+// Waits for phase `parity` of a barrier; false when the poll limit was reached.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+    uint32_t done = 0;
+    for (long long i = 0; i < SPIN_LIMIT && !done; ++i)
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                     : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done != 0;
+}
+// One box of a stored array into shared memory. The array's elements are 8 bytes (VB / 8 per voxel), so that a whole
+// row of a box is one run; a voxel starts at a multiple of 16 bytes, as the copy wants of its x coordinate.
+template <int VB>
+__device__ __forceinline__ void box_load(uint32_t dst, const CUtensorMap& map, int x, int y, int z, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(&map)), "r"(x * (VB / 8)), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
+
+// The box back out of shared memory (written there by ordinary stores), as a bulk group of the calling thread.
+template <int VB>
+__device__ __forceinline__ void box_store(const CUtensorMap& map, int x, int y, int z, uint32_t src) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];\n" ::"l"(
+                     reinterpret_cast<uint64_t>(&map)),
+                 "r"(x * (VB / 8)), "r"(y), "r"(z), "r"(src)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+}
+__device__ __forceinline__ void box_stores_read() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
+
+template <int TZ>
 __device__ __forceinline__ void tile_origin(int t, int n, int& x0, int& y0, int& z0) {
     const int tx = n / TX, ty = n / TY;
     x0 = (t % tx) * TX;
@@ -114,186 +169,403 @@ __device__ __forceinline__ void tile_origin(int t, int n, int& x0, int& y0, int&
     z0 = (t / (tx * ty)) * TZ;
 }
 
-// Stage the periodic halo tile of `in` around the output tile at (x0, y0, z0).
-__device__ __forceinline__ void stage_halo(uint8_t* sm, const __nv_bfloat16* __restrict__ in, int n, int x0, int y0,
-                                           int z0) {
-    const uint32_t base = smem_u32(sm);
-    for (int j = threadIdx.x; j < 2 * HALO; j += NTHREADS) {
-        const int h = j >> 1, k = j & 1;
-        const int hx = h % HX, hy = (h / HX) % HY, hz = h / (HX * HY);
-        int gx = x0 - 1 + hx, gy = y0 - 1 + hy, gz = z0 - 1 + hz;
-        gx += gx < 0 ? n : (gx >= n ? -n : 0);
-        gy += gy < 0 ? n : (gy >= n ? -n : 0);
-        gz += gz < 0 ? n : (gz >= n ? -n : 0);
-        const size_t v = ((size_t)gz * n + gy) * n + gx;
-        cp_async16(base + vox_off(h, k), in + v * C + k * 8);
-    }
-}
+// Byte offsets into the dynamic shared memory of k_conv.
+template <int EPI, int TZ, int VB>
+struct ConvSmem {
+    static constexpr uint32_t HALO = HX * HY * (TZ + 2) * VB;
+    static constexpr uint32_t W = HALO;                             // weights [tap][16][16]
+    static constexpr uint32_t AUX = W + 27 * C * 32;                // output tile (EPI_MASK: first the mask tile)
+    static constexpr uint32_t AUXB = TX * TY * TZ * (EPI == EPI_OUT ? 12 : 32);
+    static constexpr uint32_t BAR = AUX + AUXB;                     // one barrier of the halo, one per warp
+    static constexpr size_t BYTES = BAR + 8 * (1 + TZ);
+};
 
-template <int NT, int EPI>
-__global__ void __launch_bounds__(NTHREADS, 2) k_conv(ConvArgs a) {
-    extern __shared__ __align__(128) uint8_t sm[];
+// Implicit-GEMM convolution, persistent over tiles of 16 x 8 x TZ voxels; warp w makes output plane z = w.
+// M = 16 consecutive x voxels per mma, N = output channels (NT n-tiles of 8), K = 16 input channels of
+// one tap (VB = 16: the upper 8 are zero and are not stored).
+//
+// What bounds it: the mma.sync rate (1024 FMA per clock and SM, measured: 600 TFLOP/s), 49 us for a
+// 16-channel layer at 128^3. Each operand row (hz, hy, dx) is therefore read once per plane offset dz and used
+// for the three dy that need it (rows hy, hy - 1 and hy - 2 of the output), with the nine weights of dz
+// in registers: 30 operand loads per 144 products instead of 72. In that order every output still gets its taps
+// as (dz, dy, dx) from first to last, so the sums are the same bit for bit as tap by tap. The halo of the
+// next tile is fetched by one TMA box while this one's outputs are written, and the second CTA of
+// the SM computes while this one waits. At 128^3 a hidden layer takes 73-75 us (65% of the mma.sync rate; what is left
+// is the start and end of each tile) against 95 us with one operand load per product pair and per-thread 16-byte
+// copies, a backward one 79 against 133, the output layer 67 against 122 (153 with the loss). Row by row bulk copies
+// instead of the box took 89-95 us (about 130 cycles each), 4-plane tiles at three CTAs per SM 86 us.
+template <int NT, int EPI, int TZ, int VB>
+__global__ void __launch_bounds__(32 * TZ, TZ == 8 ? 2 : 4)
+    k_conv(ConvArgs a, const __grid_constant__ CUtensorMap halo, const __grid_constant__ CUtensorMap out,
+           const __grid_constant__ CUtensorMap mask) {
+    using S = ConvSmem<EPI, TZ, VB>;
+    extern __shared__ __align__(1024) uint8_t sm[];
     const int n = a.n;
-    int x0, y0, z0;
-    tile_origin(blockIdx.x, n, x0, y0, z0);
-    stage_halo(sm, a.in, n, x0, y0, z0);
-    {   // weights, swizzled like voxels with the output channel as the row
-        const uint32_t wb = smem_u32(sm + SMEM_HALO);
-        for (int j = threadIdx.x; j < 27 * C * 2; j += NTHREADS) {
-            const int row = j >> 1, k = j & 1;
-            cp_async16(wb + vox_off(row, k), a.w + row * C + k * 8);
-        }
+    const int ntiles = (n / TX) * (n / TY) * (n / TZ);
+    const int lane = threadIdx.x & 31, tz = threadIdx.x >> 5;
+    const int g = lane >> 2, q = lane & 3;
+    const uint32_t hb = smem_u32(sm), wb = hb + S::W, aux = hb + S::AUX + tz * (TX * TY * 32),
+                   bar = hb + S::BAR, mbar = bar + 8 + 8 * tz;
+    for (int j = threadIdx.x; j < 27 * C * 2; j += 32 * TZ) {   // weights, swizzled with the row index
+        const int row = j >> 1, k = j & 1;
+        cp_async16(wb + row * 32 + (half_slot(row, k) << 4), a.w + row * C + k * 8);
+    }
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < 1 + TZ; ++b) mbar_init(bar + 8 * b);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     cp_async_wait_all();
     __syncthreads();
+    // a run of consecutive tiles, so that every CTA has its share of those on the faces of the box, which
+    // write images too (dealt out round robin, one CTA had the same place in x every time)
+    const int tend = (int)((long long)ntiles * (blockIdx.x + 1) / gridDim.x);
+    int t = (int)((long long)ntiles * blockIdx.x / gridDim.x), x0, y0, z0;
+    tile_origin<TZ>(t, n, x0, y0, z0);
+    auto load_halo = [&]() {   // stored voxel x0 is the left neighbour of x0
+        mbar_expect(bar, S::HALO);
+        box_load<VB>(hb, halo, x0, y0, z0, bar);
+    };
+    auto load_mask = [&]() {   // this warp's plane of the mask tile
+        mbar_expect(mbar, TX * TY * 32);
+        box_load<32>(aux, mask, x0 + 1, y0 + 1, z0 + 1 + tz, mbar);
+    };
+    if (threadIdx.x == 0) load_halo();
 
-    const int lane = threadIdx.x & 31, tz = threadIdx.x >> 5;
-    const int g = lane >> 2, q = lane & 3;
-    const uint32_t hb = smem_u32(sm), wb = smem_u32(sm + SMEM_HALO);
     // ldmatrix roles: A rows (voxels) and halves; B rows (output channels) and halves
     const int ar = (lane & 7) + 8 * ((lane >> 3) & 1), ak = lane >> 4;
     const int bn = (lane & 7) + 8 * (lane >> 4), bk = (lane >> 3) & 1;
+    uint32_t aoff[3];   // this lane's operand row for each dx (stored x0 is a multiple of 16)
+#pragma unroll
+    for (int dx = 0; dx < 3; ++dx)
+        aoff[dx] = hb + tz * (HY * HX * VB) + (ar + dx) * VB + (VB == 32 ? half_slot(ar + dx, ak) << 4 : 0);
+    const uint32_t boff = wb + bn * 32 + (half_slot(bn, bk) << 4);
+    // loss: pairs of floats (sum and its rounding errors), FP64 at the end
+    float ls = 0.0f, lc = 0.0f;
 
-    float acc[TY][NT][4];
-#pragma unroll
-    for (int m = 0; m < TY; ++m)
-#pragma unroll
-        for (int j = 0; j < NT; ++j)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[m][j][e] = 0.0f;
-
-#pragma unroll 1
-    for (int tap = 0; tap < 27; ++tap) {
-        const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-        uint32_t b[4];
-        ldsm_x4(wb + vox_off(tap * C + bn, bk), b[0], b[1], b[2], b[3]);
-        const int hrow = ((tz + 1 + dz) * HY + (1 + dy)) * HX + 1 + dx + ar;
-#pragma unroll
-        for (int m = 0; m < TY; ++m) {
-            uint32_t a0, a1, a2, a3;
-            ldsm_x4(hb + vox_off(hrow + m * HX, ak), a0, a1, a2, a3);
-            mma_bf16(acc[m][0], a0, a1, a2, a3, b[0], b[1]);
-            if (NT == 2) mma_bf16(acc[m][1], a0, a1, a2, a3, b[2], b[3]);
+    uint32_t phase = 0;
+    for (; t < tend; ++t, phase ^= 1) {
+        bool ok = mbar_wait(bar, phase);
+        if (!ok) ok = (atomicOr(a.err, 4), mbar_wait(bar, phase), false);   // flag it, let the copies land, stop
+        if (!__syncthreads_and(ok)) break;
+        if (EPI != EPI_OUT && lane == 0) {
+            box_stores_read();   // the previous tile's outputs have left the buffer
+            if (EPI == EPI_MASK) load_mask();
         }
-    }
-
-    double lsum = 0.0;
+        constexpr int NPRE = EPI == EPI_OUT ? TX * TY * 3 / 32 : 1;
+        float pre[NPRE];   // EPI_OUT: the tile of target or base, in flight during the products
+        if (EPI == EPI_OUT) {
+            const float* src = a.target ? a.target : a.base;
 #pragma unroll
-    for (int m = 0; m < TY; ++m) {
+            for (int i = 0; i < NPRE; ++i) {
+                const int e = lane + 32 * i;
+                pre[i] = src ? __ldg(src + (((size_t)(z0 + tz) * n + y0 + e / (TX * 3)) * n + x0) * 3 + e % (TX * 3)) : 0.0f;
+            }
+        }
+        float acc[TY][NT][4];
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const int x = g + 8 * half;
-            const size_t v = ((size_t)(z0 + tz) * n + (y0 + m)) * n + x0 + x;
+        for (int m = 0; m < TY; ++m)
 #pragma unroll
-            for (int j = 0; j < NT; ++j) {
-                const int ch = 8 * j + 2 * q;
-                float v0 = acc[m][j][2 * half], v1 = acc[m][j][2 * half + 1];
-                if (EPI == EPI_RELU) {
-                    v0 = fmaxf(v0 + a.bias[ch], 0.0f);
-                    v1 = fmaxf(v1 + a.bias[ch + 1], 0.0f);
-                    *reinterpret_cast<__nv_bfloat162*>(a.out + v * C + ch) = __floats2bfloat162_rn(v0, v1);
-                } else if (EPI == EPI_MASK) {
-                    const __nv_bfloat162 mk = *reinterpret_cast<const __nv_bfloat162*>(a.mask + v * C + ch);
-                    v0 = __bfloat162float(mk.x) > 0.0f ? v0 : 0.0f;
-                    v1 = __bfloat162float(mk.y) > 0.0f ? v1 : 0.0f;
-                    *reinterpret_cast<__nv_bfloat162*>(a.out + v * C + ch) = __floats2bfloat162_rn(v0, v1);
-                } else if (j == 0 && q < 2) {   // EPI_OUT: channels 0..2 of n-tile 0
-                    v0 += a.bias[ch];
-                    v1 += a.bias[ch + 1];
-                    const float vv[2] = {v0, v1};
-                    float dzv[2] = {0.0f, 0.0f};
+            for (int j = 0; j < NT; ++j)
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int c = ch + e;
-                        if (c < 3) {
-                            a.y[v * 3 + c] = (a.base ? a.base[v * 3 + c] : 0.0f) + a.oscale * vv[e];
-                            if (a.target) {
-                                const float d = vv[e] - a.target[v * 3 + c] * a.tscale;
-                                lsum += (double)d * d;
-                                dzv[e] = a.gscale * d;
-                            }
-                        }
+                for (int e = 0; e < 4; ++e) acc[m][j][e] = 0.0f;
+#pragma unroll 1
+        for (int dz = 0; dz < 3; ++dz) {
+            uint32_t b[9][2 * NT];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                if (NT == 2) ldsm_x4(boff + (dz * 9 + k) * (C * 32), b[k]);
+                else ldsm_x2(boff + (dz * 9 + k) * (C * 32), b[k][0], b[k][1]);
+            }
+            const uint32_t zo = dz * (HY * HX * VB);
+#pragma unroll
+            for (int hy = 0; hy < HY; ++hy) {
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx) {
+                    uint32_t f[4];
+                    if (VB == 32) {
+                        ldsm_x4(aoff[dx] + zo + hy * (HX * VB), f);
+                    } else {
+                        ldsm_x2(aoff[dx] + zo + hy * (HX * VB), f[0], f[1]);
+                        f[2] = f[3] = 0u;
                     }
-                    if (a.target)
-                        *reinterpret_cast<__nv_bfloat162*>(a.out + v * C + ch) = __floats2bfloat162_rn(dzv[0], dzv[1]);
+#pragma unroll
+                    for (int dy = 0; dy < 3; ++dy) {
+                        const int m = hy - dy;
+                        if (m < 0 || m >= TY) continue;
+#pragma unroll
+                        for (int j = 0; j < NT; ++j) mma_bf16(acc[m][j], f, b[3 * dy + dx][2 * j], b[3 * dy + dx][2 * j + 1]);
+                    }
                 }
             }
         }
-    }
-    if (EPI == EPI_OUT && a.target) {
+        __syncthreads();   // the halo has been read
+        const int cx = x0, cy = y0, cz = z0;
+        if (t + 1 < tend) {
+            tile_origin<TZ>(t + 1, n, x0, y0, z0);
+            if (threadIdx.x == 0) load_halo();
+        }
+        if (EPI == EPI_RELU || EPI == EPI_MASK) {
+            if (EPI == EPI_MASK && !mbar_wait(mbar, phase)) {
+                atomicOr(a.err, 4);   // flag it and let the copy land
+                mbar_wait(mbar, phase);
+            }
+            float bia[NT][2];
 #pragma unroll
-        for (int o = 16; o; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-        if (lane == 0 && lsum != 0.0) atomicAdd(a.loss, lsum);
+            for (int j = 0; j < NT; ++j)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) bia[j][e] = EPI == EPI_RELU ? a.bias[8 * j + 2 * q + e] : 0.0f;
+            __syncwarp();
+            uint8_t* tile = sm + S::AUX + tz * (TX * TY * 32);   // voxels as they are stored, from x0 + 1
+#pragma unroll
+            for (int m = 0; m < TY; ++m)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int j = 0; j < NT; ++j) {
+                        float u0 = acc[m][j][2 * h], u1 = acc[m][j][2 * h + 1];
+                        __nv_bfloat162* p = reinterpret_cast<__nv_bfloat162*>(
+                            tile + (m * TX + g + 8 * h) * 32 + half_slot(g + 1, j) * 16 + 4 * q);
+                        if (EPI == EPI_RELU) {
+                            u0 = fmaxf(u0 + bia[j][0], 0.0f);
+                            u1 = fmaxf(u1 + bia[j][1], 0.0f);
+                        } else {   // the mask's value lies where the output goes
+                            const __nv_bfloat162 mk = *p;
+                            u0 = __bfloat162float(mk.x) > 0.0f ? u0 : 0.0f;
+                            u1 = __bfloat162float(mk.y) > 0.0f ? u1 : 0.0f;
+                        }
+                        *p = __floats2bfloat162_rn(u0, u1);
+                    }
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            __syncwarp();
+            if (lane == 0) box_store<32>(out, cx + 1, cy + 1, cz + tz + 1, aux);
+            // images of the voxels on the faces of the box (n voxels away: the same half slots, n a multiple of 16).
+            // Per axis a set of shifts: 0, +n on the low face, -n on the high one
+            const int z = cz + tz;
+            const unsigned mx = 1u | (cx == 0 ? 2u : 0u) | (cx + TX == n ? 4u : 0u),
+                           my = 1u | (cy == 0 ? 2u : 0u) | (cy + TY == n ? 4u : 0u),
+                           mz = 1u | (z == 0 ? 2u : 0u) | (z + 1 == n ? 4u : 0u);
+            if ((mx | my | mz) != 1u)
+                for (unsigned uz = mz; uz; uz &= uz - 1)
+                    for (unsigned uy = my; uy; uy &= uy - 1)
+                        for (unsigned ux = mx; ux; ux &= ux - 1) {
+                            const unsigned lowz = uz & -uz, lowy = uy & -uy, lowx = ux & -ux;
+                            if ((lowx | lowy | lowz) == 1u) continue;   // the voxels themselves
+                            const int nx = lowx == 1u ? TX : 1, ny = lowy == 1u ? TY : 1;
+                            const int lx = lowx == 4u ? TX - 1 : 0, ly = lowy == 4u ? TY - 1 : 0;
+                            const size_t v0 = voxel(n, cx + (lowx == 1u ? 0 : (lowx == 2u ? n : -n)),
+                                                    cy + (lowy == 1u ? 0 : (lowy == 2u ? n : -n)),
+                                                    z + (lowz == 1u ? 0 : (lowz == 2u ? n : -n)));
+                            for (int e = lane; e < 2 * nx * ny; e += 32) {
+                                const int x = lx + ((e >> 1) & (nx - 1)), y = ly + (nx == 1 ? e >> 1 : e / (2 * TX));
+                                reinterpret_cast<uint4*>(a.out)[2 * (v0 + (size_t)y * (n + 2) + x) + (e & 1)] =
+                                    reinterpret_cast<const uint4*>(tile)[2 * (y * TX + x) + (e & 1)];
+                            }
+                        }
+            __syncwarp();
+        } else {   // EPI_OUT: channels 0..2 through shared memory, so that rows leave as whole 192-byte runs
+            float* so = reinterpret_cast<float*>(sm + S::AUX) + tz * (TX * TY * 3);
+            if (q < 2) {
+                const float c0 = a.bias[2 * q], c1 = q == 0 ? a.bias[1] : 0.0f;
+#pragma unroll
+                for (int m = 0; m < TY; ++m)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        float* p = so + (m * TX + g + 8 * h) * 3 + 2 * q;
+                        p[0] = acc[m][0][2 * h] + c0;
+                        if (q == 0) p[1] = acc[m][0][2 * h + 1] + c1;
+                    }
+            }
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < NPRE; ++k) {
+                const int e = lane + 32 * k;
+                const size_t i = (((size_t)(cz + tz) * n + cy + e / (TX * 3)) * n + cx) * 3 + e % (TX * 3);
+                const float u = so[e];
+                const float b = !a.target ? pre[k] : (a.base ? a.base[i] : 0.0f);
+                a.y[i] = b + a.oscale * u;
+                if (a.target) {
+                    const float d = u - pre[k] * a.tscale;
+                    so[e] = a.gscale * d;
+                    const float p = __fmul_rn(d, d), pe = fmaf(d, d, -p), s = __fadd_rn(ls, p), z = __fsub_rn(s, ls);
+                    lc += (__fsub_rn(ls, __fsub_rn(s, z)) + __fsub_rn(p, z)) + pe;
+                    ls = s;
+                }
+            }
+            if (a.target) {
+                __syncwarp();
+                for (int e = lane; e < TX * TY; e += 32) {
+                    const __nv_bfloat162 b01 = __floats2bfloat162_rn(so[3 * e], so[3 * e + 1]);
+                    const __nv_bfloat162 b2z = __floats2bfloat162_rn(so[3 * e + 2], 0.0f);
+                    const uint4 u = make_uint4(*reinterpret_cast<const uint32_t*>(&b01), *reinterpret_cast<const uint32_t*>(&b2z), 0u, 0u);
+                    const int x = cx + e % TX, y = cy + e / TX, z = cz + tz;
+                    reinterpret_cast<uint4*>(a.out)[voxel(n, x, y, z)] = u;
+                    at_images(n, x, y, z, [&](size_t i) { reinterpret_cast<uint4*>(a.out)[i] = u; });
+                }
+            }
+            __syncwarp();   // the outputs have been read before the next tile's are written
+        }
+    }
+    if (EPI != EPI_OUT && lane == 0) box_stores_read();   // shared memory stays until it has been read
+    if (EPI == EPI_OUT && a.target) {
+        double s = (double)ls + (double)lc;
+#pragma unroll
+        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0 && s != 0.0) atomicAdd(a.loss, s);
     }
 }
 
+// Byte offsets into the dynamic shared memory of k_wgrad: two buffers of (activation halo, dz tile); at the
+// end the per-group sums take their place.
+template <int TZ, int VA, int VD>
+struct WgradSmem {
+    static constexpr uint32_t HALO = HX * HY * (TZ + 2) * VA;
+    static constexpr uint32_t BUF = HALO + TX * TY * TZ * VD;
+    static constexpr uint32_t SUMS = (TZ / 2) * LSIZE * 4;
+    static constexpr uint32_t BAR = 2 * BUF > SUMS ? 2 * BUF : SUMS;
+    static constexpr size_t BYTES = BAR + 16;
+};
+
 // Per-CTA partial weight gradients of one layer over a static round-robin share of the tiles:
-// part[blockIdx.x][slot][o][i]. Warp w owns slots {w, w + 8, w + 16, w + 24} below 28.
-__global__ void __launch_bounds__(NTHREADS, 2)
-    k_wgrad(const __nv_bfloat16* __restrict__ dz, const __nv_bfloat16* __restrict__ act, int n, float* __restrict__ part) {
-    extern __shared__ __align__(128) uint8_t sm[];
+// part[blockIdx.x][slot][o][i]. A warp takes one plane offset dz (9 taps, all accumulators in
+// registers) and two output planes of the tile: 3 x TZ / 2 warps. K = the 16 voxels of an x row.
+// ACT_A = false: M = output channels (dz rows), N = input channels; true (the last layer, whose 3 output
+// channels fit one n-tile): M = input channels, N = output channels.
+//
+// What bounds it: the mma.sync rate (49 us per 16-channel layer at 128^3). Stepping over the halo rows hy, a
+// warp loads the three shifted activation rows (dx) and one dz row, and uses them with the last three dz rows
+// (dy): 18 products for 4 operand loads, against 7 for 4.5 when each warp walked its own taps. The next
+// tile arrives in the other buffer meanwhile, as two TMA boxes. At 128^3 a 16-channel layer takes
+// 67 us (75% of that rate) against 170 us, the first and the last layer 41 and 43.
+template <bool ACT_A, int NT, int TZ, int VA, int VD>
+__global__ void __launch_bounds__(32 * 3 * (TZ / 2), 1)
+    k_wgrad(const __grid_constant__ CUtensorMap act, const __grid_constant__ CUtensorMap dz, int n,
+            float* __restrict__ part, int* err) {
+    using S = WgradSmem<TZ, VA, VD>;
+    constexpr int NTHR = 32 * 3 * (TZ / 2);
+    extern __shared__ __align__(1024) uint8_t sm[];
     const int ntiles = (n / TX) * (n / TY) * (n / TZ);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int zo = w % 3, grp = w / 3;                                      // plane offset, planes 2 grp and 2 grp + 1
     const int g = lane >> 2, q = lane & 3;
-    const uint32_t hb = smem_u32(sm), db = smem_u32(sm + SMEM_HALO);
-    const int av = (lane & 7) + 8 * (lane >> 4), ak = (lane >> 3) & 1;       // dz^T as A
-    const int bv = (lane & 7) + 8 * ((lane >> 3) & 1), bk = lane >> 4;      // shifted act as B
+    const uint32_t sb = smem_u32(sm), bar = sb + S::BAR;
+    if (threadIdx.x == 0) {
+        mbar_init(bar);
+        mbar_init(bar + 8);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    __syncthreads();
+    auto load = [&](int t, int buf) {   // halo of the activations and dz of tile t
+        int x0, y0, z0;
+        tile_origin<TZ>(t, n, x0, y0, z0);
+        const uint32_t d = sb + buf * S::BUF, b = bar + 8 * buf;
+        mbar_expect(b, S::BUF);
+        box_load<VA>(d, act, x0, y0, z0, b);
+        box_load<VD>(d + S::HALO, dz, x0 + 1, y0 + 1, z0 + 1, b);
+    };
+    // Operand rows are voxels (K), read transposed. As A (M = channels): matrices (lo channels, voxels 0-7),
+    // (hi, 0-7), (lo, 8-15), (hi, 8-15). As B (N = channels): (lo, 0-7), (lo, 8-15), (hi, 0-7), (hi, 8-15).
+    const int a_v = (lane & 7) + 8 * (lane >> 4), a_k = (lane >> 3) & 1;
+    const int b_v = (lane & 7) + 8 * ((lane >> 3) & 1), b_k = lane >> 4;
+    const int act_v = ACT_A ? a_v : b_v, act_k = ACT_A ? a_k : b_k;
+    const int dz_v = ACT_A ? b_v : a_v, dz_k = ACT_A ? b_k : a_k;
+    uint32_t ao[3];
+#pragma unroll
+    for (int dx = 0; dx < 3; ++dx)
+        ao[dx] = (VA == 32 ? (act_v + dx) * 32 + (half_slot(act_v + dx, act_k) << 4) : (((lane & 15) + dx) * 16)) +
+                 zo * (HY * HX * VA);
+    const uint32_t dof = S::HALO + (VD == 32 ? dz_v * 32 + (half_slot(dz_v + 1, dz_k) << 4) : (lane & 15) * 16);
     const uint32_t ones = 0x3F803F80u;                                      // bf16 pair (1, 1)
+    const uint32_t ones4[4] = {ones, ones, ones, ones};
 
-    float acc[4][2][4];
+    float acc[9][NT][4], accb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+    for (int s = 0; s < 9; ++s)
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
+        for (int j = 0; j < NT; ++j)
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[s][j][e] = 0.0f;
 
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        int x0, y0, z0;
-        tile_origin(t, n, x0, y0, z0);
-        stage_halo(sm, act, n, x0, y0, z0);
-        for (int j = threadIdx.x; j < 2 * TILE; j += NTHREADS) {
-            const int l = j >> 1, k = j & 1;
-            const int lx = l % TX, ly = (l / TX) % TY, lz = l / (TX * TY);
-            const size_t v = ((size_t)(z0 + lz) * n + (y0 + ly)) * n + x0 + lx;
-            cp_async16(db + vox_off(l, k), dz + v * C + k * 8);
+    if (threadIdx.x == 0 && (int)blockIdx.x < ntiles) load(blockIdx.x, 0);
+    int it = 0;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++it) {
+        const int buf = it & 1;
+        if (threadIdx.x == 0 && t + (int)gridDim.x < ntiles) load(t + gridDim.x, buf ^ 1);
+        bool ok = mbar_wait(bar + 8 * buf, (it >> 1) & 1);
+        if (!ok) ok = (atomicOr(err, 4), mbar_wait(bar + 8 * buf, (it >> 1) & 1), false);
+        if (!__syncthreads_and(ok)) {   // let the other buffer's copies land too, then stop
+            if (t + (int)gridDim.x < ntiles) mbar_wait(bar + 8 * (buf ^ 1), ((it + 1) >> 1) & 1);
+            return;
         }
-        cp_async_wait_all();
-        __syncthreads();
+        const uint32_t base = sb + buf * S::BUF;
 #pragma unroll 1
-        for (int row = 0; row < TZ * TY; ++row) {
-            const int lz = row / TY, ly = row % TY;
-            uint32_t a0, a1, a2, a3;
-            ldsm_x4_t(db + vox_off(row * TX + av, ak), a0, a1, a2, a3);
+        for (int pl = 0; pl < 2; ++pl) {
+            const uint32_t ab = base + (2 * grp + pl) * (HY * HX * VA);
+            const uint32_t db = base + dof + (2 * grp + pl) * (TY * TX * VD);
+            uint32_t d[TY][4];
 #pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const int slot = w + 8 * s;
-                if (slot >= SLOTS) break;
-                uint32_t b0, b1, b2, b3;
-                if (slot == 27) {
-                    b0 = b1 = b2 = b3 = ones;
-                } else {
-                    const int dzz = slot / 9 - 1, dyy = (slot / 3) % 3 - 1, dxx = slot % 3 - 1;
-                    const int h = ((lz + 1 + dzz) * HY + (ly + 1 + dyy)) * HX + 1 + dxx + bv;
-                    ldsm_x4_t(hb + vox_off(h, bk), b0, b1, b2, b3);
+            for (int hy = 0; hy < HY; ++hy) {
+                if (hy < TY) {
+                    if (VD == 32) {
+                        ldsm_x4_t(db + hy * (TX * VD), d[hy]);
+                    } else {   // 8 channels: two matrices, voxels 0-7 and 8-15
+                        ldsm_x2_t(db + hy * (TX * VD), d[hy][0], d[hy][1]);
+                        d[hy][2] = d[hy][3] = 0u;
+                    }
+                    if (zo == 1) {   // bias: the sum of dz
+                        if (ACT_A) mma_bf16(accb, ones4, d[hy][0], d[hy][1]);
+                        else mma_bf16(accb, d[hy], ones, ones);
+                    }
                 }
-                mma_bf16(acc[s][0], a0, a1, a2, a3, b0, b1);
-                mma_bf16(acc[s][1], a0, a1, a2, a3, b2, b3);
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx) {
+                    uint32_t f[4];
+                    if (VA == 32) ldsm_x4_t(ab + ao[dx] + hy * (HX * VA), f);
+                    else ldsm_x2_t(ab + ao[dx] + hy * (HX * VA), f[0], f[1]);
+#pragma unroll
+                    for (int dy = 0; dy < 3; ++dy) {
+                        const int m = hy - dy;   // output row of the tap (dz, dy, dx) that reads halo row hy
+                        if (m < 0 || m >= TY) continue;
+#pragma unroll
+                        for (int j = 0; j < NT; ++j) {
+                            if (ACT_A) mma_bf16(acc[3 * dy + dx][j], f, d[m][0], d[m][1]);
+                            else mma_bf16(acc[3 * dy + dx][j], d[m], f[2 * j], f[2 * j + 1]);
+                        }
+                    }
+                }
             }
         }
-        __syncthreads();
+        __syncthreads();   // this buffer has been read
     }
+    // sums of the groups, then over the groups in a fixed order
+    float* sums = reinterpret_cast<float*>(sm);
+    float* mine = sums + (size_t)grp * LSIZE;
+    auto put = [&](int slot, int m, int k, float v) { mine[slot * C * C + (ACT_A ? k * C + m : m * C + k)] = v; };
+    for (int e = threadIdx.x; e < (TZ / 2) * LSIZE; e += NTHR) sums[e] = 0.0f;
+    __syncthreads();
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const int slot = w + 8 * s;
-        if (slot >= SLOTS) break;
-        float* p = part + ((size_t)blockIdx.x * SLOTS + slot) * C * C;
+    for (int s = 0; s < 9; ++s)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int i = 8 * j + 2 * q;
-            *reinterpret_cast<float2*>(p + g * C + i) = make_float2(acc[s][j][0], acc[s][j][1]);
-            *reinterpret_cast<float2*>(p + (g + 8) * C + i) = make_float2(acc[s][j][2], acc[s][j][3]);
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) put(zo * 9 + s, g + 8 * (e >> 1), 8 * j + 2 * q + (e & 1), acc[s][j][e]);
+    if (zo == 1) {   // db[o] in column 0 of slot 27: from column 0 (M = o), or from row 0 (N = o)
+        if (ACT_A) {
+            if (g == 0) {
+                put(27, 0, 2 * q, accb[0]);
+                put(27, 0, 2 * q + 1, accb[1]);
+            }
+        } else if (q == 0) {
+            put(27, g, 0, accb[0]);
+            put(27, g + 8, 0, accb[2]);
         }
+    }
+    __syncthreads();
+    float* p = part + (size_t)blockIdx.x * LSIZE;
+    for (int e = threadIdx.x; e < LSIZE; e += NTHR) {
+        float s = sums[e];
+#pragma unroll
+        for (int k = 1; k < TZ / 2; ++k) s += sums[(size_t)k * LSIZE + e];
+        p[e] = s;
     }
 }
 
@@ -315,7 +587,6 @@ constexpr uint32_t TC_PLANE = TC_HALO * 16;                       // bytes per K
 constexpr uint32_t TC_W = 27 * 512;                               // weight bytes
 constexpr size_t TC_SMEM = 2 * (size_t)TC_PLANE + TC_W + 128;     // + mbarrier and TMEM address
 constexpr uint32_t TC_COLS = TC_ROWS * 16;                        // TMEM columns (power of two)
-constexpr long long TC_SPIN_LIMIT = 1ll << 24;
 // kind::f16 instruction descriptor: FP32 D (bits 4-5), BF16 A and B (bits 7-9, 10-12), both
 // K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28.
 constexpr uint32_t TC_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((16u >> 3) << 17) | ((128u >> 4) << 24);
@@ -325,22 +596,19 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t lbo, uint32_
            ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);   // no swizzle, base offset 0
 }
 
-// Stage the halo of tile t (periodic) into the two K-half planes with 16-byte cp.async.
-__device__ __forceinline__ void tc_stage(uint32_t sbase, const __nv_bfloat16* __restrict__ in, int n, int t) {
+// Stage the halo of tile t into the two K-half planes with 16-byte cp.async.
+// An 8-channel input (in8) fills the first plane; the second is zero and is cleared once by the caller.
+__device__ __forceinline__ void tc_stage(uint32_t sbase, const __nv_bfloat16* __restrict__ in, int n, int t, bool in8) {
     const int txn = n / 128, tyn = n / TC_TY;
     const int x0 = (t % txn) * 128, y0 = ((t / txn) % tyn) * TC_TY, z0 = (t / (txn * tyn)) * TC_TZ;
 #pragma unroll 1
     for (int row = 0; row < TC_HY * TC_HZ; ++row) {
         const int hy = row % TC_HY, hz = row / TC_HY;
-        int gy = y0 - 1 + hy, gz = z0 - 1 + hz;
-        gy += gy < 0 ? n : (gy >= n ? -n : 0);
-        gz += gz < 0 ? n : (gz >= n ? -n : 0);
-        const __nv_bfloat16* src = in + ((size_t)gz * n + gy) * n * C;
-        for (int j = threadIdx.x; j < 2 * TC_HX; j += 128) {
-            const int hx = j >> 1, k = j & 1;
-            int gx = x0 - 1 + hx;
-            gx += gx < 0 ? n : (gx >= n ? -n : 0);
-            cp_async16(sbase + k * TC_PLANE + (row * TC_HX + hx) * 16, src + (size_t)gx * C + k * 8);
+        const __nv_bfloat16* src = in + (((size_t)(z0 + hz) * (n + 2) + y0 + hy) * (n + 2) + x0) * (in8 ? 8 : C);
+        for (int j = threadIdx.x; j < (in8 ? 1 : 2) * TC_HX; j += 128) {
+            const int hx = in8 ? j : j >> 1, k = in8 ? 0 : j & 1;
+            cp_async16(sbase + k * TC_PLANE + (row * TC_HX + hx) * 16,
+                       in8 ? src + hx * 8 : src + hx * C + half_slot(hx, k) * 8);
         }
     }
     asm volatile("cp.async.commit_group;\n" ::);
@@ -350,7 +618,7 @@ __device__ __forceinline__ void tc_stage(uint32_t sbase, const __nv_bfloat16* __
 // the staged halo, issue the 27 x TC_ROWS MMAs (one thread), wait for them, start staging the next
 // tile's halo (the MMAs no longer read shared memory), then read TMEM and write the outputs.
 template <int EPI>
-__global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
+__global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a, bool in8) {
     extern __shared__ __align__(1024) uint8_t sm[];
     uint8_t* wsm = sm + 2 * TC_PLANE;
     uint64_t* mbar = reinterpret_cast<uint64_t*>(wsm + TC_W);
@@ -363,7 +631,10 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
         const int tap = j >> 5, o = (j >> 1) & 15, k = j & 1;
         cp_async16(sbase + 2 * TC_PLANE + tap * 512 + k * 256 + o * 16, a.w + (tap * C + o) * C + k * 8);
     }
-    if (blockIdx.x < ntiles) tc_stage(sbase, a.in, n, blockIdx.x);
+    if (in8)
+        for (uint32_t j = tid; j < TC_PLANE / 16; j += 128)
+            *reinterpret_cast<uint4*>(sm + TC_PLANE + j * 16) = make_uint4(0u, 0u, 0u, 0u);
+    if (blockIdx.x < ntiles) tc_stage(sbase, a.in, n, blockIdx.x, in8);
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(mbar)));
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -407,7 +678,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
                          : "memory");
         }
         uint32_t done = 0;
-        for (long long i = 0; i < TC_SPIN_LIMIT && !done; ++i) {
+        for (long long i = 0; i < SPIN_LIMIT && !done; ++i) {
             asm volatile(
                 "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
                 : "=r"(done)
@@ -420,7 +691,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
         }
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         if (!__syncthreads_and(done)) break;
-        if (t + (int)gridDim.x < ntiles) tc_stage(sbase, a.in, n, t + gridDim.x);   // overlaps the epilogue
+        if (t + (int)gridDim.x < ntiles) tc_stage(sbase, a.in, n, t + gridDim.x, in8);   // overlaps the epilogue
         const int x0 = (t % txn) * 128, y0 = ((t / txn) % tyn) * TC_TY, z0 = (t / (txn * tyn)) * TC_TZ;
 #pragma unroll 1
         for (int r = 0; r < TC_ROWS; ++r) {
@@ -432,15 +703,16 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
                 : "r"(taddr + ((uint32_t)(32 * warp) << 16) + r * 16));
             asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
             const int ry = r % TC_TY, rz = r / TC_TY;
-            const size_t v = ((size_t)(z0 + rz) * n + (y0 + ry)) * n + x0 + 32 * warp + lane;
+            const int vx = x0 + 32 * warp + lane, vy = y0 + ry, vz = z0 + rz;
+            const size_t v = ((size_t)vz * n + vy) * n + vx, vs = voxel(n, vx, vy, vz);
             float acc[16];
 #pragma unroll
             for (int c = 0; c < 16; ++c) acc[c] = __uint_as_float(q[c]);
             if (EPI == EPI_RELU || EPI == EPI_MASK) {
                 uint32_t pk[8];
                 if (EPI == EPI_MASK) {
-                    const uint4* mp = reinterpret_cast<const uint4*>(a.mask + v * C);
-                    const uint4 m0 = mp[0], m1 = mp[1];
+                    const uint4* mp = reinterpret_cast<const uint4*>(a.mask + vs * C);
+                    const uint4 m0 = mp[half_slot(lane + 1, 0)], m1 = mp[half_slot(lane + 1, 1)];
                     const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
@@ -458,9 +730,13 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
                         pk[c] = *reinterpret_cast<const uint32_t*>(&b);
                     }
                 }
-                uint4* op = reinterpret_cast<uint4*>(a.out + v * C);
-                op[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                op[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                auto put = [&](size_t i) {
+                    uint4* op = reinterpret_cast<uint4*>(a.out) + 2 * i;
+                    op[half_slot(lane + 1, 0)] = make_uint4(pk[0], pk[1], pk[2], pk[3]);   // stored at lane + 1 (mod 8)
+                    op[half_slot(lane + 1, 1)] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                };
+                put(vs);
+                at_images(n, vx, vy, vz, put);
             } else {   // EPI_OUT: channels 0..2
                 float dzv[3];
 #pragma unroll
@@ -477,8 +753,9 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
                 if (a.target) {
                     const __nv_bfloat162 b01 = __floats2bfloat162_rn(dzv[0], dzv[1]);
                     const __nv_bfloat162 b2z = __floats2bfloat162_rn(dzv[2], 0.0f);
-                    *reinterpret_cast<uint2*>(a.out + v * C) =
-                        make_uint2(*reinterpret_cast<const uint32_t*>(&b01), *reinterpret_cast<const uint32_t*>(&b2z));
+                    const uint4 u = make_uint4(*reinterpret_cast<const uint32_t*>(&b01), *reinterpret_cast<const uint32_t*>(&b2z), 0u, 0u);
+                    reinterpret_cast<uint4*>(a.out)[vs] = u;
+                    at_images(n, vx, vy, vz, [&](size_t i) { reinterpret_cast<uint4*>(a.out)[i] = u; });
                 }
             }
         }
@@ -502,18 +779,26 @@ __device__ __forceinline__ bool real_slot(int l, int slot, int o, int i) {
     return slot < 27 ? i < cin[l] : i == 0;
 }
 
-// Sum the per-CTA partials of every layer in a fixed order: grad[l][slot][o][i].
-__global__ void k_reduce_grads(const float* __restrict__ part, int nparts, float* __restrict__ grad) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= LAYERS * LSIZE) return;
+// Sum the per-CTA partials of every layer in a fixed order: grad[l][slot][o][i]. 32 slots per block, the
+// partials dealt over RG_Y rows of threads (a column of 304 sums one after the other took 23 us).
+constexpr int RG_Y = 32;
+__global__ void __launch_bounds__(32 * RG_Y) k_reduce_grads(const float* __restrict__ part, int nparts, float* __restrict__ grad) {
+    __shared__ float sh[RG_Y][33];
+    const int idx = blockIdx.x * 32 + threadIdx.x;   // LAYERS * LSIZE is a multiple of 32
     const int l = idx / LSIZE, r = idx % LSIZE;
     const int slot = r / (C * C), o = (r / C) % C, i = r % C;
+    const bool real = real_slot(l, slot, o, i);
     float s = 0.0f;
-    if (real_slot(l, slot, o, i)) {
-        const float* p = part + (size_t)l * nparts * LSIZE + r;
-        for (int b = 0; b < nparts; ++b) s += p[(size_t)b * LSIZE];
+    if (real)
+        for (int b = threadIdx.y; b < nparts; b += RG_Y) s += part[((size_t)l * nparts + b) * LSIZE + r];
+    sh[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y == 0) {
+        s = 0.0f;
+#pragma unroll
+        for (int k = 0; k < RG_Y; ++k) s += sh[k][threadIdx.x];
+        grad[idx] = real ? s : 0.0f;
     }
-    grad[idx] = s;
 }
 
 // Adam on the FP32 master copy, then the BF16 forward and flipped-transposed weights and the bias.
@@ -544,19 +829,21 @@ __global__ void k_adam(float* __restrict__ wm, float* __restrict__ m1, float* __
     }
 }
 
-// x[v][c] = bf16(psi[v][c] / s_in) for c < 3, zero for the padded channels.
-__global__ void k_pack_input(const float* __restrict__ psi, size_t nv, float inv_s, __nv_bfloat16* __restrict__ x) {
-    const size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= nv) return;
-    const __nv_bfloat162 p01 = __floats2bfloat162_rn(psi[3 * v] * inv_s, psi[3 * v + 1] * inv_s);
-    const __nv_bfloat162 p2z = __floats2bfloat162_rn(psi[3 * v + 2] * inv_s, 0.0f);
-    uint4 lo;
-    lo.x = *reinterpret_cast<const uint32_t*>(&p01);
-    lo.y = *reinterpret_cast<const uint32_t*>(&p2z);
-    lo.z = lo.w = 0u;
-    uint4* d = reinterpret_cast<uint4*>(x + v * C);
-    d[0] = lo;
-    d[1] = make_uint4(0u, 0u, 0u, 0u);
+// x[v][c] = bf16(psi[v][c] / s_in) for c < 3, zero for the other five channels; one thread per stored voxel.
+__global__ void k_pack_input(const float* __restrict__ psi, int n, float inv_s, __nv_bfloat16* __restrict__ x) {
+    const int m = n + 2, row = blockIdx.x * blockDim.y + threadIdx.y;   // stored row (z, y)
+    if (row >= m * m) return;
+    int y = row % m - 1, z = row / m - 1;
+    y += y < 0 ? n : (y >= n ? -n : 0);
+    z += z < 0 ? n : (z >= n ? -n : 0);
+    const float* src = psi + ((size_t)z * n + y) * n * 3;
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        const int gx = i == 0 ? n - 1 : (i == n + 1 ? 0 : i - 1);
+        const __nv_bfloat162 p01 = __floats2bfloat162_rn(src[3 * gx] * inv_s, src[3 * gx + 1] * inv_s);
+        const __nv_bfloat162 p2z = __floats2bfloat162_rn(src[3 * gx + 2] * inv_s, 0.0f);
+        reinterpret_cast<uint4*>(x)[(size_t)row * m + i] =
+            make_uint4(*reinterpret_cast<const uint32_t*>(&p01), *reinterpret_cast<const uint32_t*>(&p2z), 0u, 0u);
+    }
 }
 
 }  // namespace
@@ -571,11 +858,15 @@ struct colapm_nn {
     colapm_nn_config cfg{};
     cudaStream_t stream = nullptr;
     int steps = 0;
-    int nparts = 0;
+    int nparts = 0;                    // CTAs of a weight gradient (one per SM at most)
+    int sms = 0;
+    bool small = false;                // tiles of 2 planes instead of 8
     // device
-    __nv_bfloat16* act[LAYERS] = {};   // act[0] = packed input, act[l] = output of layer l (l = 1..3)
+    __nv_bfloat16* act[LAYERS] = {};   // act[0] = packed input (8 channels), act[l] = output of layer l (l = 1..3)
     __nv_bfloat16* dz[2] = {};         // gradient ping-pong
-    __nv_bfloat16* dz_out = nullptr;   // gradient at the network output (channels 0..2)
+    // TMA boxes of each array: halo and plane of a k_conv tile, halo and tile of k_wgrad
+    struct Maps { CUtensorMap halo, whalo, wtile, plane; } m_act[LAYERS], m_dz[2], m_dz_out;
+    __nv_bfloat16* dz_out = nullptr;   // gradient at the network output (8 channels, 0..2 used)
     float* y = nullptr;                // scratch output [n^3][3]
     float* wm = nullptr;               // master [4][28][16][16]
     float* m1 = nullptr;
@@ -588,7 +879,6 @@ struct colapm_nn {
     double* loss = nullptr;
     int* err = nullptr;                // device error word (bit 4: a tensor-core wait gave up)
     bool use_tc = false;               // tcgen05 convolutions (grid side a multiple of 128)
-    int tc_grid = 0;                   // persistent grid of the tcgen05 convolutions
     long long launches = 0;
 };
 
@@ -602,35 +892,57 @@ namespace {
         }                                         \
     } while (0)
 
-int conv_grid(int n) { return (n / TX) * (n / TY) * (n / TZ); }
+// Tiles of 16 x 8 x TZ voxels. TZ = 8 gives the least halo; a grid with fewer of them than half the SMs (side
+// 32 and less) is cut into planes of 2, so that up to four times as many SMs work on it: forward / training
+// step at side 32 in 35 / 110 us against 43 / 135 us with TZ = 8, at side 16 in 39 / 112 against 49 / 137, but
+// at side 48 (108 tiles of 8 planes) in 45 / 138 against 43 / 138.
+int tiles_of(int n, int tz) { return (n / TX) * (n / TY) * (n / tz); }
 
-bool configured = false;
-
-cudaError_t configure() {
-    if (configured) return cudaSuccess;
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_conv<2, EPI_RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_CONV))) return e;
-    if ((e = cudaFuncSetAttribute(k_conv<2, EPI_MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_CONV))) return e;
-    if ((e = cudaFuncSetAttribute(k_conv<1, EPI_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_CONV))) return e;
-    if ((e = cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_WGRAD))) return e;
-    if ((e = cudaFuncSetAttribute(k_conv_tc<EPI_RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM))) return e;
-    if ((e = cudaFuncSetAttribute(k_conv_tc<EPI_MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM))) return e;
-    if ((e = cudaFuncSetAttribute(k_conv_tc<EPI_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM))) return e;
-    configured = true;
-    return cudaSuccess;
+template <int NT, int EPI, int TZ, int VB>
+cudaError_t launch_conv(const colapm_nn* c, const ConvArgs& a, const CUtensorMap& halo, const CUtensorMap& out, const CUtensorMap& mask) {
+    using S = ConvSmem<EPI, TZ, VB>;
+    static colapm::GridCache cache;
+    int grid = 0;
+    cudaError_t e = colapm::cached_grid(cache, k_conv<NT, EPI, TZ, VB>, 32 * TZ, S::BYTES, &grid);
+    if (e) return e;
+    k_conv<NT, EPI, TZ, VB><<<std::min(tiles_of(c->n, TZ), grid), 32 * TZ, S::BYTES, c->stream>>>(a, halo, out, mask);
+    return cudaGetLastError();
 }
 
-template <int NT, int EPI>
-cudaError_t conv(colapm_nn* c, ConvArgs a) {
+// VB: bytes per voxel of the input (16: the packed input or the output gradient).
+template <int NT, int EPI, int VB>
+cudaError_t conv(colapm_nn* c, ConvArgs a, const colapm_nn::Maps& in, const colapm_nn::Maps& out, const colapm_nn::Maps& mask) {
     a.err = c->err;
+    ++c->launches;
     if (c->use_tc) {
         const int tiles = (c->n / 128) * (c->n / TC_TY) * (c->n / TC_TZ);
-        k_conv_tc<EPI><<<std::min(tiles, c->tc_grid), 128, TC_SMEM, c->stream>>>(a);
-    } else {
-        k_conv<NT, EPI><<<conv_grid(c->n), NTHREADS, SMEM_CONV, c->stream>>>(a);
+        static colapm::GridCache cache;
+        int grid = 0;
+        cudaError_t e = colapm::cached_grid(cache, k_conv_tc<EPI>, 128, TC_SMEM, &grid);
+        if (e) return e;
+        k_conv_tc<EPI><<<std::min(tiles, grid), 128, TC_SMEM, c->stream>>>(a, VB == 16);
+        return cudaGetLastError();
     }
-    ++c->launches;
+    return c->small ? launch_conv<NT, EPI, 2, VB>(c, a, in.halo, out.plane, mask.plane)
+                    : launch_conv<NT, EPI, CONV_TZ, VB>(c, a, in.halo, out.plane, mask.plane);
+}
+
+template <bool ACT_A, int NT, int TZ, int VA, int VD>
+cudaError_t launch_wgrad(colapm_nn* c, const CUtensorMap& dz, int l) {
+    using S = WgradSmem<TZ, VA, VD>;
+    static colapm::GridCache cache;
+    int grid = 0;   // only the shared-memory attribute: the CTAs are the network's partials
+    cudaError_t e = colapm::cached_grid(cache, k_wgrad<ACT_A, NT, TZ, VA, VD>, 96 * (TZ / 2), S::BYTES, &grid);
+    if (e) return e;
+    k_wgrad<ACT_A, NT, TZ, VA, VD><<<c->nparts, 96 * (TZ / 2), S::BYTES, c->stream>>>(
+        c->m_act[l].whalo, dz, c->n, c->part + (size_t)l * c->nparts * LSIZE, c->err);
     return cudaGetLastError();
+}
+
+template <bool ACT_A, int NT, int VA, int VD>
+cudaError_t wgrad(colapm_nn* c, const CUtensorMap& dz, int l) {
+    ++c->launches;
+    return c->small ? launch_wgrad<ACT_A, NT, 2, VA, VD>(c, dz, l) : launch_wgrad<ACT_A, NT, 8, VA, VD>(c, dz, l);
 }
 
 // Report (and clear) a device-side error of the network's kernels; synchronises.
@@ -660,7 +972,8 @@ cudaError_t publish(colapm_nn* c) {
 // Forward through all four layers; with `target`, also the output gradient and the loss sum.
 cudaError_t forward(colapm_nn* c, const float* psi, float* y, const float* base, const float* target) {
     const size_t nv = c->nv;
-    k_pack_input<<<(unsigned)((nv + 255) / 256), 256, 0, c->stream>>>(psi, nv, 1.0f / c->cfg.s_in, c->act[0]);
+    const int rows = (c->n + 2) * (c->n + 2), bx = c->n >= 62 ? 64 : 32;
+    k_pack_input<<<(rows + 3) / 4, dim3(bx, 4), 0, c->stream>>>(psi, c->n, 1.0f / c->cfg.s_in, c->act[0]);
     ++c->launches;
     cudaError_t e = cudaGetLastError();
     if (e) return e;
@@ -671,7 +984,9 @@ cudaError_t forward(colapm_nn* c, const float* psi, float* y, const float* base,
         a.bias = c->bias + l * C;
         a.n = c->n;
         a.out = c->act[l + 1];
-        if ((e = conv<2, EPI_RELU>(c, a))) return e;
+        const auto &in = c->m_act[l], &out = c->m_act[l + 1];
+        e = l == 0 ? conv<2, EPI_RELU, 16>(c, a, in, out, out) : conv<2, EPI_RELU, 32>(c, a, in, out, out);
+        if (e) return e;
     }
     ConvArgs a{};
     a.in = c->act[3];
@@ -688,18 +1003,18 @@ cudaError_t forward(colapm_nn* c, const float* psi, float* y, const float* base,
         a.loss = c->loss;
         a.out = c->dz_out;
     }
-    return conv<1, EPI_OUT>(c, a);
+    return conv<1, EPI_OUT, 32>(c, a, c->m_act[3], c->m_dz_out, c->m_dz_out);
 }
 
 // Backward through all layers into per-CTA partials, then the fixed-order reduction into grad.
 cudaError_t backward(colapm_nn* c) {
     cudaError_t e;
     const __nv_bfloat16* g = c->dz_out;
+    const colapm_nn::Maps* gm = &c->m_dz_out;
     for (int l = 3; l >= 0; --l) {
-        k_wgrad<<<c->nparts, NTHREADS, SMEM_WGRAD, c->stream>>>(g, c->act[l], c->n,
-                                                               c->part + (size_t)l * c->nparts * LSIZE);
-        ++c->launches;
-        if ((e = cudaGetLastError())) return e;
+        e = l == 3 ? wgrad<true, 1, 32, 16>(c, gm->wtile, l)
+                   : (l == 0 ? wgrad<false, 1, 16, 32>(c, gm->wtile, l) : wgrad<false, 2, 32, 32>(c, gm->wtile, l));
+        if (e) return e;
         if (l == 0) break;
         ConvArgs a{};
         a.in = g;
@@ -707,13 +1022,34 @@ cudaError_t backward(colapm_nn* c) {
         a.n = c->n;
         a.mask = c->act[l];
         a.out = c->dz[l & 1];
-        if ((e = conv<2, EPI_MASK>(c, a))) return e;
+        const colapm_nn::Maps* om = &c->m_dz[l & 1];
+        e = l == 3 ? conv<2, EPI_MASK, 16>(c, a, *gm, *om, c->m_act[l]) : conv<2, EPI_MASK, 32>(c, a, *gm, *om, c->m_act[l]);
+        if (e) return e;
         g = c->dz[l & 1];
+        gm = om;
     }
-    const int total = LAYERS * LSIZE;
-    k_reduce_grads<<<(total + 255) / 256, 256, 0, c->stream>>>(c->part, c->nparts, c->grad);
+    k_reduce_grads<<<LAYERS * LSIZE / 32, dim3(32, RG_Y), 0, c->stream>>>(c->part, c->nparts, c->grad);
     ++c->launches;
     return cudaGetLastError();
+}
+
+// Tensor maps of a stored array of (n + 2)^3 voxels of vb bytes, as 8-byte elements.
+bool encode_maps(colapm_nn::Maps& m, void* p, int n, int vb, bool small) {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult st;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &st) != cudaSuccess || !fn)
+        return false;
+    const auto encode = reinterpret_cast<decltype(&cuTensorMapEncodeTiled)>(fn);
+    const cuuint64_t e = vb / 8, s = n + 2, dims[3] = {s * e, s, s}, strides[2] = {s * vb, s * s * vb};
+    const cuuint32_t one[3] = {1, 1, 1};
+    auto box = [&](CUtensorMap* map, cuuint32_t x, cuuint32_t y, cuuint32_t z) {
+        const cuuint32_t b[3] = {(cuuint32_t)(x * e), y, z};
+        return encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, p, dims, strides, b, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                      CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    const int cz = small ? 2 : CONV_TZ, wz = small ? 2 : 8;
+    return box(&m.halo, HX, HY, cz + 2) && box(&m.whalo, HX, HY, wz + 2) && box(&m.wtile, TX, TY, wz) && box(&m.plane, TX, TY, 1);
 }
 
 // Flat parameter order: per layer W[27][cout][cin] then b[cout].
@@ -800,20 +1136,15 @@ int colapm_nn_create(int n, const colapm_nn_config* cfg, void* stream, colapm_nn
         colapm_nn_destroy(c);
         return code;
     };
-    if (configure() != cudaSuccess) return fail(COLAPM_E_CUDA);
-    int dev = 0, sms = 0, occ = 0;
-    if (cudaGetDevice(&dev) || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_wgrad, NTHREADS, SMEM_WGRAD))
-        return fail(COLAPM_E_CUDA);
-    c->nparts = std::max(1, std::min(conv_grid(n), sms * std::max(occ, 1)));
-    int occ_tc = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_tc, k_conv_tc<EPI_RELU>, 128, TC_SMEM)) return fail(COLAPM_E_CUDA);
-    c->tc_grid = sms * std::max(occ_tc, 1);
-    const size_t abytes = c->nv * C * sizeof(__nv_bfloat16);
+    int dev = 0;
+    if (cudaGetDevice(&dev) || cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev)) return fail(COLAPM_E_CUDA);
+    c->small = 2 * tiles_of(n, 8) < c->sms;
+    c->nparts = std::min(tiles_of(n, c->small ? 2 : 8), c->sms * (c->small ? 2 : 1));
+    const size_t abytes = (size_t)(n + 2) * (n + 2) * (n + 2) * C * sizeof(__nv_bfloat16);
     bool ok = true;
-    for (int l = 0; l < LAYERS; ++l) ok = ok && cudaMalloc(&c->act[l], abytes) == cudaSuccess;
+    for (int l = 0; l < LAYERS; ++l) ok = ok && cudaMalloc(&c->act[l], l == 0 ? abytes / 2 : abytes) == cudaSuccess;
     ok = ok && cudaMalloc(&c->dz[0], abytes) == cudaSuccess && cudaMalloc(&c->dz[1], abytes) == cudaSuccess &&
-         cudaMalloc(&c->dz_out, abytes) == cudaSuccess && cudaMalloc(&c->y, c->nv * 3 * sizeof(float)) == cudaSuccess;
+         cudaMalloc(&c->dz_out, abytes / 2) == cudaSuccess && cudaMalloc(&c->y, c->nv * 3 * sizeof(float)) == cudaSuccess;
     const size_t ps = (size_t)LAYERS * LSIZE * sizeof(float);
     ok = ok && cudaMalloc(&c->wm, ps) == cudaSuccess && cudaMalloc(&c->m1, ps) == cudaSuccess &&
          cudaMalloc(&c->m2, ps) == cudaSuccess && cudaMalloc(&c->grad, ps) == cudaSuccess &&
@@ -826,8 +1157,12 @@ int colapm_nn_create(int n, const colapm_nn_config* cfg, void* stream, colapm_nn
         (void)cudaGetLastError();
         return fail(COLAPM_E_NOMEM);
     }
+    for (int l = 0; l < LAYERS; ++l) ok = ok && encode_maps(c->m_act[l], c->act[l], n, l == 0 ? 16 : 32, c->small);
+    ok = ok && encode_maps(c->m_dz[0], c->dz[0], n, 32, c->small) && encode_maps(c->m_dz[1], c->dz[1], n, 32, c->small) &&
+         encode_maps(c->m_dz_out, c->dz_out, n, 16, c->small);
+    if (!ok) return fail(COLAPM_E_CUDA);
     c->use_tc = cfg->engine == 1 && n % 128 == 0;
-    if (cudaMemsetAsync(c->err, 0, sizeof(int), c->stream) || cudaMemsetAsync(c->dz_out, 0, abytes, c->stream) ||
+    if (cudaMemsetAsync(c->err, 0, sizeof(int), c->stream) ||
         cudaMemsetAsync(c->m1, 0, ps, c->stream) ||
         cudaMemsetAsync(c->m2, 0, ps, c->stream) || cudaMemsetAsync(c->grad, 0, ps, c->stream))
         return fail(COLAPM_E_CUDA);
