@@ -281,8 +281,8 @@ long long colapm_kernel_launches(const colapm_ctx* ctx);
 /* ---- autotuning ------------------------------------------------------------------------- */
 /* The mesh passes of a force computation, each on the two-stage register FFT (bit set) or on the
  * multi-stage shared-memory Stockham FFT (bit clear). A pass whose line length has no two-stage
- * plan (the lengths 64, 96, 128, 160, 192, 256, 320, 384, 512, 1024 have one: two radices in
- * {8, 10, 12, 16, 20, 24, 32}) runs on the Stockham plan either way. The initial-condition
+ * plan (the lengths 32, 48, 64, 80, 96, 128, 160, 192, 256, 320, 384, 512, 1024 have one: two radices in
+ * {4, 6, 8, 10, 12, 16, 20, 24, 32}) runs on the Stockham plan either way. The initial-condition
  * transforms on the particle grid take the same choice per kind of pass. */
 #define COLAPM_PLAN_XF 1u    /* forward x pass (r2c of the density)                  */
 #define COLAPM_PLAN_Y 2u     /* y passes, both directions                             */
@@ -315,8 +315,8 @@ int colapm_autotune(colapm_ctx* ctx, int* choice);
 int colapm_set_engine(colapm_ctx* ctx, int fused, int two_stage, int block);
 
 /* Select the plan per pass: a mask of COLAPM_PLAN_* bits (two-stage where set). The blocked
- * half-spectrum layout of the 512^3 and 1024^3 meshes needs every pass two-stage; any other mask
- * uses the plain layout there. COLAPM_E_ARG outside 0 ... COLAPM_PLAN_ALL. */
+ * half-spectrum layout of the meshes from 64^3 on needs every pass two-stage; any other mask uses the
+ * plain layout. COLAPM_E_ARG outside 0 ... COLAPM_PLAN_ALL. */
 int colapm_set_plan(colapm_ctx* ctx, int plan);
 
 /* The context's configuration: cfg (7 ints) = {plan mask, particle-kernel block size, fused x-y

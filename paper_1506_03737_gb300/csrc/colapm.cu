@@ -520,8 +520,8 @@ int colapm_create(const colapm_params* p, void* stream, colapm_ctx** out) {
     if (ok && xy_supported(c->nm))
         ok = dalloc(reinterpret_cast<char**>(&c->xy_ring), xy_ring_bytes(c->nm)) == cudaSuccess &&
              dalloc(&c->xy_ctr, xy_ctr_ints(c->nm, 3)) == cudaSuccess;
-    // blocked spectra where every pass has a two-stage plan (the x passes need N/2 in 256, 512)
-    if (ok && (c->nm == 512 || c->nm == 1024)) ok = dalloc(&c->Freal, 3 * c->nm3) == cudaSuccess;
+    // blocked spectra where every pass has a two-stage plan (lines of N and of N / 2)
+    if (ok && c->nm >= 64) ok = dalloc(&c->Freal, 3 * c->nm3) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         free_all(c);

@@ -1,6 +1,6 @@
-// Two-stage register FFT for the mesh lengths with a two-radix plan (L = 64 ... 1024).
+// Two-stage register FFT for the lengths with a two-radix plan (L = 32 ... 1024).
 //
-// A line of length L = RA * RB (radices 8 to 32) is transformed in two Stockham stages. In
+// A line of length L = RA * RB (radices 4 to 32) is transformed in two Stockham stages. In
 // stage A (stride 1) task j < L/RA takes inputs j + r L/RA (r < RA) straight from global memory
 // (or from the caller), applies the RA-point DFT in registers and writes output r to position
 // j RA + r of a shared exchange buffer. In stage B (stride RA) task j < RA reads positions
@@ -25,7 +25,10 @@ namespace colapm {
 
 template <int L>
 struct F2;
+template <> struct F2<32> { static constexpr int R1 = 8, R2 = 4; };
+template <> struct F2<48> { static constexpr int R1 = 8, R2 = 6; };
 template <> struct F2<64> { static constexpr int R1 = 8, R2 = 8; };
+template <> struct F2<80> { static constexpr int R1 = 8, R2 = 10; };
 template <> struct F2<96> { static constexpr int R1 = 8, R2 = 12; };
 template <> struct F2<128> { static constexpr int R1 = 16, R2 = 8; };
 template <> struct F2<160> { static constexpr int R1 = 16, R2 = 10; };
@@ -36,11 +39,11 @@ template <> struct F2<384> { static constexpr int R1 = 16, R2 = 24; };
 template <> struct F2<512> { static constexpr int R1 = 16, R2 = 32; };
 template <> struct F2<1024> { static constexpr int R1 = 32, R2 = 32; };
 
-// Lengths with a two-stage plan. The mixed ones (96, 160, 192, 320, 384) take a composite second
-// radix (10, 12, 20, 24), itself split into coprime factors in registers (prime-factor algorithm).
+// Lengths with a two-stage plan: every mesh side above 16, and half of every one above 32. The mixed ones (48, 80,
+// 96, 160, 192, 320, 384) take a composite second radix (6, 10, 12, 20, 24), itself split into coprime factors in registers (prime-factor algorithm).
 template <int L>
 struct F2Has {
-    static constexpr bool value = L == 64 || L == 96 || L == 128 || L == 160 || L == 192 || L == 256 || L == 320 ||
+    static constexpr bool value = L == 32 || L == 48 || L == 64 || L == 80 || L == 96 || L == 128 || L == 160 || L == 192 || L == 256 || L == 320 ||
                                   L == 384 || L == 512 || L == 1024;
 };
 
@@ -118,11 +121,22 @@ __host__ __device__ __forceinline__ size_t hs_index(int kx, int y, int z) {
     else return ((size_t)z * L + y) * (L / 2) + kx;
 }
 
-// Distance between rows y and y + d of one column when d and y are multiples of 8 apart from the
-// same residue (d a multiple of 8): what the passes add per register index.
+// Distance between rows y and y + d of one column (d a multiple of 8 in the blocked layout).
 template <int L, bool BLK>
 __host__ __device__ __forceinline__ constexpr size_t hs_ystep(int d) {
     return BLK ? (size_t)(d / 8) * L * 64 : (size_t)d * (L / 2);
+}
+
+// Offset of row j + r STEP from row 0 of a column: what the passes add per register index. A compile-time
+// multiple from row j on, except where STEP is not a multiple of 8 in the blocked layout (the mixed lengths).
+template <int L, bool BLK, int STEP>
+__host__ __device__ __forceinline__ size_t hs_row(int j, int r) {
+    if constexpr (!BLK || STEP % 8 == 0) {
+        return (BLK ? (size_t)(j >> 3) * L * 64 + (j & 7) * 8 : (size_t)j * (L / 2)) + r * hs_ystep<L, BLK>(STEP);
+    } else {
+        const int y = j + r * STEP;
+        return (size_t)(unsigned)((y >> 3) * (L * 64) + (y & 7) * 8);
+    }
 }
 
 // Stage B of a line held in exchange buffer xb (stage-A radix RA), task j < RA of line c:
@@ -151,12 +165,12 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy(float2* __restrict__ data, siz
     const int tid = threadIdx.x, c = tid & 7, j = tid >> 3;
     for (int t = blockIdx.x; t < total; t += gridDim.x) {
         const int f = t / TPF, r0 = t % TPF;
-        // rows y = j + r L/RA (stage A) and j + RA r (stage B); L/RA and RA are multiples of 8
-        float2* g = data + (size_t)f * fstride + hs_index<L, BLK>((r0 % NG) * 8 + c, j, r0 / NG);
+        // rows y = j + r L/RA (stage A) and j + RA r (stage B)
+        float2* g = data + (size_t)f * fstride + hs_index<L, BLK>((r0 % NG) * 8 + c, 0, r0 / NG);
         if (tid < K::TA) {
             float2 v[RA];
 #pragma unroll
-            for (int r = 0; r < RA; ++r) v[r] = __ldcg(g + r * hs_ystep<L, BLK>(L / RA));
+            for (int r = 0; r < RA; ++r) v[r] = __ldcg(g + hs_row<L, BLK, L / RA>(j, r));
             dft<RA, S>(v);
 #pragma unroll
             for (int r = 0; r < RA; ++r) xb[Xch<L, RA>::at(c, j * RA + r)] = v[r];
@@ -166,7 +180,7 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy(float2* __restrict__ data, siz
             float2 v[RB];
             stage_b<L, RA, RB, S>(xb, tws, c, j, v);
 #pragma unroll
-            for (int r = 0; r < RB; ++r) g[r * hs_ystep<L, BLK>(RA)] = v[r];
+            for (int r = 0; r < RB; ++r) g[hs_row<L, BLK, RA>(j, r)] = v[r];
         }
         __syncthreads();
     }
@@ -185,10 +199,11 @@ struct Z2 {
     // stage-A registers: the smaller footprint fits three CTAs per SM at C = 4, which hides the load
     // latency better than the prefetch does with two (force z pass at 1024^3: 6.0 against 6.9 ms)
     static constexpr bool PREFETCH = MODE != Z_LPT1 && !DIRECT;
-    static constexpr int MINB = DIRECT && C == 4 ? 3 : 1;                         // CTAs per SM
     static constexpr int PF = PREFETCH ? C * L : 0;                               // dense [z][C] buffer
     static constexpr int TA = C * L / R1, TB = C * L / R2, T = TA > TB ? TA : TB;
     static constexpr size_t SMEM = sizeof(float2) * ((size_t)XS * (1 + NSAVE) + PF) + sizeof(Tw2);
+    // CTAs per SM: 12 warps where a task holds 32 values, 20 (at most 102 registers) with the smaller radices
+    static constexpr int MINB = DIRECT ? (R1 == 32 || R2 == 32 ? 384 / T : 640 / T) : 1;
 };
 
 template <int L, int MODE, int C = 8, bool BLK = false, bool DIRECT = false>
@@ -412,7 +427,7 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy_force(float2* __restrict__ dat
     const int tid = threadIdx.x, c = tid & 7, j = tid >> 3;
     for (int t = blockIdx.x; t < TPF; t += gridDim.x) {
         const int kx = (t % NG) * 8 + c;
-        const size_t off = hs_index<L, true>(kx, j, t / NG);   // row j; other rows at hs_ystep offsets
+        const size_t off = hs_index<L, true>(kx, 0, t / NG);
         const float kxv = kf * (float)kx;
 #pragma unroll 1
         for (int pass = 0; pass < 3; ++pass) {
@@ -423,7 +438,7 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy_force(float2* __restrict__ dat
 #pragma unroll
                 for (int r = 0; r < RA; ++r) {
                     const int y = j + r * (L / RA);
-                    v[r] = __ldcg(src + r * hs_ystep<L, true>(L / RA));
+                    v[r] = __ldcg(src + hs_row<L, true, L / RA>(j, r));
                     if (pass == 1) v[r] = cscale(v[r], kf * (float)sbin(y, L));
                 }
                 dft<RA, +1>(v);
@@ -436,7 +451,7 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy_force(float2* __restrict__ dat
                 stage_b<L, RA, RB, +1>(xb, tws, c, j, u);
                 const float sc = pass == 2 ? kxv : 1.0f;
 #pragma unroll
-                for (int r = 0; r < RB; ++r) dst[r * hs_ystep<L, true>(RA)] = make_float2(-sc * u[r].y, sc * u[r].x);
+                for (int r = 0; r < RB; ++r) dst[hs_row<L, true, RA>(j, r)] = make_float2(-sc * u[r].y, sc * u[r].x);
             }
             __syncthreads();
         }
@@ -450,6 +465,7 @@ struct X2 {
     static constexpr int RA = F2<n>::R1, RB = F2<n>::R2;
     static constexpr int TA = 8 * n / RA, TB = 8 * n / RB, T = TA > TB ? TA : TB;
     static constexpr size_t SMEM = sizeof(float2) * (size_t)Xch<n, RA>::SIZE + sizeof(Tw2);
+    static constexpr bool SPLIT = n != 256;   // forward: the half spectrum inside stage B (see k2_fx_fwd)
     // inverse: plus a dense [8][n] staging buffer for the cp.async prefetch of the rows
     static constexpr size_t SMEM_INV = SMEM + sizeof(float2) * 8 * (size_t)n;
 };
@@ -499,12 +515,13 @@ __global__ void __launch_bounds__(X2<n>::T) k2_fx_fwd(const void* __restrict__ i
             for (int r = 0; r < RA; ++r) xb[Xch<n, RA>::at(c, j * RA + r)] = v[r];
         }
         __syncthreads();
-        // The half spectrum X[k] from Z[k] and Z[n-k]: inside stage B for n >= 512 (partner values by
-        // warp shuffle; one barrier and one shared round trip fewer, measured 3.8 -> 3.4 ms at
-        // n = 512), or in a separate loop over the exchange buffer (measured faster at n = 256).
-        if constexpr (RB == 32) {
+        // The half spectrum X[k] from Z[k] and Z[n-k]: inside stage B (partner values by warp shuffle;
+        // one barrier and one shared round trip fewer: 3.8 -> 3.4 ms at n = 512, 437 -> 182 us at n = 192 with
+        // the blocked layout), or in a separate loop over the exchange buffer (n = 256, where the step of 512^3
+        // takes 3.86 ms that way and 4.22 ms this).
+        if constexpr (X::SPLIT) {
             if (tid < X::TB) {   // stage B: Z[j + RA r], then X[k] for the same k = j + RA r
-                static_assert(RA == 16 || RA == 32, "the partner of a task must be in its warp");
+                static_assert(32 % RA == 0 && X::TB % 32 == 0, "the partner of a task must be in its warp");
                 const int c = tid / RA, j = tid % RA;
                 float2 v[RB];
                 stage_b<n, RA, RB, -1>(xb, tws, c, j, v);

@@ -475,6 +475,8 @@ __global__ void __launch_bounds__(TCfg<L>::T) k_fz(float2* __restrict__ in, ZOut
     }
 }
 
+// Meshes whose passes all have a two-stage plan (N and N / 2): they can use the blocked layout.
+#define COLAPM_FOR_BLOCKED_SIZES(X) X(64) X(96) X(128) X(160) X(192) X(256) X(320) X(384) X(512) X(1024)
 #define COLAPM_FOR_MESH_SIZES(X) X(16) X(32) X(64) X(96) X(128) X(160) X(192) X(256) X(320) X(384) X(512) X(1024)
 
 }  // namespace colapm

@@ -57,8 +57,9 @@ static cudaError_t fy_force_t(float2* data, size_t fstride, const float2* tw, cu
 
 cudaError_t launch_fy_force(int n_mesh, float2* data, size_t field_stride, const float2* tw, cudaStream_t s) {
     switch (n_mesh) {
-        case 512: return fy_force_t<512>(data, field_stride, tw, s);
-        case 1024: return fy_force_t<1024>(data, field_stride, tw, s);
+#define X(N) case N: return fy_force_t<N>(data, field_stride, tw, s);
+        COLAPM_FOR_BLOCKED_SIZES(X)
+#undef X
         default: return cudaErrorInvalidValue;
     }
 }

@@ -31,8 +31,8 @@ static cudaError_t fz2(float2* in, ZOut out, const float2* tw, const float* sinc
         // Blocked layout: 4-column tiles (32-byte rows whose 512-byte runs the neighbouring tiles
         // complete), which with the prefetch buffer measured 2% faster than 8-column ones (34% for the
         // power spectrum), and with direct loads fit three CTAs per SM. Standard layout: 8 columns
-        // (4-column rows there are 32 bytes 4 MB apart).
-        constexpr int CZ = BLK ? 4 : 8;
+        // (4-column rows there are 32 bytes 4 MB apart). Below 256, 8 columns too: enough threads per CTA.
+        constexpr int CZ = BLK && N >= 256 ? 4 : 8;
         constexpr bool DIRECT = BLK;   // blocked layout: loads straight into registers, three CTAs per SM
         using Z = Z2<N, MODE, CZ, DIRECT>;
         const size_t smem = Z::SMEM + (MODE == Z_POWER ? (size_t)pw.nbins * 24 + (size_t)(pw.nbins + 1) * 4 : 0);
