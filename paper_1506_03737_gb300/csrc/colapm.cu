@@ -68,7 +68,7 @@ struct colapm_ctx {
                                          // 8 internal (a sort slot out of range)
     // power-spectrum tables (grown on demand)
     int* pw_bin = nullptr;               // |n|^2 thresholds of the bins
-    double* pw_acc = nullptr;            // ksum[nb], psum[nb], cnt[nb] (as u64)
+    double* pw_acc = nullptr;            // ksum[nb], psum[nb], cnt[nb] (as u64), then the partial sums (power_layout)
     int pw_n2cap = 0, pw_nbcap = 0;
     float pw_lga = 0.0f, pw_lgb = 0.0f;  // log-spacing guess of the bins (PowerArgs)
     unsigned long long* d_seed = nullptr;          // device seed of the Gaussian field
@@ -710,7 +710,7 @@ int power_prepare(colapm_ctx* c, int nbins, double kmin, double kmax) {
     if (nbins > c->pw_nbcap) {
         if (c->pw_acc) cudaFree(c->pw_acc);
         c->pw_acc = nullptr;
-        if (dalloc(&c->pw_acc, (size_t)3 * nbins) != cudaSuccess) {
+        if (dalloc(&c->pw_acc, power_words(nbins, kPowerRegions)) != cudaSuccess) {
             c->pw_nbcap = 0;
             return COLAPM_E_NOMEM;
         }
@@ -737,7 +737,7 @@ int power_enqueue(colapm_ctx* c, int nbins, const DepositSrc* src = nullptr, boo
     const double box = c->prm.box;
     Phase ph(c, COLAPM_PHASE_POWER);   // all of P(k), its deposit and forward passes included
     PhaseMute mute(c);
-    CK(cudaMemsetAsync(c->pw_acc, 0, (size_t)3 * nbins * sizeof(double), c->stream));
+    CK(cudaMemsetAsync(c->pw_acc, 0, power_words(nbins, kPowerRegions) * sizeof(double), c->stream));
     int r = deposit(c, src);
     if (r) return r;
     r = density_xy(c);
@@ -745,10 +745,7 @@ int power_enqueue(colapm_ctx* c, int nbins, const DepositSrc* src = nullptr, boo
     PowerArgs pw{};
     pw.n2_lo = c->pw_bin;
     pw.kf = (float)(2.0 * M_PI / box);
-    pw.ksum = c->pw_acc;
-    pw.psum = c->pw_acc + nbins;
-    pw.cnt = reinterpret_cast<unsigned long long*>(c->pw_acc + 2 * nbins);
-    pw.nbins = nbins;
+    power_layout(pw, c->pw_acc, nbins, kPowerRegions);
     const double nm = c->nm;
     pw.pnorm = (float)(box * box * box / (nm * nm * nm * nm * nm * nm));
     pw.lga = c->pw_lga;

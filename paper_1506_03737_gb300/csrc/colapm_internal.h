@@ -47,10 +47,27 @@ struct PowerArgs {
     int nbins;
     float kf;                   // 2 pi / L (h/Mpc)
     float pnorm;                // L^3 / N^6
+    double* part;               // [regions][3 nbins] partial sums (k, P, count as u64) of the two-stage z pass, zeroed
+    unsigned* done;             // CTAs of that pass that have finished, zeroed
+    int regions;                // a power of two
     // first guess of the bin of |n|^2 for log-spaced bins, floor(lga log2 |n|^2 + lgb), corrected
     // against n2_lo (lga = 0: binary search only)
     float lga, lgb;
 };
+
+constexpr int kPowerRegions = 16;   // 64 cost up to 8 us more in the final sum and gained nothing
+// FP64 words of the accumulators of `nbins` bins: the result [3 nbins], the regions, the counter.
+__host__ __device__ constexpr size_t power_words(int nbins, int regions) { return (size_t)3 * nbins * (1 + regions) + 1; }
+// PowerArgs' accumulator pointers into such an array (all zero at the start of a pass).
+inline void power_layout(PowerArgs& pw, double* acc, int nbins, int regions) {
+    pw.ksum = acc;
+    pw.psum = acc + nbins;
+    pw.cnt = reinterpret_cast<unsigned long long*>(acc + 2 * nbins);
+    pw.part = acc + 3 * (size_t)nbins;
+    pw.done = reinterpret_cast<unsigned*>(acc + (size_t)3 * nbins * (1 + regions));
+    pw.regions = regions;
+    pw.nbins = nbins;
+}
 
 // Guess from the log-spacing of the bins (at most one or two off near an edge), then a walk to
 // the bin whose thresholds hold |n|^2; -1 outside. The same bin as the binary search.
@@ -75,11 +92,40 @@ __device__ __forceinline__ int power_bin(int n2, const int* lo, int nbins) {
     return a;
 }
 
+// Walks the bins upward along modes of growing |n|^2. thr: the thresholds lo[0 .. nbins], then INT_MAX twice;
+// e: the next threshold, so the bin is e - 1 (0: below every bin, nbins + 1: above). The threshold after it is
+// held too: a lane that leaves its bin does a compare and a load that nothing waits for, which matters
+// because the lanes of a warp leave theirs at different modes (a search there cost more than the rest).
+struct BinWalk {
+    const int* thr;
+    int e, hi, next;
+    __device__ __forceinline__ void start(int n2, const int* t, const PowerArgs& pw) {
+        thr = t;
+        if (n2 < t[0]) e = 0;
+        else if (n2 >= t[pw.nbins]) e = pw.nbins + 1;
+        else e = 1 + (pw.lga != 0.0f && n2 ? power_bin_guess(n2, t, pw) : power_bin(n2, t, pw.nbins));
+        hi = t[e];
+        next = t[min(e + 1, pw.nbins + 1)];
+    }
+    __device__ __forceinline__ bool leaves(int n2) const { return n2 >= hi; }
+    __device__ __forceinline__ void advance(int n2, int nbins) {
+        do {
+            ++e;
+            hi = next;
+            next = thr[min(e + 1, nbins + 1)];
+        } while (n2 >= hi);
+    }
+    __device__ __forceinline__ int bin(int nbins) const { return e > nbins ? -1 : e - 1; }   // -1: outside every bin
+};
+__device__ __forceinline__ void load_thresholds(int* thr, const PowerArgs& pw, int tid, int threads) {
+    for (int b = tid; b < pw.nbins + 3; b += threads) thr[b] = b <= pw.nbins ? pw.n2_lo[b] : 0x7fffffff;
+}
+
 // Bins the modes (nx, ny, nz(z)) of one column for z = z0 ... z0 + per - 1 (ny not on the Nyquist
 // plane; z = L/2 skipped) into the FP64 bins: FP32 sums over runs of consecutive modes in one bin
 // (a few dozen at most), added to the bin when the run leaves it. The current bin's |n|^2 range
 // stays in registers, so a mode of the same bin costs two compares; a new bin comes from the
-// log-spacing guess (power_bin_guess) or the binary search. value(z) gives the mode's complex
+// log-spacing guess (power_bin_guess) or the binary search. Used by the Stockham z pass. value(z) gives the mode's complex
 // amplitude, sinc2[z] the CIC window factor along z (wxy the product of the x and y factors).
 template <typename F>
 __device__ __forceinline__ void bin_column_run(int nx, int ny, int z0, int per, int L, float wxy,

@@ -202,6 +202,12 @@ struct Z2 {
     static constexpr int PF = PREFETCH ? C * L : 0;                               // dense [z][C] buffer
     static constexpr int TA = C * L / R1, TB = C * L / R2, T = TA > TB ? TA : TB;
     static constexpr size_t SMEM = sizeof(float2) * ((size_t)XS * (1 + NSAVE) + PF) + sizeof(Tw2);
+    // Z_POWER: |X|^2 of the tile, C lines of L floats; a thread bins PER z of one line and their mirror
+    // images L - z. One word of padding per PER and a pitch of 32 / C (mod 32) put the reads of a
+    // warp on 32 banks. Then the table 1 / sinc^4 of the window along z.
+    static constexpr int PER = L * C / (2 * T), PP = ((L + L / PER + 31) / 32) * 32 + 32 / C;
+    static_assert(MODE != Z_POWER || (PER * T * 2 == L * C && L % PER == 0), "the runs must cover the tile");
+    static constexpr size_t SMEM_POWER = SMEM + sizeof(float) * ((size_t)C * PP + L / 2);
     // CTAs per SM: 12 warps where a task holds 32 values, 20 (at most 102 registers) with the smaller radices
     static constexpr int MINB = DIRECT ? (R1 == 32 || R2 == 32 ? 384 / T : 640 / T) : 1;
 };
@@ -218,18 +224,18 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
     float2* save = xb + Z::XS;                                   // bases B (, C), layout Xch<L,R1>
     float2* pf = xb + Z::XS * (1 + Z::NSAVE);                    // prefetched input tile [z][8]
     Tw2* tws = reinterpret_cast<Tw2*>(pf + Z::PF);
-    double* ksum = reinterpret_cast<double*>(tws + 1);
-    double* psum = ksum + pw.nbins;
-    unsigned long long* cnt = reinterpret_cast<unsigned long long*>(psum + pw.nbins);
-    int* lo = reinterpret_cast<int*>(cnt + pw.nbins);
+    float* pbuf = reinterpret_cast<float*>(tws + 1);             // Z_POWER: [C][PP], then the window table, then the thresholds
+    float* iw2 = pbuf + (MODE == Z_POWER ? C * Z::PP : 0);
+    int* lo = reinterpret_cast<int*>(iw2 + (MODE == Z_POWER ? L / 2 : 0));
     load_tw2<L, L>(tws, tw, T);
+    double* part = nullptr;                                      // Z_POWER: the sums this CTA adds to
     if constexpr (MODE == Z_POWER) {
-        for (int b = threadIdx.x; b < pw.nbins; b += T) {
-            ksum[b] = 0.0;
-            psum[b] = 0.0;
-            cnt[b] = 0ull;
+        load_thresholds(lo, pw, threadIdx.x, T);
+        for (int z = threadIdx.x; z < L / 2; z += T) {
+            const float s2 = sinc2[z];
+            iw2[z] = 1.0f / (s2 * s2);
         }
-        for (int b = threadIdx.x; b <= pw.nbins; b += T) lo[b] = pw.n2_lo[b];
+        part = pw.part + (size_t)(blockIdx.x & (pw.regions - 1)) * 3 * pw.nbins;
     }
     __syncthreads();
     const float kf = 6.283185307179586f / (float)L;
@@ -303,20 +309,60 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
         }
 
         if constexpr (MODE == Z_POWER) {
-            // Store the spectrum of the C columns in z order, then bin runs of consecutive z.
+            // |X|^2 of the C columns in z order, then runs of consecutive z, each with its mirror image L - z (the
+            // same |n| and window), into the bins: FP32 sums of at most 2 PER modes, then one reduction each in
+            // L2 (fire and forget; shared-memory FP64 atomics are retry loops on which the lanes of a warp
+            // collide), over 16 copies of the bins. What bounded the binning was the search for the next bin,
+            // which the lanes of a warp reach at different modes (BinWalk), and a square root and a division
+            // per mode. At 64^3, 128^3, 512^3 and 1024^3 with 32 to 100 bins the pass took 17, 42, 717 and 5171 us
+            // and takes 9, 16, 290 and 1978 us. Counting the modes apart, over 1/48 of the grid, took 460 us
+            // at 1024^3: the loops were too few and too long. The next tile's stage A only touches the
+            // exchange buffer, and the barrier after it separates this tile's reads from the next tile's values.
             if (tid < TB) {
 #pragma unroll
-                for (int r = 0; r < R2; ++r) xb[Xch<L, R1, C>::at(c, j + R1 * r)] = v[r];
+                for (int r = 0; r < R2; ++r) {
+                    const int z = j + R1 * r;
+                    pbuf[c * Z::PP + z + z / Z::PER] = fmaf(v[r].x, v[r].x, v[r].y * v[r].y);
+                }
             }
             __syncthreads();
-
-            if (!nyq_y) {   // each thread a run of consecutive z of one column
-                constexpr int PER = L * C / T;
-                const int pc = tid % C;
-                bin_column_run(kx0 + pc, ny, (tid / C) * PER, PER, L, sinc2[kx0 + pc] * sinc2[ky], sinc2, lo, pw, psum,
-                               ksum, cnt, [&](int z) { return xb[Xch<L, R1, C>::at(pc, z)]; });
+            if (!nyq_y) {
+                const float wxy = sinc2[nx] * sinc2[ky];
+                const float cf = __fdividef(nx == 0 ? pw.pnorm : 2.0f * pw.pnorm, wxy * wxy);
+                const float ck = nx == 0 ? pw.kf : 2.0f * pw.kf;
+                const int nxy2 = nx * nx + ny * ny, z0 = j * Z::PER;
+                const float* p = pbuf + c * Z::PP;
+                double* psum = part + pw.nbins;
+                unsigned long long* cnt = reinterpret_cast<unsigned long long*>(part + 2 * pw.nbins);
+                BinWalk w;
+                w.start(nxy2 + z0 * z0, lo, pw);
+                float acc = 0.0f, ks = 0.0f;
+                unsigned modes = 0;
+                auto flush = [&]() {
+                    const int b = w.bin(pw.nbins);
+                    if (b >= 0) {
+                        atomicAdd(&part[b], (double)(ks * ck));
+                        atomicAdd(&psum[b], (double)(acc * cf));
+                        atomicAdd(&cnt[b], (unsigned long long)(nx == 0 ? modes : 2 * modes));
+                    }
+                    acc = 0.0f;
+                    ks = 0.0f;
+                    modes = 0;
+                };
+#pragma unroll
+                for (int zz = 0; zz < Z::PER; ++zz) {
+                    const int z = z0 + zz, m = L - z, n2 = nxy2 + z * z;
+                    const float s = p[z + z / Z::PER] + (z ? p[m + m / Z::PER] : 0.0f);
+                    if (w.leaves(n2)) {   // the run leaves its bin
+                        flush();
+                        w.advance(n2, pw.nbins);
+                    }
+                    acc = fmaf(s, iw2[z], acc);
+                    ks = fmaf(z ? 2.0f : 1.0f, sqrtf((float)n2), ks);
+                    modes += z ? 2 : 1;
+                }
+                flush();
             }
-            __syncthreads();
             continue;
         } else {
             // bases: A = g X, B = k_z A (, C = k_z^2 A); g = gnorm / (k^2 [W^d]), 0 on excluded modes
@@ -393,13 +439,26 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
         }
     }
     if constexpr (MODE == Z_POWER) {
+        // the CTA that finishes last adds up the regions (in their order) into the result
+        __shared__ unsigned last;
+        __threadfence();
         __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(pw.done, 1u) == gridDim.x - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        for (int b = threadIdx.x; b < 2 * pw.nbins; b += T) {
+            double s = 0.0;
+#pragma unroll 16
+            for (int r = 0; r < pw.regions; ++r) s += __ldcg(pw.part + (size_t)r * 3 * pw.nbins + b);
+            (b < pw.nbins ? pw.ksum : pw.psum - pw.nbins)[b] = s;
+        }
         for (int b = threadIdx.x; b < pw.nbins; b += T) {
-            if (cnt[b]) {
-                atomicAdd(&pw.psum[b], psum[b]);
-                atomicAdd(&pw.ksum[b], ksum[b]);
-                atomicAdd(&pw.cnt[b], cnt[b]);
-            }
+            unsigned long long s = 0;
+#pragma unroll 16
+            for (int r = 0; r < pw.regions; ++r)
+                s += __ldcg(reinterpret_cast<const unsigned long long*>(pw.part + (size_t)r * 3 * pw.nbins + 2 * pw.nbins + b));
+            pw.cnt[b] = s;
         }
     }
 }

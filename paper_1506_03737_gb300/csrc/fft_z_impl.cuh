@@ -35,7 +35,7 @@ static cudaError_t fz2(float2* in, ZOut out, const float2* tw, const float* sinc
         constexpr int CZ = BLK && N >= 256 ? 4 : 8;
         constexpr bool DIRECT = BLK;   // blocked layout: loads straight into registers, three CTAs per SM
         using Z = Z2<N, MODE, CZ, DIRECT>;
-        const size_t smem = Z::SMEM + (MODE == Z_POWER ? (size_t)pw.nbins * 24 + (size_t)(pw.nbins + 1) * 4 : 0);
+        const size_t smem = MODE == Z_POWER ? Z::SMEM_POWER + (size_t)(pw.nbins + 3) * 4 : Z::SMEM;
         static GridCache cache;
         int grid2 = 0;
         cudaError_t e = cached_grid(cache, k2_fz<N, MODE, CZ, BLK, DIRECT>, Z::T, smem, &grid2);

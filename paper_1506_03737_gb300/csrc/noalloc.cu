@@ -29,8 +29,8 @@ constexpr size_t kTw = align256(kSpec + sizeof(float2) * kMaxNm * kMaxNm * kMaxN
 constexpr size_t kSinc = align256(kTw + sizeof(float2) * kMaxNm);                  // float [nm]
 constexpr size_t kEdges = align256(kSinc + sizeof(float) * kMaxNm);                // double [nbins + 1]
 constexpr size_t kBin = align256(kEdges + sizeof(double) * (kMaxBins + 1));        // int [nbins + 1] thresholds
-constexpr size_t kAcc = align256(kBin + sizeof(int) * (kMaxBins + 1));             // double [3 nbins]
-constexpr size_t kOut = align256(kAcc + sizeof(double) * 3 * kMaxBins);            // k, P (double), n (i64)
+constexpr size_t kAcc = align256(kBin + sizeof(int) * (kMaxBins + 1));             // double [power_words(nbins, kPowerRegions)]
+constexpr size_t kOut = align256(kAcc + sizeof(double) * power_words(kMaxBins, kPowerRegions));            // k, P (double), n (i64)
 constexpr size_t kErr = align256(kOut + sizeof(double) * 3 * kMaxBins);            // int [4]
 constexpr size_t kBytes = align256(kErr + 4 * sizeof(int));
 
@@ -181,7 +181,7 @@ extern "C" int colapm_power_noalloc(const int* cell, const float* offset, long l
     NCK(cudaMemcpyAsync(sinc2, h_s2, sizeof(float) * nm, cudaMemcpyHostToDevice, s));
     NCK(cudaMemcpyAsync(edges, h_edges, sizeof(double) * (nbins + 1), cudaMemcpyHostToDevice, s));
     NCK(cudaMemsetAsync(rho, 0, sizeof(unsigned long long) * nm3, s));
-    NCK(cudaMemsetAsync(acc, 0, sizeof(double) * 3 * nbins, s));
+    NCK(cudaMemsetAsync(acc, 0, sizeof(double) * power_words(nbins, kPowerRegions), s));
     NCK(cudaMemsetAsync(err, 0, 4 * sizeof(int), s));
     k_bin_thresholds<<<(nbins + 128) / 128, 128, 0, s>>>(edges, nbins, kf, n2max, bin);
     NCK(cudaGetLastError());
@@ -193,10 +193,7 @@ extern "C" int colapm_power_noalloc(const int* cell, const float* offset, long l
     PowerArgs pw{};
     pw.n2_lo = bin;
     pw.kf = (float)kf;
-    pw.ksum = acc;
-    pw.psum = acc + nbins;
-    pw.cnt = reinterpret_cast<unsigned long long*>(acc + 2 * nbins);
-    pw.nbins = nbins;
+    power_layout(pw, acc, nbins, kPowerRegions);
     pw.pnorm = (float)(box * box * box / ((double)nm3 * (double)nm3));
     pw.lga = (float)(0.5 * nbins / std::log2(h_edges[nbins] / h_edges[0]));
     pw.lgb = (float)(nbins * std::log2(kf / h_edges[0]) / std::log2(h_edges[nbins] / h_edges[0]));
