@@ -392,9 +392,8 @@ void lightcone_free(colapm_ctx* c) {
 int place_particles(colapm_ctx* c, float to_mesh) {
     const Growth& g = c->table.g[0];
     if (c->lc_on) CK(cudaMemsetAsync(c->lc_count, 0, sizeof(unsigned long long), c->stream));   // a new run
-    CKL(launch_iota(c->id, c->np3, c->stream));
     c->id_order = true;
-    CKL(launch_init_particles(c->pos, c->mom, c->psi1, c->psi2, c->np, c->nm, to_mesh, (float)g.d1, (float)g.d2,
+    CKL(launch_init_particles(c->pos, c->mom, c->id, c->psi1, c->psi2, c->np, c->nm, to_mesh, (float)g.d1, (float)g.d2,
                              (float)g.p1, (float)g.p2, c->prm.cola, c->stream));
     c->step = 0;
     c->has_ics = true;
@@ -597,6 +596,7 @@ int colapm_make_ics(colapm_ctx* c) {
     if (c->seed_src == c->d_seed) CKL(launch_set_u64(c->d_seed, c->prm.seed, c->stream));
     if (int r = initial_field(c, dk, phi)) return r;
     ZOut o1{};
+    o1.vscale = (float)c->nm / np;   // the displacements in PM-mesh cells
     for (int j = 0; j < 3; ++j) o1.p[j] = p1 + j * hs;
     for (int j = 0; j < 6; ++j) o1.p[3 + j] = phi + j * hs;
     CKL(launch_fz(np, Z_LPT1, dk, o1, c->tw_p, nullptr, 0, gnorm, nullptr, c->stream, ts(c, COLAPM_PLAN_Z)));
@@ -609,11 +609,12 @@ int colapm_make_ics(colapm_ctx* c) {
     CKL(launch_fx_fwd_f32(np, c->scratch, phi, c->tw_p, c->stream, ts(c, COLAPM_PLAN_XF)));
     CKL(launch_fy(np, -1, phi, 0, 1, c->tw_p, c->stream, ts(c, COLAPM_PLAN_Y)));
     ZOut o2{};
+    o2.vscale = o1.vscale;
     for (int j = 0; j < 3; ++j) o2.p[j] = p2 + j * hs;
     CKL(launch_fz(np, Z_LPT2, phi, o2, c->tw_p, nullptr, 0, gnorm, nullptr, c->stream, ts(c, COLAPM_PLAN_Z)));
     CKL(launch_fy(np, +1, p2, hs, 3, c->tw_p, c->stream, ts(c, COLAPM_PLAN_Y)));
     CKL(launch_fx_inv(np, p2, hs, 3, c->tw_p, c->stream, ts(c, COLAPM_PLAN_XI)));
-    return place_particles(c, (float)c->nm / np);
+    return place_particles(c, 1.0f);
 }
 
 int colapm_set_displacements(colapm_ctx* c, const float* psi1, const float* psi2) {
@@ -994,15 +995,13 @@ int colapm_get_lpt(colapm_ctx* c, float* psi1, float* psi2) {
     if (int r = id_order(c)) return r;
     const float f = (float)(c->prm.box / c->nm);
     const size_t n = 3 * c->np3;
-    if (psi1) {
-        CKL(launch_scale(c->scratch, c->psi1, n, f, c->stream));
-        copy_out(c, psi1, c->scratch, n * sizeof(float));
-        CK(cudaStreamSynchronize(c->stream));
-    }
-    if (psi2) {
-        CKL(launch_scale(c->scratch, c->psi2, n, f, c->stream));
-        copy_out(c, psi2, c->scratch, n * sizeof(float));
-    }
+    // straight into a device array; through two parts of the scratch into a host one
+    float* d1 = psi1 && !is_device_ptr(psi1) ? c->scratch : psi1;
+    float* d2 = psi2 && !is_device_ptr(psi2) ? c->scratch + n : psi2;
+    if (psi1) CKL(launch_scale(d1, c->psi1, n, f, c->stream));
+    if (psi2) CKL(launch_scale(d2, c->psi2, n, f, c->stream));
+    if (psi1 && d1 != psi1) copy_out(c, psi1, d1, n * sizeof(float));
+    if (psi2 && d2 != psi2) copy_out(c, psi2, d2, n * sizeof(float));
     return pending_error(c);
 }
 
@@ -1553,7 +1552,7 @@ int batch_enqueue_lockstep(colapm_batch* b, int K) {
             w.rho = c->rho;
             w.np3 = c->np3;
             w.first = items;
-            w.nm = c->nm;
+            w.u = make_udiv(c->nm);
             w.k = coef_for(c, st);
             wh[m++] = w;
             items += multi_items(c->np3);

@@ -23,7 +23,72 @@ struct StepCoef {
 // Output pointers of a z pass (up to 9 spectra: 3 x Psi1 and 6 x phi_ij of the ICs).
 struct ZOut {
     float2* p[9];
+    float vscale = 1.0f;   // factor of the vector outputs (LPT modes: the displacements, e.g. in another cell size)
 };
+
+// Division of any 32-bit n by d >= 2 as a multiplication (Granlund & Montgomery, "Division by invariant integers
+// using multiplication", 1994, Fig. 4.1): with l = ceil(log2 d) and magic = floor(2^32 (2^l - d) / d) + 1, the
+// quotient is (t + ((n - t) >> 1)) >> (l - 1), t the high word of magic n. No branch: one in the gather (an
+// ordinary division for words of a corrupt state) cost a quarter of its speed.
+struct UDiv {
+    unsigned d = 0, magic = 0;
+    int s = 0;   // l - 1
+    __host__ __device__ __forceinline__ unsigned div(unsigned n) const {
+#ifdef __CUDA_ARCH__
+        const unsigned t = __umulhi(n, magic);
+#else
+        const unsigned t = (unsigned)(((unsigned long long)n * magic) >> 32);
+#endif
+        return (t + ((n - t) >> 1)) >> s;
+    }
+    __host__ __device__ __forceinline__ unsigned mod(unsigned n) const { return n - div(n) * d; }
+    // n = x + d (y + d z), z reduced modulo d
+    __host__ __device__ __forceinline__ void split(unsigned n, int& x, int& y, int& z) const {
+        const unsigned q = div(n), r = div(q);
+        x = (int)(n - q * d);
+        y = (int)(q - r * d);
+        z = (int)mod(r);
+    }
+    // c wrapped into [0, d): for c < 0, c = -(a + 1) wraps to d - 1 - a mod d
+    __host__ __device__ __forceinline__ int wrap(int c) const {
+        const int sign = c >> 31;
+        const int x = (int)mod((unsigned)(c ^ sign));
+        return sign ? (int)d - 1 - x : x;
+    }
+};
+inline UDiv make_udiv(int d) {
+    UDiv u;
+    u.d = (unsigned)d;
+    int l = 1;
+    while ((1 << l) < d) ++l;
+    u.s = l - 1;
+    u.magic = (unsigned)((((1ull << l) - (unsigned)d) << 32) / (unsigned)d + 1);
+    return u;
+}
+
+// Site i of the Lagrangian lattice sits at mesh coordinate i nm / np + 1/2 (spacing L / np, offset by
+// half a PM cell): i nm / np = (i mul) / 2^shift, with shift > 0 for the coarse meshes np = 2 nm, 4 nm only.
+struct Lattice {
+    UDiv np, nm;
+    int mul, shift;
+    float inv;   // 2^-shift
+    __host__ __device__ __forceinline__ void site(unsigned p, int* c) const { np.split(p, c[0], c[1], c[2]); }
+    // integer part of site i's mesh coordinate less 1/2, and its exact fractional remainder
+    __host__ __device__ __forceinline__ void at(int i, int& base, float& frac) const {
+        const int t = i * mul;
+        base = t >> shift;
+        frac = (float)(t & ((1 << shift) - 1)) * inv;
+    }
+};
+inline Lattice make_lattice(int np, int nm) {
+    Lattice l;
+    l.np = make_udiv(np);
+    l.nm = make_udiv(nm);
+    l.mul = nm >= np ? nm / np : 1;
+    l.shift = nm >= np ? 0 : (np == 2 * nm ? 1 : 2);
+    l.inv = 1.0f / (float)(1 << l.shift);
+    return l;
+}
 
 enum ZMode {
     Z_FORCE = 0,   // forward z, F_j = i k_j delta / (k^2 W^d) / N^3, inverse z, 3 outputs
@@ -235,7 +300,7 @@ struct MockWork {
     unsigned long long* rho;
     size_t np3;
     long long first;
-    int nm;
+    UDiv u;      // of the mesh side
     StepCoef k;
 };
 
@@ -252,7 +317,8 @@ cudaError_t launch_deposit(const float4* pos, size_t np3, int nm, unsigned long 
 cudaError_t launch_gather_kick_drift(float4* pos, float* mom, const float* psi1, const float* psi2,
                                      const float* force, size_t np3, int nm, StepCoef c, int drift,
                                      cudaStream_t s, int block = 256, const LightconeStep* lc = nullptr);
-cudaError_t launch_init_particles(float4* pos, float* mom, float* psi1, float* psi2, int np, int nm,
+// Particle p gets id p; psi1 / psi2 are rewritten only where to_mesh is not 1.
+cudaError_t launch_init_particles(float4* pos, float* mom, int* id, float* psi1, float* psi2, int np, int nm,
                                   float to_mesh, float d1, float d2, float p1, float p2, int cola,
                                   cudaStream_t s);
 cudaError_t launch_add_lpt_momentum(float* mom, const float* psi1, const float* psi2, size_t np3, float p1,

@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
             __syncthreads();   // forward exchange buffer free
             const float kyv = kf * (float)ny;
             const float kxv = kf * (float)nx;
-            constexpr float sg = MODE == Z_LPT2 ? -1.0f : 1.0f;
+            const float sg = MODE == Z_LPT2 ? -out.vscale : out.vscale;
             constexpr int NB = Z::NSAVE + 1;
 #pragma unroll 1
             for (int bi = 0; bi < NB; ++bi) {

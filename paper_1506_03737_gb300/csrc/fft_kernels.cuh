@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(TCfg<L>::T) k_fz(float2* __restrict__ in, ZOut
             if constexpr (Z::NBASE == 3) tile_fft<L, T, +1, L>(aux + TS, stw);
             const float kyv = kf * (float)ny;
             auto kxv = [&](int c) { return kf * (float)(kx0 + c); };
-            constexpr float sg = MODE == Z_LPT2 ? -1.0f : 1.0f;
+            const float sg = MODE == Z_LPT2 ? -out.vscale : out.vscale;
             st_cols_scaled<L, T, true>(cur, out.p[0] + base, stride, [&](int c) { return sg * kxv(c); });
             st_cols_scaled<L, T, true>(cur, out.p[1] + base, stride, [&](int) { return sg * kyv; });
             st_cols_scaled<L, T, true>(aux, out.p[2] + base, stride, [&](int) { return sg; });

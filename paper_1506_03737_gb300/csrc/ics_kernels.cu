@@ -41,41 +41,47 @@ __global__ void k_gaussian_field(int n, const unsigned long long* __restrict__ s
                                  float2* __restrict__ dk) {
     const unsigned long long seed = *seedp;
     const int h = n / 2;
-    const size_t total = (size_t)n * n * h;
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= total) return;
-    const int ix = (int)(t % h), iy = (int)((t / h) % n), iz = (int)(t / ((size_t)h * n));
-    float2 v = make_float2(0.0f, 0.0f);
-    if (iy != h && iz != h) {
-        const int nx = ix, ny = iy < h ? iy : iy - n, nz = iz < h ? iz : iz - n;
-        const int n2 = nx * nx + ny * ny + nz * nz;
-        if (n2 > 0) {
-            const unsigned long long m = ((unsigned long long)iz * n + iy) * n + ix;
-            unsigned long long src = m;
-            bool conj = false;
-            if (ix == 0) {   // the larger full-grid index of each conjugate pair mirrors its partner
-                const unsigned long long part = ((unsigned long long)((n - iz) % n) * n + (n - iy) % n) * n;
-                if (m > part) {
-                    src = part;
-                    conj = true;
+    // a row of modes per row of threads: no index division (with 64-bit ones the pass took 79 us at 256^3, 63 now)
+    const int iy = blockIdx.x * blockDim.y + threadIdx.y, iz = blockIdx.y;
+    if (iy >= n) return;
+    for (int ix = threadIdx.x; ix < h; ix += blockDim.x) {
+        const size_t t = ((size_t)iz * n + iy) * h + ix;
+        float2 v = make_float2(0.0f, 0.0f);
+        if (iy != h && iz != h) {
+            const int nx = ix, ny = iy < h ? iy : iy - n, nz = iz < h ? iz : iz - n;
+            const int n2 = nx * nx + ny * ny + nz * nz;
+            if (n2 > 0) {
+                const unsigned long long m = ((unsigned long long)iz * n + iy) * n + ix;
+                unsigned long long src = m;
+                bool conj = false;
+                if (ix == 0) {   // the larger full-grid index of each conjugate pair mirrors its partner
+                    const unsigned long long part = ((unsigned long long)(iz ? n - iz : 0) * n + (iy ? n - iy : 0)) * n;
+                    if (m > part) {
+                        src = part;
+                        conj = true;
+                    }
                 }
+                const float2 g = draw(src, seed);
+                const float a = amp_of_n2[n2];
+                v = make_float2(a * g.x, conj ? -a * g.y : a * g.y);
             }
-            const float2 g = draw(src, seed);
-            const float a = amp_of_n2[n2];
-            v = make_float2(a * g.x, conj ? -a * g.y : a * g.y);
         }
+        dk[t] = v;
     }
-    dk[t] = v;
 }
 
 // S = phi_xx phi_yy + phi_xx phi_zz + phi_yy phi_zz - phi_xy^2 - phi_xz^2 - phi_yz^2
 // (the right-hand side of the phi2 Poisson equation, §2.1); phi = [xx, yy, zz, xy, xz, yz].
-__global__ void k_lpt2_source(const float* __restrict__ phi, size_t n3, float* __restrict__ src) {
+__global__ void k_lpt2_source(const float4* __restrict__ phi, size_t n4, float4* __restrict__ src) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n3) return;
-    const float xx = phi[i], yy = phi[n3 + i], zz = phi[2 * n3 + i];
-    const float xy = phi[3 * n3 + i], xz = phi[4 * n3 + i], yz = phi[5 * n3 + i];
-    src[i] = xx * yy + xx * zz + yy * zz - xy * xy - xz * xz - yz * yz;
+    if (i >= n4) return;
+    const float4 xx = __ldcs(phi + i), yy = __ldcs(phi + n4 + i), zz = __ldcs(phi + 2 * n4 + i);
+    const float4 xy = __ldcs(phi + 3 * n4 + i), xz = __ldcs(phi + 4 * n4 + i), yz = __ldcs(phi + 5 * n4 + i);
+    auto s = [](float xx, float yy, float zz, float xy, float xz, float yz) {
+        return xx * yy + xx * zz + yy * zz - xy * xy - xz * xz - yz * yz;
+    };
+    src[i] = make_float4(s(xx.x, yy.x, zz.x, xy.x, xz.x, yz.x), s(xx.y, yy.y, zz.y, xy.y, xz.y, yz.y),
+                         s(xx.z, yy.z, zz.z, xy.z, xz.z, yz.z), s(xx.w, yy.w, zz.w, xy.w, xz.w, yz.w));
 }
 
 __global__ void k_set_u64(unsigned long long* dst, unsigned long long value) { *dst = value; }
@@ -119,13 +125,15 @@ cudaError_t launch_set_u64(unsigned long long* dst, unsigned long long value, cu
 
 cudaError_t launch_gaussian_field(int np, const unsigned long long* seed, const float* amp_of_n2, float2* dk,
                                   cudaStream_t s) {
-    const size_t total = (size_t)np * np * (np / 2);
-    k_gaussian_field<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(np, seed, amp_of_n2, dk);
+    const int bx = np / 2 < 256 ? np / 2 : 256, by = 256 / bx;   // np / 2 may not divide 256: fewer threads then
+    k_gaussian_field<<<dim3((np + by - 1) / by, np), dim3(bx, by), 0, s>>>(np, seed, amp_of_n2, dk);
     return cudaGetLastError();
 }
 
 cudaError_t launch_lpt2_source(const float* phi, size_t np3, float* src, cudaStream_t s) {
-    k_lpt2_source<<<(unsigned)((np3 + 255) / 256), 256, 0, s>>>(phi, np3, src);
+    const size_t n4 = np3 / 4;   // np is a multiple of 16
+    k_lpt2_source<<<(unsigned)((n4 + 255) / 256), 256, 0, s>>>(reinterpret_cast<const float4*>(phi), n4,
+                                                               reinterpret_cast<float4*>(src));
     return cudaGetLastError();
 }
 

@@ -22,10 +22,10 @@ struct Cic {
     int fx, fy, fz;
 };
 
-__device__ __forceinline__ Cic cic_setup(float4 P, int nm) {
-    const unsigned c = __float_as_uint(P.w);
-    const unsigned unm = (unsigned)nm;
-    int cx = (int)(c % unm), cy = (int)((c / unm) % unm), cz = (int)((c / (unm * unm)) % unm);
+__device__ __forceinline__ Cic cic_setup(float4 P, const UDiv& u) {
+    const int nm = (int)u.d;
+    int cx, cy, cz;
+    u.split(__float_as_uint(P.w), cx, cy, cz);
     int fx = __float2int_rn(P.x * 32768.0f), fy = __float2int_rn(P.y * 32768.0f), fz = __float2int_rn(P.z * 32768.0f);
     if (fx == QONE) { fx = 0; cx = cx + 1 == nm ? 0 : cx + 1; }
     if (fy == QONE) { fy = 0; cy = cy + 1 == nm ? 0 : cy + 1; }
@@ -42,9 +42,10 @@ __device__ __forceinline__ Cic cic_setup(float4 P, int nm) {
 // Two threads per particle, one per x corner (lane parity): the atomics of one warp instruction then
 // hit 16 particles x 2 neighbouring cells, which along the Lagrangian x rows are runs of consecutive
 // int64 cells (fully used 32-byte sectors), instead of every other cell of twice as many sectors.
-__device__ __forceinline__ void deposit_corner(const float4* __restrict__ pos, size_t p, int dx, int nm,
+__device__ __forceinline__ void deposit_corner(const float4* __restrict__ pos, size_t p, int dx, const UDiv& u,
                                                unsigned long long* __restrict__ rho) {
-    const Cic c = cic_setup(pos[p], nm);
+    const Cic c = cic_setup(pos[p], u);
+    const int nm = (int)u.d;
     const unsigned long long wx = (unsigned long long)(dx ? c.fx : QONE - c.fx);
     const unsigned long long wy[2] = {(unsigned long long)(QONE - c.fy), (unsigned long long)c.fy};
     const unsigned long long wz[2] = {(unsigned long long)(QONE - c.fz), (unsigned long long)c.fz};
@@ -58,11 +59,11 @@ __device__ __forceinline__ void deposit_corner(const float4* __restrict__ pos, s
         }
 }
 
-__global__ void k_deposit(const float4* __restrict__ pos, size_t np3, int nm, unsigned long long* __restrict__ rho) {
+__global__ void k_deposit(const float4* __restrict__ pos, size_t np3, UDiv u, unsigned long long* __restrict__ rho) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t p = t >> 1;
     if (p >= np3) return;
-    deposit_corner(pos, p, (int)(t & 1), nm, rho);
+    deposit_corner(pos, p, (int)(t & 1), u, rho);
 }
 
 // Tiled deposit of particles ordered by tile (a sort with the same tile shape): a CTA takes the
@@ -75,10 +76,11 @@ __global__ void k_deposit(const float4* __restrict__ pos, size_t np3, int nm, un
 constexpr int DT_T = 256;
 
 template <int TS>
-__global__ void __launch_bounds__(DT_T) k_deposit_tiles(const float4* __restrict__ pos, int nm, int xs,
+__global__ void __launch_bounds__(DT_T) k_deposit_tiles(const float4* __restrict__ pos, UDiv u, int xs,
                                                         const unsigned* __restrict__ ends, unsigned ntiles,
                                                         unsigned long long* __restrict__ rho) {
     constexpr int T = 1 << TS, RY = T + 1, RXMAX = 65;
+    const int nm = (int)u.d;
     __shared__ unsigned long long acc[RXMAX * RY * RY];
     const int RX = (1 << xs) + 1, NR = RX * RY * RY;
     const int nbx = nm >> xs, nty = nm >> TS;
@@ -93,7 +95,7 @@ __global__ void __launch_bounds__(DT_T) k_deposit_tiles(const float4* __restrict
         for (size_t slot = start * 2 + threadIdx.x; slot < end * 2; slot += DT_T) {
             const size_t p = slot >> 1;
             const int dx = (int)(slot & 1);
-            const Cic c = cic_setup(pos[p], nm);
+            const Cic c = cic_setup(pos[p], u);
             const unsigned long long wx = (unsigned long long)(dx ? c.fx : QONE - c.fx);
             const unsigned long long wy[2] = {(unsigned long long)(QONE - c.fy), (unsigned long long)c.fy};
             const unsigned long long wz[2] = {(unsigned long long)(QONE - c.fz), (unsigned long long)c.fz};
@@ -182,7 +184,7 @@ __device__ __forceinline__ void record_lightcone(const LightconeStep& lc, const 
 template <bool LC>
 __device__ __forceinline__ void gather_kick_drift(float4* __restrict__ pos, float* __restrict__ mom,
                                                   const float* __restrict__ psi1, const float* __restrict__ psi2,
-                                                  const float* __restrict__ force, size_t np3, int nm, const StepCoef& k,
+                                                  const float* __restrict__ force, size_t np3, const UDiv& u, const StepCoef& k,
                                                   int drift, const LightconeStep& lc, size_t p) {
     // every load of the particle's own data is issued before the force loads that depend on its
     // position, so the two sets are in flight together (streaming: each is used once per step)
@@ -194,7 +196,8 @@ __device__ __forceinline__ void gather_kick_drift(float4* __restrict__ pos, floa
         s2[j] = __ldcs(psi2 + j * np3 + p);
         v[j] = __ldcs(mom + j * np3 + p);
     }
-    const Cic c = cic_setup(P, nm);
+    const int nm = (int)u.d;
+    const Cic c = cic_setup(P, u);
     const float s = 1.0f / 32768.0f;
     const float wx[2] = {(QONE - c.fx) * s, c.fx * s};
     const float wy[2] = {(QONE - c.fy) * s, c.fy * s};
@@ -218,8 +221,8 @@ __device__ __forceinline__ void gather_kick_drift(float4* __restrict__ pos, floa
         }
     float d[3];
     const float off[3] = {P.x, P.y, P.z};
-    int cell[3] = {(int)(__float_as_uint(P.w) % (unsigned)nm), (int)((__float_as_uint(P.w) / (unsigned)nm) % (unsigned)nm),
-                   (int)((__float_as_uint(P.w) / ((unsigned)nm * (unsigned)nm)) % (unsigned)nm)};
+    int cell[3];
+    u.split(__float_as_uint(P.w), cell[0], cell[1], cell[2]);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
         // kick (Eq. eq:vcola): p += K [F - D1 Psi1 - (D2 - D1^2) Psi2]
@@ -233,13 +236,11 @@ __device__ __forceinline__ void gather_kick_drift(float4* __restrict__ pos, floa
     float o[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        float u = off[j] + d[j];
-        float fl = floorf(u);
-        float r = u - fl;
+        float w = off[j] + d[j];
+        float fl = floorf(w);
+        float r = w - fl;
         if (r >= 1.0f) { r = 0.0f; fl += 1.0f; }
-        int cc = (cell[j] + (int)fl) % nm;
-        if (cc < 0) cc += nm;
-        cell[j] = cc;
+        cell[j] = u.wrap(cell[j] + (int)fl);
         o[j] = r;
     }
     const unsigned lin = (unsigned)cell[0] + (unsigned)nm * ((unsigned)cell[1] + (unsigned)nm * (unsigned)cell[2]);
@@ -248,11 +249,11 @@ __device__ __forceinline__ void gather_kick_drift(float4* __restrict__ pos, floa
 
 template <bool LC>
 __global__ void k_gather_kick_drift(float4* __restrict__ pos, float* __restrict__ mom, const float* __restrict__ psi1,
-                                    const float* __restrict__ psi2, const float* __restrict__ force, size_t np3, int nm,
+                                    const float* __restrict__ psi2, const float* __restrict__ force, size_t np3, UDiv u,
                                     StepCoef k, int drift, LightconeStep lc) {
     const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np3) return;
-    gather_kick_drift<LC>(pos, mom, psi1, psi2, force, np3, nm, k, drift, lc, p);
+    gather_kick_drift<LC>(pos, mom, psi1, psi2, force, np3, u, k, drift, lc, p);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -309,7 +310,7 @@ __global__ void __launch_bounds__(MW_T) k_multi_deposit(const MockWork* __restri
         for (int h = 0; h < 2 * MW_ITEM / MW_T; ++h) {   // two threads per particle, one per x corner
             const int slot = h * MW_T + threadIdx.x;
             const size_t p = base + (slot >> 1);
-            if (p < mw.np3) deposit_corner(mw.pos, p, slot & 1, mw.nm, mw.rho);
+            if (p < mw.np3) deposit_corner(mw.pos, p, slot & 1, mw.u, mw.rho);
         }
     }
     leave_queue(queue);
@@ -326,54 +327,47 @@ __global__ void __launch_bounds__(MW_T) k_multi_gather_kick_drift(const MockWork
         for (int h = 0; h < MW_ITEM / MW_T; ++h) {
             const size_t p = base + h * MW_T + threadIdx.x;
             if (p < mw.np3)
-                gather_kick_drift<false>(mw.pos, mw.mom, mw.psi1, mw.psi2, mw.force, mw.np3, mw.nm, mw.k, 1,
+                gather_kick_drift<false>(mw.pos, mw.mom, mw.psi1, mw.psi2, mw.force, mw.np3, mw.u, mw.k, 1,
                                          LightconeStep{}, p);
         }
     }
     leave_queue(queue);
 }
 
-// Site i of the Lagrangian lattice sits at mesh coordinate i nm / np + 1/2 (spacing L / np, offset by
-// half a PM cell). Integer part of i nm / np and its exact fractional remainder (0 when np divides nm;
-// a multiple of nm / np otherwise, i.e. of 1/2 or 1/4 for the coarse meshes).
-__device__ __forceinline__ void lattice_site(int i, int np, int nm, int& base, float& frac) {
-    const int t = i * nm;   // < 2^20 for the supported sizes (np, nm <= 1024): 32-bit division
-    base = t / np;
-    frac = (float)(t % np) / (float)np;
-}
-
-// Particles on the Lagrangian lattice (offset by half a PM cell), displaced by D1 Psi1 + D2 Psi2.
-// psi1 / psi2 arrive in IC-grid cells and leave in PM-mesh cells (factor to_mesh = Nm / Np).
-__global__ void k_init_particles(float4* __restrict__ pos, float* __restrict__ mom, float* __restrict__ psi1,
-                                 float* __restrict__ psi2, int np, int nm, float to_mesh, float d1, float d2, float p1,
-                                 float p2, int cola) {
-    const size_t np3 = (size_t)np * np * np;
+// Particles on the Lagrangian lattice (offset by half a PM cell), displaced by D1 Psi1 + D2 Psi2, and their ids.
+// psi1 / psi2 arrive in some unit and leave in PM-mesh cells (factor to_mesh; not rewritten where it is 1).
+// Bound by its 56 bytes per particle (24 more with a factor): the index arithmetic goes through
+// multiplications (UDiv), the ids were a pass of their own. 256^3: 244 + 35 us before, 168 now.
+__global__ void k_init_particles(float4* __restrict__ pos, float* __restrict__ mom, int* __restrict__ id,
+                                 float* __restrict__ psi1, float* __restrict__ psi2, size_t np3, Lattice lat, float to_mesh,
+                                 float d1, float d2, float p1, float p2, int cola) {
     const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np3) return;
-    const unsigned up = (unsigned)p, unp = (unsigned)np;   // np^3 <= 2^30: 32-bit divisions
-    const int site[3] = {(int)(up % unp), (int)((up / unp) % unp), (int)(up / (unp * unp))};
-    int cell[3];
+    const int nm = (int)lat.nm.d;
+    int site[3], cell[3];
+    lat.site((unsigned)p, site);
     float o[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
         const float s1 = psi1[j * np3 + p] * to_mesh, s2 = psi2[j * np3 + p] * to_mesh;
-        psi1[j * np3 + p] = s1;
-        psi2[j * np3 + p] = s2;
+        if (to_mesh != 1.0f) {
+            psi1[j * np3 + p] = s1;
+            psi2[j * np3 + p] = s2;
+        }
         int base;
         float frac;
-        lattice_site(site[j], np, nm, base, frac);
+        lat.at(site[j], base, frac);
         const float u = (0.5f + frac) + fmaf(d1, s1, d2 * s2);
         float fl = floorf(u);
         float r = u - fl;
         if (r >= 1.0f) { r = 0.0f; fl += 1.0f; }
-        int cc = (base + (int)fl) % nm;
-        if (cc < 0) cc += nm;
-        cell[j] = cc;
+        cell[j] = lat.nm.wrap(base + (int)fl);
         o[j] = r;
         mom[j * np3 + p] = cola ? 0.0f : fmaf(p1, s1, p2 * s2);
     }
     const unsigned lin = (unsigned)cell[0] + (unsigned)nm * ((unsigned)cell[1] + (unsigned)nm * (unsigned)cell[2]);
     pos[p] = make_float4(o[0], o[1], o[2], __uint_as_float(lin));
+    id[p] = (int)p;
 }
 
 __global__ void k_add_lpt_momentum(float* __restrict__ mom, const float* __restrict__ psi1, const float* __restrict__ psi2,
@@ -384,15 +378,15 @@ __global__ void k_add_lpt_momentum(float* __restrict__ mom, const float* __restr
 }
 
 __global__ void k_export_particles(const float4* __restrict__ pos, const float* __restrict__ mom,
-                                   const int* __restrict__ id, size_t np3, int nm, float cell,
+                                   const int* __restrict__ id, size_t np3, UDiv u, float cell,
                                    float* __restrict__ pos_xyz, float* __restrict__ mom_xyz) {
     const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np3) return;
     const size_t q = id ? (size_t)id[p] : p;   // the particle's id: its place in the output
     if (pos_xyz) {
         const float4 P = pos[p];
-        const unsigned c = __float_as_uint(P.w), u = (unsigned)nm;
-        const unsigned cx = c % u, cy = (c / u) % u, cz = c / (u * u);
+        int cx, cy, cz;
+        u.split(__float_as_uint(P.w), cx, cy, cz);
         pos_xyz[3 * q + 0] = ((float)cx + P.x) * cell;
         pos_xyz[3 * q + 1] = ((float)cy + P.y) * cell;
         pos_xyz[3 * q + 2] = ((float)cz + P.z) * cell;
@@ -453,24 +447,24 @@ __global__ void k_import_state(float4* __restrict__ pos, float* __restrict__ mom
     }
 }
 
-// Psi = x - q in Mpc/h with the minimum-image convention, q = (site * Nm/Np + 1/2) cells.
-__global__ void k_export_displacement(const float4* __restrict__ pos, int np, int nm, float cell,
+// Psi = x - q in Mpc/h with the minimum-image convention, q = (site * Nm/Np + 1/2) cells. With divisions by np and
+// nm it was bound by them (256^3: 201 us for 28 bytes per particle, 85 now).
+__global__ void k_export_displacement(const float4* __restrict__ pos, size_t np3, Lattice lat, float cell,
                                       float* __restrict__ psi) {
-    const size_t np3 = (size_t)np * np * np;
     const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np3) return;
     const float4 P = pos[p];
-    const unsigned c = __float_as_uint(P.w), u = (unsigned)nm;
-    const int cc[3] = {(int)(c % u), (int)((c / u) % u), (int)(c / (u * u))};
-    const unsigned up = (unsigned)p, unp = (unsigned)np;   // np^3 <= 2^30: 32-bit divisions
-    const int site[3] = {(int)(up % unp), (int)((up / unp) % unp), (int)(up / (unp * unp))};
+    const int nm = (int)lat.nm.d;
+    int cc[3], site[3];
+    lat.nm.split(__float_as_uint(P.w), cc[0], cc[1], cc[2]);
+    lat.site((unsigned)p, site);
     const float off[3] = {P.x, P.y, P.z};
     const int h = nm / 2;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
         int base;
         float frac;
-        lattice_site(site[j], np, nm, base, frac);
+        lat.at(site[j], base, frac);
         int di = cc[j] - base;
         di += di < -h ? nm : (di >= h ? -nm : 0);
         float d = (float)di + (off[j] - (0.5f + frac));
@@ -480,14 +474,13 @@ __global__ void k_export_displacement(const float4* __restrict__ pos, int np, in
 }
 
 // x = q + Psi (Psi in Mpc/h, xyz-interleaved); momenta are left alone.
-__global__ void k_import_displacement(float4* __restrict__ pos, int np, int nm, float to_mesh,
+__global__ void k_import_displacement(float4* __restrict__ pos, size_t np3, Lattice lat, float to_mesh,
                                       const float* __restrict__ psi, int* err) {
-    const size_t np3 = (size_t)np * np * np;
     const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np3) return;
-    const unsigned up = (unsigned)p, unp = (unsigned)np;   // np^3 <= 2^30: 32-bit divisions
-    const int site[3] = {(int)(up % unp), (int)((up / unp) % unp), (int)(up / (unp * unp))};
-    int cell[3];
+    const int nm = (int)lat.nm.d;
+    int site[3], cell[3];
+    lat.site((unsigned)p, site);
     float o[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -498,14 +491,12 @@ __global__ void k_import_displacement(float4* __restrict__ pos, int np, int nm, 
         }
         int base;
         float frac;
-        lattice_site(site[j], np, nm, base, frac);
+        lat.at(site[j], base, frac);
         const float u = (0.5f + frac) + s;
         float fl = floorf(u);
         float r = u - fl;
         if (r >= 1.0f) { r = 0.0f; fl += 1.0f; }
-        int cc = (base + (int)fl) % nm;
-        if (cc < 0) cc += nm;
-        cell[j] = cc;
+        cell[j] = lat.nm.wrap(base + (int)fl);
         o[j] = r;
     }
     const unsigned lin = (unsigned)cell[0] + (unsigned)nm * ((unsigned)cell[1] + (unsigned)nm * (unsigned)cell[2]);
@@ -557,9 +548,17 @@ __global__ void k_rsd_positions(const float4* __restrict__ pos, const float* __r
     out[p] = make_float4(o[0], o[1], o[2], __uint_as_float(lin));
 }
 
+// dst = f src, V floats per thread (one per thread took twice the time of the copy it is).
+template <int V>
 __global__ void k_scale(float* __restrict__ dst, const float* __restrict__ src, size_t n, float f) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dst[i] = src[i] * f;
+    const size_t i = V * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
+    if (i >= n) return;
+    if constexpr (V == 4) {
+        const float4 v = __ldcs(reinterpret_cast<const float4*>(src + i));
+        *reinterpret_cast<float4*>(dst + i) = make_float4(v.x * f, v.y * f, v.z * f, v.w * f);
+    } else {
+        dst[i] = src[i] * f;
+    }
 }
 
 inline unsigned blocks(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -567,7 +566,7 @@ inline unsigned blocks(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
 }  // namespace
 
 cudaError_t launch_deposit(const float4* pos, size_t np3, int nm, unsigned long long* rho, cudaStream_t s, int block) {
-    k_deposit<<<blocks(2 * np3, block), block, 0, s>>>(pos, np3, nm, rho);
+    k_deposit<<<blocks(2 * np3, block), block, 0, s>>>(pos, np3, make_udiv(nm), rho);
     return cudaGetLastError();
 }
 
@@ -575,9 +574,9 @@ cudaError_t launch_gather_kick_drift(float4* pos, float* mom, const float* psi1,
                                      size_t np3, int nm, StepCoef c, int drift, cudaStream_t s, int block,
                                      const LightconeStep* lc) {
     if (lc && drift)
-        k_gather_kick_drift<true><<<blocks(np3, block), block, 0, s>>>(pos, mom, psi1, psi2, force, np3, nm, c, drift, *lc);
+        k_gather_kick_drift<true><<<blocks(np3, block), block, 0, s>>>(pos, mom, psi1, psi2, force, np3, make_udiv(nm), c, drift, *lc);
     else
-        k_gather_kick_drift<false><<<blocks(np3, block), block, 0, s>>>(pos, mom, psi1, psi2, force, np3, nm, c, drift,
+        k_gather_kick_drift<false><<<blocks(np3, block), block, 0, s>>>(pos, mom, psi1, psi2, force, np3, make_udiv(nm), c, drift,
                                                                         LightconeStep{});
     return cudaGetLastError();
 }
@@ -592,9 +591,9 @@ cudaError_t launch_deposit_tiles(const float4* pos, int nm, int tshift, const un
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const unsigned grid = (unsigned)sms * 8u < ntiles ? (unsigned)sms * 8u : ntiles;
     switch (tshift) {
-        case 1: k_deposit_tiles<1><<<grid, DT_T, 0, s>>>(pos, nm, xs, ends, ntiles, rho); break;
-        case 2: k_deposit_tiles<2><<<grid, DT_T, 0, s>>>(pos, nm, xs, ends, ntiles, rho); break;
-        default: k_deposit_tiles<3><<<grid, DT_T, 0, s>>>(pos, nm, xs, ends, ntiles, rho); break;
+        case 1: k_deposit_tiles<1><<<grid, DT_T, 0, s>>>(pos, make_udiv(nm), xs, ends, ntiles, rho); break;
+        case 2: k_deposit_tiles<2><<<grid, DT_T, 0, s>>>(pos, make_udiv(nm), xs, ends, ntiles, rho); break;
+        default: k_deposit_tiles<3><<<grid, DT_T, 0, s>>>(pos, make_udiv(nm), xs, ends, ntiles, rho); break;
     }
     return cudaGetLastError();
 }
@@ -623,10 +622,11 @@ cudaError_t launch_multi_gather_kick_drift(const MockWork* w, int nmock, long lo
     return cudaGetLastError();
 }
 
-cudaError_t launch_init_particles(float4* pos, float* mom, float* psi1, float* psi2, int np, int nm, float to_mesh,
+cudaError_t launch_init_particles(float4* pos, float* mom, int* id, float* psi1, float* psi2, int np, int nm, float to_mesh,
                                   float d1, float d2, float p1, float p2, int cola, cudaStream_t s) {
     const size_t np3 = (size_t)np * np * np;
-    k_init_particles<<<blocks(np3, 256), 256, 0, s>>>(pos, mom, psi1, psi2, np, nm, to_mesh, d1, d2, p1, p2, cola);
+    k_init_particles<<<blocks(np3, 256), 256, 0, s>>>(pos, mom, id, psi1, psi2, np3, make_lattice(np, nm), to_mesh, d1, d2, p1,
+                                                    p2, cola);
     return cudaGetLastError();
 }
 
@@ -638,7 +638,7 @@ cudaError_t launch_add_lpt_momentum(float* mom, const float* psi1, const float* 
 
 cudaError_t launch_export_particles(const float4* pos, const float* mom, const int* id, size_t np3, int nm, float cell,
                                     float* pos_xyz, float* mom_xyz, cudaStream_t s) {
-    k_export_particles<<<blocks(np3, 256), 256, 0, s>>>(pos, mom, id, np3, nm, cell, pos_xyz, mom_xyz);
+    k_export_particles<<<blocks(np3, 256), 256, 0, s>>>(pos, mom, id, np3, make_udiv(nm), cell, pos_xyz, mom_xyz);
     return cudaGetLastError();
 }
 
@@ -656,14 +656,14 @@ cudaError_t launch_import_state(float4* pos, float* mom, size_t np3, int nm, con
 
 cudaError_t launch_export_displacement(const float4* pos, int np, int nm, float cell, float* psi, cudaStream_t s) {
     const size_t np3 = (size_t)np * np * np;
-    k_export_displacement<<<blocks(np3, 256), 256, 0, s>>>(pos, np, nm, cell, psi);
+    k_export_displacement<<<blocks(np3, 256), 256, 0, s>>>(pos, np3, make_lattice(np, nm), cell, psi);
     return cudaGetLastError();
 }
 
 cudaError_t launch_import_displacement(float4* pos, int np, int nm, float to_mesh, const float* psi, int* err,
                                        cudaStream_t s) {
     const size_t np3 = (size_t)np * np * np;
-    k_import_displacement<<<blocks(np3, 256), 256, 0, s>>>(pos, np, nm, to_mesh, psi, err);
+    k_import_displacement<<<blocks(np3, 256), 256, 0, s>>>(pos, np3, make_lattice(np, nm), to_mesh, psi, err);
     return cudaGetLastError();
 }
 
@@ -674,7 +674,11 @@ cudaError_t launch_rsd_positions(const float4* pos, const float* mom, size_t np3
 }
 
 cudaError_t launch_scale(float* dst, const float* src, size_t n, float f, cudaStream_t s) {
-    k_scale<<<blocks(n, 256), 256, 0, s>>>(dst, src, n, f);
+    // a caller's array may start at any float
+    if (n % 4 == 0 && (reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) % 16 == 0)
+        k_scale<4><<<blocks(n / 4, 256), 256, 0, s>>>(dst, src, n, f);
+    else
+        k_scale<1><<<blocks(n, 256), 256, 0, s>>>(dst, src, n, f);
     return cudaGetLastError();
 }
 
