@@ -95,6 +95,7 @@ __host__ __device__ __forceinline__ void twiddle2(float2* v, const Tw2* t, int j
 }  // namespace colapm
 
 #include "colapm_internal.h"
+#include "launch_cache.h"
 
 namespace colapm {
 
@@ -159,7 +160,9 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy(float2* __restrict__ data, siz
     extern __shared__ float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
     Tw2* tws = reinterpret_cast<Tw2*>(xb + Xch<L, RA>::SIZE);
+    pdl_trigger();
     load_tw2<L, L>(tws, tw, K::T);
+    pdl_wait();
     __syncthreads();
     const int total = TPF * nfields;
     const int tid = threadIdx.x, c = tid & 7, j = tid >> 3;
@@ -227,7 +230,9 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
     float* pbuf = reinterpret_cast<float*>(tws + 1);             // Z_POWER: [C][PP], then the window table, then the thresholds
     float* iw2 = pbuf + (MODE == Z_POWER ? C * Z::PP : 0);
     int* lo = reinterpret_cast<int*>(iw2 + (MODE == Z_POWER ? L / 2 : 0));
+    pdl_trigger();
     load_tw2<L, L>(tws, tw, T);
+    pdl_wait();
     double* part = nullptr;                                      // Z_POWER: the sums this CTA adds to
     if constexpr (MODE == Z_POWER) {
         load_thresholds(lo, pw, threadIdx.x, T);
@@ -480,7 +485,9 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy_force(float2* __restrict__ dat
     extern __shared__ float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
     Tw2* tws = reinterpret_cast<Tw2*>(xb + Xch<L, RA>::SIZE);
+    pdl_trigger();
     load_tw2<L, L>(tws, tw, K::T);
+    pdl_wait();
     __syncthreads();
     const float kf = 6.283185307179586f / (float)L;
     const int tid = threadIdx.x, c = tid & 7, j = tid >> 3;
@@ -540,7 +547,9 @@ __global__ void __launch_bounds__(X2<n>::T) k2_fx_fwd(const void* __restrict__ i
     extern __shared__ float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
     Tw2* tws = reinterpret_cast<Tw2*>(xb + Xch<n, RA>::SIZE);
+    pdl_trigger();
     load_tw2<n, N>(tws, tw, X::T);
+    pdl_wait();
     __syncthreads();
     const int tid = threadIdx.x;
     bool over = false;
@@ -653,7 +662,9 @@ __global__ void __launch_bounds__(X2<n>::T, 3) k2_fx_inv(float2* __restrict__ da
     float2* xb = reinterpret_cast<float2*>(smem4);
     Tw2* tws = reinterpret_cast<Tw2*>(xb + Xch<n, RA>::SIZE);
     float2* stg = reinterpret_cast<float2*>(tws + 1);   // [8][n]
+    pdl_trigger();
     load_tw2<n, N>(tws, tw, T);
+    pdl_wait();
     const int tid = threadIdx.x;
     const int nitems = items_per_field * nfields;
     auto gptr = [&](int t) { return dst + (size_t)(t / items_per_field) * fstride + (size_t)(t % items_per_field) * 8 * n; };

@@ -136,7 +136,9 @@ __global__ void __launch_bounds__(PZ_T, MINB)
     float2* xb = reinterpret_cast<float2*>(smem4);
     float2* save = xb + X::SIZE;
     Tw2* tws = reinterpret_cast<Tw2*>(save + X::SIZE);
+    pdl_trigger();
     load_tw2<L, L>(tws, tw, PZ_T);
+    pdl_wait();
     __syncthreads();
     const float kf = 6.283185307179586f / (float)L;
     const int tid = threadIdx.x, c = tid & 3, h = (tid >> 2) & 1, j = tid >> 3;

@@ -13,8 +13,7 @@ static cudaError_t fx_fwd2(const void* in, float2* out, const float2* tw, float 
     cudaError_t e = cached_grid(cache, k2_fx_fwd<n, I64, BLK>, X::T, X::SMEM, &grid2);
     if (e != cudaSuccess) return e;
     const int items = 2 * n * 2 * n / 8;
-    k2_fx_fwd<n, I64, BLK><<<grid2 < items ? grid2 : items, X::T, X::SMEM, s>>>(in, out, tw, scale, err, items, zero);
-    return cudaGetLastError();
+    return launch_dep(overlap_mesh(2 * n), k2_fx_fwd<n, I64, BLK>, grid2 < items ? grid2 : items, X::T, X::SMEM, s, in, out, tw, scale, err, items, zero);
 }
 
 template <int N, bool I64>
@@ -44,8 +43,7 @@ static cudaError_t fx_inv2(float2* data, size_t fstride, int nfields, const floa
     cudaError_t e = cached_grid(cache, k2_fx_inv<n, BLK>, X::T, X::SMEM_INV, &grid2);
     if (e != cudaSuccess) return e;
     const int ipf = 2 * n * 2 * n / 8, items = ipf * nfields;
-    k2_fx_inv<n, BLK><<<grid2 < items ? grid2 : items, X::T, X::SMEM_INV, s>>>(data, fstride, tw, ipf, nfields, dst);
-    return cudaGetLastError();
+    return launch_dep(overlap_mesh(2 * n), k2_fx_inv<n, BLK>, grid2 < items ? grid2 : items, X::T, X::SMEM_INV, s, data, fstride, tw, ipf, nfields, dst);
 }
 
 template <int N>

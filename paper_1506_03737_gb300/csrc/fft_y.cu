@@ -13,8 +13,7 @@ static cudaError_t fy2(float2* data, size_t fstride, int nfields, const float2* 
     cudaError_t e = cached_grid(cache, k2_fy<N, S, BLK>, K::T, smem, &grid2);
     if (e != cudaSuccess) return e;
     const int total = (N / 2 / 8) * N * nfields;
-    k2_fy<N, S, BLK><<<grid2 < total ? grid2 : total, K::T, smem, s>>>(data, fstride, tw, nfields);
-    return cudaGetLastError();
+    return launch_dep(overlap_mesh(N), k2_fy<N, S, BLK>, grid2 < total ? grid2 : total, K::T, smem, s, data, fstride, tw, nfields);
 }
 
 template <int N, int S>
@@ -51,8 +50,7 @@ static cudaError_t fy_force_t(float2* data, size_t fstride, const float2* tw, cu
     cudaError_t e = cached_grid(cache, k2_fy_force<N>, K::T, smem, &grid);
     if (e != cudaSuccess) return e;
     const int total = (N / 2 / 8) * N;
-    k2_fy_force<N><<<grid < total ? grid : total, K::T, smem, s>>>(data, fstride, tw);
-    return cudaGetLastError();
+    return launch_dep(overlap_mesh(N), k2_fy_force<N>, grid < total ? grid : total, K::T, smem, s, data, fstride, tw);
 }
 
 cudaError_t launch_fy_force(int n_mesh, float2* data, size_t field_stride, const float2* tw, cudaStream_t s) {

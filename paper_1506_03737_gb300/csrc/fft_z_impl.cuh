@@ -25,8 +25,7 @@ static cudaError_t fz2(float2* in, ZOut out, const float2* tw, const float* sinc
         cudaError_t e = cached_grid(cache, k2_fz_pair<MINB>, PZ_T, PairZ<MINB>::SMEM, &grid);
         if (e != cudaSuccess) return e;
         const int total = (N / 2 / 4) * N;
-        k2_fz_pair<MINB><<<grid < total ? grid : total, PZ_T, PairZ<MINB>::SMEM, s>>>(in, out, tw, sinc2, deconv, gnorm);
-        return cudaGetLastError();
+        return launch_dep(overlap_mesh(N), k2_fz_pair<MINB>, grid < total ? grid : total, PZ_T, PairZ<MINB>::SMEM, s, in, out, tw, sinc2, deconv, gnorm);
     } else {
         // Blocked layout: 4-column tiles (32-byte rows whose 512-byte runs the neighbouring tiles
         // complete), which with the prefetch buffer measured 2% faster than 8-column ones (34% for the
@@ -41,8 +40,7 @@ static cudaError_t fz2(float2* in, ZOut out, const float2* tw, const float* sinc
         cudaError_t e = cached_grid(cache, k2_fz<N, MODE, CZ, BLK, DIRECT>, Z::T, smem, &grid2);
         if (e != cudaSuccess) return e;
         const int total = (N / 2 / CZ) * N;
-        k2_fz<N, MODE, CZ, BLK, DIRECT><<<grid2 < total ? grid2 : total, Z::T, smem, s>>>(in, out, tw, sinc2, deconv, gnorm, pw);
-        return cudaGetLastError();
+        return launch_dep(overlap_mesh(N), k2_fz<N, MODE, CZ, BLK, DIRECT>, grid2 < total ? grid2 : total, Z::T, smem, s, in, out, tw, sinc2, deconv, gnorm, pw);
     }
 }
 

@@ -1,5 +1,6 @@
 // Initial-condition kernels (§5, §2.1): Gaussian field and the 2LPT source term.
 #include "colapm_internal.h"
+#include "launch_cache.h"
 
 namespace colapm {
 
@@ -39,6 +40,8 @@ __device__ __forceinline__ float2 draw(unsigned long long m, unsigned long long 
 // One thread per half-grid mode (iz, iy, ix < N/2): delta_k = amp(|n|^2) g, Hermitian on ix = 0.
 __global__ void k_gaussian_field(int n, const unsigned long long* __restrict__ seedp, const float* __restrict__ amp_of_n2,
                                  float2* __restrict__ dk) {
+    pdl_trigger();
+    pdl_wait();
     const unsigned long long seed = *seedp;
     const int h = n / 2;
     // a row of modes per row of threads: no index division (with 64-bit ones the pass took 79 us at 256^3, 63 now)
@@ -73,6 +76,8 @@ __global__ void k_gaussian_field(int n, const unsigned long long* __restrict__ s
 // S = phi_xx phi_yy + phi_xx phi_zz + phi_yy phi_zz - phi_xy^2 - phi_xz^2 - phi_yz^2
 // (the right-hand side of the phi2 Poisson equation, §2.1); phi = [xx, yy, zz, xy, xz, yz].
 __global__ void k_lpt2_source(const float4* __restrict__ phi, size_t n4, float4* __restrict__ src) {
+    pdl_trigger();
+    pdl_wait();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n4) return;
     const float4 xx = __ldcs(phi + i), yy = __ldcs(phi + n4 + i), zz = __ldcs(phi + 2 * n4 + i);
@@ -126,15 +131,13 @@ cudaError_t launch_set_u64(unsigned long long* dst, unsigned long long value, cu
 cudaError_t launch_gaussian_field(int np, const unsigned long long* seed, const float* amp_of_n2, float2* dk,
                                   cudaStream_t s) {
     const int bx = np / 2 < 256 ? np / 2 : 256, by = 256 / bx;   // np / 2 may not divide 256: fewer threads then
-    k_gaussian_field<<<dim3((np + by - 1) / by, np), dim3(bx, by), 0, s>>>(np, seed, amp_of_n2, dk);
-    return cudaGetLastError();
+    return launch_dep(overlap_mesh(np), k_gaussian_field, dim3((np + by - 1) / by, np), dim3(bx, by), 0, s, np, seed, amp_of_n2, dk);
 }
 
 cudaError_t launch_lpt2_source(const float* phi, size_t np3, float* src, cudaStream_t s) {
     const size_t n4 = np3 / 4;   // np is a multiple of 16
-    k_lpt2_source<<<(unsigned)((n4 + 255) / 256), 256, 0, s>>>(reinterpret_cast<const float4*>(phi), n4,
+    return launch_dep(np3 <= (size_t)128 * 128 * 128, k_lpt2_source, (unsigned)((n4 + 255) / 256), 256, 0, s, reinterpret_cast<const float4*>(phi), n4,
                                                                reinterpret_cast<float4*>(src));
-    return cudaGetLastError();
 }
 
 }  // namespace colapm

@@ -206,13 +206,15 @@ __global__ void __launch_bounds__(32 * TZ, TZ == 8 ? 2 : 4)
     const int g = lane >> 2, q = lane & 3;
     const uint32_t hb = smem_u32(sm), wb = hb + S::W, aux = hb + S::AUX + tz * (TX * TY * 32),
                    bar = hb + S::BAR, mbar = bar + 8 + 8 * tz;
-    for (int j = threadIdx.x; j < 27 * C * 2; j += 32 * TZ) {   // weights, swizzled with the row index
-        const int row = j >> 1, k = j & 1;
-        cp_async16(wb + row * 32 + (half_slot(row, k) << 4), a.w + row * C + k * 8);
-    }
+    pdl_trigger();
     if (threadIdx.x == 0) {
         for (int b = 0; b < 1 + TZ; ++b) mbar_init(bar + 8 * b);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    pdl_wait();
+    for (int j = threadIdx.x; j < 27 * C * 2; j += 32 * TZ) {   // weights, swizzled with the row index
+        const int row = j >> 1, k = j & 1;
+        cp_async16(wb + row * 32 + (half_slot(row, k) << 4), a.w + row * C + k * 8);
     }
     cp_async_wait_all();
     __syncthreads();
@@ -453,6 +455,8 @@ __global__ void __launch_bounds__(32 * 3 * (TZ / 2), 1)
         mbar_init(bar + 8);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+    pdl_trigger();
+    pdl_wait();
     __syncthreads();
     auto load = [&](int t, int buf) {   // halo of the activations and dz of tile t
         int x0, y0, z0;
@@ -783,6 +787,8 @@ __device__ __forceinline__ bool real_slot(int l, int slot, int o, int i) {
 // partials dealt over RG_Y rows of threads (a column of 304 sums one after the other took 23 us).
 constexpr int RG_Y = 32;
 __global__ void __launch_bounds__(32 * RG_Y) k_reduce_grads(const float* __restrict__ part, int nparts, float* __restrict__ grad) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ float sh[RG_Y][33];
     const int idx = blockIdx.x * 32 + threadIdx.x;   // LAYERS * LSIZE is a multiple of 32
     const int l = idx / LSIZE, r = idx % LSIZE;
@@ -806,6 +812,8 @@ __global__ void k_adam(float* __restrict__ wm, float* __restrict__ m1, float* __
                        const float* __restrict__ grad, float lr, float b1, float b2, float eps, float c1, float c2,
                        int update, __nv_bfloat16* __restrict__ wf, __nv_bfloat16* __restrict__ wt,
                        float* __restrict__ bias) {
+    pdl_trigger();
+    pdl_wait();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= LAYERS * LSIZE) return;
     const int l = idx / LSIZE, r = idx % LSIZE;
@@ -831,6 +839,8 @@ __global__ void k_adam(float* __restrict__ wm, float* __restrict__ m1, float* __
 
 // x[v][c] = bf16(psi[v][c] / s_in) for c < 3, zero for the other five channels; one thread per stored voxel.
 __global__ void k_pack_input(const float* __restrict__ psi, int n, float inv_s, __nv_bfloat16* __restrict__ x) {
+    pdl_trigger();
+    pdl_wait();
     const int m = n + 2, row = blockIdx.x * blockDim.y + threadIdx.y;   // stored row (z, y)
     if (row >= m * m) return;
     int y = row % m - 1, z = row / m - 1;
@@ -905,8 +915,8 @@ cudaError_t launch_conv(const colapm_nn* c, const ConvArgs& a, const CUtensorMap
     int grid = 0;
     cudaError_t e = colapm::cached_grid(cache, k_conv<NT, EPI, TZ, VB>, 32 * TZ, S::BYTES, &grid);
     if (e) return e;
-    k_conv<NT, EPI, TZ, VB><<<std::min(tiles_of(c->n, TZ), grid), 32 * TZ, S::BYTES, c->stream>>>(a, halo, out, mask);
-    return cudaGetLastError();
+    return colapm::launch_dep(true, k_conv<NT, EPI, TZ, VB>, std::min(tiles_of(c->n, TZ), grid), 32 * TZ, S::BYTES, c->stream, a, halo,
+                              out, mask);
 }
 
 // VB: bytes per voxel of the input (16: the packed input or the output gradient).
@@ -934,9 +944,8 @@ cudaError_t launch_wgrad(colapm_nn* c, const CUtensorMap& dz, int l) {
     int grid = 0;   // only the shared-memory attribute: the CTAs are the network's partials
     cudaError_t e = colapm::cached_grid(cache, k_wgrad<ACT_A, NT, TZ, VA, VD>, 96 * (TZ / 2), S::BYTES, &grid);
     if (e) return e;
-    k_wgrad<ACT_A, NT, TZ, VA, VD><<<c->nparts, 96 * (TZ / 2), S::BYTES, c->stream>>>(
-        c->m_act[l].whalo, dz, c->n, c->part + (size_t)l * c->nparts * LSIZE, c->err);
-    return cudaGetLastError();
+    return colapm::launch_dep(true, k_wgrad<ACT_A, NT, TZ, VA, VD>, c->nparts, 96 * (TZ / 2), S::BYTES, c->stream, c->m_act[l].whalo,
+                              dz, c->n, c->part + (size_t)l * c->nparts * LSIZE, c->err);
 }
 
 template <bool ACT_A, int NT, int VA, int VD>
@@ -973,9 +982,9 @@ cudaError_t publish(colapm_nn* c) {
 cudaError_t forward(colapm_nn* c, const float* psi, float* y, const float* base, const float* target) {
     const size_t nv = c->nv;
     const int rows = (c->n + 2) * (c->n + 2), bx = c->n >= 62 ? 64 : 32;
-    k_pack_input<<<(rows + 3) / 4, dim3(bx, 4), 0, c->stream>>>(psi, c->n, 1.0f / c->cfg.s_in, c->act[0]);
     ++c->launches;
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = colapm::launch_dep(true, k_pack_input, (rows + 3) / 4, dim3(bx, 4), 0, c->stream, psi, c->n, 1.0f / c->cfg.s_in,
+                                       c->act[0]);
     if (e) return e;
     for (int l = 0; l < 3; ++l) {
         ConvArgs a{};
@@ -1028,9 +1037,8 @@ cudaError_t backward(colapm_nn* c) {
         g = c->dz[l & 1];
         gm = om;
     }
-    k_reduce_grads<<<LAYERS * LSIZE / 32, dim3(32, RG_Y), 0, c->stream>>>(c->part, c->nparts, c->grad);
     ++c->launches;
-    return cudaGetLastError();
+    return colapm::launch_dep(true, k_reduce_grads, LAYERS * LSIZE / 32, dim3(32, RG_Y), 0, c->stream, c->part, c->nparts, c->grad);
 }
 
 // Tensor maps of a stored array of (n + 2)^3 voxels of vb bytes, as 8-byte elements.
@@ -1248,10 +1256,9 @@ int colapm_nn_train_step(colapm_nn* c, const float* psi, const float* target, do
     const float c1 = 1.0f - std::pow(c->cfg.beta1, (float)c->steps);
     const float c2 = 1.0f - std::pow(c->cfg.beta2, (float)c->steps);
     const int total = LAYERS * LSIZE;
-    k_adam<<<(total + 255) / 256, 256, 0, c->stream>>>(c->wm, c->m1, c->m2, c->grad, c->cfg.lr, c->cfg.beta1,
-                                                       c->cfg.beta2, c->cfg.eps, c1, c2, 1, c->wf, c->wt, c->bias);
     ++c->launches;
-    NN_CK(cudaGetLastError());
+    NN_CK(colapm::launch_dep(true, k_adam, (total + 255) / 256, 256, 0, c->stream, c->wm, c->m1, c->m2, c->grad, c->cfg.lr,
+                             c->cfg.beta1, c->cfg.beta2, c->cfg.eps, c1, c2, 1, c->wf, c->wt, c->bias));
     if (loss) {
         double h = 0.0;
         NN_CK(cudaMemcpyAsync(&h, c->loss, sizeof(double), cudaMemcpyDeviceToHost, c->stream));

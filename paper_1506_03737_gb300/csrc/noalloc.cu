@@ -14,6 +14,7 @@
 #include <mutex>
 
 #include "colapm_internal.h"
+#include "launch_cache.h"
 
 namespace colapm {
 namespace {
@@ -39,6 +40,8 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kBytes];
 // Fixed-point CIC deposit of xyz cell / offset arrays (the definition of pm_kernels.cu).
 __global__ void k_deposit_xyz(const int* __restrict__ cell, const float* __restrict__ off, long long n, int nm,
                               unsigned long long* __restrict__ rho, int* err) {
+    pdl_trigger();
+    pdl_wait();
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     int c[3], f[3];
@@ -75,6 +78,8 @@ __global__ void k_deposit_xyz(const int* __restrict__ cell, const float* __restr
 // (sqrt correctly rounded), n2max + 1 if none; one thread per edge, binary search over |n|^2.
 __global__ void k_bin_thresholds(const double* __restrict__ edges, int nbins, double kf, int n2max,
                                  int* __restrict__ lo) {
+    pdl_trigger();
+    pdl_wait();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b > nbins) return;
     int a = 0, z = n2max + 1;   // find the first n2 in [0, n2max + 1) with kf sqrt(n2) >= edges[b]
@@ -86,6 +91,8 @@ __global__ void k_bin_thresholds(const double* __restrict__ edges, int nbins, do
 }
 
 __global__ void k_finish(const double* __restrict__ acc, int nbins, double* __restrict__ out) {
+    pdl_trigger();
+    pdl_wait();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nbins) return;
     unsigned long long cnt;
@@ -183,10 +190,8 @@ extern "C" int colapm_power_noalloc(const int* cell, const float* offset, long l
     NCK(cudaMemsetAsync(rho, 0, sizeof(unsigned long long) * nm3, s));
     NCK(cudaMemsetAsync(acc, 0, sizeof(double) * power_words(nbins, kPowerRegions), s));
     NCK(cudaMemsetAsync(err, 0, 4 * sizeof(int), s));
-    k_bin_thresholds<<<(nbins + 128) / 128, 128, 0, s>>>(edges, nbins, kf, n2max, bin);
-    NCK(cudaGetLastError());
-    k_deposit_xyz<<<(unsigned)((n_particles + 255) / 256), 256, 0, s>>>(cell, offset, n_particles, nm, rho, err);
-    NCK(cudaGetLastError());
+    NCK(launch_dep(true, k_bin_thresholds, (nbins + 128) / 128, 128, 0, s, edges, nbins, kf, n2max, bin));
+    NCK(launch_dep(true, k_deposit_xyz, (unsigned)((n_particles + 255) / 256), 256, 0, s, cell, offset, n_particles, nm, rho, err));
     const double ratio = (double)nm3 / (double)n_particles;   // cells per particle
     NCK(launch_fx_fwd_i64(nm, rho, spec, tw, (float)(ratio * std::ldexp(1.0, -45)), err, s));
     NCK(launch_fy(nm, -1, spec, 0, 1, tw, s));
@@ -198,8 +203,7 @@ extern "C" int colapm_power_noalloc(const int* cell, const float* offset, long l
     pw.lga = (float)(0.5 * nbins / std::log2(h_edges[nbins] / h_edges[0]));
     pw.lgb = (float)(nbins * std::log2(kf / h_edges[0]) / std::log2(h_edges[nbins] / h_edges[0]));
     NCK(launch_fz(nm, Z_POWER, spec, ZOut{}, tw, sinc2, 0, 1.0f, &pw, s));
-    k_finish<<<(nbins + 127) / 128, 128, 0, s>>>(acc, nbins, out);
-    NCK(cudaGetLastError());
+    NCK(launch_dep(true, k_finish, (nbins + 127) / 128, 128, 0, s, acc, nbins, out));
     int h_err = 0;
     NCK(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     NCK(cudaMemcpyAsync(k_out, out, sizeof(double) * nbins, cudaMemcpyDefault, s));

@@ -60,6 +60,8 @@ __device__ __forceinline__ void deposit_corner(const float4* __restrict__ pos, s
 }
 
 __global__ void k_deposit(const float4* __restrict__ pos, size_t np3, UDiv u, unsigned long long* __restrict__ rho) {
+    pdl_trigger();
+    pdl_wait();
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t p = t >> 1;
     if (p >= np3) return;
@@ -251,6 +253,8 @@ template <bool LC>
 __global__ void k_gather_kick_drift(float4* __restrict__ pos, float* __restrict__ mom, const float* __restrict__ psi1,
                                     const float* __restrict__ psi2, const float* __restrict__ force, size_t np3, UDiv u,
                                     StepCoef k, int drift, LightconeStep lc) {
+    pdl_trigger();
+    pdl_wait();
     const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np3) return;
     gather_kick_drift<LC>(pos, mom, psi1, psi2, force, np3, u, k, drift, lc, p);
@@ -301,6 +305,8 @@ __device__ __forceinline__ void leave_queue(unsigned long long* queue) {
 
 __global__ void __launch_bounds__(MW_T) k_multi_deposit(const MockWork* __restrict__ w, int nmock, long long nitems,
                                                         unsigned long long* queue) {
+    pdl_trigger();
+    pdl_wait();
     long long item;
     int m;
     while (next_item(w, nmock, nitems, queue, item, m)) {
@@ -318,6 +324,8 @@ __global__ void __launch_bounds__(MW_T) k_multi_deposit(const MockWork* __restri
 
 __global__ void __launch_bounds__(MW_T) k_multi_gather_kick_drift(const MockWork* __restrict__ w, int nmock,
                                                                   long long nitems, unsigned long long* queue) {
+    pdl_trigger();
+    pdl_wait();
     long long item;
     int m;
     while (next_item(w, nmock, nitems, queue, item, m)) {
@@ -341,6 +349,8 @@ __global__ void __launch_bounds__(MW_T) k_multi_gather_kick_drift(const MockWork
 __global__ void k_init_particles(float4* __restrict__ pos, float* __restrict__ mom, int* __restrict__ id,
                                  float* __restrict__ psi1, float* __restrict__ psi2, size_t np3, Lattice lat, float to_mesh,
                                  float d1, float d2, float p1, float p2, int cola) {
+    pdl_trigger();
+    pdl_wait();
     const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np3) return;
     const int nm = (int)lat.nm.d;
@@ -372,6 +382,8 @@ __global__ void k_init_particles(float4* __restrict__ pos, float* __restrict__ m
 
 __global__ void k_add_lpt_momentum(float* __restrict__ mom, const float* __restrict__ psi1, const float* __restrict__ psi2,
                                    size_t n3, float p1, float p2) {
+    pdl_trigger();
+    pdl_wait();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n3) return;
     mom[i] = fmaf(p1, psi1[i], fmaf(p2, psi2[i], mom[i]));
@@ -380,6 +392,8 @@ __global__ void k_add_lpt_momentum(float* __restrict__ mom, const float* __restr
 __global__ void k_export_particles(const float4* __restrict__ pos, const float* __restrict__ mom,
                                    const int* __restrict__ id, size_t np3, UDiv u, float cell,
                                    float* __restrict__ pos_xyz, float* __restrict__ mom_xyz) {
+    pdl_trigger();
+    pdl_wait();
     const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np3) return;
     const size_t q = id ? (size_t)id[p] : p;   // the particle's id: its place in the output
@@ -399,6 +413,8 @@ __global__ void k_export_particles(const float4* __restrict__ pos, const float* 
 
 __global__ void k_export_state(const float4* __restrict__ pos, const float* __restrict__ mom, size_t np3, int nm,
                                int* __restrict__ cell_xyz, float* __restrict__ off_xyz, float* __restrict__ mom_xyz) {
+    pdl_trigger();
+    pdl_wait();
     const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np3) return;
     const float4 P = pos[p];
@@ -451,6 +467,8 @@ __global__ void k_import_state(float4* __restrict__ pos, float* __restrict__ mom
 // nm it was bound by them (256^3: 201 us for 28 bytes per particle, 85 now).
 __global__ void k_export_displacement(const float4* __restrict__ pos, size_t np3, Lattice lat, float cell,
                                       float* __restrict__ psi) {
+    pdl_trigger();
+    pdl_wait();
     const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= np3) return;
     const float4 P = pos[p];
@@ -551,6 +569,8 @@ __global__ void k_rsd_positions(const float4* __restrict__ pos, const float* __r
 // dst = f src, V floats per thread (one per thread took twice the time of the copy it is).
 template <int V>
 __global__ void k_scale(float* __restrict__ dst, const float* __restrict__ src, size_t n, float f) {
+    pdl_trigger();
+    pdl_wait();
     const size_t i = V * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= n) return;
     if constexpr (V == 4) {
@@ -566,19 +586,17 @@ inline unsigned blocks(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
 }  // namespace
 
 cudaError_t launch_deposit(const float4* pos, size_t np3, int nm, unsigned long long* rho, cudaStream_t s, int block) {
-    k_deposit<<<blocks(2 * np3, block), block, 0, s>>>(pos, np3, make_udiv(nm), rho);
-    return cudaGetLastError();
+    return launch_dep(overlap_mesh(nm), k_deposit, blocks(2 * np3, block), block, 0, s, pos, np3, make_udiv(nm), rho);
 }
 
 cudaError_t launch_gather_kick_drift(float4* pos, float* mom, const float* psi1, const float* psi2, const float* force,
                                      size_t np3, int nm, StepCoef c, int drift, cudaStream_t s, int block,
                                      const LightconeStep* lc) {
     if (lc && drift)
-        k_gather_kick_drift<true><<<blocks(np3, block), block, 0, s>>>(pos, mom, psi1, psi2, force, np3, make_udiv(nm), c, drift, *lc);
-    else
-        k_gather_kick_drift<false><<<blocks(np3, block), block, 0, s>>>(pos, mom, psi1, psi2, force, np3, make_udiv(nm), c, drift,
-                                                                        LightconeStep{});
-    return cudaGetLastError();
+        return launch_dep(overlap_mesh(nm), k_gather_kick_drift<true>, blocks(np3, block), block, 0, s, pos, mom, psi1, psi2, force, np3,
+                          make_udiv(nm), c, drift, *lc);
+    return launch_dep(overlap_mesh(nm), k_gather_kick_drift<false>, blocks(np3, block), block, 0, s, pos, mom, psi1, psi2, force, np3,
+                      make_udiv(nm), c, drift, LightconeStep{});
 }
 
 cudaError_t launch_deposit_tiles(const float4* pos, int nm, int tshift, const unsigned* ends, unsigned long long* rho,
@@ -607,8 +625,7 @@ cudaError_t launch_multi_deposit(const MockWork* w, int nmock, long long nitems,
     cudaError_t e = cached_grid(cache, k_multi_deposit, MW_T, 0, &grid);
     if (e != cudaSuccess) return e;
     if (nitems < 1 || nmock < 1) return cudaSuccess;
-    k_multi_deposit<<<nitems < grid ? (int)nitems : grid, MW_T, 0, s>>>(w, nmock, nitems, queue);
-    return cudaGetLastError();
+    return launch_dep(false, k_multi_deposit, nitems < grid ? (int)nitems : grid, MW_T, 0, s, w, nmock, nitems, queue);
 }
 
 cudaError_t launch_multi_gather_kick_drift(const MockWork* w, int nmock, long long nitems, unsigned long long* queue,
@@ -618,34 +635,29 @@ cudaError_t launch_multi_gather_kick_drift(const MockWork* w, int nmock, long lo
     cudaError_t e = cached_grid(cache, k_multi_gather_kick_drift, MW_T, 0, &grid);
     if (e != cudaSuccess) return e;
     if (nitems < 1 || nmock < 1) return cudaSuccess;
-    k_multi_gather_kick_drift<<<nitems < grid ? (int)nitems : grid, MW_T, 0, s>>>(w, nmock, nitems, queue);
-    return cudaGetLastError();
+    return launch_dep(false, k_multi_gather_kick_drift, nitems < grid ? (int)nitems : grid, MW_T, 0, s, w, nmock, nitems, queue);
 }
 
 cudaError_t launch_init_particles(float4* pos, float* mom, int* id, float* psi1, float* psi2, int np, int nm, float to_mesh,
                                   float d1, float d2, float p1, float p2, int cola, cudaStream_t s) {
     const size_t np3 = (size_t)np * np * np;
-    k_init_particles<<<blocks(np3, 256), 256, 0, s>>>(pos, mom, id, psi1, psi2, np3, make_lattice(np, nm), to_mesh, d1, d2, p1,
+    return launch_dep(overlap_mesh(nm), k_init_particles, blocks(np3, 256), 256, 0, s, pos, mom, id, psi1, psi2, np3, make_lattice(np, nm), to_mesh, d1, d2, p1,
                                                     p2, cola);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_add_lpt_momentum(float* mom, const float* psi1, const float* psi2, size_t np3, float p1, float p2,
                                     cudaStream_t s) {
-    k_add_lpt_momentum<<<blocks(3 * np3, 256), 256, 0, s>>>(mom, psi1, psi2, 3 * np3, p1, p2);
-    return cudaGetLastError();
+    return launch_dep(np3 <= (size_t)128 * 128 * 128, k_add_lpt_momentum, blocks(3 * np3, 256), 256, 0, s, mom, psi1, psi2, 3 * np3, p1, p2);
 }
 
 cudaError_t launch_export_particles(const float4* pos, const float* mom, const int* id, size_t np3, int nm, float cell,
                                     float* pos_xyz, float* mom_xyz, cudaStream_t s) {
-    k_export_particles<<<blocks(np3, 256), 256, 0, s>>>(pos, mom, id, np3, make_udiv(nm), cell, pos_xyz, mom_xyz);
-    return cudaGetLastError();
+    return launch_dep(overlap_mesh(nm), k_export_particles, blocks(np3, 256), 256, 0, s, pos, mom, id, np3, make_udiv(nm), cell, pos_xyz, mom_xyz);
 }
 
 cudaError_t launch_export_state(const float4* pos, const float* mom, size_t np3, int nm, int* cell_xyz, float* off_xyz,
                                 float* mom_xyz, cudaStream_t s) {
-    k_export_state<<<blocks(np3, 256), 256, 0, s>>>(pos, mom, np3, nm, cell_xyz, off_xyz, mom_xyz);
-    return cudaGetLastError();
+    return launch_dep(overlap_mesh(nm), k_export_state, blocks(np3, 256), 256, 0, s, pos, mom, np3, nm, cell_xyz, off_xyz, mom_xyz);
 }
 
 cudaError_t launch_import_state(float4* pos, float* mom, size_t np3, int nm, const int* cell_xyz, const float* off_xyz,
@@ -656,8 +668,7 @@ cudaError_t launch_import_state(float4* pos, float* mom, size_t np3, int nm, con
 
 cudaError_t launch_export_displacement(const float4* pos, int np, int nm, float cell, float* psi, cudaStream_t s) {
     const size_t np3 = (size_t)np * np * np;
-    k_export_displacement<<<blocks(np3, 256), 256, 0, s>>>(pos, np3, make_lattice(np, nm), cell, psi);
-    return cudaGetLastError();
+    return launch_dep(overlap_mesh(nm), k_export_displacement, blocks(np3, 256), 256, 0, s, pos, np3, make_lattice(np, nm), cell, psi);
 }
 
 cudaError_t launch_import_displacement(float4* pos, int np, int nm, float to_mesh, const float* psi, int* err,
@@ -676,10 +687,8 @@ cudaError_t launch_rsd_positions(const float4* pos, const float* mom, size_t np3
 cudaError_t launch_scale(float* dst, const float* src, size_t n, float f, cudaStream_t s) {
     // a caller's array may start at any float
     if (n % 4 == 0 && (reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) % 16 == 0)
-        k_scale<4><<<blocks(n / 4, 256), 256, 0, s>>>(dst, src, n, f);
-    else
-        k_scale<1><<<blocks(n, 256), 256, 0, s>>>(dst, src, n, f);
-    return cudaGetLastError();
+        return launch_dep(n <= (size_t)3 * 128 * 128 * 128, k_scale<4>, blocks(n / 4, 256), 256, 0, s, dst, src, n, f);
+    return launch_dep(n <= (size_t)3 * 128 * 128 * 128, k_scale<1>, blocks(n, 256), 256, 0, s, dst, src, n, f);
 }
 
 }  // namespace colapm
