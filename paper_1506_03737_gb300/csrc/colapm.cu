@@ -64,6 +64,11 @@ struct colapm_ctx {
     float2* tw_p = nullptr;              // exp(-2 pi i t / np)
     float* sinc2_m = nullptr;            // sinc^2(pi n / nm) per FFT bin, then nm ones (no window)
     float* amp_p = nullptr;              // Gaussian-field amplitude per integer |n|^2 of the IC grid
+    int* err_h = nullptr;                // pinned host copy of err
+    int* pw_host = nullptr;              // pinned: thresholds, then sums of up to three spectra (grown on demand)
+    int pw_hostcap = 0;                  // its bins
+    int pw_nbins = 0;                    // the binning that pw_bin holds
+    double pw_kmin = 0.0, pw_kmax = 0.0;
     int* err = nullptr;                  // device error bits: 1 overflow, 2 bad state import, 4 wait timeout,
                                          // 8 internal (a sort slot out of range)
     // power-spectrum tables (grown on demand)
@@ -147,6 +152,8 @@ void free_all(colapm_ctx* c) {
                     c->fnl_tab, c->fnl_sum, c->lc_out, c->lc_count, c->lc_tab, c->lc_reps};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    if (c->err_h) cudaFreeHost(c->err_h);
+    if (c->pw_host) cudaFreeHost(c->pw_host);
     for (auto& v : c->ev)
         for (auto& pr : v) {
             cudaEventDestroy(pr.first);
@@ -167,9 +174,9 @@ std::vector<float2> twiddles(int n) {
 }
 
 int pending_error(colapm_ctx* c) {
-    int h = 0;
-    CK(cudaMemcpyAsync(&h, c->err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(c->err_h, c->err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    const int h = *c->err_h;
     if (h) CK(cudaMemsetAsync(c->err, 0, sizeof(int), c->stream));
     if (h & 1) return COLAPM_E_OVERFLOW;
     if (h & 2) return COLAPM_E_ARG;
@@ -515,7 +522,8 @@ int colapm_create(const colapm_params* p, void* stream, colapm_ctx** out) {
               dalloc(&c->mom_alt, 3 * c->np3) == cudaSuccess && dalloc(&c->psi1_alt, 3 * c->np3) == cudaSuccess &&
               dalloc(&c->psi2_alt, 3 * c->np3) == cudaSuccess && dalloc(&c->id_alt, c->np3) == cudaSuccess &&
               dalloc(&c->sort_cnt, sort_buckets(c->nm)) == cudaSuccess &&
-              dalloc(&c->sort_tile, sort_tiles(c->nm)) == cudaSuccess;
+              dalloc(&c->sort_tile, sort_tiles(c->nm)) == cudaSuccess &&
+              cudaMallocHost(&c->err_h, sizeof(int)) == cudaSuccess;
     if (ok && xy_supported(c->nm))
         ok = dalloc(reinterpret_cast<char**>(&c->xy_ring), xy_ring_bytes(c->nm)) == cudaSuccess &&
              dalloc(&c->xy_ctr, xy_ctr_ints(c->nm, 3)) == cudaSuccess;
@@ -682,23 +690,21 @@ namespace {
 // accumulators. Bin membership of every integer |n|^2 is decided in FP64 with the same
 // expressions as the definition: |k| = (2 pi / L) sqrt(n^2), e_b = kmin (kmax / kmin)^(b / nbins),
 // e_b <= |k| < e_{b+1}; it is monotone in n^2, so n2_lo[b] = the smallest n^2 with |k| >= e_b.
+// The pinned host block: sums of three spectra (9 pw_hostcap doubles), then the thresholds. Pinned, because every copy
+// to or from pageable memory waits for the stream by itself.
+double* power_host_sums(const colapm_ctx* c) { return reinterpret_cast<double*>(c->pw_host); }
+int* power_host_thresholds(const colapm_ctx* c) { return reinterpret_cast<int*>(power_host_sums(c) + 9 * (size_t)c->pw_hostcap); }
+
 int power_prepare(colapm_ctx* c, int nbins, double kmin, double kmax) {
     if (nbins < 1 || nbins > 4096) return COLAPM_E_ARG;
     const double box = c->prm.box, kf = 2.0 * M_PI / box;
     if (kmin <= 0) kmin = kf;
     if (kmax <= 0) kmax = M_PI * c->nm / box;
     if (!(kmax > kmin)) return COLAPM_E_ARG;
+    if (nbins == c->pw_nbins && kmin == c->pw_kmin && kmax == c->pw_kmax) return COLAPM_OK;   // the device has them
     const int h = c->nm / 2, n2max = 3 * h * h;
-    std::vector<double> edges(nbins + 1);
-    for (int b = 0; b <= nbins; ++b) edges[b] = kmin * std::pow(kmax / kmin, (double)b / nbins);
-    std::vector<int> lo(nbins + 1, n2max + 1);
-    {
-        int b = 0;
-        for (int n2 = 0; n2 <= n2max && b <= nbins; ++n2) {
-            const double km = kf * std::sqrt((double)n2);
-            while (b <= nbins && km >= edges[b]) lo[b++] = n2;   // first n^2 at or above edge b
-        }
-    }
+    CK(cudaStreamSynchronize(c->stream));   // nothing in flight uses the buffers below
+    c->pw_nbins = 0;
     if (nbins + 1 > c->pw_n2cap) {
         if (c->pw_bin) cudaFree(c->pw_bin);
         c->pw_bin = nullptr;
@@ -717,8 +723,22 @@ int power_prepare(colapm_ctx* c, int nbins, double kmin, double kmax) {
         }
         c->pw_nbcap = nbins;
     }
-    CK(cudaMemcpyAsync(c->pw_bin, lo.data(), lo.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
+    if (nbins > c->pw_hostcap) {
+        if (c->pw_host) cudaFreeHost(c->pw_host);
+        c->pw_host = nullptr;
+        c->pw_hostcap = 0;
+        if (cudaMallocHost(&c->pw_host, 9 * (size_t)nbins * sizeof(double) + ((size_t)nbins + 1) * sizeof(int)) != cudaSuccess) {
+            cudaGetLastError();
+            return COLAPM_E_NOMEM;
+        }
+        c->pw_hostcap = nbins;
+    }
+    int* lo = power_host_thresholds(c);
+    power_thresholds(nbins, kmin, kmax, kf, n2max, lo);
+    CK(cudaMemcpyAsync(c->pw_bin, lo, (nbins + 1) * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    c->pw_nbins = nbins;
+    c->pw_kmin = kmin;
+    c->pw_kmax = kmax;
     const double lr = std::log2(kmax / kmin);
     c->pw_lga = (float)(0.5 * nbins / lr);
     c->pw_lgb = (float)(nbins * std::log2(kf / kmin) / lr);
@@ -767,6 +787,35 @@ void power_finish(const double* acc, int nbins, double* ko, double* po, long lon
     }
 }
 
+// Results of a spectrum call into caller arrays that may be host or device (nothing else is in flight).
+int power_deliver(colapm_ctx* c, int nbins, const double* ko, const double* po, const long long* no, double* k_out,
+                  double* p_out, long long* nmodes_out) {
+    bool dev = false;
+    const void* src[3] = {ko, po, no};
+    void* dst[3] = {k_out, p_out, nmodes_out};
+    for (int i = 0; i < 3; ++i) {
+        if (is_device_ptr(dst[i])) {
+            CK(cudaMemcpyAsync(dst[i], src[i], nbins * 8, cudaMemcpyDefault, c->stream));
+            dev = true;
+        } else {
+            std::memcpy(dst[i], src[i], nbins * 8);
+        }
+    }
+    if (dev) CK(cudaStreamSynchronize(c->stream));
+    return COLAPM_OK;
+}
+
+// The spectrum that power_enqueue has queued, into the caller's arrays.
+int power_result(colapm_ctx* c, int nbins, double* k_out, double* p_out, long long* nmodes_out) {
+    double* acc = power_host_sums(c);
+    CK(cudaMemcpyAsync(acc, c->pw_acc, 3 * (size_t)nbins * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    if (int r = pending_error(c)) return r;   // synchronises
+    std::vector<double> ko(nbins), po(nbins);
+    std::vector<long long> no(nbins);
+    power_finish(acc, nbins, ko.data(), po.data(), no.data());
+    return power_deliver(c, nbins, ko.data(), po.data(), no.data(), k_out, p_out, nmodes_out);
+}
+
 }  // namespace
 
 extern "C" {
@@ -779,18 +828,7 @@ int colapm_power(colapm_ctx* c, int nbins, double kmin, double kmax, double* k_o
     if (r) return r;
     r = power_enqueue(c, nbins);
     if (r) return r;
-    std::vector<double> acc(3 * nbins);
-    CK(cudaMemcpyAsync(acc.data(), c->pw_acc, acc.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    r = pending_error(c);   // synchronises
-    if (r) return r;
-    std::vector<double> ko(nbins), po(nbins);
-    std::vector<long long> no(nbins);
-    power_finish(acc.data(), nbins, ko.data(), po.data(), no.data());
-    CK(cudaMemcpyAsync(k_out, ko.data(), nbins * sizeof(double), cudaMemcpyDefault, c->stream));
-    CK(cudaMemcpyAsync(p_out, po.data(), nbins * sizeof(double), cudaMemcpyDefault, c->stream));
-    CK(cudaMemcpyAsync(nmodes_out, no.data(), nbins * sizeof(long long), cudaMemcpyDefault, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    return COLAPM_OK;
+    return power_result(c, nbins, k_out, p_out, nmodes_out);
 }
 
 int colapm_cross_correlation(colapm_ctx* a, colapm_ctx* b, int nbins, double kmin, double kmax, double* k_out,
@@ -804,7 +842,7 @@ int colapm_cross_correlation(colapm_ctx* a, colapm_ctx* b, int nbins, double kmi
     // Bin sums of |delta_a|^2, |delta_b|^2 and |delta_a + delta_b|^2 (the masses of both deposited
     // into one mesh; the transform is linear), without the window: Re(delta_a delta_b^*) is half of
     // the third minus the first two, mode by mode, so also bin by bin.
-    std::vector<double> acc(9 * (size_t)nbins);
+    double* acc = power_host_sums(a);
     DepositSrc src[3];
     src[0] = own_particles(a);
     src[1] = own_particles(b);
@@ -814,22 +852,18 @@ int colapm_cross_correlation(colapm_ctx* a, colapm_ctx* b, int nbins, double kmi
     for (int pass = 0; pass < 3; ++pass) {
         r = power_enqueue(a, nbins, &src[pass], false);
         if (r) return r;
-        CK(cudaMemcpyAsync(acc.data() + (size_t)pass * 3 * nbins, a->pw_acc, 3 * (size_t)nbins * sizeof(double),
+        CK(cudaMemcpyAsync(acc + (size_t)pass * 3 * nbins, a->pw_acc, 3 * (size_t)nbins * sizeof(double),
                            cudaMemcpyDeviceToHost, a->stream));
-        r = pending_error(a);   // synchronises
-        if (r) return r;
     }
+    r = pending_error(a);   // synchronises
+    if (r) return r;
     std::vector<double> ko(nbins), ro(nbins), pa(nbins), pb(nbins), pab(nbins);
     std::vector<long long> no(nbins);
-    power_finish(acc.data(), nbins, ko.data(), pa.data(), no.data());
-    power_finish(acc.data() + 3 * (size_t)nbins, nbins, ko.data(), pb.data(), no.data());
-    power_finish(acc.data() + 6 * (size_t)nbins, nbins, ko.data(), pab.data(), no.data());
+    power_finish(acc, nbins, ko.data(), pa.data(), no.data());
+    power_finish(acc + 3 * (size_t)nbins, nbins, ko.data(), pb.data(), no.data());
+    power_finish(acc + 6 * (size_t)nbins, nbins, ko.data(), pab.data(), no.data());
     for (int i = 0; i < nbins; ++i) ro[i] = no[i] ? 0.5 * (pab[i] - pa[i] - pb[i]) / std::sqrt(pa[i] * pb[i]) : NAN;
-    CK(cudaMemcpyAsync(k_out, ko.data(), nbins * sizeof(double), cudaMemcpyDefault, a->stream));
-    CK(cudaMemcpyAsync(r_out, ro.data(), nbins * sizeof(double), cudaMemcpyDefault, a->stream));
-    CK(cudaMemcpyAsync(nmodes_out, no.data(), nbins * sizeof(long long), cudaMemcpyDefault, a->stream));
-    CK(cudaStreamSynchronize(a->stream));
-    return COLAPM_OK;
+    return power_deliver(a, nbins, ko.data(), ro.data(), no.data(), k_out, r_out, nmodes_out);
 }
 
 int colapm_power_rsd(colapm_ctx* c, int los, int nbins, double kmin, double kmax, double* k_out, double* p_out,
@@ -847,18 +881,7 @@ int colapm_power_rsd(colapm_ctx* c, int los, int nbins, double kmin, double kmax
     src.n[0] = c->np3;
     r = power_enqueue(c, nbins, &src);
     if (r) return r;
-    std::vector<double> acc(3 * nbins);
-    CK(cudaMemcpyAsync(acc.data(), c->pw_acc, acc.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    r = pending_error(c);
-    if (r) return r;
-    std::vector<double> ko(nbins), po(nbins);
-    std::vector<long long> no(nbins);
-    power_finish(acc.data(), nbins, ko.data(), po.data(), no.data());
-    CK(cudaMemcpyAsync(k_out, ko.data(), nbins * sizeof(double), cudaMemcpyDefault, c->stream));
-    CK(cudaMemcpyAsync(p_out, po.data(), nbins * sizeof(double), cudaMemcpyDefault, c->stream));
-    CK(cudaMemcpyAsync(nmodes_out, no.data(), nbins * sizeof(long long), cudaMemcpyDefault, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    return COLAPM_OK;
+    return power_result(c, nbins, k_out, p_out, nmodes_out);
 }
 
 int colapm_get_particles(colapm_ctx* c, float* pos, float* mom) {

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 
@@ -119,6 +120,19 @@ struct PowerArgs {
     // against n2_lo (lga = 0: binary search only)
     float lga, lgb;
 };
+
+// The thresholds n2_lo[0 .. nbins]: the smallest integer |n|^2 <= n2max with kf sqrt(|n|^2) >= kmin (kmax / kmin)^(b / nbins)
+// in FP64, n2max + 1 if none. A first guess from the square of the edge, walked to the place where the comparison
+// itself turns (|k| grows with |n|^2).
+inline void power_thresholds(int nbins, double kmin, double kmax, double kf, int n2max, int* lo) {
+    for (int b = 0; b <= nbins; ++b) {
+        const double edge = kmin * std::pow(kmax / kmin, (double)b / nbins), x = (edge / kf) * (edge / kf);
+        int n = !(x < (double)n2max + 1.0) ? n2max + 1 : (int)x;
+        while (n > 0 && kf * std::sqrt((double)(n - 1)) >= edge) --n;
+        while (n <= n2max && !(kf * std::sqrt((double)n) >= edge)) ++n;
+        lo[b] = n;
+    }
+}
 
 constexpr int kPowerRegions = 16;   // 64 cost up to 8 us more in the final sum and gained nothing
 // FP64 words of the accumulators of `nbins` bins: the result [3 nbins], the regions, the counter.

@@ -26,14 +26,17 @@ constexpr int kMaxBins = COLAPM_NOALLOC_MAX_BINS;
 constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t kRho = 0;                                                        // u64 [nm^3]
 constexpr size_t kSpec = align256(kRho + sizeof(unsigned long long) * kMaxNm * kMaxNm * kMaxNm);   // float2 [nm^3/2]
-constexpr size_t kTw = align256(kSpec + sizeof(float2) * kMaxNm * kMaxNm * kMaxNm / 2);            // float2 [nm]
-constexpr size_t kSinc = align256(kTw + sizeof(float2) * kMaxNm);                  // float [nm]
-constexpr size_t kEdges = align256(kSinc + sizeof(float) * kMaxNm);                // double [nbins + 1]
-constexpr size_t kBin = align256(kEdges + sizeof(double) * (kMaxBins + 1));        // int [nbins + 1] thresholds
-constexpr size_t kAcc = align256(kBin + sizeof(int) * (kMaxBins + 1));             // double [power_words(nbins, kPowerRegions)]
-constexpr size_t kOut = align256(kAcc + sizeof(double) * power_words(kMaxBins, kPowerRegions));            // k, P (double), n (i64)
-constexpr size_t kErr = align256(kOut + sizeof(double) * 3 * kMaxBins);            // int [4]
-constexpr size_t kBytes = align256(kErr + 4 * sizeof(int));
+constexpr size_t kTab = align256(kSpec + sizeof(float2) * kMaxNm * kMaxNm * kMaxNm / 2);           // Tables
+constexpr size_t kErr = align256(kTab + sizeof(float2) * kMaxNm + sizeof(float) * kMaxNm + sizeof(int) * (kMaxBins + 1));   // int
+constexpr size_t kAcc = kErr + 256;                                                // double [power_words(nbins, kPowerRegions)]
+constexpr size_t kBytes = align256(kAcc + sizeof(double) * power_words(kMaxBins, kPowerRegions));
+
+// Constant tables of a call, uploaded in one copy: exp(-2 pi i t / nm), sinc^2 per FFT bin, bin thresholds.
+struct Tables {
+    float2 tw[kMaxNm];
+    float sinc2[kMaxNm];
+    int lo[kMaxBins + 1];
+};
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kBytes];
 
@@ -74,35 +77,6 @@ __global__ void k_deposit_xyz(const int* __restrict__ cell, const float* __restr
             }
 }
 
-// Bin thresholds in FP64: n2_lo[b] = smallest integer |n|^2 with kf sqrt(|n|^2) >= edges[b]
-// (sqrt correctly rounded), n2max + 1 if none; one thread per edge, binary search over |n|^2.
-__global__ void k_bin_thresholds(const double* __restrict__ edges, int nbins, double kf, int n2max,
-                                 int* __restrict__ lo) {
-    pdl_trigger();
-    pdl_wait();
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b > nbins) return;
-    int a = 0, z = n2max + 1;   // find the first n2 in [0, n2max + 1) with kf sqrt(n2) >= edges[b]
-    while (a < z) {
-        const int m = (a + z) >> 1;
-        if (kf * sqrt((double)m) >= edges[b]) z = m; else a = m + 1;
-    }
-    lo[b] = a;
-}
-
-__global__ void k_finish(const double* __restrict__ acc, int nbins, double* __restrict__ out) {
-    pdl_trigger();
-    pdl_wait();
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nbins) return;
-    unsigned long long cnt;
-    memcpy(&cnt, &acc[2 * nbins + b], sizeof(cnt));
-    out[b] = cnt ? acc[b] / (double)cnt : NAN;
-    out[nbins + b] = cnt ? acc[nbins + b] / (double)cnt : NAN;
-    const long long n = (long long)cnt;
-    memcpy(&out[2 * nbins + b], &n, sizeof(n));
-}
-
 std::mutex g_mu;
 unsigned char* g_dev_ptr[64] = {};
 
@@ -116,6 +90,16 @@ bool device_resident(const void* p, int dev) {
     }
     if (a.type == cudaMemoryTypeManaged) return true;
     return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
+// Memory that the host may write (not a device or managed array).
+bool host_memory(const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return a.type != cudaMemoryTypeDevice && a.type != cudaMemoryTypeManaged;
 }
 
 }  // namespace
@@ -151,28 +135,21 @@ extern "C" int colapm_power_noalloc(const int* cell, const float* offset, long l
     }
     auto* rho = reinterpret_cast<unsigned long long*>(base + kRho);
     auto* spec = reinterpret_cast<float2*>(base + kSpec);
-    auto* tw = reinterpret_cast<float2*>(base + kTw);
-    auto* sinc2 = reinterpret_cast<float*>(base + kSinc);
-    auto* edges = reinterpret_cast<double*>(base + kEdges);
-    auto* bin = reinterpret_cast<int*>(base + kBin);
-    auto* acc = reinterpret_cast<double*>(base + kAcc);
-    auto* out = reinterpret_cast<double*>(base + kOut);
+    auto* tab = reinterpret_cast<Tables*>(base + kTab);
     auto* err = reinterpret_cast<int*>(base + kErr);
+    auto* acc = reinterpret_cast<double*>(base + kAcc);
 
     // Host tables on the stack (copied before this call returns; the call synchronises).
-    float2 h_tw[kMaxNm];
-    float h_s2[kMaxNm];
-    double h_edges[kMaxBins + 1];
+    Tables h;
     for (int i = 0; i < nm; ++i) {
         const double ang = 2.0 * M_PI * (double)i / nm;
-        h_tw[i] = make_float2((float)std::cos(ang), (float)-std::sin(ang));
+        h.tw[i] = make_float2((float)std::cos(ang), (float)-std::sin(ang));
         const int sg = i < nm / 2 ? i : i - nm;
         const double x = M_PI * sg / nm;
         const double v = sg == 0 ? 1.0 : std::sin(x) / x;
-        h_s2[i] = (float)(v * v);
+        h.sinc2[i] = (float)(v * v);
     }
-    for (int b = 0; b <= nbins; ++b) h_edges[b] = kmin * std::pow(kmax / kmin, (double)b / nbins);
-    const int n2max = 3 * (nm / 2) * (nm / 2);
+    power_thresholds(nbins, kmin, kmax, kf, 3 * (nm / 2) * (nm / 2), h.lo);
     const size_t nm3 = (size_t)nm * nm * nm;
 
     // Once work is queued, an error return first waits (best effort) for what was queued, so that no
@@ -184,31 +161,45 @@ extern "C" int colapm_power_noalloc(const int* cell, const float* offset, long l
             return COLAPM_E_CUDA;               \
         }                                       \
     } while (0)
-    NCK(cudaMemcpyAsync(tw, h_tw, sizeof(float2) * nm, cudaMemcpyHostToDevice, s));
-    NCK(cudaMemcpyAsync(sinc2, h_s2, sizeof(float) * nm, cudaMemcpyHostToDevice, s));
-    NCK(cudaMemcpyAsync(edges, h_edges, sizeof(double) * (nbins + 1), cudaMemcpyHostToDevice, s));
+    NCK(cudaMemcpyAsync(tab, &h, offsetof(Tables, lo) + sizeof(int) * (nbins + 1), cudaMemcpyHostToDevice, s));
     NCK(cudaMemsetAsync(rho, 0, sizeof(unsigned long long) * nm3, s));
-    NCK(cudaMemsetAsync(acc, 0, sizeof(double) * power_words(nbins, kPowerRegions), s));
-    NCK(cudaMemsetAsync(err, 0, 4 * sizeof(int), s));
-    NCK(launch_dep(true, k_bin_thresholds, (nbins + 128) / 128, 128, 0, s, edges, nbins, kf, n2max, bin));
+    NCK(cudaMemsetAsync(err, 0, (kAcc - kErr) + sizeof(double) * power_words(nbins, kPowerRegions), s));
     NCK(launch_dep(true, k_deposit_xyz, (unsigned)((n_particles + 255) / 256), 256, 0, s, cell, offset, n_particles, nm, rho, err));
     const double ratio = (double)nm3 / (double)n_particles;   // cells per particle
-    NCK(launch_fx_fwd_i64(nm, rho, spec, tw, (float)(ratio * std::ldexp(1.0, -45)), err, s));
-    NCK(launch_fy(nm, -1, spec, 0, 1, tw, s));
+    NCK(launch_fx_fwd_i64(nm, rho, spec, tab->tw, (float)(ratio * std::ldexp(1.0, -45)), err, s));
+    NCK(launch_fy(nm, -1, spec, 0, 1, tab->tw, s));
     PowerArgs pw{};
-    pw.n2_lo = bin;
+    pw.n2_lo = tab->lo;
     pw.kf = (float)kf;
     power_layout(pw, acc, nbins, kPowerRegions);
     pw.pnorm = (float)(box * box * box / ((double)nm3 * (double)nm3));
-    pw.lga = (float)(0.5 * nbins / std::log2(h_edges[nbins] / h_edges[0]));
-    pw.lgb = (float)(nbins * std::log2(kf / h_edges[0]) / std::log2(h_edges[nbins] / h_edges[0]));
-    NCK(launch_fz(nm, Z_POWER, spec, ZOut{}, tw, sinc2, 0, 1.0f, &pw, s));
-    NCK(launch_dep(true, k_finish, (nbins + 127) / 128, 128, 0, s, acc, nbins, out));
-    int h_err = 0;
-    NCK(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
-    NCK(cudaMemcpyAsync(k_out, out, sizeof(double) * nbins, cudaMemcpyDefault, s));
-    NCK(cudaMemcpyAsync(p_out, out + nbins, sizeof(double) * nbins, cudaMemcpyDefault, s));
-    NCK(cudaMemcpyAsync(nmodes_out, out + 2 * nbins, sizeof(long long) * nbins, cudaMemcpyDefault, s));
+    const double lr = std::log2(kmax / kmin);
+    pw.lga = (float)(0.5 * nbins / lr);
+    pw.lgb = (float)(nbins * std::log2(kf / kmin) / lr);
+    NCK(launch_fz(nm, Z_POWER, spec, ZOut{}, tab->tw, tab->sinc2, 0, 1.0f, &pw, s));
+    // the error word and the sums in one copy; the means are formed here
+    struct {
+        int err[(kAcc - kErr) / sizeof(int)];
+        double acc[3 * kMaxBins];
+    } r;
+    NCK(cudaMemcpyAsync(&r, err, (kAcc - kErr) + 3 * (size_t)nbins * sizeof(double), cudaMemcpyDeviceToHost, s));
+    NCK(cudaStreamSynchronize(s));
+    const int h_err = r.err[0];
+    double ko[kMaxBins], po[kMaxBins];
+    long long no[kMaxBins];
+    for (int b = 0; b < nbins; ++b) {
+        unsigned long long cnt;
+        std::memcpy(&cnt, &r.acc[2 * nbins + b], sizeof(cnt));
+        no[b] = (long long)cnt;
+        ko[b] = cnt ? r.acc[b] / (double)cnt : NAN;
+        po[b] = cnt ? r.acc[nbins + b] / (double)cnt : NAN;
+    }
+    const void* src[3] = {ko, po, no};
+    void* dst[3] = {k_out, p_out, nmodes_out};
+    for (int i = 0; i < 3; ++i) {
+        if (host_memory(dst[i])) std::memcpy(dst[i], src[i], nbins * 8);
+        else NCK(cudaMemcpyAsync(dst[i], src[i], nbins * 8, cudaMemcpyDefault, s));
+    }
     NCK(cudaStreamSynchronize(s));
 #undef NCK
     if (h_err & 2) return COLAPM_E_ARG;

@@ -1,5 +1,5 @@
 // Host check of the index arithmetic of the particle kernels: UDiv against the ordinary division, and the
-// Lattice sites against their definition i nm / np.
+// Lattice sites against their definition i nm / np, and the P(k) bin thresholds against a search through every |n|^2.
 #include <cstdio>
 
 #include "../paper_1506_03737_gb300/csrc/colapm_internal.h"
@@ -41,6 +41,22 @@ int main() {
                 bad += base != t / np || frac != (float)(t % np) / (float)np;
             }
         }
+    for (int nm : {16, 64, 96, 256})
+        for (int nbins : {1, 7, 100, 700})
+            for (double box : {100.0, 256.0, 512.7})
+                for (int k = 0; k < 4; ++k) {   // default range, edges on modes, a narrow range, edges beyond the mesh
+                    const double kf = 2.0 * M_PI / box, ny = M_PI * nm / box;
+                    const double kmin = k == 1 ? 2.0 * kf : (k == 2 ? 0.31 * ny : (k == 3 ? 0.01 * kf : kf));
+                    const double kmax = k == 1 ? 6.0 * kf : (k == 2 ? 0.33 * ny : (k == 3 ? 100.0 * ny : ny));
+                    const int n2max = 3 * (nm / 2) * (nm / 2);
+                    static int lo[701];
+                    colapm::power_thresholds(nbins, kmin, kmax, kf, n2max, lo);
+                    for (int b = 0, n2 = 0; b <= nbins; ++b) {
+                        const double edge = kmin * std::pow(kmax / kmin, (double)b / nbins);
+                        while (n2 <= n2max && !(kf * std::sqrt((double)n2) >= edge)) ++n2;   // edges grow
+                        bad += lo[b] != n2;
+                    }
+                }
     printf("%ld mismatches\n", bad);
     return bad != 0;
 }
