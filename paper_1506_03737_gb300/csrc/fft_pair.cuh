@@ -1,4 +1,4 @@
-// Paired-lane 32-point transforms for the 1024-point z pass of the force (L = 32 x 32).
+// Paired-lane 32-point transforms for the z passes of the force of 1024 (32 x 32) and 512 points (16 x 32).
 //
 // The two-stage z pass gives every radix-32 task to one thread, which then holds 32 complex
 // values: with the saved base in shared memory that allows 12 warps per SM. Here a task is split
@@ -91,7 +91,7 @@ __host__ __device__ __forceinline__ void pair_twiddle(float2* v, const Tw2* t, i
 
 #ifdef __CUDACC__
 __device__ __forceinline__ float2 pair_swap(float2 a) {
-    return make_float2(__shfl_xor_sync(0xffffffffu, a.x, 4), __shfl_xor_sync(0xffffffffu, a.y, 4));
+    return make_float2(__shfl_xor_sync(0xffffffffu, a.x, 16), __shfl_xor_sync(0xffffffffu, a.y, 16));
 }
 // The exchanges on the device: every send first, then the shuffles, then every finish (the same
 // arithmetic as index by index; measured faster than interleaving them at 2 CTAs per SM).
@@ -119,10 +119,12 @@ __device__ __forceinline__ void pair_dif(float2* v, int h) {
 
 // ---------------------------------------------------------------------------------------------
 // Force z pass, 1024-point lines, blocked layout, 4-column tiles, 256 threads: thread
-// (c, h, j) = (tid & 3, (tid >> 2) & 1, tid >> 3) is half h of task j of column c (the partner is
-// lane ^ 4). The chain is that of k2_fz<1024, Z_FORCE, 4, true>: forward z (stage A DIT from
-// global memory, exchange, stage B DIT), the Green's function with CIC deconvolution, the saved
-// base B = k_z A in shared memory, and two inverse z transforms (stage A DIF, exchange, stage B
+// c = tid & 3, h = (tid >> 4) & 1, j = the other bits is half h of task j of column c. The partner is
+// lane ^ 16, so that the 16 lanes of a shared-memory phase are 4 columns x 4 tasks of one half: with the
+// exchange buffer's pitch (4 mod 16) they fall on 16 different 8-byte banks (as lane ^ 4 the halves met two
+// by two: 4.93 ms per pass at 1024^3, 4.59 now). The chain is that of k2_fz<1024, Z_FORCE, 4, true>: forward
+// z (stage A DIT from global memory, exchange, stage B DIT), the Green's function with CIC deconvolution,
+// the saved base B = k_z A in shared memory, and two inverse z transforms (stage A DIF, exchange, stage B
 // DIT) written as the bases A' (field 0) and B' (field 2).
 constexpr int PZ_T = 256;
 
@@ -141,7 +143,7 @@ __global__ void __launch_bounds__(PZ_T, MINB)
     pdl_wait();
     __syncthreads();
     const float kf = 6.283185307179586f / (float)L;
-    const int tid = threadIdx.x, c = tid & 3, h = (tid >> 2) & 1, j = tid >> 3;
+    const int tid = threadIdx.x, c = tid & 3, h = (tid >> 4) & 1, j = ((tid >> 2) & 3) + 4 * (tid >> 5);
     // tile -> (ky, kx0) as in k2_fz (blocked layout, 4-column tiles)
     auto tile_of = [&](int tt, int& ky_, int& kx0_) {
         const int qq = tt >> 3;
@@ -219,6 +221,96 @@ __global__ void __launch_bounds__(PZ_T, MINB)
         }
     }
 }
+
+// ---------------------------------------------------------------------------------------------
+// The same pass for 512-point lines (L = 16 x 32): the radix-16 stages keep one thread per task, the radix-32 ones
+// use a pair, so that all 128 threads of a 4-column tile work in every stage with 16 values each. With one
+// thread per task the radix-32 stages left half of the threads waiting at the barrier and held 32
+// values: 530 us at 512^3 with 3 CTAs per SM, 457 now with 4 (500 with 5, 587 with 6: more tiles in flight
+// only queue for the L1 data path, which is 71% busy; a 32-byte row of the mesh costs it as much as
+// 128 bytes of shared memory).
+constexpr int PZ5_T = 128, PZ5_MINB = 4;
+
+static __global__ void __launch_bounds__(PZ5_T, PZ5_MINB)
+    k2_fz_pair512(const float2* __restrict__ in, ZOut out, const float2* __restrict__ tw, const float* __restrict__ sinc2,
+                  int deconv, float gnorm) {
+    constexpr int L = 512, RA = 16, RB = 32, n = L / 2, C = 4, NTILE = (n / C) * L;
+    using XF = Xch<L, RA, C>;   // forward exchange (and the saved base)
+    using XI = Xch<L, RB, C>;   // inverse exchange
+    extern __shared__ float4 smem4[];
+    float2* xb = reinterpret_cast<float2*>(smem4);
+    float2* save = xb + (XF::SIZE > XI::SIZE ? XF::SIZE : XI::SIZE);
+    Tw2* tws = reinterpret_cast<Tw2*>(save + XF::SIZE);
+    pdl_trigger();
+    load_tw2<L, L>(tws, tw, PZ5_T);
+    pdl_wait();
+    __syncthreads();
+    const float kf = 6.283185307179586f / (float)L;
+    const int tid = threadIdx.x, c = tid & 3;
+    const int ja = tid >> 2;                                                              // radix-16 task (32 of them)
+    const int h = (tid >> 4) & 1, jb = ((tid >> 2) & 3) + 4 * (tid >> 5);                 // half of a radix-32 task (16)
+    for (int t = blockIdx.x; t < NTILE; t += gridDim.x) {
+        // tile -> (ky, kx0) as in k2_fz (blocked layout, 4-column tiles)
+        const int qq = t >> 3;
+        const int ky = 8 * (qq / (2 * (n / 8))) + (t & 7), kx0 = ((qq / 2) % (n / 8)) * 8 + (qq % 2) * C;
+        const size_t base = hs_index<L, true>(kx0 + c, ky, 0);
+        const int ny = sbin(ky, L), nx = kx0 + c;
+        const bool nyq_y = ky == L / 2;
+        float2 v[16];
+        // forward stage A: inputs z = ja + 32 r
+#pragma unroll
+        for (int r = 0; r < RA; ++r) v[r] = __ldcg(in + base + (size_t)(ja + RB * r) * 64);
+        dft<RA, -1>(v);
+#pragma unroll
+        for (int r = 0; r < RA; ++r) xb[XF::at(c, ja * RA + r)] = v[r];
+        __syncthreads();
+        // forward stage B: inputs jb + 16 r, r = 2m + h; outputs X[jb + 16 r], r = pair_dit_r(q, h)
+#pragma unroll
+        for (int m = 0; m < 16; ++m) v[m] = xb[XF::at(c, jb + RA * (2 * m + h))];
+        pair_twiddle<-1>(v, tws, jb, h);
+        dft<16, -1>(v);
+        pair_dit<-1>(v, h);
+        // bases: A = g X, B = k_z A; g = gnorm / (k^2 W^d), 0 on excluded modes
+        const int nxy2 = nx * nx + ny * ny;
+        const float wxy = deconv ? sinc2[nx] * sinc2[ky] : 1.0f;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            const int z = jb + RA * pair_dit_r(q, h);
+            const int nz = sbin(z, L);
+            const int n2 = nxy2 + nz * nz;
+            float w = 1.0f;
+            if (deconv) {
+                w = wxy * sinc2[z];
+                if (deconv == 2) w *= w;
+            }
+            const float g = !nyq_y && z != L / 2 && n2 != 0 ? __fdividef(gnorm, kf * kf * (float)n2 * w) : 0.0f;
+            v[q] = cscale(v[q], g);
+            save[XF::at(c, z)] = cscale(v[q], kf * (float)nz);
+        }
+        __syncthreads();   // forward exchange buffer free
+#pragma unroll 1
+        for (int bi = 0; bi < 2; ++bi) {
+            if (bi > 0) {
+#pragma unroll
+                for (int q = 0; q < 16; ++q) v[q] = save[XF::at(c, jb + RA * pair_dit_r(q, h))];
+            }
+            // inverse stage A (radix 32, DIF): outputs 2m + h of task jb
+            pair_dif<+1>(v, h);
+#pragma unroll
+            for (int m = 0; m < 16; ++m) xb[XI::at(c, jb * RB + 2 * m + h)] = v[m];
+            __syncthreads();
+            // inverse stage B (radix 16): inputs and outputs ja + 32 r
+            stage_b<L, RB, RA, +1, C>(xb, tws, c, ja, v);
+            float2* dst = out.p[bi == 0 ? 0 : 2];
+#pragma unroll
+            for (int r = 0; r < RA; ++r) dst[base + (size_t)(ja + RB * r) * 64] = v[r];
+            __syncthreads();   // exchange buffer free for the next base / tile
+        }
+    }
+}
+constexpr size_t PZ5_SMEM =
+    sizeof(float2) * ((size_t)(Xch<512, 16, 4>::SIZE > Xch<512, 32, 4>::SIZE ? Xch<512, 16, 4>::SIZE : Xch<512, 32, 4>::SIZE) +
+                      Xch<512, 16, 4>::SIZE) + sizeof(Tw2);
 
 template <int MINB>
 struct PairZ {
