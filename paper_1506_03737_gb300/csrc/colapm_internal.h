@@ -331,10 +331,10 @@ cudaError_t launch_deposit(const float4* pos, size_t np3, int nm, unsigned long 
 cudaError_t launch_gather_kick_drift(float4* pos, float* mom, const float* psi1, const float* psi2,
                                      const float* force, size_t np3, int nm, StepCoef c, int drift,
                                      cudaStream_t s, int block = 256, const LightconeStep* lc = nullptr);
-// Particle p gets id p; psi1 / psi2 are rewritten only where to_mesh is not 1.
-cudaError_t launch_init_particles(float4* pos, float* mom, int* id, float* psi1, float* psi2, int np, int nm,
-                                  float to_mesh, float d1, float d2, float p1, float p2, int cola,
-                                  cudaStream_t s);
+// Particle p gets id p and the displacements src1 / src2 (both psi1 / psi2, or neither: other arrays) times to_mesh.
+cudaError_t launch_init_particles(float4* pos, float* mom, int* id, const float* src1, const float* src2, float* psi1,
+                                  float* psi2, int np, int nm, float to_mesh, float d1, float d2, float p1, float p2,
+                                  int cola, cudaStream_t s);
 cudaError_t launch_add_lpt_momentum(float* mom, const float* psi1, const float* psi2, size_t np3, float p1,
                                     float p2, cudaStream_t s);
 // Writes particle p's values at its id (id may be NULL: slot order is id order).

@@ -343,12 +343,13 @@ __global__ void __launch_bounds__(MW_T) k_multi_gather_kick_drift(const MockWork
 }
 
 // Particles on the Lagrangian lattice (offset by half a PM cell), displaced by D1 Psi1 + D2 Psi2, and their ids.
-// psi1 / psi2 arrive in some unit and leave in PM-mesh cells (factor to_mesh; not rewritten where it is 1).
+// src1 / src2 hold the displacements in some unit, psi1 / psi2 receive them in PM-mesh cells (factor to_mesh;
+// not rewritten where they are the same arrays and the factor is 1).
 // Bound by its 56 bytes per particle (24 more with a factor): the index arithmetic goes through
 // multiplications (UDiv), the ids were a pass of their own. 256^3: 244 + 35 us before, 168 now.
 __global__ void k_init_particles(float4* __restrict__ pos, float* __restrict__ mom, int* __restrict__ id,
-                                 float* __restrict__ psi1, float* __restrict__ psi2, size_t np3, Lattice lat, float to_mesh,
-                                 float d1, float d2, float p1, float p2, int cola) {
+                                 const float* src1, const float* src2, float* psi1, float* psi2, size_t np3, Lattice lat,
+                                 float to_mesh, float d1, float d2, float p1, float p2, int cola) {
     pdl_trigger();
     pdl_wait();
     const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -359,8 +360,8 @@ __global__ void k_init_particles(float4* __restrict__ pos, float* __restrict__ m
     float o[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        const float s1 = psi1[j * np3 + p] * to_mesh, s2 = psi2[j * np3 + p] * to_mesh;
-        if (to_mesh != 1.0f) {
+        const float s1 = src1[j * np3 + p] * to_mesh, s2 = src2[j * np3 + p] * to_mesh;
+        if (to_mesh != 1.0f || src1 != psi1) {
             psi1[j * np3 + p] = s1;
             psi2[j * np3 + p] = s2;
         }
@@ -638,10 +639,10 @@ cudaError_t launch_multi_gather_kick_drift(const MockWork* w, int nmock, long lo
     return launch_dep(false, k_multi_gather_kick_drift, nitems < grid ? (int)nitems : grid, MW_T, 0, s, w, nmock, nitems, queue);
 }
 
-cudaError_t launch_init_particles(float4* pos, float* mom, int* id, float* psi1, float* psi2, int np, int nm, float to_mesh,
+cudaError_t launch_init_particles(float4* pos, float* mom, int* id, const float* src1, const float* src2, float* psi1, float* psi2, int np, int nm, float to_mesh,
                                   float d1, float d2, float p1, float p2, int cola, cudaStream_t s) {
     const size_t np3 = (size_t)np * np * np;
-    return launch_dep(overlap_mesh(nm), k_init_particles, blocks(np3, 256), 256, 0, s, pos, mom, id, psi1, psi2, np3, make_lattice(np, nm), to_mesh, d1, d2, p1,
+    return launch_dep(overlap_mesh(nm), k_init_particles, blocks(np3, 256), 256, 0, s, pos, mom, id, src1, src2, psi1, psi2, np3, make_lattice(np, nm), to_mesh, d1, d2, p1,
                                                     p2, cola);
 }
 
