@@ -10,6 +10,7 @@
 
 #include "colapm_internal.h"
 #include "cosmology.h"
+#include "tma.cuh"
 
 using namespace colapm;
 
@@ -22,6 +23,7 @@ struct colapm_ctx {
     // device buffers
     unsigned long long* rho = nullptr;   // nm^3 int64 fixed-point density
     float* F = nullptr;                  // 3 nm^3: density spectrum, then the three force meshes
+    CUtensorMap zmaps[2];                // boxes of fields 0 and 2 of F for the force z pass (512, 1024; ZOut)
     float* Freal = nullptr;              // 3 nm^3: the real force meshes when the spectra use the blocked layout
     float4* pos = nullptr;               // np^3 (offsets, cell bits)
     float* mom = nullptr;                // 3 np^3, cells
@@ -325,6 +327,8 @@ int force_from_density(colapm_ctx* c, float* dst = nullptr) {
         out.p[0] = d;
         out.p[1] = d + fs;
         out.p[2] = d + 2 * fs;
+        out.maps = c->zmaps;
+        out.err = c->err;
         const float gnorm = (float)(1.0 / ((double)c->nm * c->nm * c->nm));
         CKL(launch_fz(c->nm, Z_FORCE, d, out, c->tw_m, c->sinc2_m, c->prm.deconv, gnorm, nullptr, c->stream,
                       ts(c, COLAPM_PLAN_Z), use_blocked(c)));
@@ -546,6 +550,16 @@ int colapm_create(const colapm_params* p, void* stream, colapm_ctx** out) {
         free_all(c);
         delete c;
         return COLAPM_E_NOMEM;
+    }
+    if (c->nm == 512 || c->nm == 1024) {   // [kx/8][y/8][z][y%8][kx%8]: 64 complex per z of an 8 x 8 block of columns
+        const cuuint64_t n = c->nm, dims[3] = {64, n, n / 16 * (n / 8)}, strides[2] = {512, n * 512};
+        const cuuint32_t box[3] = {4, 256, 1};
+        for (int f = 0; f < 2; ++f)
+            if (!encode_box3(&c->zmaps[f], c->F + 2 * f * c->nm3, dims, strides, box)) {
+                free_all(c);
+                delete c;
+                return COLAPM_E_CUDA;
+            }
     }
     std::vector<float2> tm = twiddles(c->nm), tp = twiddles(c->np);
     std::vector<float> s2(2 * c->nm, 1.0f);

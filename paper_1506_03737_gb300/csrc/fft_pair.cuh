@@ -22,6 +22,7 @@
 #pragma once
 
 #include "fft2.cuh"
+#include "tma.cuh"
 
 namespace colapm {
 
@@ -128,49 +129,80 @@ __device__ __forceinline__ void pair_dif(float2* v, int h) {
 // DIT) written as the bases A' (field 0) and B' (field 2).
 constexpr int PZ_T = 256;
 
+// Tile t of the blocked layout: its columns (ky, kx0 .. kx0 + 3) as in k2_fz, and its place in the tensor maps.
+template <int L>
+__device__ __forceinline__ void pair_tile(int t, int& ky, int& kx0) {
+    constexpr int n = L / 2;
+    const int q = t >> 3;
+    ky = 8 * (q / (2 * (n / 8))) + (t & 7);
+    kx0 = ((q / 2) % (n / 8)) * 8 + (q % 2) * 4;
+}
+
+// The tile buffer: [z][4 columns] dense in shared memory, moved by boxes of 256 z each. Through the L1 data path
+// a 32-byte row costs a whole wavefront, in each direction, which was what bounded the pass (71% busy at
+// 512^3); the boxes bypass it, and the tile after this one arrives while the second base is transformed.
+template <int L>
+__device__ __forceinline__ void pair_load(float2* buf, const CUtensorMap& map, int t, uint32_t bar) {
+    int ky, kx0;
+    pair_tile<L>(t, ky, kx0);
+    mbar_expect(bar, L * 32);
+#pragma unroll
+    for (int z = 0; z < L; z += 256)
+        box_load(smem_u32(buf + 4 * z), map, (ky & 7) * 8 + (kx0 & 7), z, (kx0 >> 3) * (L / 8) + (ky >> 3), bar);
+}
+template <int L>
+__device__ __forceinline__ void pair_store(const float2* buf, const CUtensorMap& map, int ky, int kx0) {
+#pragma unroll
+    for (int z = 0; z < L; z += 256)
+        box_store(map, (ky & 7) * 8 + (kx0 & 7), z, (kx0 >> 3) * (L / 8) + (ky >> 3), smem_u32(buf + 4 * z));
+}
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
+
 template <int MINB>
 __global__ void __launch_bounds__(PZ_T, MINB)
-    k2_fz_pair(const float2* __restrict__ in, ZOut out, const float2* __restrict__ tw, const float* __restrict__ sinc2,
-               int deconv, float gnorm) {
+    k2_fz_pair(const __grid_constant__ CUtensorMap f0, const __grid_constant__ CUtensorMap f2, const float2* __restrict__ tw,
+               const float* __restrict__ sinc2, int deconv, float gnorm, int* err) {
     constexpr int L = 1024, R = 32, n = L / 2, C = 4, NTILE = (n / C) * L;
     using X = Xch<L, R, C>;
-    extern __shared__ float4 smem4[];
+    extern __shared__ __align__(128) float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
-    float2* save = xb + X::SIZE;
-    Tw2* tws = reinterpret_cast<Tw2*>(save + X::SIZE);
+    float2* save = xb + X::SIZE;   // the saved base, then the tile of the second output
+    float2* buf = save + X::SIZE;  // the input tile, then that of the first output
+    static_assert(X::SIZE * sizeof(float2) % 128 == 0 && X::SIZE >= L * C, "box copies start at multiples of 128 bytes");
+    Tw2* tws = reinterpret_cast<Tw2*>(buf + L * C);
+    const uint32_t bar = smem_u32(tws + 1);
     pdl_trigger();
     load_tw2<L, L>(tws, tw, PZ_T);
+    if (threadIdx.x == 0) {
+        mbar_init(bar);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
     pdl_wait();
     __syncthreads();
+    if (threadIdx.x == 0 && blockIdx.x < NTILE) pair_load<L>(buf, f0, blockIdx.x, bar);
     const float kf = 6.283185307179586f / (float)L;
     const int tid = threadIdx.x, c = tid & 3, h = (tid >> 4) & 1, j = ((tid >> 2) & 3) + 4 * (tid >> 5);
-    // tile -> (ky, kx0) as in k2_fz (blocked layout, 4-column tiles)
-    auto tile_of = [&](int tt, int& ky_, int& kx0_) {
-        const int qq = tt >> 3;
-        ky_ = 8 * (qq / (2 * (n / 8))) + (tt & 7);
-        kx0_ = ((qq / 2) % (n / 8)) * 8 + (qq % 2) * C;
-    };
-    auto load_a = [&](int tt, float2* dst) {
-        int ky_, kx0_;
-        tile_of(tt, ky_, kx0_);
-        const size_t b = hs_index<L, true>(kx0_ + c, ky_, 0);
-#pragma unroll
-        for (int m = 0; m < 16; ++m) dst[m] = __ldcg(in + b + (size_t)(j + R * (2 * m + h)) * 64);
-    };
-    for (int t = blockIdx.x; t < NTILE; t += gridDim.x) {
+    uint32_t phase = 0;
+    for (int t = blockIdx.x; t < NTILE; t += gridDim.x, phase ^= 1) {
         int ky, kx0;
-        tile_of(t, ky, kx0);
-        const size_t base = hs_index<L, true>(kx0 + c, ky, 0);
+        pair_tile<L>(t, ky, kx0);
         const int ny = sbin(ky, L), nx = kx0 + c;
         const bool nyq_y = ky == L / 2;
         float2 v[16];
         // forward stage A: inputs z = j + 32 r, r = 2m + h
-        load_a(t, v);
+        bool ok = mbar_wait(bar, phase);
+        if (!ok) {   // flag it, let the copy land, stop
+            atomicOr(err, 4);
+            mbar_wait(bar, phase);
+        }
+#pragma unroll
+        for (int m = 0; m < 16; ++m) v[m] = buf[(j + R * (2 * m + h)) * C + c];
         dft<16, -1>(v);
         pair_dit<-1>(v, h);
 #pragma unroll
         for (int q = 0; q < 16; ++q) xb[X::at(c, j * R + pair_dit_r(q, h))] = v[q];
-        __syncthreads();
+        if (tid == 0) box_stores_read();   // the last tile's second output has left `save`
+        if (!__syncthreads_and(ok)) break;
         // forward stage B: inputs j + 32 r, r = 2m + h; outputs X[j + 32 r], r = pair_dit_r(q, h)
 #pragma unroll
         for (int m = 0; m < 16; ++m) v[m] = xb[X::at(c, j + R * (2 * m + h))];
@@ -207,6 +239,10 @@ __global__ void __launch_bounds__(PZ_T, MINB)
             pair_dif<+1>(v, h);
 #pragma unroll
             for (int m = 0; m < 16; ++m) xb[X::at(c, j * R + 2 * m + h)] = v[m];
+            if (bi > 0 && tid == 0) {   // the first output has left the tile buffer: the next tile
+                box_stores_read();
+                if (t + (int)gridDim.x < NTILE) pair_load<L>(buf, f0, t + gridDim.x, bar);
+            }
             __syncthreads();
             // inverse stage B: inputs j + 32 r, r = 2m + h; outputs z = j + 32 pair_dit_r(q, h)
 #pragma unroll
@@ -214,12 +250,15 @@ __global__ void __launch_bounds__(PZ_T, MINB)
             pair_twiddle<+1>(v, tws, j, h);
             dft<16, +1>(v);
             pair_dit<+1>(v, h);
-            float2* dst = out.p[bi == 0 ? 0 : 2];
+            float2* dst = bi == 0 ? buf : save;
 #pragma unroll
-            for (int q = 0; q < 16; ++q) dst[base + (size_t)(j + R * pair_dit_r(q, h)) * 64] = v[q];
-            __syncthreads();   // exchange buffer free for the next base / tile
+            for (int q = 0; q < 16; ++q) dst[(j + R * pair_dit_r(q, h)) * C + c] = v[q];
+            fence_async_smem();
+            __syncthreads();   // the output tile is complete, the exchange buffer free for the next base / tile
+            if (tid == 0) pair_store<L>(dst, bi == 0 ? f0 : f2, ky, kx0);
         }
     }
+    if (tid == 0) box_stores_done();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -232,38 +271,52 @@ __global__ void __launch_bounds__(PZ_T, MINB)
 constexpr int PZ5_T = 128, PZ5_MINB = 4;
 
 static __global__ void __launch_bounds__(PZ5_T, PZ5_MINB)
-    k2_fz_pair512(const float2* __restrict__ in, ZOut out, const float2* __restrict__ tw, const float* __restrict__ sinc2,
-                  int deconv, float gnorm) {
+    k2_fz_pair512(const __grid_constant__ CUtensorMap f0, const __grid_constant__ CUtensorMap f2, const float2* __restrict__ tw,
+                  const float* __restrict__ sinc2, int deconv, float gnorm, int* err) {
     constexpr int L = 512, RA = 16, RB = 32, n = L / 2, C = 4, NTILE = (n / C) * L;
     using XF = Xch<L, RA, C>;   // forward exchange (and the saved base)
     using XI = Xch<L, RB, C>;   // inverse exchange
-    extern __shared__ float4 smem4[];
+    constexpr int XS = XF::SIZE > XI::SIZE ? XF::SIZE : XI::SIZE;
+    static_assert(XS * sizeof(float2) % 128 == 0 && XF::SIZE * sizeof(float2) % 128 == 0 && XF::SIZE >= L * C, "box copies");
+    extern __shared__ __align__(128) float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
-    float2* save = xb + (XF::SIZE > XI::SIZE ? XF::SIZE : XI::SIZE);
-    Tw2* tws = reinterpret_cast<Tw2*>(save + XF::SIZE);
+    float2* save = xb + XS;            // the saved base, then the tile of the second output
+    float2* buf = save + XF::SIZE;     // the input tile, then that of the first output
+    Tw2* tws = reinterpret_cast<Tw2*>(buf + L * C);
+    const uint32_t bar = smem_u32(tws + 1);
     pdl_trigger();
     load_tw2<L, L>(tws, tw, PZ5_T);
+    if (threadIdx.x == 0) {
+        mbar_init(bar);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
     pdl_wait();
     __syncthreads();
+    if (threadIdx.x == 0 && blockIdx.x < NTILE) pair_load<L>(buf, f0, blockIdx.x, bar);
     const float kf = 6.283185307179586f / (float)L;
     const int tid = threadIdx.x, c = tid & 3;
     const int ja = tid >> 2;                                                              // radix-16 task (32 of them)
     const int h = (tid >> 4) & 1, jb = ((tid >> 2) & 3) + 4 * (tid >> 5);                 // half of a radix-32 task (16)
-    for (int t = blockIdx.x; t < NTILE; t += gridDim.x) {
-        // tile -> (ky, kx0) as in k2_fz (blocked layout, 4-column tiles)
-        const int qq = t >> 3;
-        const int ky = 8 * (qq / (2 * (n / 8))) + (t & 7), kx0 = ((qq / 2) % (n / 8)) * 8 + (qq % 2) * C;
-        const size_t base = hs_index<L, true>(kx0 + c, ky, 0);
+    uint32_t phase = 0;
+    for (int t = blockIdx.x; t < NTILE; t += gridDim.x, phase ^= 1) {
+        int ky, kx0;
+        pair_tile<L>(t, ky, kx0);
         const int ny = sbin(ky, L), nx = kx0 + c;
         const bool nyq_y = ky == L / 2;
         float2 v[16];
         // forward stage A: inputs z = ja + 32 r
+        bool ok = mbar_wait(bar, phase);
+        if (!ok) {   // flag it, let the copy land, stop
+            atomicOr(err, 4);
+            mbar_wait(bar, phase);
+        }
 #pragma unroll
-        for (int r = 0; r < RA; ++r) v[r] = __ldcg(in + base + (size_t)(ja + RB * r) * 64);
+        for (int r = 0; r < RA; ++r) v[r] = buf[(ja + RB * r) * C + c];
         dft<RA, -1>(v);
 #pragma unroll
         for (int r = 0; r < RA; ++r) xb[XF::at(c, ja * RA + r)] = v[r];
-        __syncthreads();
+        if (tid == 0) box_stores_read();   // the last tile's second output has left `save`
+        if (!__syncthreads_and(ok)) break;
         // forward stage B: inputs jb + 16 r, r = 2m + h; outputs X[jb + 16 r], r = pair_dit_r(q, h)
 #pragma unroll
         for (int m = 0; m < 16; ++m) v[m] = xb[XF::at(c, jb + RA * (2 * m + h))];
@@ -298,23 +351,30 @@ static __global__ void __launch_bounds__(PZ5_T, PZ5_MINB)
             pair_dif<+1>(v, h);
 #pragma unroll
             for (int m = 0; m < 16; ++m) xb[XI::at(c, jb * RB + 2 * m + h)] = v[m];
+            if (bi > 0 && tid == 0) {   // the first output has left the tile buffer: the next tile
+                box_stores_read();
+                if (t + (int)gridDim.x < NTILE) pair_load<L>(buf, f0, t + gridDim.x, bar);
+            }
             __syncthreads();
             // inverse stage B (radix 16): inputs and outputs ja + 32 r
             stage_b<L, RB, RA, +1, C>(xb, tws, c, ja, v);
-            float2* dst = out.p[bi == 0 ? 0 : 2];
+            float2* dst = bi == 0 ? buf : save;
 #pragma unroll
-            for (int r = 0; r < RA; ++r) dst[base + (size_t)(ja + RB * r) * 64] = v[r];
-            __syncthreads();   // exchange buffer free for the next base / tile
+            for (int r = 0; r < RA; ++r) dst[(ja + RB * r) * C + c] = v[r];
+            fence_async_smem();
+            __syncthreads();   // the output tile is complete, the exchange buffer free for the next base / tile
+            if (tid == 0) pair_store<L>(dst, bi == 0 ? f0 : f2, ky, kx0);
         }
     }
+    if (tid == 0) box_stores_done();
 }
 constexpr size_t PZ5_SMEM =
     sizeof(float2) * ((size_t)(Xch<512, 16, 4>::SIZE > Xch<512, 32, 4>::SIZE ? Xch<512, 16, 4>::SIZE : Xch<512, 32, 4>::SIZE) +
-                      Xch<512, 16, 4>::SIZE) + sizeof(Tw2);
+                      Xch<512, 16, 4>::SIZE + 512 * 4) + sizeof(Tw2) + 8;
 
 template <int MINB>
 struct PairZ {
-    static constexpr size_t SMEM = sizeof(float2) * 2 * (size_t)Xch<1024, 32, 4>::SIZE + sizeof(Tw2);
+    static constexpr size_t SMEM = sizeof(float2) * (2 * (size_t)Xch<1024, 32, 4>::SIZE + 1024 * 4) + sizeof(Tw2) + 8;
 };
 #endif
 

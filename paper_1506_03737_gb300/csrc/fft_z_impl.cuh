@@ -20,20 +20,25 @@ static cudaError_t fz2(float2* in, ZOut out, const float2* tw, const float* sinc
         // held to 80 registers for three CTAs, 5.32 ms with the next tile's inputs loaded into
         // registers during the inverse transforms)
         constexpr int MINB = 2;
+        const auto* maps = static_cast<const CUtensorMap*>(out.maps);
+        if (!maps) return cudaErrorInvalidValue;
         static GridCache cache;
         int grid = 0;
         cudaError_t e = cached_grid(cache, k2_fz_pair<MINB>, PZ_T, PairZ<MINB>::SMEM, &grid);
         if (e != cudaSuccess) return e;
         const int total = (N / 2 / 4) * N;
-        return launch_dep(overlap_mesh(N), k2_fz_pair<MINB>, grid < total ? grid : total, PZ_T, PairZ<MINB>::SMEM, s, in, out, tw, sinc2, deconv, gnorm);
+        return launch_dep(overlap_mesh(N), k2_fz_pair<MINB>, grid < total ? grid : total, PZ_T, PairZ<MINB>::SMEM, s, maps[0], maps[1], tw, sinc2,
+                          deconv, gnorm, out.err);
     } else if constexpr (N == 512 && MODE == Z_FORCE && BLK) {
+        const auto* maps = static_cast<const CUtensorMap*>(out.maps);
+        if (!maps) return cudaErrorInvalidValue;
         static GridCache cache;
         int grid = 0;
         cudaError_t e = cached_grid(cache, k2_fz_pair512, PZ5_T, PZ5_SMEM, &grid);
         if (e != cudaSuccess) return e;
         const int total = (N / 2 / 4) * N;
-        return launch_dep(overlap_mesh(N), k2_fz_pair512, grid < total ? grid : total, PZ5_T, PZ5_SMEM, s, in, out, tw, sinc2,
-                          deconv, gnorm);
+        return launch_dep(overlap_mesh(N), k2_fz_pair512, grid < total ? grid : total, PZ5_T, PZ5_SMEM, s, maps[0], maps[1],
+                          tw, sinc2, deconv, gnorm, out.err);
     } else {
         // Blocked layout: 4-column tiles (32-byte rows whose 512-byte runs the neighbouring tiles
         // complete), which with the prefetch buffer measured 2% faster than 8-column ones (34% for the

@@ -28,7 +28,6 @@
 //   backward-data  da[u][i]   = sum_tap sum_o W[tap][o][i] dz[u - d_tap][o]
 //                             = forward with W'[tap][i][o] = W[26 - tap][o][i], no bias
 //   weight grad    dW[tap][o][i] = sum_v dz[v][o] a[v + d_tap][i];  db[o] = sum_v dz[v][o]
-#include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -42,6 +41,7 @@
 #include "../../include/colapm_nn.h"
 #include "colapm_internal.h"
 #include "launch_cache.h"
+#include "tma.cuh"
 
 namespace colapm {
 namespace nn {
@@ -56,7 +56,6 @@ constexpr int LAYERS = 4;
 constexpr int LSIZE = SLOTS * C * C;           // 7168 master slots per layer
 constexpr int CIN[LAYERS] = {3, 16, 16, 16};
 constexpr int COUT[LAYERS] = {16, 16, 16, 3};
-constexpr long long SPIN_LIMIT = 1ll << 24;    // polls of a bounded wait
 
 enum Epi { EPI_RELU = 0, EPI_OUT = 1, EPI_MASK = 2 };
 
@@ -75,8 +74,6 @@ struct ConvArgs {
     double* loss;                // sum of squared normalised errors
     int* err;                    // bit 4: a bounded wait gave up
 };
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t* r) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
@@ -125,41 +122,6 @@ __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.commit_group;\n" ::);
     asm volatile("cp.async.wait_group 0;\n" ::);
 }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
-}
-// Waits for phase `parity` of a barrier; false when the poll limit was reached.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    uint32_t done = 0;
-    for (long long i = 0; i < SPIN_LIMIT && !done; ++i)
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-                     : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    return done != 0;
-}
-// One box of a stored array into shared memory. The array's elements are 8 bytes (VB / 8 per voxel), so that a whole
-// row of a box is one run; a voxel starts at a multiple of 16 bytes, as the copy wants of its x coordinate.
-template <int VB>
-__device__ __forceinline__ void box_load(uint32_t dst, const CUtensorMap& map, int x, int y, int z, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(&map)), "r"(x * (VB / 8)), "r"(y), "r"(z), "r"(bar)
-        : "memory");
-}
-
-// The box back out of shared memory (written there by ordinary stores), as a bulk group of the calling thread.
-template <int VB>
-__device__ __forceinline__ void box_store(const CUtensorMap& map, int x, int y, int z, uint32_t src) {
-    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];\n" ::"l"(
-                     reinterpret_cast<uint64_t>(&map)),
-                 "r"(x * (VB / 8)), "r"(y), "r"(z), "r"(src)
-                 : "memory");
-    asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
-}
-__device__ __forceinline__ void box_stores_read() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
 
 template <int TZ>
 __device__ __forceinline__ void tile_origin(int t, int n, int& x0, int& y0, int& z0) {
@@ -225,11 +187,11 @@ __global__ void __launch_bounds__(32 * TZ, TZ == 8 ? 2 : 4)
     tile_origin<TZ>(t, n, x0, y0, z0);
     auto load_halo = [&]() {   // stored voxel x0 is the left neighbour of x0
         mbar_expect(bar, S::HALO);
-        box_load<VB>(hb, halo, x0, y0, z0, bar);
+        box_load(hb, halo, x0 * (VB / 8), y0, z0, bar);
     };
     auto load_mask = [&]() {   // this warp's plane of the mask tile
         mbar_expect(mbar, TX * TY * 32);
-        box_load<32>(aux, mask, x0 + 1, y0 + 1, z0 + 1 + tz, mbar);
+        box_load(aux, mask, (x0 + 1) * 4, y0 + 1, z0 + 1 + tz, mbar);
     };
     if (threadIdx.x == 0) load_halo();
 
@@ -339,7 +301,7 @@ __global__ void __launch_bounds__(32 * TZ, TZ == 8 ? 2 : 4)
                     }
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
             __syncwarp();
-            if (lane == 0) box_store<32>(out, cx + 1, cy + 1, cz + tz + 1, aux);
+            if (lane == 0) box_store(out, (cx + 1) * 4, cy + 1, cz + tz + 1, aux);
             // images of the voxels on the faces of the box (n voxels away: the same half slots, n a multiple of 16).
             // Per axis a set of shifts: 0, +n on the low face, -n on the high one
             const int z = cz + tz;
@@ -463,8 +425,8 @@ __global__ void __launch_bounds__(32 * 3 * (TZ / 2), 1)
         tile_origin<TZ>(t, n, x0, y0, z0);
         const uint32_t d = sb + buf * S::BUF, b = bar + 8 * buf;
         mbar_expect(b, S::BUF);
-        box_load<VA>(d, act, x0, y0, z0, b);
-        box_load<VD>(d + S::HALO, dz, x0 + 1, y0 + 1, z0 + 1, b);
+        box_load(d, act, x0 * (VA / 8), y0, z0, b);
+        box_load(d + S::HALO, dz, (x0 + 1) * (VD / 8), y0 + 1, z0 + 1, b);
     };
     // Operand rows are voxels (K), read transposed. As A (M = channels): matrices (lo channels, voxels 0-7),
     // (hi, 0-7), (lo, 8-15), (hi, 8-15). As B (N = channels): (lo, 0-7), (lo, 8-15), (hi, 0-7), (hi, 8-15).
@@ -1043,18 +1005,10 @@ cudaError_t backward(colapm_nn* c) {
 
 // Tensor maps of a stored array of (n + 2)^3 voxels of vb bytes, as 8-byte elements.
 bool encode_maps(colapm_nn::Maps& m, void* p, int n, int vb, bool small) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult st;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &st) != cudaSuccess || !fn)
-        return false;
-    const auto encode = reinterpret_cast<decltype(&cuTensorMapEncodeTiled)>(fn);
     const cuuint64_t e = vb / 8, s = n + 2, dims[3] = {s * e, s, s}, strides[2] = {s * vb, s * s * vb};
-    const cuuint32_t one[3] = {1, 1, 1};
     auto box = [&](CUtensorMap* map, cuuint32_t x, cuuint32_t y, cuuint32_t z) {
         const cuuint32_t b[3] = {(cuuint32_t)(x * e), y, z};
-        return encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, p, dims, strides, b, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                      CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+        return colapm::encode_box3(map, p, dims, strides, b);
     };
     const int cz = small ? 2 : CONV_TZ, wz = small ? 2 : 8;
     return box(&m.halo, HX, HY, cz + 2) && box(&m.whalo, HX, HY, wz + 2) && box(&m.wtile, TX, TY, wz) && box(&m.plane, TX, TY, 1);
