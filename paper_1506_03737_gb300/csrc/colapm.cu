@@ -23,7 +23,7 @@ struct colapm_ctx {
     // device buffers
     unsigned long long* rho = nullptr;   // nm^3 int64 fixed-point density
     float* F = nullptr;                  // 3 nm^3: density spectrum, then the three force meshes
-    CUtensorMap zmaps[2];                // boxes of fields 0 and 2 of F for the force z pass (512, 1024; ZOut)
+    CUtensorMap zmaps[2];                // boxes of fields 0 and 2 of F for the blocked force z pass from 256^3 on (ZOut)
     float* Freal = nullptr;              // 3 nm^3: the real force meshes when the spectra use the blocked layout
     float4* pos = nullptr;               // np^3 (offsets, cell bits)
     float* mom = nullptr;                // 3 np^3, cells
@@ -551,9 +551,9 @@ int colapm_create(const colapm_params* p, void* stream, colapm_ctx** out) {
         delete c;
         return COLAPM_E_NOMEM;
     }
-    if (c->nm == 512 || c->nm == 1024) {   // [kx/8][y/8][z][y%8][kx%8]: 64 complex per z of an 8 x 8 block of columns
+    if (c->nm >= 256) {   // [kx/8][y/8][z][y%8][kx%8]: 64 complex per z of an 8 x 8 block of columns
         const cuuint64_t n = c->nm, dims[3] = {64, n, n / 16 * (n / 8)}, strides[2] = {512, n * 512};
-        const cuuint32_t box[3] = {4, 256, 1};
+        const cuuint32_t box[3] = {4, c->nm >= 512 ? 256u : (c->nm > 256 ? (cuuint32_t)c->nm / 2 : (cuuint32_t)c->nm), 1};
         for (int f = 0; f < 2; ++f)
             if (!encode_box3(&c->zmaps[f], c->F + 2 * f * c->nm3, dims, strides, box)) {
                 free_all(c);

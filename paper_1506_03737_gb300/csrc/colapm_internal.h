@@ -24,7 +24,7 @@ struct StepCoef {
 // Output pointers of a z pass (up to 9 spectra: 3 x Psi1 and 6 x phi_ij of the ICs).
 struct ZOut {
     float2* p[9];
-    // blocked force pass of 512 and 1024 points: boxes of 4 columns x 256 z of fields 0 and 2 (host), and the
+    // blocked force pass: tensor maps of the tile boxes of fields 0 and 2 (two CUtensorMap, host), and the
     // device error word (bit 4: a bounded wait gave up)
     const void* maps = nullptr;
     int* err = nullptr;

@@ -142,12 +142,12 @@ __host__ __device__ __forceinline__ size_t hs_row(int j, int r) {
 
 // Stage B of a line held in exchange buffer xb (stage-A radix RA), task j < RA of line c:
 // loads j + RA r, twiddles, RB-point DFT. Returns X[j + RA r] in v.
-template <int L, int RA, int RB, int S, int LINES = 8>
+template <int L, int RA, int RB, int S, int LINES = 8, bool TRIV = false>
 __host__ __device__ __forceinline__ void stage_b(const float2* xb, const Tw2* tw, int c, int j, float2* v) {
 #pragma unroll
     for (int r = 0; r < RB; ++r) v[r] = xb[Xch<L, RA, LINES>::at(c, j + RA * r)];
     twiddle2<RB, S>(v, tw, j);
-    dft<RB, S>(v);
+    dft<RB, S, TRIV>(v);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -259,6 +259,7 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
         }
     };
     static_assert(!BLK || C == 8 || C == 4, "blocked layout needs 8- or 4-column tiles");
+    static_assert(!BLK || MODE == Z_POWER || L < 256, "the blocked force pass of the longer lines is in fft_pair.cuh");
     const int tid = threadIdx.x, c = tid % C, j = tid / C;
     constexpr int TA = Z::TA, TB = Z::TB;   // forward stage-A / stage-B tasks
     auto prefetch = [&](int tt) {   // 16-byte cp.async.cg of rows z = 0..L-1, C columns, into pf

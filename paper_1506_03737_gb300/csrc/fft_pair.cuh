@@ -1,4 +1,5 @@
-// Paired-lane 32-point transforms for the z passes of the force of 1024 (32 x 32) and 512 points (16 x 32).
+// Force z passes of the blocked layout from 256 points on: tiles moved by TMA boxes, and, for 1024 (32 x 32) and 512
+// points (16 x 32), 32-point transforms on pairs of lanes.
 //
 // The two-stage z pass gives every radix-32 task to one thread, which then holds 32 complex
 // values: with the saved base in shared memory that allows 12 warps per SM. Here a task is split
@@ -65,7 +66,7 @@ __host__ __device__ __forceinline__ void pair_dif_finish(float2* v, int h, int i
     v[i + 8] = csel(h != 0, v[i + 8], recv);      // Y_h[i + 8]
 }
 template <int S>
-__host__ __device__ __forceinline__ void pair_dif_dft(float2* v) { dft<16, S>(v); }
+__host__ __device__ __forceinline__ void pair_dif_dft(float2* v) { dft<16, S, true>(v); }
 
 // Twiddles of stage B for task j, inputs r = 2m + h: v[m] *= w^(S j r), w = exp(-2 pi i / L), from
 // the tables w^(8 M j) (M = r >> 3 = m >> 2) and w^j (r & 7 = 2 (m & 3) + h).
@@ -156,6 +157,22 @@ __device__ __forceinline__ void pair_store(const float2* buf, const CUtensorMap&
     for (int z = 0; z < L; z += 256)
         box_store(map, (ky & 7) * 8 + (kx0 & 7), z, (kx0 >> 3) * (L / 8) + (ky >> 3), smem_u32(buf + 4 * z));
 }
+// Green's function with the CIC window at index z of a column: gnorm / (k^2 W^d), 0 on excluded modes (nxy2 and wxy: the
+// column's nx^2 + ny^2 and window factor). A table of it per z in shared memory took the L1 that the window
+// factors live in, and was slower.
+template <int L>
+__device__ __forceinline__ float green_at(int z, int nz, int nxy2, float wxy, bool nyq_y, const float* __restrict__ sinc2,
+                                          int deconv, float gnorm) {
+    const float kf = 6.283185307179586f / (float)L;
+    const int n2 = nxy2 + nz * nz;   // 0 only at k = 0
+    float w = 1.0f;
+    if (deconv) {
+        w = wxy * sinc2[z];
+        if (deconv == 2) w *= w;
+    }
+    // fast division (within 2 ulp; k^2 W is far from the range where it flushes)
+    return !nyq_y && z != L / 2 && n2 != 0 ? __fdividef(gnorm, kf * kf * (float)n2 * w) : 0.0f;
+}
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
 template <int MINB>
@@ -197,7 +214,7 @@ __global__ void __launch_bounds__(PZ_T, MINB)
         }
 #pragma unroll
         for (int m = 0; m < 16; ++m) v[m] = buf[(j + R * (2 * m + h)) * C + c];
-        dft<16, -1>(v);
+        dft<16, -1, true>(v);
         pair_dit<-1>(v, h);
 #pragma unroll
         for (int q = 0; q < 16; ++q) xb[X::at(c, j * R + pair_dit_r(q, h))] = v[q];
@@ -207,7 +224,7 @@ __global__ void __launch_bounds__(PZ_T, MINB)
 #pragma unroll
         for (int m = 0; m < 16; ++m) v[m] = xb[X::at(c, j + R * (2 * m + h))];
         pair_twiddle<-1>(v, tws, j, h);
-        dft<16, -1>(v);
+        dft<16, -1, true>(v);
         pair_dit<-1>(v, h);
         // bases: A = g X, B = k_z A; g = gnorm / (k^2 W^d), 0 on excluded modes
         {
@@ -215,16 +232,8 @@ __global__ void __launch_bounds__(PZ_T, MINB)
             const float wxy = deconv ? sinc2[nx] * sinc2[ky] : 1.0f;
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
-                const int z = j + R * pair_dit_r(q, h);
-                const int nz = sbin(z, L);
-                const int n2 = nxy2 + nz * nz;
-                float w = 1.0f;
-                if (deconv) {
-                    w = wxy * sinc2[z];
-                    if (deconv == 2) w *= w;
-                }
-                const float g = !nyq_y && z != L / 2 && n2 != 0 ? __fdividef(gnorm, kf * kf * (float)n2 * w) : 0.0f;
-                v[q] = cscale(v[q], g);
+                const int z = j + R * pair_dit_r(q, h), nz = sbin(z, L);
+                v[q] = cscale(v[q], green_at<L>(z, nz, nxy2, wxy, nyq_y, sinc2, deconv, gnorm));
                 save[X::at(c, z)] = cscale(v[q], kf * (float)nz);
             }
         }
@@ -248,7 +257,7 @@ __global__ void __launch_bounds__(PZ_T, MINB)
 #pragma unroll
             for (int m = 0; m < 16; ++m) v[m] = xb[X::at(c, j + R * (2 * m + h))];
             pair_twiddle<+1>(v, tws, j, h);
-            dft<16, +1>(v);
+            dft<16, +1, true>(v);
             pair_dit<+1>(v, h);
             float2* dst = bi == 0 ? buf : save;
 #pragma unroll
@@ -312,7 +321,7 @@ static __global__ void __launch_bounds__(PZ5_T, PZ5_MINB)
         }
 #pragma unroll
         for (int r = 0; r < RA; ++r) v[r] = buf[(ja + RB * r) * C + c];
-        dft<RA, -1>(v);
+        dft<RA, -1, true>(v);
 #pragma unroll
         for (int r = 0; r < RA; ++r) xb[XF::at(c, ja * RA + r)] = v[r];
         if (tid == 0) box_stores_read();   // the last tile's second output has left `save`
@@ -321,23 +330,15 @@ static __global__ void __launch_bounds__(PZ5_T, PZ5_MINB)
 #pragma unroll
         for (int m = 0; m < 16; ++m) v[m] = xb[XF::at(c, jb + RA * (2 * m + h))];
         pair_twiddle<-1>(v, tws, jb, h);
-        dft<16, -1>(v);
+        dft<16, -1, true>(v);
         pair_dit<-1>(v, h);
         // bases: A = g X, B = k_z A; g = gnorm / (k^2 W^d), 0 on excluded modes
         const int nxy2 = nx * nx + ny * ny;
         const float wxy = deconv ? sinc2[nx] * sinc2[ky] : 1.0f;
 #pragma unroll
         for (int q = 0; q < 16; ++q) {
-            const int z = jb + RA * pair_dit_r(q, h);
-            const int nz = sbin(z, L);
-            const int n2 = nxy2 + nz * nz;
-            float w = 1.0f;
-            if (deconv) {
-                w = wxy * sinc2[z];
-                if (deconv == 2) w *= w;
-            }
-            const float g = !nyq_y && z != L / 2 && n2 != 0 ? __fdividef(gnorm, kf * kf * (float)n2 * w) : 0.0f;
-            v[q] = cscale(v[q], g);
+            const int z = jb + RA * pair_dit_r(q, h), nz = sbin(z, L);
+            v[q] = cscale(v[q], green_at<L>(z, nz, nxy2, wxy, nyq_y, sinc2, deconv, gnorm));
             save[XF::at(c, z)] = cscale(v[q], kf * (float)nz);
         }
         __syncthreads();   // forward exchange buffer free
@@ -357,7 +358,7 @@ static __global__ void __launch_bounds__(PZ5_T, PZ5_MINB)
             }
             __syncthreads();
             // inverse stage B (radix 16): inputs and outputs ja + 32 r
-            stage_b<L, RB, RA, +1, C>(xb, tws, c, ja, v);
+            stage_b<L, RB, RA, +1, C, true>(xb, tws, c, ja, v);
             float2* dst = bi == 0 ? buf : save;
 #pragma unroll
             for (int r = 0; r < RA; ++r) dst[(ja + RB * r) * C + c] = v[r];
@@ -371,6 +372,126 @@ static __global__ void __launch_bounds__(PZ5_T, PZ5_MINB)
 constexpr size_t PZ5_SMEM =
     sizeof(float2) * ((size_t)(Xch<512, 16, 4>::SIZE > Xch<512, 32, 4>::SIZE ? Xch<512, 16, 4>::SIZE : Xch<512, 32, 4>::SIZE) +
                       Xch<512, 16, 4>::SIZE + 512 * 4) + sizeof(Tw2) + 8;
+
+// ---------------------------------------------------------------------------------------------
+// The same pass for lines of 256, 320 and 384 points, one thread per task, tiles of 4 columns moved by boxes as above
+// (one box of all 256 z, two halves above). With loads and stores through L1 (k2_fz) the pass took 52, 127 and
+// 221 us on these meshes, with boxes 41, 105 and 155. The shorter lines stay with k2_fz: their meshes live in L2, and a box
+// costs more than it saves (128^3: 9.9 us against 10.9).
+template <int L>
+struct ZBox {
+    static constexpr int C = 4;                                    // columns
+    static constexpr int R1 = F2<L>::R1, R2 = F2<L>::R2;
+    static constexpr int TA = C * L / R1, TB = C * L / R2, T = TA > TB ? TA : TB;
+    using XF = Xch<L, R1, C>;
+    using XI = Xch<L, R2, C>;
+    static constexpr int up(int n) { return (n + 15) / 16 * 16; }  // to 128 bytes
+    static constexpr int XS = up(XF::SIZE > XI::SIZE ? XF::SIZE : XI::SIZE), SV = up(XF::SIZE), BOXZ = L <= 256 ? L : L / 2;
+    static constexpr size_t SMEM = sizeof(float2) * ((size_t)XS + SV + L * C) + sizeof(Tw2) + 8;
+    static constexpr int MINB = 512 / T;
+};
+
+template <int L>
+__global__ void __launch_bounds__(ZBox<L>::T, ZBox<L>::MINB)
+    k2_fz_box(const __grid_constant__ CUtensorMap f0, const __grid_constant__ CUtensorMap f2, const float2* __restrict__ tw,
+              const float* __restrict__ sinc2, int deconv, float gnorm, int* err) {
+    using Z = ZBox<L>;
+    using XF = typename Z::XF;
+    using XI = typename Z::XI;
+    constexpr int C = Z::C, R1 = Z::R1, R2 = Z::R2, n = L / 2, NTILE = (n / C) * L;
+    extern __shared__ __align__(128) float4 smem4[];
+    float2* xb = reinterpret_cast<float2*>(smem4);
+    float2* save = xb + Z::XS;         // the saved base, then the tile of the second output
+    float2* buf = save + Z::SV;        // the input tile, then that of the first output
+    Tw2* tws = reinterpret_cast<Tw2*>(buf + L * C);
+    const uint32_t bar = smem_u32(tws + 1);
+    pdl_trigger();
+    load_tw2<L, L>(tws, tw, Z::T);
+    if (threadIdx.x == 0) {
+        mbar_init(bar);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    pdl_wait();
+    __syncthreads();
+    auto load = [&](int t) {
+        int ky, kx0;
+        pair_tile<L>(t, ky, kx0);
+        mbar_expect(bar, L * C * 8);
+#pragma unroll
+        for (int z = 0; z < L; z += Z::BOXZ)
+            box_load(smem_u32(buf + C * z), f0, (ky & 7) * 8 + (kx0 & 7), z, (kx0 >> 3) * (L / 8) + (ky >> 3), bar);
+    };
+    const int tid = threadIdx.x, c = tid % C, j = tid / C;
+    const float kf = 6.283185307179586f / (float)L;
+    if (tid == 0 && blockIdx.x < NTILE) load(blockIdx.x);
+    uint32_t phase = 0;
+    for (int t = blockIdx.x; t < NTILE; t += gridDim.x, phase ^= 1) {
+        int ky, kx0;
+        pair_tile<L>(t, ky, kx0);
+        const int ny = sbin(ky, L), nx = kx0 + c;
+        bool ok = mbar_wait(bar, phase);
+        if (!ok) {   // flag it, let the copy land, stop
+            atomicOr(err, 4);
+            mbar_wait(bar, phase);
+        }
+        float2 v[R2];
+        if (tid < Z::TA) {   // forward stage A: inputs z = j + r L / R1
+            float2 a[R1];
+#pragma unroll
+            for (int r = 0; r < R1; ++r) a[r] = buf[(j + r * (L / R1)) * C + c];
+            dft<R1, -1, true>(a);
+#pragma unroll
+            for (int r = 0; r < R1; ++r) xb[XF::at(c, j * R1 + r)] = a[r];
+        }
+        if (tid == 0) box_stores_read();   // the last tile's second output has left `save`
+        if (!__syncthreads_and(ok)) break;
+        if (tid < Z::TB) {   // forward stage B, then the bases A = g X (kept) and B = k_z A (saved)
+            stage_b<L, R1, R2, -1, C, true>(xb, tws, c, j, v);
+            const int nxy2 = nx * nx + ny * ny;
+            const float wxy = deconv ? sinc2[nx] * sinc2[ky] : 1.0f;
+#pragma unroll
+            for (int r = 0; r < R2; ++r) {
+                const int z = j + R1 * r, nz = sbin(z, L);
+                v[r] = cscale(v[r], green_at<L>(z, nz, nxy2, wxy, ky == L / 2, sinc2, deconv, gnorm));
+                save[XF::at(c, z)] = cscale(v[r], kf * (float)nz);
+            }
+        }
+        __syncthreads();   // forward exchange buffer free
+#pragma unroll 1
+        for (int bi = 0; bi < 2; ++bi) {
+            if (tid < Z::TB) {   // inverse stage A (radix R2)
+                if (bi > 0) {
+#pragma unroll
+                    for (int r = 0; r < R2; ++r) v[r] = save[XF::at(c, j + R1 * r)];
+                }
+                dft<R2, +1, true>(v);
+#pragma unroll
+                for (int r = 0; r < R2; ++r) xb[XI::at(c, j * R2 + r)] = v[r];
+            }
+            if (bi > 0 && tid == 0) {   // the first output has left the tile buffer: the next tile
+                box_stores_read();
+                if (t + (int)gridDim.x < NTILE) load(t + gridDim.x);
+            }
+            __syncthreads();
+            float2* dst = bi == 0 ? buf : save;
+            if (tid < Z::TA) {   // inverse stage B (radix R1): outputs z = j + R2 r
+                float2 u[R1];
+                stage_b<L, R2, R1, +1, C, true>(xb, tws, c, j, u);
+#pragma unroll
+                for (int r = 0; r < R1; ++r) dst[(j + R2 * r) * C + c] = u[r];
+            }
+            fence_async_smem();
+            __syncthreads();   // the output tile is complete, the exchange buffer free for the next base / tile
+            if (tid == 0) {
+#pragma unroll
+                for (int z = 0; z < L; z += Z::BOXZ)
+                    box_store(bi == 0 ? f0 : f2, (ky & 7) * 8 + (kx0 & 7), z, (kx0 >> 3) * (L / 8) + (ky >> 3),
+                              smem_u32(dst + C * z));
+            }
+        }
+    }
+    if (tid == 0) box_stores_done();
+}
 
 template <int MINB>
 struct PairZ {

@@ -15,10 +15,9 @@ static cudaError_t fz2(float2* in, ZOut out, const float2* tw, const float* sinc
                        cudaStream_t s) {
     if constexpr (N == 1024 && MODE == Z_FORCE && BLK) {
         // 1024-point force lines: each radix-32 task on a pair of lanes (16 values per thread),
-        // two CTAs of 256 threads per SM (measured at 1024^3: 4.93 ms against 5.50 for the
+        // two CTAs of 256 threads per SM (before the boxes, at 1024^3: 4.93 ms against 5.50 for the
         // one-thread-per-task kernel at three CTAs of 128 threads, 6.1-6.4 ms with the pair kernel
-        // held to 80 registers for three CTAs, 5.32 ms with the next tile's inputs loaded into
-        // registers during the inverse transforms)
+        // held to 80 registers for three CTAs; with them 3.39)
         constexpr int MINB = 2;
         const auto* maps = static_cast<const CUtensorMap*>(out.maps);
         if (!maps) return cudaErrorInvalidValue;
@@ -39,6 +38,17 @@ static cudaError_t fz2(float2* in, ZOut out, const float2* tw, const float* sinc
         const int total = (N / 2 / 4) * N;
         return launch_dep(overlap_mesh(N), k2_fz_pair512, grid < total ? grid : total, PZ5_T, PZ5_SMEM, s, maps[0], maps[1],
                           tw, sinc2, deconv, gnorm, out.err);
+    } else if constexpr (MODE == Z_FORCE && BLK && N >= 256) {
+        using Z = ZBox<N>;
+        const auto* maps = static_cast<const CUtensorMap*>(out.maps);
+        if (!maps) return cudaErrorInvalidValue;
+        static GridCache cache;
+        int grid = 0;
+        cudaError_t e = cached_grid(cache, k2_fz_box<N>, Z::T, Z::SMEM, &grid);
+        if (e != cudaSuccess) return e;
+        const int total = (N / 2 / Z::C) * N;
+        return launch_dep(overlap_mesh(N), k2_fz_box<N>, grid < total ? grid : total, Z::T, Z::SMEM, s, maps[0], maps[1], tw, sinc2,
+                          deconv, gnorm, out.err);
     } else {
         // Blocked layout: 4-column tiles (32-byte rows whose 512-byte runs the neighbouring tiles
         // complete), which with the prefetch buffer measured 2% faster than 8-column ones (34% for the
