@@ -378,9 +378,10 @@ int colapm_batch_run(colapm_batch* b, const unsigned long long* seeds, int nbins
 int colapm_batch_streams(const colapm_batch* b);
 
 /* Schedule of the batch's steps. on = 1 (the default): lockstep -- the mocks advance one step at a
- * time together; each step is one multi-mock deposit of every mock still running, the mesh passes
- * of each mock, and one multi-mock gather-kick-drift. The two multi-mock kernels are persistent:
- * their CTAs take work items (mock, chunk of 256 particles) from a ticket counter across all the
+ * time together; each step is one multi-mock deposit of the small mocks still running (fewer than 2^19
+ * particles), the mesh passes of each mock, and one multi-mock gather-kick-drift of the small ones; a large
+ * mock's own deposit and gather run with its mesh passes. The two multi-mock kernels are persistent:
+ * their CTAs take work items (mock, chunk of 256 particles) from a ticket counter across all their
  * mocks, whatever their sizes. on = 0: each mock runs its ICs, steps and P(k) in turn (on worker
  * streams). Both give the same particles bit for bit (the per-particle code is the same and the
  * fixed-point deposit does not depend on order), and the same P(k) up to the order of its FP64 bin

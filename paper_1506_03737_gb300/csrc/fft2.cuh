@@ -532,7 +532,7 @@ struct X2 {
     static constexpr int RA = F2<n>::R1, RB = F2<n>::R2;
     static constexpr int TA = 8 * n / RA, TB = 8 * n / RB, T = TA > TB ? TA : TB;
     static constexpr size_t SMEM = sizeof(float2) * (size_t)Xch<n, RA>::SIZE + sizeof(Tw2);
-    static constexpr bool SPLIT = n != 256;   // forward: the half spectrum inside stage B (see k2_fx_fwd)
+    static constexpr bool SPLIT = n != 128 && n != 256;   // forward: the half spectrum inside stage B (see k2_fx_fwd)
     // inverse: plus a dense [8][n] staging buffer for the cp.async prefetch of the rows
     static constexpr size_t SMEM_INV = SMEM + sizeof(float2) * 8 * (size_t)n;
 };
@@ -585,9 +585,10 @@ __global__ void __launch_bounds__(X2<n>::T) k2_fx_fwd(const void* __restrict__ i
         }
         __syncthreads();
         // The half spectrum X[k] from Z[k] and Z[n-k]: inside stage B (partner values by warp shuffle;
-        // one barrier and one shared round trip fewer: 3.8 -> 3.4 ms at n = 512, 437 -> 182 us at n = 192 with
-        // the blocked layout), or in a separate loop over the exchange buffer (n = 256, where the step of 512^3
-        // takes 3.86 ms that way and 4.22 ms this).
+        // one barrier and one shared round trip fewer), or in a separate loop over the exchange buffer. Blocked
+        // layout, us with one / the other: n = 32 5.5 / 5.9, 48 8.4 / 8.9, 64 9.5 / 11.6, 80 14.9 / 18.4, 96 20.6 /
+        // 27.4, 160 111 / 287, 192 186 / 461, 512 3400 / 3800; but 128 162 / 60, and 256 about 790 / 440: there
+        // all CTAs write the same few blocks at once, a power of two apart, and wait for them.
         if constexpr (X::SPLIT) {
             if (tid < X::TB) {   // stage B: Z[j + RA r], then X[k] for the same k = j + RA r
                 static_assert(32 % RA == 0 && X::TB % 32 == 0, "the partner of a task must be in its warp");
