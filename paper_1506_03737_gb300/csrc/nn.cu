@@ -72,8 +72,24 @@ struct ConvArgs {
     const float* target;         // EPI_OUT training: [n^3][3] physical; normalised by tscale
     float tscale, gscale;        // gscale = 2 / (3 n^3)
     double* loss;                // sum of squared normalised errors
+    bool wide;                   // EPI_OUT: y, base and target start at multiples of 16 bytes
     int* err;                    // bit 4: a bounded wait gave up
 };
+
+// Four consecutive floats of a caller's array, as one access where it is aligned.
+__device__ __forceinline__ float4 load4(const float* p, bool wide) {
+    return wide ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+}
+__device__ __forceinline__ void store4(float* p, float4 v, bool wide) {
+    if (wide) {
+        *reinterpret_cast<float4*>(p) = v;
+    } else {
+        p[0] = v.x;
+        p[1] = v.y;
+        p[2] = v.z;
+        p[3] = v.w;
+    }
+}
 
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t* r) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
@@ -154,7 +170,7 @@ struct ConvSmem {
 // next tile is fetched by one TMA box while this one's outputs are written, and the second CTA of
 // the SM computes while this one waits. At 128^3 a hidden layer takes 73-75 us (65% of the mma.sync rate; what is left
 // is the start and end of each tile) against 95 us with one operand load per product pair and per-thread 16-byte
-// copies, a backward one 79 against 133, the output layer 67 against 122 (153 with the loss). Row by row bulk copies
+// copies, a backward one 79 against 133, the output layer 64 against 122 (153 with the loss). Row by row bulk copies
 // instead of the box took 89-95 us (about 130 cycles each), 4-plane tiles at three CTAs per SM 86 us.
 template <int NT, int EPI, int TZ, int VB>
 __global__ void __launch_bounds__(32 * TZ, TZ == 8 ? 2 : 4)
@@ -215,14 +231,15 @@ __global__ void __launch_bounds__(32 * TZ, TZ == 8 ? 2 : 4)
             box_stores_read();   // the previous tile's outputs have left the buffer
             if (EPI == EPI_MASK) load_mask();
         }
-        constexpr int NPRE = EPI == EPI_OUT ? TX * TY * 3 / 32 : 1;
-        float pre[NPRE];   // EPI_OUT: the tile of target or base, in flight during the products
+        constexpr int NPRE = EPI == EPI_OUT ? TX * TY * 3 / 128 : 1;
+        float4 pre[NPRE];   // EPI_OUT: the tile of target or base, in flight during the products
         if (EPI == EPI_OUT) {
             const float* src = a.target ? a.target : a.base;
 #pragma unroll
             for (int i = 0; i < NPRE; ++i) {
-                const int e = lane + 32 * i;
-                pre[i] = src ? __ldg(src + (((size_t)(z0 + tz) * n + y0 + e / (TX * 3)) * n + x0) * 3 + e % (TX * 3)) : 0.0f;
+                const int e = 4 * (lane + 32 * i);
+                const size_t at = (((size_t)(z0 + tz) * n + y0 + e / (TX * 3)) * n + x0) * 3 + e % (TX * 3);
+                pre[i] = src ? load4(src + at, a.wide) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             }
         }
         float acc[TY][NT][4];
@@ -341,19 +358,26 @@ __global__ void __launch_bounds__(32 * TZ, TZ == 8 ? 2 : 4)
             }
             __syncwarp();
 #pragma unroll
-            for (int k = 0; k < NPRE; ++k) {
-                const int e = lane + 32 * k;
+            for (int k = 0; k < NPRE; ++k) {   // four values a lane: rows are 48 values, all multiples of 4
+                const int e = 4 * (lane + 32 * k);
                 const size_t i = (((size_t)(cz + tz) * n + cy + e / (TX * 3)) * n + cx) * 3 + e % (TX * 3);
-                const float u = so[e];
-                const float b = !a.target ? pre[k] : (a.base ? a.base[i] : 0.0f);
-                a.y[i] = b + a.oscale * u;
-                if (a.target) {
-                    const float d = u - pre[k] * a.tscale;
-                    so[e] = a.gscale * d;
-                    const float p = __fmul_rn(d, d), pe = fmaf(d, d, -p), s = __fadd_rn(ls, p), z = __fsub_rn(s, ls);
-                    lc += (__fsub_rn(ls, __fsub_rn(s, z)) + __fsub_rn(p, z)) + pe;
-                    ls = s;
+                const float4 u4 = *reinterpret_cast<const float4*>(so + e);
+                const float u[4] = {u4.x, u4.y, u4.z, u4.w}, q4[4] = {pre[k].x, pre[k].y, pre[k].z, pre[k].w};
+                float yv[4], g4[4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const float b = !a.target ? q4[m] : (a.base ? a.base[i + m] : 0.0f);
+                    yv[m] = b + a.oscale * u[m];
+                    if (a.target) {
+                        const float d = u[m] - q4[m] * a.tscale;
+                        g4[m] = a.gscale * d;
+                        const float p = __fmul_rn(d, d), pe = fmaf(d, d, -p), s = __fadd_rn(ls, p), z = __fsub_rn(s, ls);
+                        lc += (__fsub_rn(ls, __fsub_rn(s, z)) + __fsub_rn(p, z)) + pe;
+                        ls = s;
+                    }
                 }
+                store4(a.y + i, make_float4(yv[0], yv[1], yv[2], yv[3]), a.wide);
+                if (a.target) *reinterpret_cast<float4*>(so + e) = make_float4(g4[0], g4[1], g4[2], g4[3]);
             }
             if (a.target) {
                 __syncwarp();
@@ -967,6 +991,7 @@ cudaError_t forward(colapm_nn* c, const float* psi, float* y, const float* base,
     a.y = y;
     a.base = base;
     a.oscale = c->cfg.s_out;
+    a.wide = (reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(base) | reinterpret_cast<uintptr_t>(target)) % 16 == 0;
     if (target) {
         a.target = target;
         a.tscale = 1.0f / c->cfg.s_out;
