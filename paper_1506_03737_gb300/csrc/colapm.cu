@@ -629,24 +629,36 @@ int colapm_make_ics(colapm_ctx* c) {
     const float gnorm = (float)(1.0 / ((double)np * np * np));
     if (c->seed_src == c->d_seed) CKL(launch_set_u64(c->d_seed, c->prm.seed, c->stream));
     if (int r = initial_field(c, dk, phi)) return r;
-    ZOut o1{};
-    o1.vscale = (float)c->nm / np;   // the displacements in PM-mesh cells
-    for (int j = 0; j < 3; ++j) o1.p[j] = p1 + j * hs;
-    for (int j = 0; j < 6; ++j) o1.p[3 + j] = phi + j * hs;
-    CKL(launch_fz(np, Z_LPT1, dk, o1, c->tw_p, nullptr, 0, gnorm, nullptr, c->stream, ts(c, COLAPM_PLAN_Z)));
-    CKL(launch_fy(np, +1, p1, hs, 3, c->tw_p, c->stream, ts(c, COLAPM_PLAN_Y)));
-    CKL(launch_fy(np, +1, phi, hs, 6, c->tw_p, c->stream, ts(c, COLAPM_PLAN_Y)));
-    CKL(launch_fx_inv(np, p1, hs, 3, c->tw_p, c->stream, ts(c, COLAPM_PLAN_XI)));
-    CKL(launch_fx_inv(np, phi, hs, 6, c->tw_p, c->stream, ts(c, COLAPM_PLAN_XI)));
-    // 2LPT: S from the six phi_ij, then Psi2 = -i k S_k / k^2.
-    CKL(launch_lpt2_source(c->scratch + np3, np3, c->scratch, c->stream));
+    const float vs = (float)c->nm / np;   // the displacements in PM-mesh cells
+    ZOut o1{}, o2{};
+    o1.vscale = o2.vscale = vs;
+    for (int j = 0; j < 3; ++j) o2.p[j] = p2 + j * hs;
+    float2* src = dk;   // the second-order source, where the initial field was
+    const unsigned inv = COLAPM_PLAN_Y | COLAPM_PLAN_Z | COLAPM_PLAN_XI;
+    const bool fused = lpt_fused(np) && (c->plan & inv) == inv;
+    if (fused) {
+        // three bases of the z pass (in psi1's space), six spectra, then Psi1 and the 2LPT source S at once
+        for (int j = 0; j < 3; ++j) o1.p[j] = p1 + j * hs;
+        CKL(launch_fz(np, Z_LPT1_BASES, dk, o1, c->tw_p, nullptr, 0, gnorm, nullptr, c->stream, true));
+        CKL(launch_fy_lpt(np, p1, phi, hs, c->tw_p, c->stream));
+        CKL(launch_fx_lpt(np, phi, hs, p1, src, c->tw_p, vs, c->stream));
+        std::swap(o2.p[1], o2.p[2]);   // the second base goes to field 2
+    } else {
+        for (int j = 0; j < 3; ++j) o1.p[j] = p1 + j * hs;
+        for (int j = 0; j < 6; ++j) o1.p[3 + j] = phi + j * hs;
+        CKL(launch_fz(np, Z_LPT1, dk, o1, c->tw_p, nullptr, 0, gnorm, nullptr, c->stream, ts(c, COLAPM_PLAN_Z)));
+        CKL(launch_fy(np, +1, p1, hs, 3, c->tw_p, c->stream, ts(c, COLAPM_PLAN_Y)));
+        CKL(launch_fy(np, +1, phi, hs, 6, c->tw_p, c->stream, ts(c, COLAPM_PLAN_Y)));
+        CKL(launch_fx_inv(np, p1, hs, 3, c->tw_p, c->stream, ts(c, COLAPM_PLAN_XI)));
+        CKL(launch_fx_inv(np, phi, hs, 6, c->tw_p, c->stream, ts(c, COLAPM_PLAN_XI)));
+        CKL(launch_lpt2_source(c->scratch + np3, np3, c->scratch, c->stream));   // S from the six phi_ij
+    }
+    // 2LPT: Psi2 = -i k S_k / k^2.
     CKL(launch_fx_fwd_f32(np, c->scratch, phi, c->tw_p, c->stream, ts(c, COLAPM_PLAN_XF)));
     CKL(launch_fy(np, -1, phi, 0, 1, c->tw_p, c->stream, ts(c, COLAPM_PLAN_Y)));
-    ZOut o2{};
-    o2.vscale = o1.vscale;
-    for (int j = 0; j < 3; ++j) o2.p[j] = p2 + j * hs;
-    CKL(launch_fz(np, Z_LPT2, phi, o2, c->tw_p, nullptr, 0, gnorm, nullptr, c->stream, ts(c, COLAPM_PLAN_Z)));
-    CKL(launch_fy(np, +1, p2, hs, 3, c->tw_p, c->stream, ts(c, COLAPM_PLAN_Y)));
+    CKL(launch_fz(np, fused ? Z_LPT2_BASES : Z_LPT2, phi, o2, c->tw_p, nullptr, 0, gnorm, nullptr, c->stream, ts(c, COLAPM_PLAN_Z)));
+    if (fused) CKL(launch_fy_force(np, p2, hs, c->tw_p, c->stream, false, -vs));
+    else CKL(launch_fy(np, +1, p2, hs, 3, c->tw_p, c->stream, ts(c, COLAPM_PLAN_Y)));
     CKL(launch_fx_inv(np, p2, hs, 3, c->tw_p, c->stream, ts(c, COLAPM_PLAN_XI)));
     return place_particles(c, c->psi1, c->psi2, 1.0f);
 }

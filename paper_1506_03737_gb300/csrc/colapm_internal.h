@@ -102,7 +102,10 @@ enum ZMode {
     Z_POWER = 3,   // forward z, bin |delta|^2 / W^2
     // (Stockham engine only) per-mode scaling by a table indexed by |n|^2, passed in place of sinc2:
     Z_SCALE_FWD = 4,   // forward z, then multiply: 1 output in k-space
-    Z_SCALE_INV = 5    // (input already transformed) multiply, then inverse z: 1 output
+    Z_SCALE_INV = 5,   // (input already transformed) multiply, then inverse z: 1 output
+    // (two-stage engine only) the LPT modes up to their bases A, B (, C) = IFFT_z(g X), (k_z g X) (, k_z^2 g X): 2 (3) outputs
+    Z_LPT1_BASES = 6,
+    Z_LPT2_BASES = 7
 };
 
 // Power-spectrum binning. Bin membership is decided in FP64 on the host (or once per call on
@@ -275,7 +278,17 @@ cudaError_t launch_fy(int n_mesh, int sign, float2* data, size_t field_stride, i
 // Inverse y pass of the force in the blocked layout (N >= 64): from the z pass's two bases in
 // fields 0 and 2 to the three force spectra in fields 0, 1, 2 (the blocked force z pass writes
 // the bases instead of the three spectra).
-cudaError_t launch_fy_force(int n_mesh, float2* data, size_t field_stride, const float2* tw, cudaStream_t s);
+// With blocked = false in the plain layout, times sg (the second-order displacements).
+cudaError_t launch_fy_force(int n_mesh, float2* data, size_t field_stride, const float2* tw, cudaStream_t s, bool blocked = true,
+                            float sg = 1.0f);
+// First-order LPT after the z pass has left its three bases A, B, C (Z_LPT1_BASES) in `bases` (lpt_fused(np) only):
+// inverse y to the six spectra of A, k_y A, k_y^2 A, B, k_y B, C (`field_stride` complex apart, as the bases are), then
+// inverse x to the displacements psi (three real fields, times vscale) and the second-order source
+// S = xx yy + xx zz + yy zz - xy^2 - xz^2 - yz^2 of the second derivatives, which are never stored.
+bool lpt_fused(int np);
+cudaError_t launch_fy_lpt(int np, const float2* bases, float2* spectra, size_t field_stride, const float2* tw, cudaStream_t s);
+cudaError_t launch_fx_lpt(int np, const float2* spectra, size_t field_stride, float2* psi, float2* src, const float2* tw,
+                          float vscale, cudaStream_t s);
 // z pass with the spectral multiply fused.
 // Fused x-y passes (N = 512, 1024): forward r2c x + y of the int64 density into the half
 // spectrum `out`; inverse y + c2r x of `nfields` spectra in place. `ring` holds xy_ring_bytes(N)

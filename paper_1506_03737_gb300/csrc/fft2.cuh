@@ -197,11 +197,12 @@ template <int L, int MODE, int C = 8, bool DIRECT = false>
 struct Z2 {
     static constexpr int R1 = F2<L>::R1, R2 = F2<L>::R2;
     static constexpr int XS = Xch<L, R1, C>::SIZE > Xch<L, R2, C>::SIZE ? Xch<L, R1, C>::SIZE : Xch<L, R2, C>::SIZE;
-    static constexpr int NSAVE = MODE == Z_LPT1 ? 2 : (MODE == Z_POWER ? 0 : 1);   // saved bases B (, C)
+    static constexpr bool LPT1 = MODE == Z_LPT1 || MODE == Z_LPT1_BASES, BASES = MODE == Z_LPT1_BASES || MODE == Z_LPT2_BASES;
+    static constexpr int NSAVE = LPT1 ? 2 : (MODE == Z_POWER ? 0 : 1);   // saved bases B (, C)
     // next tile via cp.async into a shared buffer, or (DIRECT) straight from global memory into the
     // stage-A registers: the smaller footprint fits three CTAs per SM at C = 4, which hides the load
     // latency better than the prefetch does with two (force z pass at 1024^3: 6.0 against 6.9 ms)
-    static constexpr bool PREFETCH = MODE != Z_LPT1 && !DIRECT;
+    static constexpr bool PREFETCH = !LPT1 && !DIRECT;
     static constexpr int PF = PREFETCH ? C * L : 0;                               // dense [z][C] buffer
     static constexpr int TA = C * L / R1, TB = C * L / R2, T = TA > TB ? TA : TB;
     static constexpr size_t SMEM = sizeof(float2) * ((size_t)XS * (1 + NSAVE) + PF) + sizeof(Tw2);
@@ -211,8 +212,9 @@ struct Z2 {
     static constexpr int PER = L * C / (2 * T), PP = ((L + L / PER + 31) / 32) * 32 + 32 / C;
     static_assert(MODE != Z_POWER || (PER * T * 2 == L * C && L % PER == 0), "the runs must cover the tile");
     static constexpr size_t SMEM_POWER = SMEM + sizeof(float) * ((size_t)C * PP + L / 2);
-    // CTAs per SM: 12 warps where a task holds 32 values, 20 (at most 102 registers) with the smaller radices
-    static constexpr int MINB = DIRECT ? (R1 == 32 || R2 == 32 ? 384 / T : 640 / T) : 1;
+    // CTAs per SM: 16 warps for the LPT bases (at most 128 registers; 256 points: 103 and 78 us without the bound, 80 and
+    // 54 with it); 12 warps where a task holds 32 values, 20 (at most 102 registers) with the smaller radices
+    static constexpr int MINB = DIRECT ? (R1 == 32 || R2 == 32 ? 384 / T : 640 / T) : (BASES ? 512 / T : 1);
 };
 
 template <int L, int MODE, int C = 8, bool BLK = false, bool DIRECT = false>
@@ -285,7 +287,7 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
         const size_t base = hs_index<L, BLK>(kx0 + c, ky, 0);
         const int nx = kx0 + c;
         float2 v[R2];   // stage-B results: X[j + R1 r] (j < R1), or the LPT1 input spectrum
-        if constexpr (MODE == Z_LPT1) {
+        if constexpr (Z::LPT1) {
             if (tid < TB) {
 #pragma unroll
                 for (int r = 0; r < R2; ++r) v[r] = __ldcg(in + base + (size_t)(j + R1 * r) * stride);
@@ -421,6 +423,8 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
                         const float2 ia = make_float2(-a.y, a.x);   // i * a
                         if (MODE == Z_FORCE && BLK) {   // bases only; k2_fy_force applies i k_x, i k_y, i
                             out.p[bi == 0 ? 0 : 2][o] = a;
+                        } else if (Z::BASES) {
+                            out.p[bi][o] = a;
                         } else if (bi == 0) {
                             out.p[0][o] = cscale(ia, sg * kxv);
                             out.p[1][o] = cscale(ia, sg * kyv);
@@ -478,9 +482,9 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
 //   F_y = i IFFT_y(k_y A')     -> field 1
 //   F_x = i k_x IFFT_y(A')     -> field 0 (in place; A' is read twice, the second time from L2)
 // It reads 8 bytes per cell instead of the 12 of three separate spectra.
-template <int L>
+template <int L, bool BLK>
 __global__ void __launch_bounds__(K2<L>::T) k2_fy_force(float2* __restrict__ data, size_t fstride,
-                                                        const float2* __restrict__ tw) {
+                                                        const float2* __restrict__ tw, float sg) {
     using K = K2<L>;
     constexpr int RA = K::RA, RB = K::RB, n = L / 2, NG = n / 8, TPF = NG * L;
     extern __shared__ float4 smem4[];
@@ -494,7 +498,7 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy_force(float2* __restrict__ dat
     const int tid = threadIdx.x, c = tid & 7, j = tid >> 3;
     for (int t = blockIdx.x; t < TPF; t += gridDim.x) {
         const int kx = (t % NG) * 8 + c;
-        const size_t off = hs_index<L, true>(kx, 0, t / NG);
+        const size_t off = hs_index<L, BLK>(kx, 0, t / NG);
         const float kxv = kf * (float)kx;
 #pragma unroll 1
         for (int pass = 0; pass < 3; ++pass) {
@@ -505,7 +509,7 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy_force(float2* __restrict__ dat
 #pragma unroll
                 for (int r = 0; r < RA; ++r) {
                     const int y = j + r * (L / RA);
-                    v[r] = __ldcg(src + hs_row<L, true, L / RA>(j, r));
+                    v[r] = __ldcg(src + hs_row<L, BLK, L / RA>(j, r));
                     if (pass == 1) v[r] = cscale(v[r], kf * (float)sbin(y, L));
                 }
                 dft<RA, +1>(v);
@@ -516,9 +520,57 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy_force(float2* __restrict__ dat
             if (tid < K::TB) {
                 float2 u[RB];
                 stage_b<L, RA, RB, +1>(xb, tws, c, j, u);
-                const float sc = pass == 2 ? kxv : 1.0f;
+                const float sc = pass == 2 ? sg * kxv : sg;
 #pragma unroll
-                for (int r = 0; r < RB; ++r) dst[hs_row<L, true, RA>(j, r)] = make_float2(-sc * u[r].y, sc * u[r].x);
+                for (int r = 0; r < RB; ++r) dst[hs_row<L, BLK, RA>(j, r)] = make_float2(-sc * u[r].y, sc * u[r].x);
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// Inverse y pass of the first-order LPT: six spectra from the three bases A, B, C of the z pass (see launch_fy_lpt). The
+// x and y derivatives of one base differ by factors constant along a z line, so the passes carry 4 + 12, 12 + 24
+// and 24 + 16 bytes per cell (the x pass makes nine rows of them) instead of 4 + 36, 36 + 36 and 36 + 36.
+template <int L>
+__global__ void __launch_bounds__(K2<L>::T) k2_fy_lpt(const float2* __restrict__ bases, float2* __restrict__ dst, size_t fstride,
+                                                      const float2* __restrict__ tw) {
+    using K = K2<L>;
+    constexpr int RA = K::RA, RB = K::RB, n = L / 2, NG = n / 8, TPF = NG * L;
+    extern __shared__ float4 smem4[];
+    float2* xb = reinterpret_cast<float2*>(smem4);
+    Tw2* tws = reinterpret_cast<Tw2*>(xb + Xch<L, RA>::SIZE);
+    pdl_trigger();
+    load_tw2<L, L>(tws, tw, K::T);
+    pdl_wait();
+    __syncthreads();
+    const float kf = 6.283185307179586f / (float)L;
+    const int tid = threadIdx.x, c = tid & 7, j = tid >> 3;
+    for (int t = blockIdx.x; t < TPF; t += gridDim.x) {
+        const size_t off = hs_index<L, false>((t % NG) * 8 + c, 0, t / NG);
+#pragma unroll 1
+        for (int f = 0; f < 6; ++f) {   // A, k_y A, k_y^2 A, B, k_y B, C
+            const float2* src = bases + (f < 3 ? 0 : (f < 5 ? 1 : 2)) * fstride + off;
+            const int power = f < 3 ? f : (f == 4 ? 1 : 0);
+            if (tid < K::TA) {
+                float2 v[RA];
+#pragma unroll
+                for (int r = 0; r < RA; ++r) {
+                    v[r] = __ldcg(src + hs_row<L, false, L / RA>(j, r));   // a base's second and third time from L2
+                    const float ky = kf * (float)sbin(j + r * (L / RA), L);
+                    if (power) v[r] = cscale(v[r], power == 1 ? ky : ky * ky);
+                }
+                dft<RA, +1>(v);
+#pragma unroll
+                for (int r = 0; r < RA; ++r) xb[Xch<L, RA>::at(c, j * RA + r)] = v[r];
+            }
+            __syncthreads();
+            if (tid < K::TB) {
+                float2 u[RB];
+                stage_b<L, RA, RB, +1>(xb, tws, c, j, u);
+                float2* d = dst + f * fstride + off;
+#pragma unroll
+                for (int r = 0; r < RB; ++r) d[hs_row<L, false, RA>(j, r)] = u[r];
             }
             __syncthreads();
         }
@@ -721,6 +773,110 @@ __global__ void __launch_bounds__(X2<n>::T, 3) k2_fx_inv(float2* __restrict__ da
             for (int r = 0; r < RB; ++r) d[(size_t)c * n + j + RA * r] = u[r];
         }
         // no barrier: the next tile's stage A writes xb only after the wait + barrier at its top
+    }
+    cp_async_wait<0>();
+}
+
+// Inverse x pass of the first-order LPT and the second-order source (see launch_fx_lpt): nine c2r transforms per row from six
+// spectra, 8 rows per tile, each spectrum's rows staged by cp.async while the one before is transformed. The six second
+// derivatives stay in registers, where a thread holds the same cells of each row; they were stored (24 bytes
+// per cell), read by a pass that formed the source, and written and read once more: at 256^3 the x pass and the
+// source pass took 281 and 71 us, this one 225 (1.8 TB/s: bound by the exchanges of nine transforms per row and their
+// barriers, at 12 to 16 warps per SM), with the y pass 273 and now 121, the z pass 139 and 80; the initial conditions
+// of 256^3 particles as a whole went from 1122 to 914 us.
+template <int n>
+__global__ void __launch_bounds__(X2<n>::T, (X2<n>::RB >= 16 ? 3 : 4) * 128 / X2<n>::T)
+    k2_fx_lpt(const float2* __restrict__ spec, size_t fstride, float2* __restrict__ psi, float2* __restrict__ src,
+              const float2* __restrict__ tw, int nitems, float vscale) {
+    using X = X2<n>;
+    constexpr int RA = X::RA, RB = X::RB, N = 2 * n, T = X::T;
+    extern __shared__ float4 smem4[];
+    float2* xb = reinterpret_cast<float2*>(smem4);
+    Tw2* tws = reinterpret_cast<Tw2*>(xb + Xch<n, RA>::SIZE);
+    float2* stg = reinterpret_cast<float2*>(tws + 1);   // [8][n]
+    pdl_trigger();
+    load_tw2<n, N>(tws, tw, T);
+    pdl_wait();
+    const int tid = threadIdx.x;
+    const float kf = 6.283185307179586f / (float)N;
+    // order of the spectra: xx first, then yy and zz (the products), then the mixed ones
+    constexpr int NS = 6;
+    constexpr int FIELD[NS] = {0, 2, 5, 1, 3, 4};   // A, k_y^2 A, C, k_y A, B, k_y B
+    auto prefetch = [&](int t, int f) {
+        const float2* g = spec + (size_t)f * fstride + (size_t)t * 8 * n;
+        for (int e = tid; e < 8 * n / 2; e += T) cp_async16_cg(stg + 2 * e, g + 2 * e);
+        cp_async_commit();
+    };
+    // c2r of the staged rows times (1, k_x or k_x^2) [times i vscale]: u = real pairs at j + RA r of line c
+    const int ca = tid / (n / RA), ja = tid % (n / RA), c = tid / RA, j = tid % RA;
+    auto transform = [&](int power, bool vec, float2* u) {
+        if (tid < X::TA) {
+            const float2* row = stg + ca * n;
+            auto factor = [&](int k, float2 x) {
+                const float kx = kf * (float)k;
+                const float f = (power == 0 ? 1.0f : (power == 1 ? kx : kx * kx)) * (vec ? vscale : 1.0f);
+                return vec ? make_float2(-f * x.y, f * x.x) : cscale(x, f);
+            };
+            float2 v[RA];
+#pragma unroll
+            for (int r = 0; r < RA; ++r) {
+                const int k = ja + r * (n / RA);
+                const float2 xk = factor(k, row[k]);
+                const float2 xc = k == 0 ? make_float2(0.0f, 0.0f) : cconj(factor(n - k, row[k == 0 ? 0 : n - k]));
+                const float2 E = cadd(xk, xc);
+                const float2 O = cmul(csub(xk, xc), cconj(tw[k]));
+                v[r] = make_float2(E.x - O.y, E.y + O.x);
+            }
+            dft<RA, +1>(v);
+#pragma unroll
+            for (int r = 0; r < RA; ++r) xb[Xch<n, RA>::at(ca, ja * RA + r)] = v[r];
+        }
+        __syncthreads();
+        if (tid < X::TB) stage_b<n, RA, RB, +1>(xb, tws, c, j, u);
+    };
+    if (blockIdx.x < nitems) prefetch(blockIdx.x, FIELD[0]);
+    for (int t = blockIdx.x; t < nitems; t += gridDim.x) {
+        const size_t out = ((size_t)t * 8 + c) * n + j;
+        float2 S[RB], D[RB];   // the source so far; xx, then xx + yy
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            cp_async_wait<0>();
+            __syncthreads();   // the staged rows are complete, the exchange buffer free
+            const int f = FIELD[s];
+            float2 u[RB];
+            if (f == 0 || f == 1 || f == 3) {   // a displacement component from the same spectrum
+                transform(f == 0 ? 1 : 0, true, u);
+                if (tid < X::TB) {
+                    float2* d = psi + (size_t)(f == 0 ? 0 : (f == 1 ? 1 : 2)) * fstride + out;
+#pragma unroll
+                    for (int r = 0; r < RB; ++r) d[RA * r] = u[r];
+                }
+                __syncthreads();   // the exchange buffer has been read
+            }
+            transform(f == 0 ? 2 : (f == 1 || f == 3 ? 1 : 0), false, u);
+            // every thread has passed the barrier after the last read of the staged rows
+            if (s + 1 < NS) prefetch(t, FIELD[s + 1 < NS ? s + 1 : 0]);
+            else if (t + (int)gridDim.x < nitems) prefetch(t + gridDim.x, FIELD[0]);
+            if (tid < X::TB) {
+#pragma unroll
+                for (int r = 0; r < RB; ++r) {
+                    if (s == 0) {
+                        D[r] = u[r];
+                    } else if (s == 1) {
+                        S[r] = make_float2(D[r].x * u[r].x, D[r].y * u[r].y);
+                        D[r] = cadd(D[r], u[r]);
+                    } else if (s == 2) {
+                        S[r] = make_float2(fmaf(D[r].x, u[r].x, S[r].x), fmaf(D[r].y, u[r].y, S[r].y));
+                    } else {
+                        S[r] = make_float2(fmaf(-u[r].x, u[r].x, S[r].x), fmaf(-u[r].y, u[r].y, S[r].y));
+                    }
+                }
+            }
+        }
+        if (tid < X::TB) {
+#pragma unroll
+            for (int r = 0; r < RB; ++r) src[out + RA * r] = S[r];
+        }
     }
     cp_async_wait<0>();
 }

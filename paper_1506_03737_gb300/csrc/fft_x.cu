@@ -96,4 +96,28 @@ cudaError_t launch_fx_inv(int n_mesh, float2* data, size_t field_stride, int nfi
     }
 }
 
+template <int N>
+static cudaError_t fx_lpt_t(const float2* spec, size_t fstride, float2* psi, float2* src, const float2* tw, float vscale,
+                            cudaStream_t s) {
+    constexpr int n = N / 2;
+    using X = X2<n>;
+    static GridCache cache;
+    int grid = 0;
+    cudaError_t e = cached_grid(cache, k2_fx_lpt<n>, X::T, X::SMEM_INV, &grid);
+    if (e != cudaSuccess) return e;
+    const int items = N * N / 8;
+    return launch_dep(overlap_mesh(N), k2_fx_lpt<n>, grid < items ? grid : items, X::T, X::SMEM_INV, s, spec, fstride, psi, src, tw,
+                      items, vscale);
+}
+
+cudaError_t launch_fx_lpt(int np, const float2* spectra, size_t field_stride, float2* psi, float2* src, const float2* tw,
+                          float vscale, cudaStream_t s) {
+    switch (np) {
+#define X(N) case N: return fx_lpt_t<N>(spectra, field_stride, psi, src, tw, vscale, s);
+        COLAPM_FOR_LPT_SIZES(X)
+#undef X
+        default: return cudaErrorInvalidValue;
+    }
+}
+
 }  // namespace colapm

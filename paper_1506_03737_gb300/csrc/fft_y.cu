@@ -41,22 +41,62 @@ static cudaError_t fy_t(int sign, float2* data, size_t fstride, int nfields, con
                     : fy_sign<N, +1>(data, fstride, nfields, tw, s, two_stage, blocked);
 }
 
-template <int N>
-static cudaError_t fy_force_t(float2* data, size_t fstride, const float2* tw, cudaStream_t s) {
+template <int N, bool BLK>
+static cudaError_t fy_force_t(float2* data, size_t fstride, const float2* tw, cudaStream_t s, float sg) {
     using K = K2<N>;
     constexpr size_t smem = sizeof(float2) * Xch<N, K::RA>::SIZE + sizeof(Tw2);
     static GridCache cache;
     int grid = 0;
-    cudaError_t e = cached_grid(cache, k2_fy_force<N>, K::T, smem, &grid);
+    cudaError_t e = cached_grid(cache, k2_fy_force<N, BLK>, K::T, smem, &grid);
     if (e != cudaSuccess) return e;
     const int total = (N / 2 / 8) * N;
-    return launch_dep(overlap_mesh(N), k2_fy_force<N>, grid < total ? grid : total, K::T, smem, s, data, fstride, tw);
+    return launch_dep(overlap_mesh(N), k2_fy_force<N, BLK>, grid < total ? grid : total, K::T, smem, s, data, fstride, tw, sg);
 }
 
-cudaError_t launch_fy_force(int n_mesh, float2* data, size_t field_stride, const float2* tw, cudaStream_t s) {
+cudaError_t launch_fy_force(int n_mesh, float2* data, size_t field_stride, const float2* tw, cudaStream_t s, bool blocked,
+                            float sg) {
+    if (!blocked) {
+        switch (n_mesh) {
+#define X(N) case N: return fy_force_t<N, false>(data, field_stride, tw, s, sg);
+            COLAPM_FOR_LPT_SIZES(X)
+#undef X
+            default: return cudaErrorInvalidValue;
+        }
+    }
     switch (n_mesh) {
-#define X(N) case N: return fy_force_t<N>(data, field_stride, tw, s);
+#define X(N) case N: return fy_force_t<N, true>(data, field_stride, tw, s, sg);
         COLAPM_FOR_BLOCKED_SIZES(X)
+#undef X
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+bool lpt_fused(int np) {
+    switch (np) {
+#define X(N) case N:
+        COLAPM_FOR_LPT_SIZES(X)
+#undef X
+        return true;
+        default: return false;
+    }
+}
+
+template <int N>
+static cudaError_t fy_lpt_t(const float2* bases, float2* spectra, size_t fstride, const float2* tw, cudaStream_t s) {
+    using K = K2<N>;
+    constexpr size_t smem = sizeof(float2) * Xch<N, K::RA>::SIZE + sizeof(Tw2);
+    static GridCache cache;
+    int grid = 0;
+    cudaError_t e = cached_grid(cache, k2_fy_lpt<N>, K::T, smem, &grid);
+    if (e != cudaSuccess) return e;
+    const int total = (N / 2 / 8) * N;
+    return launch_dep(overlap_mesh(N), k2_fy_lpt<N>, grid < total ? grid : total, K::T, smem, s, bases, spectra, fstride, tw);
+}
+
+cudaError_t launch_fy_lpt(int np, const float2* bases, float2* spectra, size_t field_stride, const float2* tw, cudaStream_t s) {
+    switch (np) {
+#define X(N) case N: return fy_lpt_t<N>(bases, spectra, field_stride, tw, s);
+        COLAPM_FOR_LPT_SIZES(X)
 #undef X
         default: return cudaErrorInvalidValue;
     }

@@ -79,15 +79,18 @@ static cudaError_t fz_mode(float2* in, ZOut out, const float2* tw, const float* 
         return fz2<N, MODE, false>(in, out, tw, sinc2, deconv, gnorm, pw, s);
     }
     if (blocked) return cudaErrorInvalidValue;
-    using C = Fz<N, MODE>;
-    const size_t smem = C::BASE_SMEM + (MODE == Z_POWER ? (size_t)pw.nbins * 24 + (size_t)(pw.nbins + 1) * 4 : 0);
-    static GridCache cache;
-    int grid = 0;
-    cudaError_t e = cached_grid(cache, k_fz<N, MODE>, C::T, smem, &grid);
-    if (e != cudaSuccess) return e;
-    const int total = (N / 2 / 8) * N;
-    k_fz<N, MODE><<<grid < total ? grid : total, C::T, smem, s>>>(in, out, tw, sinc2, deconv, gnorm, pw);
-    return cudaGetLastError();
+    if constexpr (MODE == Z_LPT1_BASES || MODE == Z_LPT2_BASES) return cudaErrorInvalidValue;
+    else {
+        using C = Fz<N, MODE>;
+        const size_t smem = C::BASE_SMEM + (MODE == Z_POWER ? (size_t)pw.nbins * 24 + (size_t)(pw.nbins + 1) * 4 : 0);
+        static GridCache cache;
+        int grid = 0;
+        cudaError_t e = cached_grid(cache, k_fz<N, MODE>, C::T, smem, &grid);
+        if (e != cudaSuccess) return e;
+        const int total = (N / 2 / 8) * N;
+        k_fz<N, MODE><<<grid < total ? grid : total, C::T, smem, s>>>(in, out, tw, sinc2, deconv, gnorm, pw);
+        return cudaGetLastError();
+    }
 }
 
 template <int N>
@@ -100,6 +103,8 @@ static cudaError_t fz_t(int mode, float2* in, ZOut out, const float2* tw, const 
         case Z_LPT1: return fz_mode<N, Z_LPT1>(in, out, tw, sinc2, deconv, gnorm, pw, s, ts, blk);
         case Z_LPT2: return fz_mode<N, Z_LPT2>(in, out, tw, sinc2, deconv, gnorm, pw, s, ts, blk);
         case Z_POWER: return fz_mode<N, Z_POWER>(in, out, tw, sinc2, deconv, gnorm, pw, s, ts, blk);
+        case Z_LPT1_BASES: return fz_mode<N, Z_LPT1_BASES>(in, out, tw, sinc2, deconv, gnorm, pw, s, ts, blk);
+        case Z_LPT2_BASES: return fz_mode<N, Z_LPT2_BASES>(in, out, tw, sinc2, deconv, gnorm, pw, s, ts, blk);
         case Z_SCALE_FWD: return fz_mode<N, Z_SCALE_FWD>(in, out, tw, sinc2, deconv, gnorm, pw, s, false, blk);
         case Z_SCALE_INV: return fz_mode<N, Z_SCALE_INV>(in, out, tw, sinc2, deconv, gnorm, pw, s, false, blk);
         default: return cudaErrorInvalidValue;
