@@ -814,7 +814,10 @@ int power_enqueue(colapm_ctx* c, int nbins, const DepositSrc* src = nullptr, boo
     pw.pnorm = (float)(box * box * box / (nm * nm * nm * nm * nm * nm));
     pw.lga = c->pw_lga;
     pw.lgb = c->pw_lgb;
-    CKL(launch_fz(c->nm, Z_POWER, reinterpret_cast<float2*>(c->F), ZOut{}, c->tw_m, c->sinc2_m + (window ? 0 : c->nm), 0, 1.0f, &pw,
+    ZOut out{};
+    out.maps = c->zmaps;
+    out.err = c->err;
+    CKL(launch_fz(c->nm, Z_POWER, reinterpret_cast<float2*>(c->F), out, c->tw_m, c->sinc2_m + (window ? 0 : c->nm), 0, 1.0f, &pw,
                   c->stream, ts(c, COLAPM_PLAN_Z), use_blocked(c)));
     return COLAPM_OK;
 }

@@ -189,6 +189,97 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy(float2* __restrict__ data, siz
     }
 }
 
+// P(k) of a tile of C columns (k_y = ky, k_x = kx0 + c): pbuf holds |X|^2, C lines of PP floats with one word of padding per
+// PER z; each of the T threads bins PER consecutive z of one line, and their mirror images L - z, which have the same
+// |n| and window (iw2: 1 / sinc^4 along z): FP32 sums of at most 2 PER modes, then one reduction each in L2
+// (fire and forget; shared-memory FP64 atomics are retry loops on which the lanes of a warp collide), over 16
+// copies of the bins. What bounded the binning was the search for the next bin, which the lanes of a warp reach
+// at different modes (BinWalk), and a square root and a division per mode. At 64^3, 128^3, 512^3 and 1024^3 with
+// 32 to 100 bins the pass took 17, 42, 717 and 5171 us with them, then 9, 16, 290 and 1978 us (512^3
+// with its tiles moved by boxes, k2_power_box: 228). Counting the modes apart, over 1/48 of the grid, took
+// 460 us at 1024^3: the loops were too few and too long.
+template <int L, int C, int T>
+struct PowerTile {
+    static constexpr int PER = L * C / (2 * T), PP = ((L + L / PER + 31) / 32) * 32 + 32 / C;   // the reads of a warp on 32 banks
+    static_assert(PER * T * 2 == L * C && L % PER == 0, "the runs must cover the tile");
+    __device__ __forceinline__ static int at(int c, int z) { return c * PP + z + z / PER; }
+};
+template <int L, int C, int T>
+__device__ __forceinline__ void power_bin_tile(const float* pbuf, int kx0, int ky, const float* __restrict__ sinc2,
+                                               const float* iw2, const int* lo, const PowerArgs& pw, double* part) {
+    using P = PowerTile<L, C, T>;
+    const int c = threadIdx.x % C, j = threadIdx.x / C, nx = kx0 + c, ny = sbin(ky, L);
+    const float wxy = sinc2[nx] * sinc2[ky];
+    const float cf = __fdividef(nx == 0 ? pw.pnorm : 2.0f * pw.pnorm, wxy * wxy);
+    const float ck = nx == 0 ? pw.kf : 2.0f * pw.kf;
+    const int nxy2 = nx * nx + ny * ny, z0 = j * P::PER;
+    double* psum = part + pw.nbins;
+    unsigned long long* cnt = reinterpret_cast<unsigned long long*>(part + 2 * pw.nbins);
+    BinWalk w;
+    w.start(nxy2 + z0 * z0, lo, pw);
+    float acc = 0.0f, ks = 0.0f;
+    unsigned modes = 0;
+    auto flush = [&]() {
+        const int b = w.bin(pw.nbins);
+        if (b >= 0) {
+            atomicAdd(&part[b], (double)(ks * ck));
+            atomicAdd(&psum[b], (double)(acc * cf));
+            atomicAdd(&cnt[b], (unsigned long long)(nx == 0 ? modes : 2 * modes));
+        }
+        acc = 0.0f;
+        ks = 0.0f;
+        modes = 0;
+    };
+#pragma unroll
+    for (int zz = 0; zz < P::PER; ++zz) {
+        const int z = z0 + zz, m = L - z, n2 = nxy2 + z * z;
+        const float s = pbuf[P::at(c, z)] + (z ? pbuf[P::at(c, m)] : 0.0f);
+        if (w.leaves(n2)) {   // the run leaves its bin
+            flush();
+            w.advance(n2, pw.nbins);
+        }
+        acc = fmaf(s, iw2[z], acc);
+        ks = fmaf(z ? 2.0f : 1.0f, sqrtf((float)n2), ks);
+        modes += z ? 2 : 1;
+    }
+    flush();
+}
+// The CTA that finishes last adds up the regions (in their order) into the result.
+__device__ __forceinline__ void power_sum_regions(const PowerArgs& pw, int T) {
+    __shared__ unsigned last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(pw.done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int b = threadIdx.x; b < 2 * pw.nbins; b += T) {
+        double s = 0.0;
+#pragma unroll 16
+        for (int r = 0; r < pw.regions; ++r) s += __ldcg(pw.part + (size_t)r * 3 * pw.nbins + b);
+        (b < pw.nbins ? pw.ksum : pw.psum - pw.nbins)[b] = s;
+    }
+    for (int b = threadIdx.x; b < pw.nbins; b += T) {
+        unsigned long long s = 0;
+#pragma unroll 16
+        for (int r = 0; r < pw.regions; ++r)
+            s += __ldcg(reinterpret_cast<const unsigned long long*>(pw.part + (size_t)r * 3 * pw.nbins + 2 * pw.nbins + b));
+        pw.cnt[b] = s;
+    }
+}
+// The tables of a P(k) pass: 1 / sinc^4 along z, the thresholds.
+template <int L>
+__device__ __forceinline__ void power_tables(float* iw2, int* lo, const float* __restrict__ sinc2, const PowerArgs& pw, int T) {
+    load_thresholds(lo, pw, threadIdx.x, T);
+    for (int z = threadIdx.x; z < L / 2; z += T) {
+        const float s2 = sinc2[z];
+        iw2[z] = 1.0f / (s2 * s2);
+    }
+}
+__device__ __forceinline__ double* power_region(const PowerArgs& pw) {
+    return pw.part + (size_t)(blockIdx.x & (pw.regions - 1)) * 3 * pw.nbins;
+}
+
 // ---------------------------------------------------------------------------------------------
 // z pass with the spectral operator fused (see k_fz in fft_kernels.cuh for the algebra):
 // forward z (radices R1, R2) -> bases in registers -> inverse z (radices R2, R1) per base.
@@ -206,11 +297,7 @@ struct Z2 {
     static constexpr int PF = PREFETCH ? C * L : 0;                               // dense [z][C] buffer
     static constexpr int TA = C * L / R1, TB = C * L / R2, T = TA > TB ? TA : TB;
     static constexpr size_t SMEM = sizeof(float2) * ((size_t)XS * (1 + NSAVE) + PF) + sizeof(Tw2);
-    // Z_POWER: |X|^2 of the tile, C lines of L floats; a thread bins PER z of one line and their mirror
-    // images L - z. One word of padding per PER and a pitch of 32 / C (mod 32) put the reads of a
-    // warp on 32 banks. Then the table 1 / sinc^4 of the window along z.
-    static constexpr int PER = L * C / (2 * T), PP = ((L + L / PER + 31) / 32) * 32 + 32 / C;
-    static_assert(MODE != Z_POWER || (PER * T * 2 == L * C && L % PER == 0), "the runs must cover the tile");
+    static constexpr int PP = PowerTile<L, C, MODE == Z_POWER ? T : L * C / 16>::PP;   // of the |X|^2 lines
     static constexpr size_t SMEM_POWER = SMEM + sizeof(float) * ((size_t)C * PP + L / 2);
     // CTAs per SM: 16 warps for the LPT bases (at most 128 registers; 256 points: 103 and 78 us without the bound, 80 and
     // 54 with it); 12 warps where a task holds 32 values, 20 (at most 102 registers) with the smaller radices
@@ -237,12 +324,8 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
     pdl_wait();
     double* part = nullptr;                                      // Z_POWER: the sums this CTA adds to
     if constexpr (MODE == Z_POWER) {
-        load_thresholds(lo, pw, threadIdx.x, T);
-        for (int z = threadIdx.x; z < L / 2; z += T) {
-            const float s2 = sinc2[z];
-            iw2[z] = 1.0f / (s2 * s2);
-        }
-        part = pw.part + (size_t)(blockIdx.x & (pw.regions - 1)) * 3 * pw.nbins;
+        power_tables<L>(iw2, lo, sinc2, pw, T);
+        part = power_region(pw);
     }
     __syncthreads();
     const float kf = 6.283185307179586f / (float)L;
@@ -317,60 +400,16 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
         }
 
         if constexpr (MODE == Z_POWER) {
-            // |X|^2 of the C columns in z order, then runs of consecutive z, each with its mirror image L - z (the
-            // same |n| and window), into the bins: FP32 sums of at most 2 PER modes, then one reduction each in
-            // L2 (fire and forget; shared-memory FP64 atomics are retry loops on which the lanes of a warp
-            // collide), over 16 copies of the bins. What bounded the binning was the search for the next bin,
-            // which the lanes of a warp reach at different modes (BinWalk), and a square root and a division
-            // per mode. At 64^3, 128^3, 512^3 and 1024^3 with 32 to 100 bins the pass took 17, 42, 717 and 5171 us
-            // and takes 9, 16, 290 and 1978 us. Counting the modes apart, over 1/48 of the grid, took 460 us
-            // at 1024^3: the loops were too few and too long. The next tile's stage A only touches the
-            // exchange buffer, and the barrier after it separates this tile's reads from the next tile's values.
+            // |X|^2 in z order, then the bins (power_bin_tile)
             if (tid < TB) {
 #pragma unroll
                 for (int r = 0; r < R2; ++r) {
                     const int z = j + R1 * r;
-                    pbuf[c * Z::PP + z + z / Z::PER] = fmaf(v[r].x, v[r].x, v[r].y * v[r].y);
+                    pbuf[PowerTile<L, C, T>::at(c, z)] = fmaf(v[r].x, v[r].x, v[r].y * v[r].y);
                 }
             }
             __syncthreads();
-            if (!nyq_y) {
-                const float wxy = sinc2[nx] * sinc2[ky];
-                const float cf = __fdividef(nx == 0 ? pw.pnorm : 2.0f * pw.pnorm, wxy * wxy);
-                const float ck = nx == 0 ? pw.kf : 2.0f * pw.kf;
-                const int nxy2 = nx * nx + ny * ny, z0 = j * Z::PER;
-                const float* p = pbuf + c * Z::PP;
-                double* psum = part + pw.nbins;
-                unsigned long long* cnt = reinterpret_cast<unsigned long long*>(part + 2 * pw.nbins);
-                BinWalk w;
-                w.start(nxy2 + z0 * z0, lo, pw);
-                float acc = 0.0f, ks = 0.0f;
-                unsigned modes = 0;
-                auto flush = [&]() {
-                    const int b = w.bin(pw.nbins);
-                    if (b >= 0) {
-                        atomicAdd(&part[b], (double)(ks * ck));
-                        atomicAdd(&psum[b], (double)(acc * cf));
-                        atomicAdd(&cnt[b], (unsigned long long)(nx == 0 ? modes : 2 * modes));
-                    }
-                    acc = 0.0f;
-                    ks = 0.0f;
-                    modes = 0;
-                };
-#pragma unroll
-                for (int zz = 0; zz < Z::PER; ++zz) {
-                    const int z = z0 + zz, m = L - z, n2 = nxy2 + z * z;
-                    const float s = p[z + z / Z::PER] + (z ? p[m + m / Z::PER] : 0.0f);
-                    if (w.leaves(n2)) {   // the run leaves its bin
-                        flush();
-                        w.advance(n2, pw.nbins);
-                    }
-                    acc = fmaf(s, iw2[z], acc);
-                    ks = fmaf(z ? 2.0f : 1.0f, sqrtf((float)n2), ks);
-                    modes += z ? 2 : 1;
-                }
-                flush();
-            }
+            if (!nyq_y) power_bin_tile<L, C, T>(pbuf, kx0, ky, sinc2, iw2, lo, pw, part);
             continue;
         } else {
             // bases: A = g X, B = k_z A (, C = k_z^2 A); g = gnorm / (k^2 [W^d]), 0 on excluded modes
@@ -449,27 +488,7 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
         }
     }
     if constexpr (MODE == Z_POWER) {
-        // the CTA that finishes last adds up the regions (in their order) into the result
-        __shared__ unsigned last;
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) last = atomicAdd(pw.done, 1u) == gridDim.x - 1;
-        __syncthreads();
-        if (!last) return;
-        __threadfence();
-        for (int b = threadIdx.x; b < 2 * pw.nbins; b += T) {
-            double s = 0.0;
-#pragma unroll 16
-            for (int r = 0; r < pw.regions; ++r) s += __ldcg(pw.part + (size_t)r * 3 * pw.nbins + b);
-            (b < pw.nbins ? pw.ksum : pw.psum - pw.nbins)[b] = s;
-        }
-        for (int b = threadIdx.x; b < pw.nbins; b += T) {
-            unsigned long long s = 0;
-#pragma unroll 16
-            for (int r = 0; r < pw.regions; ++r)
-                s += __ldcg(reinterpret_cast<const unsigned long long*>(pw.part + (size_t)r * 3 * pw.nbins + 2 * pw.nbins + b));
-            pw.cnt[b] = s;
-        }
+        power_sum_regions(pw, T);
     }
 }
 

@@ -493,6 +493,110 @@ __global__ void __launch_bounds__(ZBox<L>::T, ZBox<L>::MINB)
     if (tid == 0) box_stores_done();
 }
 
+// ---------------------------------------------------------------------------------------------
+// P(k) z pass of the blocked layout at 256, 384 and 512 points: 4-column tiles by boxes, stages as in the force passes above (the
+// radix-32 ones on pairs), |X|^2 into shared memory, power_bin_tile. The next tile arrives during stage B and
+// the binning, which bounds the pass (one search and one flush per run, three reductions in L2 each). Against
+// k2_fz: 49 -> 46, 115 -> 112 and 287 -> 228 us at 256, 384 and 512 points (100 bins). Not at 320 (68 -> 69), and not at
+// 1024: its stages need 256 threads, and runs of 8 modes then double the reductions (1.98 -> 3.11 ms; binning by
+// half of the threads 2.07; the same at 512 points 259 us).
+template <int L>
+struct PowBox {
+    static constexpr int C = 4, R1 = F2<L>::R1, R2 = F2<L>::R2;
+    static constexpr bool PA = R1 == 32, PB = R2 == 32;                                  // stages on pairs
+    static constexpr int TA = C * L / R1 * (PA ? 2 : 1), TB = C * L / R2 * (PB ? 2 : 1), T = TA > TB ? TA : TB;
+    using X = Xch<L, R1, C>;
+    static constexpr int BOXZ = ZBox<L>::BOXZ > 256 ? 256 : ZBox<L>::BOXZ;
+    static constexpr size_t SMEM = sizeof(float2) * ((size_t)L * C + X::SIZE) + sizeof(Tw2) +
+                                   sizeof(float) * ((size_t)C * PowerTile<L, C, T>::PP + L / 2) + 8;   // then the thresholds
+    static constexpr int MINB = 512 / T;
+};
+
+template <int L>
+__global__ void __launch_bounds__(PowBox<L>::T, PowBox<L>::MINB)
+    k2_power_box(const __grid_constant__ CUtensorMap f0, const float2* __restrict__ tw, const float* __restrict__ sinc2, PowerArgs pw,
+                 int* err) {
+    using Z = PowBox<L>;
+    using X = typename Z::X;
+    using P = PowerTile<L, Z::C, Z::T>;
+    constexpr int C = Z::C, R1 = Z::R1, R2 = Z::R2, T = Z::T, NTILE = (L / 2 / C) * L;
+    extern __shared__ __align__(128) float4 smem4[];
+    float2* buf = reinterpret_cast<float2*>(smem4);
+    float2* xb = buf + L * C;
+    Tw2* tws = reinterpret_cast<Tw2*>(xb + X::SIZE);
+    const uint32_t bar = smem_u32(tws + 1);
+    float* pbuf = reinterpret_cast<float*>(tws + 1) + 2;
+    float* iw2 = pbuf + C * P::PP;
+    int* lo = reinterpret_cast<int*>(iw2 + L / 2);
+    pdl_trigger();
+    load_tw2<L, L>(tws, tw, T);
+    if (threadIdx.x == 0) {
+        mbar_init(bar);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    pdl_wait();
+    power_tables<L>(iw2, lo, sinc2, pw, T);
+    double* part = power_region(pw);
+    __syncthreads();
+    auto load = [&](int t) {
+        int ky, kx0;
+        pair_tile<L>(t, ky, kx0);
+        mbar_expect(bar, L * C * 8);
+#pragma unroll
+        for (int z = 0; z < L; z += Z::BOXZ)
+            box_load(smem_u32(buf + C * z), f0, (ky & 7) * 8 + (kx0 & 7), z, (kx0 >> 3) * (L / 8) + (ky >> 3), bar);
+    };
+    const int tid = threadIdx.x, c = tid & 3;
+    const int js = tid >> 2, h = (tid >> 4) & 1, jp = ((tid >> 2) & 3) + 4 * (tid >> 5);   // task alone, or half of one
+    if (tid == 0 && blockIdx.x < NTILE) load(blockIdx.x);
+    uint32_t phase = 0;
+    for (int t = blockIdx.x; t < NTILE; t += gridDim.x, phase ^= 1) {
+        int ky, kx0;
+        pair_tile<L>(t, ky, kx0);
+        bool ok = mbar_wait(bar, phase);
+        if (!ok) {   // flag it, let the copy land, stop
+            atomicOr(err, 4);
+            mbar_wait(bar, phase);
+        }
+        if constexpr (Z::PA) {
+            float2 v[16];
+#pragma unroll
+            for (int m = 0; m < 16; ++m) v[m] = buf[(jp + (L / R1) * (2 * m + h)) * C + c];
+            dft<16, -1, true>(v);
+            pair_dit<-1>(v, h);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) xb[X::at(c, jp * R1 + pair_dit_r(q, h))] = v[q];
+        } else if (tid < Z::TA) {
+            float2 v[R1];
+#pragma unroll
+            for (int r = 0; r < R1; ++r) v[r] = buf[(js + r * (L / R1)) * C + c];
+            dft<R1, -1, true>(v);
+#pragma unroll
+            for (int r = 0; r < R1; ++r) xb[X::at(c, js * R1 + r)] = v[r];
+        }
+        if (!__syncthreads_and(ok)) break;   // the tile has been read; the last tile's values have been binned
+        if (tid == 0 && t + (int)gridDim.x < NTILE) load(t + gridDim.x);
+        if constexpr (Z::PB) {
+            float2 v[16];
+#pragma unroll
+            for (int m = 0; m < 16; ++m) v[m] = xb[X::at(c, jp + R1 * (2 * m + h))];
+            pair_twiddle<-1>(v, tws, jp, h);
+            dft<16, -1, true>(v);
+            pair_dit<-1>(v, h);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) pbuf[P::at(c, jp + R1 * pair_dit_r(q, h))] = fmaf(v[q].x, v[q].x, v[q].y * v[q].y);
+        } else if (tid < Z::TB) {
+            float2 v[R2];
+            stage_b<L, R1, R2, -1, C, true>(xb, tws, c, js, v);
+#pragma unroll
+            for (int r = 0; r < R2; ++r) pbuf[P::at(c, js + R1 * r)] = fmaf(v[r].x, v[r].x, v[r].y * v[r].y);
+        }
+        __syncthreads();
+        if (ky != L / 2) power_bin_tile<L, C, T>(pbuf, kx0, ky, sinc2, iw2, lo, pw, part);
+    }
+    power_sum_regions(pw, T);
+}
+
 template <int MINB>
 struct PairZ {
     static constexpr size_t SMEM = sizeof(float2) * (2 * (size_t)Xch<1024, 32, 4>::SIZE + 1024 * 4) + sizeof(Tw2) + 8;

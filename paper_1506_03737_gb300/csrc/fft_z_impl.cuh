@@ -49,6 +49,18 @@ static cudaError_t fz2(float2* in, ZOut out, const float2* tw, const float* sinc
         const int total = (N / 2 / Z::C) * N;
         return launch_dep(overlap_mesh(N), k2_fz_box<N>, grid < total ? grid : total, Z::T, Z::SMEM, s, maps[0], maps[1], tw, sinc2,
                           deconv, gnorm, out.err);
+    } else if constexpr (MODE == Z_POWER && BLK && N >= 256 && N < 1024 && N % 128 == 0) {
+        using Z = PowBox<N>;
+        const auto* maps = static_cast<const CUtensorMap*>(out.maps);
+        if (!maps) return cudaErrorInvalidValue;
+        const size_t smem = Z::SMEM + (size_t)(pw.nbins + 3) * 4;
+        static GridCache cache;
+        int grid = 0;
+        cudaError_t e = cached_grid(cache, k2_power_box<N>, Z::T, smem, &grid);
+        if (e != cudaSuccess) return e;
+        const int total = (N / 2 / Z::C) * N;
+        return launch_dep(overlap_mesh(N), k2_power_box<N>, grid < total ? grid : total, Z::T, smem, s, maps[0], tw, sinc2, pw,
+                          out.err);
     } else {
         // Blocked layout: 4-column tiles (32-byte rows whose 512-byte runs the neighbouring tiles
         // complete), which with the prefetch buffer measured 2% faster than 8-column ones (34% for the
