@@ -47,7 +47,7 @@ typedef struct {
 /* s_in = s_out = 1, lr = 1e-3, beta1 = 0.9, beta2 = 0.999, eps = 1e-8, engine = 0, seed = 1. */
 void colapm_nn_default_config(colapm_nn_config* cfg);
 
-/* A network for n^3 fields (n a multiple of 16, 16..1024); allocates about 7 n^3 x 32 bytes of
+/* A network for n^3 fields (n a multiple of 16, 16..1024); allocates about 6 (n + 2)^3 x 32 bytes of
  * activations plus a few MB. `stream` is a cudaStream_t (may be NULL). Synchronises. */
 int colapm_nn_create(int n, const colapm_nn_config* cfg, void* stream, colapm_nn** out);
 int colapm_nn_destroy(colapm_nn* nn);

@@ -24,6 +24,7 @@ struct colapm_ctx {
     unsigned long long* rho = nullptr;   // nm^3 int64 fixed-point density
     float* F = nullptr;                  // 3 nm^3: density spectrum, then the three force meshes
     CUtensorMap zmaps[2];                // boxes of fields 0 and 2 of F for the blocked force z pass from 256^3 on (ZOut)
+    CUtensorMap ymaps[3];                // and of fields 0, 1 and 2 for the inverse y pass
     float* Freal = nullptr;              // 3 nm^3: the real force meshes when the spectra use the blocked layout
     float4* pos = nullptr;               // np^3 (offsets, cell bits)
     float* mom = nullptr;                // 3 np^3, cells
@@ -342,7 +343,7 @@ int force_from_density(colapm_ctx* c, float* dst = nullptr) {
     {
         Phase ph(c, COLAPM_PHASE_FFT_INV);
         if (blk) {
-            CKL(launch_fy_force(c->nm, d, fs, c->tw_m, c->stream));   // bases -> three spectra
+            CKL(launch_fy_force(c->nm, d, fs, c->tw_m, c->stream, true, 1.0f, c->ymaps, c->err));   // bases -> three spectra
         } else {
             CKL(launch_fy(c->nm, +1, d, fs, 3, c->tw_m, c->stream, ts(c, COLAPM_PLAN_Y), blk));
         }
@@ -554,6 +555,14 @@ int colapm_create(const colapm_params* p, void* stream, colapm_ctx** out) {
     if (c->nm >= 256) {   // [kx/8][y/8][z][y%8][kx%8]: 64 complex per z of an 8 x 8 block of columns
         const cuuint64_t n = c->nm, dims[3] = {64, n, n / 16 * (n / 8)}, strides[2] = {512, n * 512};
         const cuuint32_t box[3] = {4, c->nm >= 512 ? 256u : (c->nm > 256 ? (cuuint32_t)c->nm / 2 : (cuuint32_t)c->nm), 1};
+        const cuuint64_t ydims[4] = {8, 8, n, n / 16 * (n / 8)}, ystrides[3] = {64, 512, n * 512};
+        const cuuint32_t ybox[4] = {4, 8, 1, (cuuint32_t)c->nm / 8};
+        for (int f = 0; f < 3; ++f)
+            if (!encode_box<4>(&c->ymaps[f], c->F + f * c->nm3, ydims, ystrides, ybox)) {
+                free_all(c);
+                delete c;
+                return COLAPM_E_CUDA;
+            }
         for (int f = 0; f < 2; ++f)
             if (!encode_box3(&c->zmaps[f], c->F + 2 * f * c->nm3, dims, strides, box)) {
                 free_all(c);

@@ -24,7 +24,7 @@ struct StepCoef {
 // Output pointers of a z pass (up to 9 spectra: 3 x Psi1 and 6 x phi_ij of the ICs).
 struct ZOut {
     float2* p[9];
-    // blocked force pass: tensor maps of the tile boxes of fields 0 and 2 (two CUtensorMap, host), and the
+    // blocked force and P(k) passes: tensor maps of the tile boxes of fields 0 and 2 (two CUtensorMap, host), and the
     // device error word (bit 4: a bounded wait gave up)
     const void* maps = nullptr;
     int* err = nullptr;
@@ -260,10 +260,10 @@ __device__ __forceinline__ void bin_column_run(int nx, int ny, int z0, int per, 
 // Forward x pass (r2c) of N^2 rows of N reals into N^2 rows of N/2 complex (Nyquist dropped).
 // in_i64: int64 fixed-point density converted to delta = rho * scale - 1 (flags err[0] bit 0
 // when a cell has its top bit set); in_f32: real field.
-// `two_stage` selects the two-stage register FFT where it exists (256, 512, 1024 lines); the
+// `two_stage` selects the two-stage register FFT where it exists (F2Has); the
 // shared-memory Stockham kernels otherwise.
 // zero_input: clear the int64 mesh as it is read, so that the next deposit needs no memset.
-// blocked: write the half spectrum in the blocked layout [kx/8][z][y][kx%8] (two-stage engine only).
+// blocked: write the half spectrum in the blocked layout [kx/8][y/8][z][y%8][kx%8] (two-stage engine only).
 cudaError_t launch_fx_fwd_i64(int n_mesh, const unsigned long long* in, float2* out, const float2* tw,
                               float scale, int* err, cudaStream_t s, bool two_stage = true, bool zero_input = false,
                               bool blocked = false);
@@ -280,7 +280,7 @@ cudaError_t launch_fy(int n_mesh, int sign, float2* data, size_t field_stride, i
 // the bases instead of the three spectra).
 // With blocked = false in the plain layout, times sg (the second-order displacements).
 cudaError_t launch_fy_force(int n_mesh, float2* data, size_t field_stride, const float2* tw, cudaStream_t s, bool blocked = true,
-                            float sg = 1.0f);
+                            float sg = 1.0f, const void* maps = nullptr, int* err = nullptr);   // maps, err: as in ZOut, fields 0, 1, 2
 // First-order LPT after the z pass has left its three bases A, B, C (Z_LPT1_BASES) in `bases` (lpt_fused(np) only):
 // inverse y to the six spectra of A, k_y A, k_y^2 A, B, k_y B, C (`field_stride` complex apart, as the bases are), then
 // inverse x to the displacements psi (three real fields, times vscale) and the second-order source

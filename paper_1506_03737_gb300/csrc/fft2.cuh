@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
 //   F_z = i IFFT_y(B')         -> field 2 (in place)
 //   F_y = i IFFT_y(k_y A')     -> field 1
 //   F_x = i k_x IFFT_y(A')     -> field 0 (in place; A' is read twice, the second time from L2)
-// It reads 8 bytes per cell instead of the 12 of three separate spectra.
+// It reads 8 bytes per cell instead of the 12 of three separate spectra. (512 and 1024 points: k2_fy_box.)
 template <int L, bool BLK>
 __global__ void __launch_bounds__(K2<L>::T) k2_fy_force(float2* __restrict__ data, size_t fstride,
                                                         const float2* __restrict__ tw, float sg) {

@@ -1,5 +1,5 @@
-// Force z passes of the blocked layout from 256 points on: tiles moved by TMA boxes, and, for 1024 (32 x 32) and 512
-// points (16 x 32), 32-point transforms on pairs of lanes.
+// Passes of the blocked layout whose tiles are moved by TMA boxes (force and P(k) along z, force along y), and, for 1024
+// (32 x 32) and 512 points (16 x 32), 32-point transforms on pairs of lanes.
 //
 // The two-stage z pass gives every radix-32 task to one thread, which then holds 32 complex
 // values: with the saved base in shared memory that allows 12 warps per SM. Here a task is split
@@ -124,7 +124,7 @@ __device__ __forceinline__ void pair_dif(float2* v, int h) {
 // c = tid & 3, h = (tid >> 4) & 1, j = the other bits is half h of task j of column c. The partner is
 // lane ^ 16, so that the 16 lanes of a shared-memory phase are 4 columns x 4 tasks of one half: with the
 // exchange buffer's pitch (4 mod 16) they fall on 16 different 8-byte banks (as lane ^ 4 the halves met two
-// by two: 4.93 ms per pass at 1024^3, 4.59 now). The chain is that of k2_fz<1024, Z_FORCE, 4, true>: forward
+// by two: 4.93 ms per pass at 1024^3, then 4.59, and 3.39 with the boxes below). The chain is that of k2_fz<1024, Z_FORCE, 4, true>: forward
 // z (stage A DIT from global memory, exchange, stage B DIT), the Green's function with CIC deconvolution,
 // the saved base B = k_z A in shared memory, and two inverse z transforms (stage A DIF, exchange, stage B
 // DIT) written as the bases A' (field 0) and B' (field 2).
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(PZ_T, MINB)
 // The same pass for 512-point lines (L = 16 x 32): the radix-16 stages keep one thread per task, the radix-32 ones
 // use a pair, so that all 128 threads of a 4-column tile work in every stage with 16 values each. With one
 // thread per task the radix-32 stages left half of the threads waiting at the barrier and held 32
-// values: 530 us at 512^3 with 3 CTAs per SM, 457 now with 4 (500 with 5, 587 with 6: more tiles in flight
+// values: 530 us at 512^3 with 3 CTAs per SM, 457 with 4, 364 with the boxes (500 with 5, 587 with 6: more tiles in flight
 // only queue for the L1 data path, which is 71% busy; a 32-byte row of the mesh costs it as much as
 // 128 bytes of shared memory).
 constexpr int PZ5_T = 128, PZ5_MINB = 4;
@@ -494,8 +494,126 @@ __global__ void __launch_bounds__(ZBox<L>::T, ZBox<L>::MINB)
 }
 
 // ---------------------------------------------------------------------------------------------
-// P(k) z pass of the blocked layout at 256, 384 and 512 points: 4-column tiles by boxes, stages as in the force passes above (the
-// radix-32 ones on pairs), |X|^2 into shared memory, power_bin_tile. The next tile arrives during stage B and
+// Inverse y pass of the force (k2_fy_force in fft2.cuh) with tiles of 4 columns moved by boxes: A' of the tile is read once
+// for its two transforms, B' arrives while the second one's stage B runs, the next tile's A' during the third one's.
+// What bounded k2_fy_force was latency: 16 warps per SM at 127 registers and no load in flight while a tile is
+// transformed (66 to 69% of the DRAM's cycles). From 512 points on the pass went from 512 to 464 us and, at 1024, from 3.93
+// to 3.81 ms (84% of the copy bandwidth); below, the boxes lose: 53 -> 59, 111 -> 115 and 186 -> 195 us at 256, 320, 384.
+#define COLAPM_FOR_FY_BOX_SIZES(X) X(512) X(1024)
+template <int L>
+struct FyBox {
+    static constexpr int C = 4, R1 = F2<L>::R1, R2 = F2<L>::R2;
+    static constexpr bool PA = R1 == 32, PB = R2 == 32;                                  // stages on pairs
+    static constexpr int TA = C * L / R1 * (PA ? 2 : 1), TB = C * L / R2 * (PB ? 2 : 1), T = TA > TB ? TA : TB;
+    using X = Xch<L, R1, C>;
+    static constexpr int XS = (X::SIZE + 15) / 16 * 16;   // to 128 bytes
+    static constexpr size_t SMEM = sizeof(float2) * ((size_t)XS + 2 * L * C) + sizeof(Tw2) + 8;
+    static constexpr int MINB = 512 / T;
+};
+
+template <int L>
+__global__ void __launch_bounds__(FyBox<L>::T, FyBox<L>::MINB)
+    k2_fy_box(const __grid_constant__ CUtensorMap f0, const __grid_constant__ CUtensorMap f1, const __grid_constant__ CUtensorMap f2,
+              const float2* __restrict__ tw, int* err) {
+    using Z = FyBox<L>;
+    using X = typename Z::X;
+    constexpr int C = Z::C, R1 = Z::R1, R2 = Z::R2, T = Z::T, n = L / 2, NTILE = (n / C) * L;
+    extern __shared__ __align__(128) float4 smem4[];
+    float2* xb = reinterpret_cast<float2*>(smem4);
+    float2* in = xb + Z::XS;            // [y][4]: A', then B'
+    float2* ob = in + L * C;            // the tile of each output
+    Tw2* tws = reinterpret_cast<Tw2*>(ob + L * C);
+    const uint32_t bar = smem_u32(tws + 1);
+    pdl_trigger();
+    load_tw2<L, L>(tws, tw, T);
+    if (threadIdx.x == 0) {
+        mbar_init(bar);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    pdl_wait();
+    __syncthreads();
+    // tile t: columns kx0 .. kx0 + 3 of plane z; the two halves of a block on neighbouring CTAs
+    auto load = [&](int t, const CUtensorMap& f) {
+        const int q = t % (n / C);
+        mbar_expect(bar, L * C * 8);
+        box_load4(smem_u32(in), f, (q & 1) * 4, 0, t / (n / C), (q >> 1) * (L / 8), bar);
+    };
+    const int tid = threadIdx.x, c = tid & 3;
+    const int js = tid >> 2, h = (tid >> 4) & 1, jp = ((tid >> 2) & 3) + 4 * (tid >> 5);   // task alone, or half of one
+    const float kf = 6.283185307179586f / (float)L;
+    if (tid == 0 && blockIdx.x < NTILE) load(blockIdx.x, f0);
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < NTILE && ok; t += gridDim.x) {
+        const int q = t % (n / C), z = t / (n / C);
+        const float kxv = kf * (float)(4 * q + c);
+#pragma unroll 1
+        for (int pass = 0; pass < 3; ++pass) {   // F_y from k_y A', F_x from A', F_z from B'
+            if (pass != 1) {
+                ok = mbar_wait(bar, phase);
+                if (!ok) {   // flag it, let the copy land, stop
+                    atomicOr(err, 4);
+                    mbar_wait(bar, phase);
+                }
+                phase ^= 1;
+            }
+            auto value = [&](int y) {
+                const float2 a = in[y * C + c];
+                return pass == 0 ? cscale(a, kf * (float)sbin(y, L)) : a;
+            };
+            if constexpr (Z::PA) {
+                float2 v[16];
+#pragma unroll
+                for (int m = 0; m < 16; ++m) v[m] = value(jp + (L / R1) * (2 * m + h));
+                dft<16, +1, true>(v);
+                pair_dit<+1>(v, h);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) xb[X::at(c, jp * R1 + pair_dit_r(i, h))] = v[i];
+            } else if (tid < Z::TA) {
+                float2 v[R1];
+#pragma unroll
+                for (int r = 0; r < R1; ++r) v[r] = value(js + r * (L / R1));
+                dft<R1, +1, true>(v);
+#pragma unroll
+                for (int r = 0; r < R1; ++r) xb[X::at(c, js * R1 + r)] = v[r];
+            }
+            if (tid == 0) box_stores_read();   // the output before has left `ob`
+            ok = __syncthreads_and(ok);        // the tile has been read as well
+            if (!ok) break;
+            if (tid == 0) {
+                if (pass == 1) load(t, f2);
+                if (pass == 2 && t + (int)gridDim.x < NTILE) load(t + gridDim.x, f0);
+            }
+            const float sc = pass == 1 ? kxv : 1.0f;
+            if constexpr (Z::PB) {
+                float2 v[16];
+#pragma unroll
+                for (int m = 0; m < 16; ++m) v[m] = xb[X::at(c, jp + R1 * (2 * m + h))];
+                pair_twiddle<+1>(v, tws, jp, h);
+                dft<16, +1, true>(v);
+                pair_dit<+1>(v, h);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) ob[(jp + R1 * pair_dit_r(i, h)) * C + c] = make_float2(-sc * v[i].y, sc * v[i].x);
+            } else if (tid < Z::TB) {
+                float2 v[R2];
+                stage_b<L, R1, R2, +1, C, true>(xb, tws, c, js, v);
+#pragma unroll
+                for (int r = 0; r < R2; ++r) ob[(js + R1 * r) * C + c] = make_float2(-sc * v[r].y, sc * v[r].x);
+            }
+            fence_async_smem();
+            __syncthreads();   // the output tile is complete, the exchange buffer free
+            if (tid == 0) {
+                const CUtensorMap& f = pass == 0 ? f1 : (pass == 1 ? f0 : f2);
+                box_store4(f, (q & 1) * 4, 0, z, (q >> 1) * (L / 8), smem_u32(ob));
+            }
+        }
+    }
+    if (tid == 0) box_stores_done();
+}
+
+// ---------------------------------------------------------------------------------------------
+// P(k) z pass of the blocked layout at 256, 384 and 512 points: 4-column tiles by boxes, stages as in the passes above
+// (the radix-32 ones on pairs), |X|^2 into shared memory, power_bin_tile. The next tile arrives during stage B and
 // the binning, which bounds the pass (one search and one flush per run, three reductions in L2 each). Against
 // k2_fz: 49 -> 46, 115 -> 112 and 287 -> 228 us at 256, 384 and 512 points (100 bins). Not at 320 (68 -> 69), and not at
 // 1024: its stages need 256 threads, and runs of 8 modes then double the reductions (1.98 -> 3.11 ms; binning by

@@ -1,5 +1,5 @@
 // y passes (strided columns, both directions) for every supported mesh size.
-#include "fft2.cuh"
+#include "fft_pair.cuh"
 #include "fft_kernels.cuh"
 
 namespace colapm {
@@ -53,8 +53,28 @@ static cudaError_t fy_force_t(float2* data, size_t fstride, const float2* tw, cu
     return launch_dep(overlap_mesh(N), k2_fy_force<N, BLK>, grid < total ? grid : total, K::T, smem, s, data, fstride, tw, sg);
 }
 
+template <int N>
+static cudaError_t fy_box_t(const CUtensorMap* maps, const float2* tw, cudaStream_t s, int* err) {
+    using Z = FyBox<N>;
+    static GridCache cache;
+    int grid = 0;
+    cudaError_t e = cached_grid(cache, k2_fy_box<N>, Z::T, Z::SMEM, &grid);
+    if (e != cudaSuccess) return e;
+    const int total = (N / 2 / Z::C) * N;
+    return launch_dep(overlap_mesh(N), k2_fy_box<N>, grid < total ? grid : total, Z::T, Z::SMEM, s, maps[0], maps[1], maps[2], tw, err);
+}
+
 cudaError_t launch_fy_force(int n_mesh, float2* data, size_t field_stride, const float2* tw, cudaStream_t s, bool blocked,
-                            float sg) {
+                            float sg, const void* maps, int* err) {
+    if (maps && blocked) {
+        const auto* m = static_cast<const CUtensorMap*>(maps);
+        switch (n_mesh) {
+#define X(N) case N: return fy_box_t<N>(m, tw, s, err);
+            COLAPM_FOR_FY_BOX_SIZES(X)
+#undef X
+            default: break;
+        }
+    }
     if (!blocked) {
         switch (n_mesh) {
 #define X(N) case N: return fy_force_t<N, false>(data, field_stride, tw, s, sg);

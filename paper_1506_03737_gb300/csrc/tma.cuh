@@ -1,4 +1,4 @@
-// TMA box copies of 3-D arrays of 8-byte elements, and the barriers that count them. Every wait is bounded.
+// TMA box copies of 3-D and 4-D arrays of 8-byte elements, and the barriers that count them. Every wait is bounded.
 #pragma once
 
 #include <cuda.h>
@@ -34,6 +34,12 @@ __device__ __forceinline__ void box_load(uint32_t dst, const CUtensorMap& map, i
         "l"(reinterpret_cast<uint64_t>(&map)), "r"(x), "r"(y), "r"(z), "r"(bar)
         : "memory");
 }
+__device__ __forceinline__ void box_load4(uint32_t dst, const CUtensorMap& map, int x, int y, int z, int w, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(&map)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
+        : "memory");
+}
 
 // The box back out of shared memory (written there by ordinary stores), as a bulk group of the calling thread.
 __device__ __forceinline__ void box_store(const CUtensorMap& map, int x, int y, int z, uint32_t src) {
@@ -43,21 +49,32 @@ __device__ __forceinline__ void box_store(const CUtensorMap& map, int x, int y, 
                  : "memory");
     asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
 }
+__device__ __forceinline__ void box_store4(const CUtensorMap& map, int x, int y, int z, int w, uint32_t src) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];\n" ::"l"(
+                     reinterpret_cast<uint64_t>(&map)),
+                 "r"(x), "r"(y), "r"(z), "r"(w), "r"(src)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+}
 __device__ __forceinline__ void box_stores_read() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
 __device__ __forceinline__ void box_stores_done() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
 
-// Tensor map of boxes of a 3-D array of 8-byte elements: extents, byte strides of the two outer dimensions, box.
-inline bool encode_box3(CUtensorMap* map, void* p, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
+// Tensor map of boxes of a RANK-D array of 8-byte elements: extents, byte strides of the outer dimensions, box.
+template <int RANK>
+inline bool encode_box(CUtensorMap* map, void* p, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult st;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &st) != cudaSuccess || !fn) {
         (void)cudaGetLastError();
         return false;
     }
-    const cuuint32_t one[3] = {1, 1, 1};
+    const cuuint32_t one[4] = {1, 1, 1, 1};
     return reinterpret_cast<decltype(&cuTensorMapEncodeTiled)>(fn)(
-               map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, p, dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, RANK, p, dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+inline bool encode_box3(CUtensorMap* map, void* p, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
+    return encode_box<3>(map, p, dims, strides, box);
 }
 
 }  // namespace colapm
