@@ -56,11 +56,33 @@ struct Xch {
     __host__ __device__ __forceinline__ static int at(int c, int e) { return c * PITCH + e + e / RA; }
 };
 
-// Twiddle tables for length L: w1[j] = w^j, w8[m][j] = w^(8 m j), w = exp(-2 pi i / L).
+// Twiddle tables for length L: w1[j] = w^j, w8[m][j] = w^(8 m j), w = exp(-2 pi i / L). w^(j r) is w8[r >> 3][j] times a
+// power of w1[j], made by a chain of products.
 struct Tw2 {
     float2 w1[32];
     float2 w8[4][32];
 };
+// The same with the powers too, each rounded once: w[k][j] = w^(k j), k < 8, j < JN. A chain repeats the rounding of w1[j] in
+// every power, and whatever it takes from a root's modulus it takes from each line alike, so that it stays in the mean of
+// a P(k) bin. For the lengths that would otherwise get their roots from the full table (32, 48 and 80 points, which
+// the Stockham engine transformed): power lost per line 6.9e-8, 4.0e-8 and 3.9e-8 by chains, 3.8e-8, 3.7e-8 and
+// nothing by this table (2.8e-8, 1.8e-8 and nothing there).
+template <int JN>
+struct Tw8 {
+    static_assert(JN == 16 || JN == 32, "");
+    float2 w[8][JN];
+    float2 w8[4][JN];
+};
+template <int L>
+struct TwSel {
+    using type = Tw2;
+};
+template <> struct TwSel<32> { using type = Tw8<16>; };
+template <> struct TwSel<48> { using type = Tw8<16>; };
+template <> struct TwSel<80> { using type = Tw8<16>; };
+template <int L>
+using TwOf = typename TwSel<L>::type;
+
 template <int L, int TWN>
 __device__ __forceinline__ void load_tw2(Tw2* t, const float2* __restrict__ g, int T) {
     for (int e = threadIdx.x; e < 32 * 5; e += T) {
@@ -70,16 +92,35 @@ __device__ __forceinline__ void load_tw2(Tw2* t, const float2* __restrict__ g, i
         if (m == 0) t->w1[j] = v; else t->w8[m - 1][j] = v;
     }
 }
+template <int L, int TWN, int JN>
+__device__ __forceinline__ void load_tw2(Tw8<JN>* t, const float2* __restrict__ g, int T) {
+    for (int e = threadIdx.x; e < JN * 12; e += T) {
+        const int k = e / JN, j = e % JN;
+        const float2 v = g[((k < 8 ? k : 8 * (k - 8)) * j) % L * (TWN / L)];
+        if (k < 8) t->w[k][j] = v; else t->w8[k - 8][j] = v;
+    }
+}
 
-// Multiply v[r] by w^(S j r) for r < R (j < 32).
-template <int R, int S>
-__host__ __device__ __forceinline__ void twiddle2(float2* v, const Tw2* t, int j) {
-    float2 p[8];
+// p[k] = w^(S j k), k < N <= 8.
+template <int N, int S>
+__host__ __device__ __forceinline__ void tw_powers(float2* p, const Tw2* t, int j) {
     float2 w1 = t->w1[j];
     if (S > 0) w1 = cconj(w1);
     p[0] = make_float2(1.0f, 0.0f);
 #pragma unroll
-    for (int k = 1; k < 8; ++k) p[k] = cmul(p[k - 1], w1);
+    for (int k = 1; k < N; ++k) p[k] = cmul(p[k - 1], w1);
+}
+template <int N, int S, int JN>
+__host__ __device__ __forceinline__ void tw_powers(float2* p, const Tw8<JN>* t, int j) {
+    p[0] = make_float2(1.0f, 0.0f);
+#pragma unroll
+    for (int k = 1; k < N; ++k) p[k] = S > 0 ? cconj(t->w[k][j]) : t->w[k][j];
+}
+// Multiply v[r] by w^(S j r) for r < R (j < 32).
+template <int R, int S, class TW>
+__host__ __device__ __forceinline__ void twiddle2(float2* v, const TW* t, int j) {
+    float2 p[8];
+    tw_powers<(R < 8 ? R : 8), S>(p, t, j);
 #pragma unroll
     for (int r = 1; r < R; ++r) {
         float2 w = p[r & 7];
@@ -142,8 +183,8 @@ __host__ __device__ __forceinline__ size_t hs_row(int j, int r) {
 
 // Stage B of a line held in exchange buffer xb (stage-A radix RA), task j < RA of line c:
 // loads j + RA r, twiddles, RB-point DFT. Returns X[j + RA r] in v.
-template <int L, int RA, int RB, int S, int LINES = 8, bool TRIV = false>
-__host__ __device__ __forceinline__ void stage_b(const float2* xb, const Tw2* tw, int c, int j, float2* v) {
+template <int L, int RA, int RB, int S, int LINES = 8, bool TRIV = false, class TW = Tw2>
+__host__ __device__ __forceinline__ void stage_b(const float2* xb, const TW* tw, int c, int j, float2* v) {
 #pragma unroll
     for (int r = 0; r < RB; ++r) v[r] = xb[Xch<L, RA, LINES>::at(c, j + RA * r)];
     twiddle2<RB, S>(v, tw, j);
@@ -159,7 +200,7 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy(float2* __restrict__ data, siz
     constexpr int RA = K::RA, RB = K::RB, n = L / 2, NG = n / 8, TPF = NG * L;
     extern __shared__ float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
-    Tw2* tws = reinterpret_cast<Tw2*>(xb + Xch<L, RA>::SIZE);
+    auto* tws = reinterpret_cast<TwOf<L>*>(xb + Xch<L, RA>::SIZE);
     pdl_trigger();
     load_tw2<L, L>(tws, tw, K::T);
     pdl_wait();
@@ -296,7 +337,7 @@ struct Z2 {
     static constexpr bool PREFETCH = !LPT1 && !DIRECT;
     static constexpr int PF = PREFETCH ? C * L : 0;                               // dense [z][C] buffer
     static constexpr int TA = C * L / R1, TB = C * L / R2, T = TA > TB ? TA : TB;
-    static constexpr size_t SMEM = sizeof(float2) * ((size_t)XS * (1 + NSAVE) + PF) + sizeof(Tw2);
+    static constexpr size_t SMEM = sizeof(float2) * ((size_t)XS * (1 + NSAVE) + PF) + sizeof(TwOf<L>);
     static constexpr int PP = PowerTile<L, C, MODE == Z_POWER ? T : L * C / 16>::PP;   // of the |X|^2 lines
     static constexpr size_t SMEM_POWER = SMEM + sizeof(float) * ((size_t)C * PP + L / 2);
     // CTAs per SM: 16 warps for the LPT bases (at most 128 registers; 256 points: 103 and 78 us without the bound, 80 and
@@ -315,7 +356,7 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
     float2* xb = reinterpret_cast<float2*>(smem4);
     float2* save = xb + Z::XS;                                   // bases B (, C), layout Xch<L,R1>
     float2* pf = xb + Z::XS * (1 + Z::NSAVE);                    // prefetched input tile [z][8]
-    Tw2* tws = reinterpret_cast<Tw2*>(pf + Z::PF);
+    auto* tws = reinterpret_cast<TwOf<L>*>(pf + Z::PF);
     float* pbuf = reinterpret_cast<float*>(tws + 1);             // Z_POWER: [C][PP], then the window table, then the thresholds
     float* iw2 = pbuf + (MODE == Z_POWER ? C * Z::PP : 0);
     int* lo = reinterpret_cast<int*>(iw2 + (MODE == Z_POWER ? L / 2 : 0));
@@ -508,7 +549,7 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy_force(float2* __restrict__ dat
     constexpr int RA = K::RA, RB = K::RB, n = L / 2, NG = n / 8, TPF = NG * L;
     extern __shared__ float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
-    Tw2* tws = reinterpret_cast<Tw2*>(xb + Xch<L, RA>::SIZE);
+    auto* tws = reinterpret_cast<TwOf<L>*>(xb + Xch<L, RA>::SIZE);
     pdl_trigger();
     load_tw2<L, L>(tws, tw, K::T);
     pdl_wait();
@@ -558,7 +599,7 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy_lpt(const float2* __restrict__
     constexpr int RA = K::RA, RB = K::RB, n = L / 2, NG = n / 8, TPF = NG * L;
     extern __shared__ float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
-    Tw2* tws = reinterpret_cast<Tw2*>(xb + Xch<L, RA>::SIZE);
+    auto* tws = reinterpret_cast<TwOf<L>*>(xb + Xch<L, RA>::SIZE);
     pdl_trigger();
     load_tw2<L, L>(tws, tw, K::T);
     pdl_wait();
@@ -602,7 +643,7 @@ template <int n>
 struct X2 {
     static constexpr int RA = F2<n>::R1, RB = F2<n>::R2;
     static constexpr int TA = 8 * n / RA, TB = 8 * n / RB, T = TA > TB ? TA : TB;
-    static constexpr size_t SMEM = sizeof(float2) * (size_t)Xch<n, RA>::SIZE + sizeof(Tw2);
+    static constexpr size_t SMEM = sizeof(float2) * (size_t)Xch<n, RA>::SIZE + sizeof(TwOf<n>);
     static constexpr bool SPLIT = n != 128 && n != 256;   // forward: the half spectrum inside stage B (see k2_fx_fwd)
     // inverse: plus a dense [8][n] staging buffer for the cp.async prefetch of the rows
     static constexpr size_t SMEM_INV = SMEM + sizeof(float2) * 8 * (size_t)n;
@@ -618,7 +659,7 @@ __global__ void __launch_bounds__(X2<n>::T) k2_fx_fwd(const void* __restrict__ i
     constexpr int RA = X::RA, RB = X::RB, N = 2 * n;
     extern __shared__ float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
-    Tw2* tws = reinterpret_cast<Tw2*>(xb + Xch<n, RA>::SIZE);
+    auto* tws = reinterpret_cast<TwOf<n>*>(xb + Xch<n, RA>::SIZE);
     pdl_trigger();
     load_tw2<n, N>(tws, tw, X::T);
     pdl_wait();
@@ -733,7 +774,7 @@ __global__ void __launch_bounds__(X2<n>::T, 3) k2_fx_inv(float2* __restrict__ da
     constexpr int RA = X::RA, RB = X::RB, N = 2 * n, T = X::T;
     extern __shared__ float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
-    Tw2* tws = reinterpret_cast<Tw2*>(xb + Xch<n, RA>::SIZE);
+    auto* tws = reinterpret_cast<TwOf<n>*>(xb + Xch<n, RA>::SIZE);
     float2* stg = reinterpret_cast<float2*>(tws + 1);   // [8][n]
     pdl_trigger();
     load_tw2<n, N>(tws, tw, T);
@@ -811,7 +852,7 @@ __global__ void __launch_bounds__(X2<n>::T, (X2<n>::RB >= 16 ? 3 : 4) * 128 / X2
     constexpr int RA = X::RA, RB = X::RB, N = 2 * n, T = X::T;
     extern __shared__ float4 smem4[];
     float2* xb = reinterpret_cast<float2*>(smem4);
-    Tw2* tws = reinterpret_cast<Tw2*>(xb + Xch<n, RA>::SIZE);
+    auto* tws = reinterpret_cast<TwOf<n>*>(xb + Xch<n, RA>::SIZE);
     float2* stg = reinterpret_cast<float2*>(tws + 1);   // [8][n]
     pdl_trigger();
     load_tw2<n, N>(tws, tw, T);

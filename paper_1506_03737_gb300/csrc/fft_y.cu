@@ -7,7 +7,7 @@ namespace colapm {
 template <int N, int S, bool BLK>
 static cudaError_t fy2(float2* data, size_t fstride, int nfields, const float2* tw, cudaStream_t s) {
     using K = K2<N>;
-    constexpr size_t smem = sizeof(float2) * Xch<N, K::RA>::SIZE + sizeof(Tw2);
+    constexpr size_t smem = sizeof(float2) * Xch<N, K::RA>::SIZE + sizeof(TwOf<N>);
     static GridCache cache;
     int grid2 = 0;
     cudaError_t e = cached_grid(cache, k2_fy<N, S, BLK>, K::T, smem, &grid2);
@@ -44,7 +44,7 @@ static cudaError_t fy_t(int sign, float2* data, size_t fstride, int nfields, con
 template <int N, bool BLK>
 static cudaError_t fy_force_t(float2* data, size_t fstride, const float2* tw, cudaStream_t s, float sg) {
     using K = K2<N>;
-    constexpr size_t smem = sizeof(float2) * Xch<N, K::RA>::SIZE + sizeof(Tw2);
+    constexpr size_t smem = sizeof(float2) * Xch<N, K::RA>::SIZE + sizeof(TwOf<N>);
     static GridCache cache;
     int grid = 0;
     cudaError_t e = cached_grid(cache, k2_fy_force<N, BLK>, K::T, smem, &grid);
@@ -104,7 +104,7 @@ bool lpt_fused(int np) {
 template <int N>
 static cudaError_t fy_lpt_t(const float2* bases, float2* spectra, size_t fstride, const float2* tw, cudaStream_t s) {
     using K = K2<N>;
-    constexpr size_t smem = sizeof(float2) * Xch<N, K::RA>::SIZE + sizeof(Tw2);
+    constexpr size_t smem = sizeof(float2) * Xch<N, K::RA>::SIZE + sizeof(TwOf<N>);
     static GridCache cache;
     int grid = 0;
     cudaError_t e = cached_grid(cache, k2_fy_lpt<N>, K::T, smem, &grid);
