@@ -817,7 +817,8 @@ int power_enqueue(colapm_ctx* c, int nbins, const DepositSrc* src = nullptr, boo
     if (r) return r;
     PowerArgs pw{};
     pw.n2_lo = c->pw_bin;
-    pw.kf = (float)(2.0 * M_PI / box);
+    pw.kfd = 2.0 * M_PI / box;
+    pw.kf = (float)pw.kfd;
     power_layout(pw, c->pw_acc, nbins, kPowerRegions);
     const double nm = c->nm;
     pw.pnorm = (float)(box * box * box / (nm * nm * nm * nm * nm * nm));

@@ -119,6 +119,7 @@ struct PowerArgs {
     unsigned long long* cnt;    // [nbins]
     int nbins;
     float kf;                   // 2 pi / L (h/Mpc)
+    double kfd;                 // the same; the two-stage z pass sums |n| and applies it to the sums
     float pnorm;                // L^3 / N^6
     double* part;               // [regions][3 nbins] partial sums (k, P, count as u64) of the two-stage z pass, zeroed
     unsigned* done;             // CTAs of that pass that have finished, zeroed

@@ -232,13 +232,16 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy(float2* __restrict__ data, siz
 
 // P(k) of a tile of C columns (k_y = ky, k_x = kx0 + c): pbuf holds |X|^2, C lines of PP floats with one word of padding per
 // PER z; each of the T threads bins PER consecutive z of one line, and their mirror images L - z, which have the same
-// |n| and window (iw2: 1 / sinc^4 along z): FP32 sums of at most 2 PER modes, then one reduction each in L2
+// |n| and window (win: sinc^2 along z): FP32 sums of at most 2 PER modes, then one reduction each in L2
 // (fire and forget; shared-memory FP64 atomics are retry loops on which the lanes of a warp collide), over 16
 // copies of the bins. What bounded the binning was the search for the next bin, which the lanes of a warp reach
 // at different modes (BinWalk), and a square root and a division per mode. At 64^3, 128^3, 512^3 and 1024^3 with
 // 32 to 100 bins the pass took 17, 42, 717 and 5171 us with them, then 9, 16, 290 and 1978 us (512^3
 // with its tiles moved by boxes, k2_power_box: 228). Counting the modes apart, over 1/48 of the grid, took
-// 460 us at 1024^3: the loops were too few and too long.
+// 460 us at 1024^3: the loops were too few and too long. Every pair of modes is divided by its own window: a factor
+// per column times a table per z is 4 us less at 512^3 (1722 of 1726 for the call), but their few roundings
+// stay in a bin's mean (P(k) off by 1.60, 1.77 and 2.37e-7 at 128^3, 192^3 and 384^3 instead of 1.51, 1.62 and 2.33e-7).
+// |n| is summed in units of the fundamental, which is applied to the sums in FP64.
 template <int L, int C, int T>
 struct PowerTile {
     static constexpr int PER = L * C / (2 * T), PP = ((L + L / PER + 31) / 32) * 32 + 32 / C;   // the reads of a warp on 32 banks
@@ -247,12 +250,11 @@ struct PowerTile {
 };
 template <int L, int C, int T>
 __device__ __forceinline__ void power_bin_tile(const float* pbuf, int kx0, int ky, const float* __restrict__ sinc2,
-                                               const float* iw2, const int* lo, const PowerArgs& pw, double* part) {
+                                               const float* win, const int* lo, const PowerArgs& pw, double* part) {
     using P = PowerTile<L, C, T>;
     const int c = threadIdx.x % C, j = threadIdx.x / C, nx = kx0 + c, ny = sbin(ky, L);
     const float wxy = sinc2[nx] * sinc2[ky];
-    const float cf = __fdividef(nx == 0 ? pw.pnorm : 2.0f * pw.pnorm, wxy * wxy);
-    const float ck = nx == 0 ? pw.kf : 2.0f * pw.kf;
+    const float mult = nx == 0 ? 1.0f : 2.0f, cp = mult * pw.pnorm;
     const int nxy2 = nx * nx + ny * ny, z0 = j * P::PER;
     double* psum = part + pw.nbins;
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(part + 2 * pw.nbins);
@@ -263,8 +265,8 @@ __device__ __forceinline__ void power_bin_tile(const float* pbuf, int kx0, int k
     auto flush = [&]() {
         const int b = w.bin(pw.nbins);
         if (b >= 0) {
-            atomicAdd(&part[b], (double)(ks * ck));
-            atomicAdd(&psum[b], (double)(acc * cf));
+            atomicAdd(&part[b], (double)ks);
+            atomicAdd(&psum[b], (double)acc);
             atomicAdd(&cnt[b], (unsigned long long)(nx == 0 ? modes : 2 * modes));
         }
         acc = 0.0f;
@@ -279,8 +281,9 @@ __device__ __forceinline__ void power_bin_tile(const float* pbuf, int kx0, int k
             flush();
             w.advance(n2, pw.nbins);
         }
-        acc = fmaf(s, iw2[z], acc);
-        ks = fmaf(z ? 2.0f : 1.0f, sqrtf((float)n2), ks);
+        const float w = wxy * win[z];
+        acc += __fdividef(cp * s, w * w);
+        ks = fmaf(z ? 2.0f * mult : mult, sqrtf((float)n2), ks);
         modes += z ? 2 : 1;
     }
     flush();
@@ -298,7 +301,8 @@ __device__ __forceinline__ void power_sum_regions(const PowerArgs& pw, int T) {
         double s = 0.0;
 #pragma unroll 16
         for (int r = 0; r < pw.regions; ++r) s += __ldcg(pw.part + (size_t)r * 3 * pw.nbins + b);
-        (b < pw.nbins ? pw.ksum : pw.psum - pw.nbins)[b] = s;
+        if (b < pw.nbins) pw.ksum[b] = pw.kfd * s;
+        else pw.psum[b - pw.nbins] = s;
     }
     for (int b = threadIdx.x; b < pw.nbins; b += T) {
         unsigned long long s = 0;
@@ -308,14 +312,11 @@ __device__ __forceinline__ void power_sum_regions(const PowerArgs& pw, int T) {
         pw.cnt[b] = s;
     }
 }
-// The tables of a P(k) pass: 1 / sinc^4 along z, the thresholds.
+// The tables of a P(k) pass: sinc^2 along z, the thresholds.
 template <int L>
-__device__ __forceinline__ void power_tables(float* iw2, int* lo, const float* __restrict__ sinc2, const PowerArgs& pw, int T) {
+__device__ __forceinline__ void power_tables(float* win, int* lo, const float* __restrict__ sinc2, const PowerArgs& pw, int T) {
     load_thresholds(lo, pw, threadIdx.x, T);
-    for (int z = threadIdx.x; z < L / 2; z += T) {
-        const float s2 = sinc2[z];
-        iw2[z] = 1.0f / (s2 * s2);
-    }
+    for (int z = threadIdx.x; z < L / 2; z += T) win[z] = sinc2[z];
 }
 __device__ __forceinline__ double* power_region(const PowerArgs& pw) {
     return pw.part + (size_t)(blockIdx.x & (pw.regions - 1)) * 3 * pw.nbins;
@@ -358,14 +359,14 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
     float2* pf = xb + Z::XS * (1 + Z::NSAVE);                    // prefetched input tile [z][8]
     auto* tws = reinterpret_cast<TwOf<L>*>(pf + Z::PF);
     float* pbuf = reinterpret_cast<float*>(tws + 1);             // Z_POWER: [C][PP], then the window table, then the thresholds
-    float* iw2 = pbuf + (MODE == Z_POWER ? C * Z::PP : 0);
-    int* lo = reinterpret_cast<int*>(iw2 + (MODE == Z_POWER ? L / 2 : 0));
+    float* win = pbuf + (MODE == Z_POWER ? C * Z::PP : 0);
+    int* lo = reinterpret_cast<int*>(win + (MODE == Z_POWER ? L / 2 : 0));
     pdl_trigger();
     load_tw2<L, L>(tws, tw, T);
     pdl_wait();
     double* part = nullptr;                                      // Z_POWER: the sums this CTA adds to
     if constexpr (MODE == Z_POWER) {
-        power_tables<L>(iw2, lo, sinc2, pw, T);
+        power_tables<L>(win, lo, sinc2, pw, T);
         part = power_region(pw);
     }
     __syncthreads();
@@ -450,7 +451,7 @@ __global__ void __launch_bounds__(Z2<L, MODE, C, DIRECT>::T, Z2<L, MODE, C, DIRE
                 }
             }
             __syncthreads();
-            if (!nyq_y) power_bin_tile<L, C, T>(pbuf, kx0, ky, sinc2, iw2, lo, pw, part);
+            if (!nyq_y) power_bin_tile<L, C, T>(pbuf, kx0, ky, sinc2, win, lo, pw, part);
             continue;
         } else {
             // bases: A = g X, B = k_z A (, C = k_z^2 A); g = gnorm / (k^2 [W^d]), 0 on excluded modes

@@ -644,8 +644,8 @@ __global__ void __launch_bounds__(PowBox<L>::T, PowBox<L>::MINB)
     Tw2* tws = reinterpret_cast<Tw2*>(xb + X::SIZE);
     const uint32_t bar = smem_u32(tws + 1);
     float* pbuf = reinterpret_cast<float*>(tws + 1) + 2;
-    float* iw2 = pbuf + C * P::PP;
-    int* lo = reinterpret_cast<int*>(iw2 + L / 2);
+    float* win = pbuf + C * P::PP;
+    int* lo = reinterpret_cast<int*>(win + L / 2);
     pdl_trigger();
     load_tw2<L, L>(tws, tw, T);
     if (threadIdx.x == 0) {
@@ -653,7 +653,7 @@ __global__ void __launch_bounds__(PowBox<L>::T, PowBox<L>::MINB)
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     pdl_wait();
-    power_tables<L>(iw2, lo, sinc2, pw, T);
+    power_tables<L>(win, lo, sinc2, pw, T);
     double* part = power_region(pw);
     __syncthreads();
     auto load = [&](int t) {
@@ -710,7 +710,7 @@ __global__ void __launch_bounds__(PowBox<L>::T, PowBox<L>::MINB)
             for (int r = 0; r < R2; ++r) pbuf[P::at(c, js + R1 * r)] = fmaf(v[r].x, v[r].x, v[r].y * v[r].y);
         }
         __syncthreads();
-        if (ky != L / 2) power_bin_tile<L, C, T>(pbuf, kx0, ky, sinc2, iw2, lo, pw, part);
+        if (ky != L / 2) power_bin_tile<L, C, T>(pbuf, kx0, ky, sinc2, win, lo, pw, part);
     }
     power_sum_regions(pw, T);
 }

@@ -171,6 +171,7 @@ extern "C" int colapm_power_noalloc(const int* cell, const float* offset, long l
     PowerArgs pw{};
     pw.n2_lo = tab->lo;
     pw.kf = (float)kf;
+    pw.kfd = kf;
     power_layout(pw, acc, nbins, kPowerRegions);
     pw.pnorm = (float)(box * box * box / ((double)nm3 * (double)nm3));
     const double lr = std::log2(kmax / kmin);
