@@ -219,8 +219,7 @@ __global__ void __launch_bounds__(32 * TZ, TZ == 8 ? 2 : 4)
     for (int dx = 0; dx < 3; ++dx)
         aoff[dx] = hb + tz * (HY * HX * VB) + (ar + dx) * VB + (VB == 32 ? half_slot(ar + dx, ak) << 4 : 0);
     const uint32_t boff = wb + bn * 32 + (half_slot(bn, bk) << 4);
-    // loss: pairs of floats (sum and its rounding errors), FP64 at the end
-    float ls = 0.0f, lc = 0.0f;
+    double lsum = 0.0;   // loss: the sum over this lane's tiles
 
     uint32_t phase = 0;
     for (; t < tend; ++t, phase ^= 1) {
@@ -357,13 +356,14 @@ __global__ void __launch_bounds__(32 * TZ, TZ == 8 ? 2 : 4)
                     }
             }
             __syncwarp();
+            float ls = 0.0f, lc = 0.0f;   // the tile's squares: their sum and its rounding errors
 #pragma unroll
             for (int k = 0; k < NPRE; ++k) {   // four values a lane: rows are 48 values, all multiples of 4
                 const int e = 4 * (lane + 32 * k);
                 const size_t i = (((size_t)(cz + tz) * n + cy + e / (TX * 3)) * n + cx) * 3 + e % (TX * 3);
                 const float4 u4 = *reinterpret_cast<const float4*>(so + e);
                 const float u[4] = {u4.x, u4.y, u4.z, u4.w}, q4[4] = {pre[k].x, pre[k].y, pre[k].z, pre[k].w};
-                float yv[4], g4[4];
+                float yv[4], g4[4], d4[4];
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
                     const float b = !a.target ? q4[m] : (a.base ? a.base[i + m] : 0.0f);
@@ -371,15 +371,31 @@ __global__ void __launch_bounds__(32 * TZ, TZ == 8 ? 2 : 4)
                     if (a.target) {
                         const float d = u[m] - q4[m] * a.tscale;
                         g4[m] = a.gscale * d;
+                        d4[m] = d;
                         const float p = __fmul_rn(d, d), pe = fmaf(d, d, -p), s = __fadd_rn(ls, p), z = __fsub_rn(s, ls);
                         lc += (__fsub_rn(ls, __fsub_rn(s, z)) + __fsub_rn(p, z)) + pe;
                         ls = s;
                     }
                 }
                 store4(a.y + i, make_float4(yv[0], yv[1], yv[2], yv[3]), a.wide);
-                if (a.target) *reinterpret_cast<float4*>(so + e) = make_float4(g4[0], g4[1], g4[2], g4[3]);
+                if (a.target) {
+                    *reinterpret_cast<float4*>(so + e) = make_float4(g4[0], g4[1], g4[2], g4[3]);
+                    pre[k] = make_float4(d4[0], d4[1], d4[2], d4[3]);
+                }
             }
             if (a.target) {
+                // Twelve squares as an exact sum of floats (Knuth's two-sum and the product's error by fma), then one
+                // FP64 addition, of which the GPU does few. Where the sum is not well inside the range of a
+                // float, in which the errors are floats too, and for infinities and NaN, the squares in FP64.
+                if (ls >= 0x1p-48f && ls < 0x1p120f) {
+                    lsum += (double)ls + (double)lc;
+                } else {
+#pragma unroll
+                    for (int k = 0; k < NPRE; ++k) {
+                        const float4 d = pre[k];
+                        lsum += ((double)d.x * d.x + (double)d.y * d.y) + ((double)d.z * d.z + (double)d.w * d.w);
+                    }
+                }
                 __syncwarp();
                 for (int e = lane; e < TX * TY; e += 32) {
                     const __nv_bfloat162 b01 = __floats2bfloat162_rn(so[3 * e], so[3 * e + 1]);
@@ -395,10 +411,9 @@ __global__ void __launch_bounds__(32 * TZ, TZ == 8 ? 2 : 4)
     }
     if (EPI != EPI_OUT && lane == 0) box_stores_read();   // shared memory stays until it has been read
     if (EPI == EPI_OUT && a.target) {
-        double s = (double)ls + (double)lc;
 #pragma unroll
-        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0 && s != 0.0) atomicAdd(a.loss, s);
+        for (int o = 16; o; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+        if (lane == 0 && lsum != 0.0) atomicAdd(a.loss, lsum);
     }
 }
 
