@@ -53,7 +53,8 @@ int colapm_nn_create(int n, const colapm_nn_config* cfg, void* stream, colapm_nn
 int colapm_nn_destroy(colapm_nn* nn);
 
 /* Replace or read the FP32 master parameters (host arrays of COLAPM_NN_PARAMS floats). Setting
- * them leaves the Adam moments and step count alone. Both synchronise. */
+ * them leaves the Adam moments and step count alone. Both synchronise; reading reports
+ * COLAPM_E_TIMEOUT as colapm_nn_sync does. */
 int colapm_nn_set_params(colapm_nn* nn, const float* params);
 int colapm_nn_get_params(colapm_nn* nn, float* params);
 
@@ -66,11 +67,12 @@ int colapm_nn_forward(colapm_nn* nn, const float* psi, float* out, int add);
 int colapm_nn_grads(colapm_nn* nn, const float* psi, const float* target, float* grads, double* loss);
 
 /* One Adam step on one pair (Psi_coarse, dPsi_target). *loss (or NULL) receives the loss before
- * the update (synchronises when requested). */
+ * the update (synchronises when requested). Where a bounded device-side wait has given up and that has
+ * not been reported yet, the step leaves the parameters and the Adam moments as they are. */
 int colapm_nn_train_step(colapm_nn* nn, const float* psi, const float* target, double* loss);
 
 /* Adam steps taken; kernels launched by this network so far; wait for its stream (and report
- * COLAPM_E_TIMEOUT if a bounded device-side wait of a tensor-core convolution gave up). */
+ * COLAPM_E_TIMEOUT if a bounded device-side wait gave up). */
 int colapm_nn_steps(colapm_nn* nn);
 long long colapm_nn_launches(colapm_nn* nn);
 int colapm_nn_sync(colapm_nn* nn);

@@ -808,11 +808,12 @@ __global__ void __launch_bounds__(32 * RG_Y) k_reduce_grads(const float* __restr
     }
 }
 
-// Adam on the FP32 master copy, then the BF16 forward and flipped-transposed weights and the bias.
+// Adam on the FP32 master copy, then the BF16 forward and flipped-transposed weights and the bias. No update after a wait that
+// gave up (err), until that has been reported: the partial gradients are then not all written.
 __global__ void k_adam(float* __restrict__ wm, float* __restrict__ m1, float* __restrict__ m2,
                        const float* __restrict__ grad, float lr, float b1, float b2, float eps, float c1, float c2,
                        int update, __nv_bfloat16* __restrict__ wf, __nv_bfloat16* __restrict__ wt,
-                       float* __restrict__ bias) {
+                       float* __restrict__ bias, const int* err) {
     pdl_trigger();
     pdl_wait();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -820,7 +821,7 @@ __global__ void k_adam(float* __restrict__ wm, float* __restrict__ m1, float* __
     const int l = idx / LSIZE, r = idx % LSIZE;
     const int slot = r / (C * C), o = (r / C) % C, i = r % C;
     float w = wm[idx];
-    if (update && real_slot(l, slot, o, i)) {
+    if (update && !*err && real_slot(l, slot, o, i)) {
         const float g = grad[idx];
         const float m = b1 * m1[idx] + (1.0f - b1) * g;
         const float v = b2 * m2[idx] + (1.0f - b2) * g * g;
@@ -879,7 +880,7 @@ struct colapm_nn {
     struct Maps { CUtensorMap halo, whalo, wtile, plane; } m_act[LAYERS], m_dz[2], m_dz_out;
     __nv_bfloat16* dz_out = nullptr;   // gradient at the network output (8 channels, 0..2 used)
     float* y = nullptr;                // scratch output [n^3][3]
-    float* wm = nullptr;               // master [4][28][16][16]
+    float* wm = nullptr;               // master [4][28][16][16], then the error word
     float* m1 = nullptr;
     float* m2 = nullptr;
     float* grad = nullptr;
@@ -888,7 +889,7 @@ struct colapm_nn {
     __nv_bfloat16* wt = nullptr;
     float* bias = nullptr;             // [4][16]
     double* loss = nullptr;
-    int* err = nullptr;                // device error word (bit 4: a tensor-core wait gave up)
+    int* err = nullptr;                // device error word (bit 4: a bounded wait gave up, in either engine): after wm, to be read with it
     bool use_tc = false;               // tcgen05 convolutions (grid side a multiple of 128)
     long long launches = 0;
 };
@@ -955,7 +956,13 @@ cudaError_t wgrad(colapm_nn* c, const CUtensorMap& dz, int l) {
     return c->small ? launch_wgrad<ACT_A, NT, 2, VA, VD>(c, dz, l) : launch_wgrad<ACT_A, NT, 8, VA, VD>(c, dz, l);
 }
 
-// Report (and clear) a device-side error of the network's kernels; synchronises.
+// Report (and clear) a device-side error of the network's kernels, whose word has been read.
+int report_err(colapm_nn* c, int h) {
+    if (!h) return COLAPM_OK;
+    (void)cudaMemsetAsync(c->err, 0, sizeof(int), c->stream);
+    return COLAPM_E_TIMEOUT;
+}
+// The same; synchronises.
 int check_err(colapm_nn* c) {
     int h = 0;
     if (cudaMemcpyAsync(&h, c->err, sizeof(int), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
@@ -963,18 +970,14 @@ int check_err(colapm_nn* c) {
         (void)cudaGetLastError();
         return COLAPM_E_CUDA;
     }
-    if (h) {
-        (void)cudaMemsetAsync(c->err, 0, sizeof(int), c->stream);
-        return COLAPM_E_TIMEOUT;
-    }
-    return COLAPM_OK;
+    return report_err(c, h);
 }
 
 // Weights (padded master layout) -> bf16 copies and bias, with no update.
 cudaError_t publish(colapm_nn* c) {
     const int total = LAYERS * LSIZE;
     k_adam<<<(total + 255) / 256, 256, 0, c->stream>>>(c->wm, c->m1, c->m2, c->grad, 0.f, 0.f, 0.f, 0.f, 1.f, 1.f, 0,
-                                                       c->wf, c->wt, c->bias);
+                                                       c->wf, c->wt, c->bias, c->err);
     ++c->launches;
     return cudaGetLastError();
 }
@@ -1148,17 +1151,18 @@ int colapm_nn_create(int n, const colapm_nn_config* cfg, void* stream, colapm_nn
     ok = ok && cudaMalloc(&c->dz[0], abytes) == cudaSuccess && cudaMalloc(&c->dz[1], abytes) == cudaSuccess &&
          cudaMalloc(&c->dz_out, abytes / 2) == cudaSuccess && cudaMalloc(&c->y, c->nv * 3 * sizeof(float)) == cudaSuccess;
     const size_t ps = (size_t)LAYERS * LSIZE * sizeof(float);
-    ok = ok && cudaMalloc(&c->wm, ps) == cudaSuccess && cudaMalloc(&c->m1, ps) == cudaSuccess &&
+    ok = ok && cudaMalloc(&c->wm, ps + sizeof(int)) == cudaSuccess && cudaMalloc(&c->m1, ps) == cudaSuccess &&
          cudaMalloc(&c->m2, ps) == cudaSuccess && cudaMalloc(&c->grad, ps) == cudaSuccess &&
          cudaMalloc(&c->part, ps * c->nparts) == cudaSuccess &&
          cudaMalloc(&c->wf, (size_t)LAYERS * 27 * C * C * sizeof(__nv_bfloat16)) == cudaSuccess &&
          cudaMalloc(&c->wt, (size_t)LAYERS * 27 * C * C * sizeof(__nv_bfloat16)) == cudaSuccess &&
          cudaMalloc(&c->bias, LAYERS * C * sizeof(float)) == cudaSuccess &&
-         cudaMalloc(&c->loss, sizeof(double)) == cudaSuccess && cudaMalloc(&c->err, sizeof(int)) == cudaSuccess;
+         cudaMalloc(&c->loss, sizeof(double)) == cudaSuccess;
     if (!ok) {
         (void)cudaGetLastError();
         return fail(COLAPM_E_NOMEM);
     }
+    c->err = reinterpret_cast<int*>(c->wm + LAYERS * LSIZE);
     for (int l = 0; l < LAYERS; ++l) ok = ok && encode_maps(c->m_act[l], c->act[l], n, l == 0 ? 16 : 32, c->small);
     ok = ok && encode_maps(c->m_dz[0], c->dz[0], n, 32, c->small) && encode_maps(c->m_dz[1], c->dz[1], n, 32, c->small) &&
          encode_maps(c->m_dz_out, c->dz_out, n, 16, c->small);
@@ -1188,7 +1192,6 @@ int colapm_nn_destroy(colapm_nn* c) {
     cudaFree(c->wf);
     cudaFree(c->wt);
     cudaFree(c->loss);
-    cudaFree(c->err);
     (void)cudaGetLastError();
     delete c;
     return COLAPM_OK;
@@ -1202,9 +1205,12 @@ int colapm_nn_set_params(colapm_nn* c, const float* params) {
 
 int colapm_nn_get_params(colapm_nn* c, float* params) {
     if (!c || !params) return COLAPM_E_ARG;
-    std::vector<float> pad((size_t)LAYERS * LSIZE);
+    std::vector<float> pad((size_t)LAYERS * LSIZE + 1);   // the parameters and the error word
     NN_CK(cudaMemcpyAsync(pad.data(), c->wm, pad.size() * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
     NN_CK(cudaStreamSynchronize(c->stream));
+    int h;
+    std::memcpy(&h, &pad[(size_t)LAYERS * LSIZE], sizeof(h));
+    if (int r = report_err(c, h)) return r;
     for_each_param([&](size_t k, size_t slot) { params[k] = pad[slot]; });
     return COLAPM_OK;
 }
@@ -1252,7 +1258,7 @@ int colapm_nn_train_step(colapm_nn* c, const float* psi, const float* target, do
     const int total = LAYERS * LSIZE;
     ++c->launches;
     NN_CK(colapm::launch_dep(true, k_adam, (total + 255) / 256, 256, 0, c->stream, c->wm, c->m1, c->m2, c->grad, c->cfg.lr,
-                             c->cfg.beta1, c->cfg.beta2, c->cfg.eps, c1, c2, 1, c->wf, c->wt, c->bias));
+                             c->cfg.beta1, c->cfg.beta2, c->cfg.eps, c1, c2, 1, c->wf, c->wt, c->bias, c->err));
     if (loss) {
         double h = 0.0;
         NN_CK(cudaMemcpyAsync(&h, c->loss, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
