@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy_force(float2* __restrict__ dat
 // x and y derivatives of one base differ by factors constant along a z line, so the passes carry 4 + 12, 12 + 24
 // and 24 + 16 bytes per cell (the x pass makes nine rows of them) instead of 4 + 36, 36 + 36 and 36 + 36.
 template <int L>
-__global__ void __launch_bounds__(K2<L>::T) k2_fy_lpt(const float2* __restrict__ bases, float2* __restrict__ dst, size_t fstride,
+__global__ void __launch_bounds__(K2<L>::T) k2_fy_lpt(const float2* bases, float2* __restrict__ dst, size_t fstride,
                                                       const float2* __restrict__ tw) {
     using K = K2<L>;
     constexpr int RA = K::RA, RB = K::RB, n = L / 2, NG = n / 8, TPF = NG * L;
@@ -653,7 +653,7 @@ struct X2 {
 // forward r2c: in = int64 density pairs (I64, converted to rho * scale - 1) or float reals.
 // zero (optional): the int64 input itself, cleared as it is read (the next deposit then needs no memset).
 template <int n, bool I64, bool BLK = false>
-__global__ void __launch_bounds__(X2<n>::T) k2_fx_fwd(const void* __restrict__ in_, float2* __restrict__ out,
+__global__ void __launch_bounds__(X2<n>::T) k2_fx_fwd(const void* in_, float2* __restrict__ out,
                                                        const float2* __restrict__ tw, float scale, int* err,
                                                        int nitems, unsigned long long* zero) {
     using X = X2<n>;
@@ -847,7 +847,7 @@ __global__ void __launch_bounds__(X2<n>::T, 3) k2_fx_inv(float2* __restrict__ da
 // of 256^3 particles as a whole went from 1122 to 914 us.
 template <int n>
 __global__ void __launch_bounds__(X2<n>::T, (X2<n>::RB >= 16 ? 3 : 4) * 128 / X2<n>::T)
-    k2_fx_lpt(const float2* __restrict__ spec, size_t fstride, float2* __restrict__ psi, float2* __restrict__ src,
+    k2_fx_lpt(const float2* spec, size_t fstride, float2* __restrict__ psi, float2* __restrict__ src,
               const float2* __restrict__ tw, int nitems, float vscale) {
     using X = X2<n>;
     constexpr int RA = X::RA, RB = X::RB, N = 2 * n, T = X::T;

@@ -38,7 +38,7 @@ __device__ __forceinline__ float2 draw(unsigned long long m, unsigned long long 
 }
 
 // One thread per half-grid mode (iz, iy, ix < N/2): delta_k = amp(|n|^2) g, Hermitian on ix = 0.
-__global__ void k_gaussian_field(int n, const unsigned long long* __restrict__ seedp, const float* __restrict__ amp_of_n2,
+__global__ void k_gaussian_field(int n, const unsigned long long* seedp, const float* __restrict__ amp_of_n2,
                                  float2* __restrict__ dk) {
     pdl_trigger();
     pdl_wait();
@@ -75,7 +75,7 @@ __global__ void k_gaussian_field(int n, const unsigned long long* __restrict__ s
 
 // S = phi_xx phi_yy + phi_xx phi_zz + phi_yy phi_zz - phi_xy^2 - phi_xz^2 - phi_yz^2
 // (the right-hand side of the phi2 Poisson equation, §2.1); phi = [xx, yy, zz, xy, xz, yz].
-__global__ void k_lpt2_source(const float4* __restrict__ phi, size_t n4, float4* __restrict__ src) {
+__global__ void k_lpt2_source(const float4* phi, size_t n4, float4* __restrict__ src) {
     pdl_trigger();
     pdl_wait();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;

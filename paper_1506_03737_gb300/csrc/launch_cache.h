@@ -58,6 +58,9 @@ static cudaError_t cached_grid(GridCache& c, K kernel, int threads, size_t smem,
 // constant tables and wait in pdl_wait() until the kernel before has completed and its writes are visible.
 // Every kernel launched by launch_dep calls pdl_wait() before it touches anything but constant tables (written
 // before the stream's work began); kernels whose predecessors did the same are then ordered as without it.
+// What that kernel may still be writing is read through plain pointers (or __ldcg, __ldcs): `const T* __restrict__` and
+// __ldg promise that the memory does not change while the kernel runs, which leaves the compiler free to load it on
+// the path that is not coherent, or before the wait.
 // A step on a 64^3 or 128^3 mesh is a chain of 3-12 us kernels, of which the start and the table loads
 // were 1-2 us each: a step at 64^3 went from 89 to 76 us, ten at 128^3 with P(k) from 908 to 817 us.
 // `overlap` is for such short kernels only (overlap_mesh): kernels that follow one another without a gap

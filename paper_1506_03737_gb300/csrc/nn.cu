@@ -787,7 +787,7 @@ __device__ __forceinline__ bool real_slot(int l, int slot, int o, int i) {
 // Sum the per-CTA partials of every layer in a fixed order: grad[l][slot][o][i]. 32 slots per block, the
 // partials dealt over RG_Y rows of threads (a column of 304 sums one after the other took 23 us).
 constexpr int RG_Y = 32;
-__global__ void __launch_bounds__(32 * RG_Y) k_reduce_grads(const float* __restrict__ part, int nparts, float* __restrict__ grad) {
+__global__ void __launch_bounds__(32 * RG_Y) k_reduce_grads(const float* part, int nparts, float* __restrict__ grad) {
     pdl_trigger();
     pdl_wait();
     __shared__ float sh[RG_Y][33];
@@ -811,7 +811,7 @@ __global__ void __launch_bounds__(32 * RG_Y) k_reduce_grads(const float* __restr
 // Adam on the FP32 master copy, then the BF16 forward and flipped-transposed weights and the bias. No update after a wait that
 // gave up (err), until that has been reported: the partial gradients are then not all written.
 __global__ void k_adam(float* __restrict__ wm, float* __restrict__ m1, float* __restrict__ m2,
-                       const float* __restrict__ grad, float lr, float b1, float b2, float eps, float c1, float c2,
+                       const float* grad, float lr, float b1, float b2, float eps, float c1, float c2,
                        int update, __nv_bfloat16* __restrict__ wf, __nv_bfloat16* __restrict__ wt,
                        float* __restrict__ bias, const int* err) {
     pdl_trigger();
@@ -840,7 +840,7 @@ __global__ void k_adam(float* __restrict__ wm, float* __restrict__ m1, float* __
 }
 
 // x[v][c] = bf16(psi[v][c] / s_in) for c < 3, zero for the other five channels; one thread per stored voxel.
-__global__ void k_pack_input(const float* __restrict__ psi, int n, float inv_s, __nv_bfloat16* __restrict__ x) {
+__global__ void k_pack_input(const float* psi, int n, float inv_s, __nv_bfloat16* __restrict__ x) {
     pdl_trigger();
     pdl_wait();
     const int m = n + 2, row = blockIdx.x * blockDim.y + threadIdx.y;   // stored row (z, y)

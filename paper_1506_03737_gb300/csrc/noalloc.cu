@@ -41,7 +41,7 @@ struct Tables {
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kBytes];
 
 // Fixed-point CIC deposit of xyz cell / offset arrays (the definition of pm_kernels.cu).
-__global__ void k_deposit_xyz(const int* __restrict__ cell, const float* __restrict__ off, long long n, int nm,
+__global__ void k_deposit_xyz(const int* cell, const float* off, long long n, int nm,
                               unsigned long long* __restrict__ rho, int* err) {
     pdl_trigger();
     pdl_wait();

@@ -42,7 +42,7 @@ __device__ __forceinline__ Cic cic_setup(float4 P, const UDiv& u) {
 // Two threads per particle, one per x corner (lane parity): the atomics of one warp instruction then
 // hit 16 particles x 2 neighbouring cells, which along the Lagrangian x rows are runs of consecutive
 // int64 cells (fully used 32-byte sectors), instead of every other cell of twice as many sectors.
-__device__ __forceinline__ void deposit_corner(const float4* __restrict__ pos, size_t p, int dx, const UDiv& u,
+__device__ __forceinline__ void deposit_corner(const float4* pos, size_t p, int dx, const UDiv& u,
                                                unsigned long long* __restrict__ rho) {
     const Cic c = cic_setup(pos[p], u);
     const int nm = (int)u.d;
@@ -59,7 +59,7 @@ __device__ __forceinline__ void deposit_corner(const float4* __restrict__ pos, s
         }
 }
 
-__global__ void k_deposit(const float4* __restrict__ pos, size_t np3, UDiv u, unsigned long long* __restrict__ rho) {
+__global__ void k_deposit(const float4* pos, size_t np3, UDiv u, unsigned long long* __restrict__ rho) {
     pdl_trigger();
     pdl_wait();
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -74,7 +74,7 @@ __global__ void k_deposit(const float4* __restrict__ pos, size_t np3, UDiv u, un
 // particles on 64^3 and 32^3 cells 54 us against 91 with k_deposit, 256^3 on 128^3 and 64^3 324 against 494. With
 // as many cells as particles, passing right-hand corners on to the next lane's left-hand ones cost more than the
 // reductions it saved (53 against 46 us at 128^3): k_deposit from there on.
-__global__ void k_deposit_dense(const float4* __restrict__ pos, size_t np3, UDiv u, unsigned long long* __restrict__ rho) {
+__global__ void k_deposit_dense(const float4* pos, size_t np3, UDiv u, unsigned long long* __restrict__ rho) {
     pdl_trigger();
     pdl_wait();
     const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -223,8 +223,7 @@ __device__ __forceinline__ void record_lightcone(const LightconeStep& lc, const 
 
 template <bool LC>
 __device__ __forceinline__ void gather_kick_drift(float4* __restrict__ pos, float* __restrict__ mom,
-                                                  const float* __restrict__ psi1, const float* __restrict__ psi2,
-                                                  const float* __restrict__ force, size_t np3, const UDiv& u, const StepCoef& k,
+                                                  const float* psi1, const float* psi2, const float* force, size_t np3, const UDiv& u, const StepCoef& k,
                                                   int drift, const LightconeStep& lc, size_t p) {
     // every load of the particle's own data is issued before the force loads that depend on its
     // position, so the two sets are in flight together (streaming: each is used once per step)
@@ -256,7 +255,7 @@ __device__ __forceinline__ void gather_kick_drift(float4* __restrict__ pos, floa
                 const float w = wx[dx] * wyz;
                 const size_t i = row + xs[dx];
 #pragma unroll
-                for (int j = 0; j < 3; ++j) f[j] = fmaf(w, __ldg(force + j * m3 + i), f[j]);
+                for (int j = 0; j < 3; ++j) f[j] = fmaf(w, force[j * m3 + i], f[j]);
             }
         }
     float d[3];
@@ -288,8 +287,8 @@ __device__ __forceinline__ void gather_kick_drift(float4* __restrict__ pos, floa
 }
 
 template <bool LC>
-__global__ void k_gather_kick_drift(float4* __restrict__ pos, float* __restrict__ mom, const float* __restrict__ psi1,
-                                    const float* __restrict__ psi2, const float* __restrict__ force, size_t np3, UDiv u,
+__global__ void k_gather_kick_drift(float4* __restrict__ pos, float* __restrict__ mom, const float* psi1,
+                                    const float* psi2, const float* force, size_t np3, UDiv u,
                                     StepCoef k, int drift, LightconeStep lc) {
     pdl_trigger();
     pdl_wait();
@@ -309,7 +308,7 @@ __global__ void k_gather_kick_drift(float4* __restrict__ pos, float* __restrict_
 constexpr int MW_ITEM = 256;
 constexpr int MW_T = 256;
 
-__device__ __forceinline__ bool next_item(const MockWork* __restrict__ w, int nmock, long long nitems,
+__device__ __forceinline__ bool next_item(const MockWork* w, int nmock, long long nitems,
                                           unsigned long long* queue, long long& item, int& mock) {
     __shared__ long long s_item;
     __shared__ int s_mock;
@@ -341,7 +340,7 @@ __device__ __forceinline__ void leave_queue(unsigned long long* queue) {
     }
 }
 
-__global__ void __launch_bounds__(MW_T) k_multi_deposit(const MockWork* __restrict__ w, int nmock, long long nitems,
+__global__ void __launch_bounds__(MW_T) k_multi_deposit(const MockWork* w, int nmock, long long nitems,
                                                         unsigned long long* queue) {
     pdl_trigger();
     pdl_wait();
@@ -360,7 +359,7 @@ __global__ void __launch_bounds__(MW_T) k_multi_deposit(const MockWork* __restri
     leave_queue(queue);
 }
 
-__global__ void __launch_bounds__(MW_T) k_multi_gather_kick_drift(const MockWork* __restrict__ w, int nmock,
+__global__ void __launch_bounds__(MW_T) k_multi_gather_kick_drift(const MockWork* w, int nmock,
                                                                   long long nitems, unsigned long long* queue) {
     pdl_trigger();
     pdl_wait();
@@ -419,7 +418,7 @@ __global__ void k_init_particles(float4* __restrict__ pos, float* __restrict__ m
     id[p] = (int)p;
 }
 
-__global__ void k_add_lpt_momentum(float* __restrict__ mom, const float* __restrict__ psi1, const float* __restrict__ psi2,
+__global__ void k_add_lpt_momentum(float* __restrict__ mom, const float* psi1, const float* psi2,
                                    size_t n3, float p1, float p2) {
     pdl_trigger();
     pdl_wait();
@@ -428,8 +427,7 @@ __global__ void k_add_lpt_momentum(float* __restrict__ mom, const float* __restr
     mom[i] = fmaf(p1, psi1[i], fmaf(p2, psi2[i], mom[i]));
 }
 
-__global__ void k_export_particles(const float4* __restrict__ pos, const float* __restrict__ mom,
-                                   const int* __restrict__ id, size_t np3, UDiv u, float cell,
+__global__ void k_export_particles(const float4* pos, const float* mom, const int* id, size_t np3, UDiv u, float cell,
                                    float* __restrict__ pos_xyz, float* __restrict__ mom_xyz) {
     pdl_trigger();
     pdl_wait();
@@ -445,12 +443,15 @@ __global__ void k_export_particles(const float4* __restrict__ pos, const float* 
         pos_xyz[3 * q + 2] = ((float)cz + P.z) * cell;
     }
     if (mom_xyz) {
+        float v[3];   // all loads before the first store
 #pragma unroll
-        for (int j = 0; j < 3; ++j) mom_xyz[3 * q + j] = mom[j * np3 + p] * cell;
+        for (int j = 0; j < 3; ++j) v[j] = mom[j * np3 + p];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) mom_xyz[3 * q + j] = v[j] * cell;
     }
 }
 
-__global__ void k_export_state(const float4* __restrict__ pos, const float* __restrict__ mom, size_t np3, int nm,
+__global__ void k_export_state(const float4* pos, const float* mom, size_t np3, int nm,
                                int* __restrict__ cell_xyz, float* __restrict__ off_xyz, float* __restrict__ mom_xyz) {
     pdl_trigger();
     pdl_wait();
@@ -469,8 +470,11 @@ __global__ void k_export_state(const float4* __restrict__ pos, const float* __re
         off_xyz[3 * p + 2] = P.z;
     }
     if (mom_xyz) {
+        float v[3];
 #pragma unroll
-        for (int j = 0; j < 3; ++j) mom_xyz[3 * p + j] = mom[j * np3 + p];
+        for (int j = 0; j < 3; ++j) v[j] = mom[j * np3 + p];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) mom_xyz[3 * p + j] = v[j];
     }
 }
 
@@ -504,7 +508,7 @@ __global__ void k_import_state(float4* __restrict__ pos, float* __restrict__ mom
 
 // Psi = x - q in Mpc/h with the minimum-image convention, q = (site * Nm/Np + 1/2) cells. With divisions by np and
 // nm it was bound by them (256^3: 201 us for 28 bytes per particle, 85 now).
-__global__ void k_export_displacement(const float4* __restrict__ pos, size_t np3, Lattice lat, float cell,
+__global__ void k_export_displacement(const float4* pos, size_t np3, Lattice lat, float cell,
                                       float* __restrict__ psi) {
     pdl_trigger();
     pdl_wait();
@@ -607,7 +611,7 @@ __global__ void k_rsd_positions(const float4* __restrict__ pos, const float* __r
 
 // dst = f src, V floats per thread (one per thread took twice the time of the copy it is).
 template <int V>
-__global__ void k_scale(float* __restrict__ dst, const float* __restrict__ src, size_t n, float f) {
+__global__ void k_scale(float* __restrict__ dst, const float* src, size_t n, float f) {
     pdl_trigger();
     pdl_wait();
     const size_t i = V * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
