@@ -76,8 +76,11 @@ typedef struct colapm_ctx colapm_ctx;   /* opaque; owns all device memory */
 void colapm_default_params(colapm_params* p);
 
 /* Create a context on the current CUDA device: validates *p (COLAPM_E_ARG), computes the FP64
- * timestep table and the linear P(k) normalisation on the host, allocates every device buffer
- * (COLAPM_E_NOMEM). `stream` is a cudaStream_t (may be NULL). On success *out owns the memory
+ * timestep table and the linear P(k) normalisation on the host, allocates its device buffers
+ * (COLAPM_E_NOMEM): 148 B per particle (positions, momenta, both displacements, ids, each twice, and 36 B of
+ * scratch), 20 B per mesh cell, 32 B from 512^3 cells on. On meshes of 64^3 to 384^3 cells 12 B per cell more
+ * serve the faster layout of the spectra: taken here up to 256^3, by the first step above and in batches; where
+ * they do not fit, steps use the plain layout. `stream` is a cudaStream_t (may be NULL). On success *out owns the memory
  * until colapm_destroy. */
 int colapm_create(const colapm_params* p, void* stream, colapm_ctx** out);
 

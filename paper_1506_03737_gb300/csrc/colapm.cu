@@ -25,7 +25,8 @@ struct colapm_ctx {
     float* F = nullptr;                  // 3 nm^3: density spectrum, then the three force meshes
     CUtensorMap zmaps[2];                // boxes of fields 0 and 2 of F for the blocked force z pass from 256^3 on (ZOut)
     CUtensorMap ymaps[3];                // and of fields 0, 1 and 2 for the inverse y pass
-    float* Freal = nullptr;              // 3 nm^3: the real force meshes when the spectra use the blocked layout
+    float* Freal = nullptr;              // 3 nm^3: the real force meshes when the spectra use the blocked layout (force_blocked)
+    bool freal_failed = false;           // it did not fit: the plain layout from then on
     float4* pos = nullptr;               // np^3 (offsets, cell bits)
     float* mom = nullptr;                // 3 np^3, cells
     float* psi1 = nullptr;               // 3 np^3, cells
@@ -251,14 +252,42 @@ bool use_xy(const colapm_ctx* c, int bit) { return (c->fused & bit) && c->xy_rin
 bool ts(const colapm_ctx* c, unsigned bit) { return (c->plan & bit) != 0; }
 
 // The two-stage engine keeps the half spectra in the blocked layout (see hs_index) when every pass
-// runs on it and the fused x-y passes are off; the inverse x pass then writes the real force
-// meshes to Freal.
-bool use_blocked(const colapm_ctx* c) {
-    return c->plan == COLAPM_PLAN_ALL && !(c->fused & 3) && c->Freal != nullptr;
+// runs on it (lines of N and of N / 2 have two-stage plans) and the fused x-y passes are off.
+bool use_blocked(const colapm_ctx* c) { return c->plan == COLAPM_PLAN_ALL && !(c->fused & 3) && c->nm >= 64; }
+
+// Whether a force computation into the context's own mesh uses the blocked layout. The inverse x pass then writes the real
+// force meshes to an array of their own. Below 512^3 cells it is no condition of a context: up to 256^3 (0.2 GB, less than a
+// thousandth of the memory) it is allocated with the context where it fits, above, and for the mocks of a batch, here, on
+// first use: 70 to 90 us of a first step, as much as the step itself at 64^3. Where it does not fit, or is missing while the
+// stream is being captured, the plain layout is used.
+bool force_blocked(colapm_ctx* c) {
+    if (!use_blocked(c)) return false;
+    if (c->Freal || c->freal_failed) return c->Freal != nullptr;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    if (dalloc(&c->Freal, 3 * c->nm3) != cudaSuccess) {
+        cudaGetLastError();
+        c->Freal = nullptr;
+        c->freal_failed = true;
+    }
+    return c->Freal != nullptr;
+}
+
+// Gives that array back where another one of the context needs the room; true if there was one (try again).
+bool release_freal(colapm_ctx* c) {
+    if (!c->Freal || c->nm >= 512 || cudaStreamSynchronize(c->stream) != cudaSuccess) return false;
+    cudaGetLastError();
+    cudaFree(c->Freal);
+    c->Freal = nullptr;
+    c->freal_failed = true;
+    return true;
 }
 
 // The three real force meshes of the last force computation.
-const float* force_mesh(const colapm_ctx* c) { return use_blocked(c) ? c->Freal : c->F; }
+const float* force_mesh(colapm_ctx* c) { return force_blocked(c) ? c->Freal : c->F; }
 
 SortBuffers sort_buffers(colapm_ctx* c) {
     return SortBuffers{c->pos, c->mom, c->psi1, c->psi2, c->id, c->pos_alt, c->mom_alt, c->psi1_alt, c->psi2_alt,
@@ -297,8 +326,8 @@ float density_scale(const colapm_ctx* c) {
     return (float)(m * m * m * std::ldexp(1.0, -45));
 }
 
-// Forward x and y passes of the current density into F (half spectrum, z still in real space).
-int density_xy(colapm_ctx* c) {
+// Forward x and y passes of the current density into F (half spectrum, z still in real space; `blk`: in the blocked layout).
+int density_xy(colapm_ctx* c, bool blk) {
     Phase ph(c, COLAPM_PHASE_FFT_FWD);
     float2* d = reinterpret_cast<float2*>(c->F);
     c->rho_clean = false;
@@ -307,7 +336,6 @@ int density_xy(colapm_ctx* c) {
         c->rho_clean = true;
         return COLAPM_OK;
     }
-    const bool blk = use_blocked(c);
     CKL(launch_fx_fwd_i64(c->nm, c->rho, d, c->tw_m, density_scale(c), c->err, c->stream, ts(c, COLAPM_PLAN_XF), true,
                           blk));
     c->rho_clean = true;
@@ -318,7 +346,8 @@ int density_xy(colapm_ctx* c) {
 // §2.4 steps 2-3 from the deposited density: the three real force meshes in force_mesh(c)
 // (or, blocked, in `dst`: 3 nm^3 floats of the caller's, 8-byte aligned).
 int force_from_density(colapm_ctx* c, float* dst = nullptr) {
-    int r = density_xy(c);
+    const bool blk = dst ? use_blocked(c) : force_blocked(c);
+    int r = density_xy(c, blk);
     if (r) return r;
     float2* d = reinterpret_cast<float2*>(c->F);
     const size_t fs = c->nm3 / 2;   // complex stride between the three meshes
@@ -332,14 +361,13 @@ int force_from_density(colapm_ctx* c, float* dst = nullptr) {
         out.err = c->err;
         const float gnorm = (float)(1.0 / ((double)c->nm * c->nm * c->nm));
         CKL(launch_fz(c->nm, Z_FORCE, d, out, c->tw_m, c->sinc2_m, c->prm.deconv, gnorm, nullptr, c->stream,
-                      ts(c, COLAPM_PLAN_Z), use_blocked(c)));
+                      ts(c, COLAPM_PLAN_Z), blk));
     }
     if (use_xy(c, 2)) {
         Phase ph(c, COLAPM_PHASE_FFT_INV);
         CKL(launch_xy_inv(c->nm, d, fs, 3, c->tw_m, c->xy_ring, c->xy_ctr, c->err, c->stream));
         return COLAPM_OK;
     }
-    const bool blk = use_blocked(c);
     {
         Phase ph(c, COLAPM_PHASE_FFT_INV);
         if (blk) {
@@ -511,9 +539,16 @@ struct Tuned {
 };
 static std::map<std::pair<int, int>, Tuned> g_tuned;   // (np, nm) -> choice
 
+static int create_context(const colapm_params* p, void* stream, colapm_ctx** out, bool early);
+
 extern "C" {
 
-int colapm_create(const colapm_params* p, void* stream, colapm_ctx** out) {
+int colapm_create(const colapm_params* p, void* stream, colapm_ctx** out) { return create_context(p, stream, out, true); }
+
+}  // extern "C"
+
+// `early`: allocate the blocked layout's mesh of a small context now (see force_blocked).
+static int create_context(const colapm_params* p, void* stream, colapm_ctx** out, bool early) {
     if (!out) return COLAPM_E_ARG;
     *out = nullptr;
     int r = validate(p);
@@ -544,8 +579,11 @@ int colapm_create(const colapm_params* p, void* stream, colapm_ctx** out) {
     if (ok && xy_supported(c->nm))
         ok = dalloc(reinterpret_cast<char**>(&c->xy_ring), xy_ring_bytes(c->nm)) == cudaSuccess &&
              dalloc(&c->xy_ctr, xy_ctr_ints(c->nm, 3)) == cudaSuccess;
-    // blocked spectra where every pass has a two-stage plan (lines of N and of N / 2)
-    if (ok && c->nm >= 64) ok = dalloc(&c->Freal, 3 * c->nm3) == cudaSuccess;
+    if (ok && c->nm >= 512) ok = dalloc(&c->Freal, 3 * c->nm3) == cudaSuccess;   // smaller meshes: see force_blocked
+    if (ok && early && c->nm >= 64 && c->nm <= 256 && dalloc(&c->Freal, 3 * c->nm3) != cudaSuccess) {
+        cudaGetLastError();
+        c->Freal = nullptr;
+    }
     if (!ok) {
         cudaGetLastError();
         free_all(c);
@@ -617,6 +655,8 @@ int colapm_create(const colapm_params* p, void* stream, colapm_ctx** out) {
     *out = c;
     return COLAPM_OK;
 }
+
+extern "C" {
 
 void colapm_destroy(colapm_ctx* c) {
     if (!c) return;
@@ -769,7 +809,10 @@ int power_prepare(colapm_ctx* c, int nbins, double kmin, double kmax) {
     if (nbins > c->pw_nbcap) {
         if (c->pw_acc) cudaFree(c->pw_acc);
         c->pw_acc = nullptr;
-        if (dalloc(&c->pw_acc, power_words(nbins, kPowerRegions)) != cudaSuccess) {
+        if (dalloc(&c->pw_acc, power_words(nbins, kPowerRegions)) != cudaSuccess &&
+            !(release_freal(c) && dalloc(&c->pw_acc, power_words(nbins, kPowerRegions)) == cudaSuccess)) {
+            cudaGetLastError();
+            c->pw_acc = nullptr;
             c->pw_nbcap = 0;
             return COLAPM_E_NOMEM;
         }
@@ -813,7 +856,7 @@ int power_enqueue(colapm_ctx* c, int nbins, const DepositSrc* src = nullptr, boo
     CK(cudaMemsetAsync(c->pw_acc, 0, power_words(nbins, kPowerRegions) * sizeof(double), c->stream));
     int r = deposit(c, src);
     if (r) return r;
-    r = density_xy(c);
+    r = density_xy(c, use_blocked(c));
     if (r) return r;
     PowerArgs pw{};
     pw.n2_lo = c->pw_bin;
@@ -956,7 +999,8 @@ int colapm_get_particles_async(colapm_ctx* c, float* pos, float* mom) {
     if (!c) return COLAPM_E_ARG;
     if (!c->has_ics) return COLAPM_E_STATE;
     if (!c->xfer) {
-        if (dalloc(&c->xfer, 6 * c->np3) != cudaSuccess) {
+        if (dalloc(&c->xfer, 6 * c->np3) != cudaSuccess &&
+            !(release_freal(c) && dalloc(&c->xfer, 6 * c->np3) == cudaSuccess)) {
             c->xfer = nullptr;
             cudaGetLastError();
             return COLAPM_E_NOMEM;
@@ -1185,8 +1229,10 @@ int colapm_set_lightcone(colapm_ctx* c, const colapm_lightcone* lc, long long ca
         c->lc_rep_n.push_back(cnt);
     }
     if (reps.empty()) reps.assign(3, 0);
-    if (dalloc(&c->lc_out, 2 * (size_t)capacity) != cudaSuccess || dalloc(&c->lc_count, 1) != cudaSuccess ||
-        dalloc(&c->lc_tab, tab.size()) != cudaSuccess || dalloc(&c->lc_reps, reps.size()) != cudaSuccess) {
+    if ((dalloc(&c->lc_out, 2 * (size_t)capacity) != cudaSuccess &&
+         !(release_freal(c) && dalloc(&c->lc_out, 2 * (size_t)capacity) == cudaSuccess)) ||
+        dalloc(&c->lc_count, 1) != cudaSuccess || dalloc(&c->lc_tab, tab.size()) != cudaSuccess ||
+        dalloc(&c->lc_reps, reps.size()) != cudaSuccess) {
         cudaGetLastError();
         lightcone_free(c);
         return COLAPM_E_NOMEM;
@@ -1779,7 +1825,7 @@ int colapm_batch_create(int n, const colapm_params* ps, int nstreams, void* stre
          cudaMemset(b->queue_d, 0, 4 * sizeof(unsigned long long)) != cudaSuccess))
         r = COLAPM_E_NOMEM;
     for (int i = 0; i < n && !r; ++i) {
-        r = colapm_create(&ps[i], b->ws[0], &b->ctx[i]);
+        r = create_context(&ps[i], b->ws[0], &b->ctx[i], false);
         if (!r) {
             b->ctx[i]->seed_src = b->seeds_d + i;
             b->seeds_h[i] = ps[i].seed;
@@ -1800,6 +1846,8 @@ int colapm_batch_run(colapm_batch* b, const unsigned long long* seeds, int nbins
     if (!b || !k_out || !p_out || !nmodes_out || nbins < 1 || nbins > 4096) return COLAPM_E_ARG;
     CK(cudaStreamSynchronize(b->caller));   // work the caller issued before this call comes first
     if (!b->exec || nbins != b->nbins || kmin != b->kmin || kmax != b->kmax) {
+        if (b->exec) cudaGraphExecDestroy(b->exec);   // it holds arrays that may be replaced here
+        b->exec = nullptr;
         for (colapm_ctx* c : b->ctx) {
             c->stream = b->ws[0];
             int r = power_prepare(c, nbins, kmin, kmax);
