@@ -148,8 +148,10 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Memory that a kernel on the current device may use in place of a copy (another GPU's needs the copy).
+// Memory that a kernel on the current device may use in place of a copy (another GPU's needs the copy, and so do floats at
+// addresses that are no multiple of their size).
 bool is_local_ptr(const void* p) {
+    if (reinterpret_cast<uintptr_t>(p) % sizeof(float)) return false;
     cudaPointerAttributes a;
     int dev = 0;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
