@@ -24,7 +24,7 @@ struct colapm_ctx {
     unsigned long long* rho = nullptr;   // nm^3 int64 fixed-point density
     float* F = nullptr;                  // 3 nm^3: density spectrum, then the three force meshes
     CUtensorMap zmaps[2];                // boxes of fields 0 and 2 of F for the blocked force z pass from 256^3 on (ZOut)
-    CUtensorMap ymaps[3];                // and of fields 0, 1 and 2 for the inverse y pass
+    CUtensorMap ymaps[3];                // and of fields 0, 1 and 2 for the inverse y pass from 512^3 on
     float* Freal = nullptr;              // 3 nm^3: the real force meshes when the spectra use the blocked layout (force_blocked)
     bool freal_failed = false;           // it did not fit: the plain layout from then on
     float4* pos = nullptr;               // np^3 (offsets, cell bits)
@@ -69,7 +69,7 @@ struct colapm_ctx {
     float* sinc2_m = nullptr;            // sinc^2(pi n / nm) per FFT bin, then nm ones (no window)
     float* amp_p = nullptr;              // Gaussian-field amplitude per integer |n|^2 of the IC grid
     int* err_h = nullptr;                // pinned host copy of err
-    int* pw_host = nullptr;              // pinned: thresholds, then sums of up to three spectra (grown on demand)
+    int* pw_host = nullptr;              // pinned: sums of up to three spectra, then thresholds (grown on demand)
     int pw_hostcap = 0;                  // its bins
     int pw_nbins = 0;                    // the binning that pw_bin holds
     double pw_kmin = 0.0, pw_kmax = 0.0;
@@ -597,7 +597,7 @@ static int create_context(const colapm_params* p, void* stream, colapm_ctx** out
         const cuuint32_t box[3] = {4, c->nm >= 512 ? 256u : (c->nm > 256 ? (cuuint32_t)c->nm / 2 : (cuuint32_t)c->nm), 1};
         const cuuint64_t ydims[4] = {8, 8, n, n / 16 * (n / 8)}, ystrides[3] = {64, 512, n * 512};
         const cuuint32_t ybox[4] = {4, 8, 1, (cuuint32_t)c->nm / 8};
-        for (int f = 0; f < 3; ++f)
+        for (int f = 0; f < 3 && c->nm >= 512; ++f)
             if (!encode_box<4>(&c->ymaps[f], c->F + f * c->nm3, ydims, ystrides, ybox)) {
                 free_all(c);
                 delete c;
@@ -1637,8 +1637,9 @@ void batch_free(colapm_batch* b) {
 
 // Mocks below this many particles share the multi-mock particle kernels; the others take the plain kernels, which
 // are faster once they fill the GPU (their CTAs go through the mesh in order, not by ticket) and find a mock's
-// mesh in L2 between its passes: ten mocks of 64^3 to 192^3 particles take 59.1 ms that way, 63.9 with the
-// multi-mock kernels for all.
+// mesh in L2 between its passes. With the plain ones from here on, against the multi-mock kernels for all: ten mocks of 64^3
+// to 192^3 particles 58.7 ms against 63.3, 8 (32) equal ones of 96^3 on 192^3 cells 13.6 (54.0) against 15.0 (59.3), on 96^3
+// cells 5.1 (20.0) against 6.7 (27.0), 8 of 128^3 33.2 against 35.4; 16 of 64^3 and 96^3 19.8 against 19.7.
 constexpr size_t kSharedParticles = (size_t)1 << 19;
 
 // Lockstep schedule: ICs of every mock (worker stream i mod K), then per step s one multi-mock

@@ -475,8 +475,9 @@ __global__ void __launch_bounds__(TCfg<L>::T) k_fz(float2* __restrict__ in, ZOut
     }
 }
 
-// Meshes whose passes all have a two-stage plan (N and N / 2): they can use the blocked layout.
-#define COLAPM_FOR_BLOCKED_SIZES(X) X(64) X(96) X(128) X(160) X(192) X(256) X(320) X(384) X(512) X(1024)
+// Meshes that can use the blocked layout (two-stage plans for N and N / 2: 64 to 1024) and whose force y pass does not go by
+// boxes (COLAPM_FOR_FY_BOX_SIZES).
+#define COLAPM_FOR_FY_PLAIN_SIZES(X) X(64) X(96) X(128) X(160) X(192) X(256) X(320) X(384)
 // Particle grids whose first-order LPT runs fused: those with two-stage plans from 128 (initial conditions of 128^3, 160^3,
 // 192^3, 320^3 and 384^3 particles 156, 320, 517, 2325 and 3940 us in separate passes, 134, 283, 438, 1803 and 2985
 // fused; 64^3 48.5 and 48.0, 96^3 83.6 and 87.4, too few tiles) up to 512 (9.11 and 7.57 ms; at 1024 a row's sums

@@ -66,15 +66,6 @@ static cudaError_t fy_box_t(const CUtensorMap* maps, const float2* tw, cudaStrea
 
 cudaError_t launch_fy_force(int n_mesh, float2* data, size_t field_stride, const float2* tw, cudaStream_t s, bool blocked,
                             float sg, const void* maps, int* err) {
-    if (maps && blocked) {
-        const auto* m = static_cast<const CUtensorMap*>(maps);
-        switch (n_mesh) {
-#define X(N) case N: return fy_box_t<N>(m, tw, s, err);
-            COLAPM_FOR_FY_BOX_SIZES(X)
-#undef X
-            default: break;
-        }
-    }
     if (!blocked) {
         switch (n_mesh) {
 #define X(N) case N: return fy_force_t<N, false>(data, field_stride, tw, s, sg);
@@ -83,9 +74,13 @@ cudaError_t launch_fy_force(int n_mesh, float2* data, size_t field_stride, const
             default: return cudaErrorInvalidValue;
         }
     }
+    const auto* m = static_cast<const CUtensorMap*>(maps);
     switch (n_mesh) {
+#define X(N) case N: return m ? fy_box_t<N>(m, tw, s, err) : cudaErrorInvalidValue;
+        COLAPM_FOR_FY_BOX_SIZES(X)
+#undef X
 #define X(N) case N: return fy_force_t<N, true>(data, field_stride, tw, s, sg);
-        COLAPM_FOR_BLOCKED_SIZES(X)
+        COLAPM_FOR_FY_PLAIN_SIZES(X)
 #undef X
         default: return cudaErrorInvalidValue;
     }
