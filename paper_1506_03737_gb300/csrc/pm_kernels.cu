@@ -69,41 +69,39 @@ __global__ void k_deposit(const float4* pos, size_t np3, UDiv u, unsigned long l
 }
 
 // Deposit on a mesh coarser than the particle grid (n_p^3 > n_m^3), where neighbouring particles share cells and the pass
-// is bound by the number of reductions (about 0.9 a clock and SM): one thread per particle, and an even lane whose
-// base cell is that of the odd lane after it gives its eight weights to that lane. Ten-step means: 128^3
-// particles on 64^3 and 32^3 cells 54 us against 91 with k_deposit, 256^3 on 128^3 and 64^3 324 against 494. With
-// as many cells as particles, passing right-hand corners on to the next lane's left-hand ones cost more than the
+// is bound by the number of reductions (about 0.9 a clock and SM): two threads per particle as above, and the two of an
+// even particle whose base cell is that of the particle after it give their weights to that one's. us with k_deposit / here:
+// initial conditions of 128^3 particles on 64^3 cells 41 / 35, after the steps 61 / 46, an evolved state with a fifth of the
+// particles in clumps 53 / 49, random positions 46 / 46; 256^3 on 128^3 267 / 236, 377 / 293, 351 / 328, 349 / 348; on 64^3
+// 611 / 383, 687 / 433, 617 / 497, 358 / 359. One thread per particle is faster where all lanes merge (29 for the
+// first of these) but loses the neighbouring x corners of an instruction where they do not (71 for the clumps, 76 for random).
+// With as many cells as particles, passing right-hand corners on to the next lane's left-hand ones cost more than the
 // reductions it saved (53 against 46 us at 128^3): k_deposit from there on.
 __global__ void k_deposit_dense(const float4* pos, size_t np3, UDiv u, unsigned long long* __restrict__ rho) {
     pdl_trigger();
     pdl_wait();
-    const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t p = t >> 1;
     const bool in = p < np3;   // every lane takes part in the exchange
-    const int nm = (int)u.d, odd = threadIdx.x & 1;
+    const int nm = (int)u.d, dx = (int)(t & 1);
     const Cic c = cic_setup(in ? pos[p] : make_float4(0.0f, 0.0f, 0.0f, 0.0f), u);
-    const unsigned wx[2] = {(unsigned)(QONE - c.fx), (unsigned)c.fx};
+    const unsigned wx = (unsigned)(dx ? c.fx : QONE - c.fx);
     const unsigned wy[2] = {(unsigned)(QONE - c.fy), (unsigned)c.fy};
     const unsigned wz[2] = {(unsigned)(QONE - c.fz), (unsigned)c.fz};
     const int cell = in ? (c.z0 * nm + c.y0) * nm + c.x0 : -1;   // nm <= 512 here
-    const int other = __shfl_xor_sync(0xffffffffu, cell, 1);
-    const bool same = in && other == cell;
-    unsigned long long w[4][2];   // [2 dz + dy][dx]
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int dx = 0; dx < 2; ++dx) {
-            w[r][dx] = (unsigned long long)(wy[r & 1] * wz[r >> 1]) * wx[dx];
-            const unsigned long long v = __shfl_xor_sync(0xffffffffu, w[r][dx], 1);
-            if (same) w[r][dx] += v;
-        }
-    if (!in || (same && !odd)) return;
-    const int ys[2] = {c.y0, c.y1}, zs[2] = {c.z0, c.z1};
+    const bool same = in && __shfl_xor_sync(0xffffffffu, cell, 2) == cell;
+    unsigned long long w[4];   // [2 dz + dy]
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-        unsigned long long* cells = rho + ((size_t)zs[r >> 1] * nm + ys[r & 1]) * nm;
-        if (w[r][0]) atomicAdd(cells + c.x0, w[r][0]);
-        if (w[r][1]) atomicAdd(cells + c.x1, w[r][1]);
+        w[r] = (unsigned long long)(wy[r & 1] * wz[r >> 1]) * wx;
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, w[r], 2);
+        if (same) w[r] += v;
     }
+    if (!in || (same && !(threadIdx.x & 2))) return;
+    const int x = dx ? c.x1 : c.x0, ys[2] = {c.y0, c.y1}, zs[2] = {c.z0, c.z1};
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+        if (w[r]) atomicAdd(rho + ((size_t)zs[r >> 1] * nm + ys[r & 1]) * nm + x, w[r]);
 }
 
 // Tiled deposit of particles ordered by tile (a sort with the same tile shape): a CTA takes the
@@ -630,7 +628,7 @@ inline unsigned blocks(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 cudaError_t launch_deposit(const float4* pos, size_t np3, int nm, unsigned long long* rho, cudaStream_t s, int block) {
     if (np3 > (size_t)nm * nm * nm)
-        return launch_dep(overlap_mesh(nm), k_deposit_dense, blocks(np3, block), block, 0, s, pos, np3, make_udiv(nm), rho);
+        return launch_dep(overlap_mesh(nm), k_deposit_dense, blocks(2 * np3, block), block, 0, s, pos, np3, make_udiv(nm), rho);
     return launch_dep(overlap_mesh(nm), k_deposit, blocks(2 * np3, block), block, 0, s, pos, np3, make_udiv(nm), rho);
 }
 
