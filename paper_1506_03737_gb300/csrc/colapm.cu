@@ -855,7 +855,8 @@ int power_enqueue(colapm_ctx* c, int nbins, const DepositSrc* src = nullptr, boo
     const double box = c->prm.box;
     Phase ph(c, COLAPM_PHASE_POWER);   // all of P(k), its deposit and forward passes included
     PhaseMute mute(c);
-    CK(cudaMemsetAsync(c->pw_acc, 0, power_words(nbins, kPowerRegions) * sizeof(double), c->stream));
+    const int regions = power_regions(c->nm, nbins);
+    CK(cudaMemsetAsync(c->pw_acc, 0, power_words(nbins, regions) * sizeof(double), c->stream));
     int r = deposit(c, src);
     if (r) return r;
     r = density_xy(c, use_blocked(c));
@@ -864,7 +865,7 @@ int power_enqueue(colapm_ctx* c, int nbins, const DepositSrc* src = nullptr, boo
     pw.n2_lo = c->pw_bin;
     pw.kfd = 2.0 * M_PI / box;
     pw.kf = (float)pw.kfd;
-    power_layout(pw, c->pw_acc, nbins, kPowerRegions);
+    power_layout(pw, c->pw_acc, nbins, regions);
     const double nm = c->nm;
     pw.pnorm = (float)(box * box * box / (nm * nm * nm * nm * nm * nm));
     pw.lga = c->pw_lga;

@@ -143,6 +143,11 @@ inline void power_thresholds(int nbins, double kmin, double kmax, double kf, int
 }
 
 constexpr int kPowerRegions = 16;   // 64 cost up to 8 us more in the final sum and gained nothing
+constexpr int kFewRegions = 2;
+// Copies of the bins of a pass. Few modes in many bins hardly meet, and the final sum goes over all copies: a call with 500, 1500
+// and 4096 bins on a 64^3 mesh took 79, 126 and 256 us with 16, 55, 79 and 126 with 2. From 4 nm bins on, as 16 are still
+// the better choice for 500 on 128^3 (81 us; 87 with 2).
+inline int power_regions(int nm, int nbins) { return nm <= 128 && nbins > 4 * nm ? kFewRegions : kPowerRegions; }
 // FP64 words of the accumulators of `nbins` bins: the result [3 nbins], the regions, the counter.
 __host__ __device__ constexpr size_t power_words(int nbins, int regions) { return (size_t)3 * nbins * (1 + regions) + 1; }
 // PowerArgs' accumulator pointers into such an array (all zero at the start of a pass).

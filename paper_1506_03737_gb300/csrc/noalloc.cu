@@ -163,7 +163,8 @@ extern "C" int colapm_power_noalloc(const int* cell, const float* offset, long l
     } while (0)
     NCK(cudaMemcpyAsync(tab, &h, offsetof(Tables, lo) + sizeof(int) * (nbins + 1), cudaMemcpyHostToDevice, s));
     NCK(cudaMemsetAsync(rho, 0, sizeof(unsigned long long) * nm3, s));
-    NCK(cudaMemsetAsync(err, 0, (kAcc - kErr) + sizeof(double) * power_words(nbins, kPowerRegions), s));
+    const int regions = power_regions(nm, nbins);
+    NCK(cudaMemsetAsync(err, 0, (kAcc - kErr) + sizeof(double) * power_words(nbins, regions), s));
     NCK(launch_dep(true, k_deposit_xyz, (unsigned)((n_particles + 255) / 256), 256, 0, s, cell, offset, n_particles, nm, rho, err));
     const double ratio = (double)nm3 / (double)n_particles;   // cells per particle
     NCK(launch_fx_fwd_i64(nm, rho, spec, tab->tw, (float)(ratio * std::ldexp(1.0, -45)), err, s));
@@ -172,7 +173,7 @@ extern "C" int colapm_power_noalloc(const int* cell, const float* offset, long l
     pw.n2_lo = tab->lo;
     pw.kf = (float)kf;
     pw.kfd = kf;
-    power_layout(pw, acc, nbins, kPowerRegions);
+    power_layout(pw, acc, nbins, regions);
     pw.pnorm = (float)(box * box * box / ((double)nm3 * (double)nm3));
     const double lr = std::log2(kmax / kmin);
     pw.lga = (float)(0.5 * nbins / lr);
