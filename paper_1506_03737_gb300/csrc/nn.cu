@@ -120,15 +120,13 @@ __host__ __device__ __forceinline__ int half_slot(int x, int k) { return k ^ ((x
 __device__ __forceinline__ size_t voxel(int n, int x, int y, int z) {
     return ((size_t)(z + 1) * (n + 2) + (y + 1)) * (n + 2) + (x + 1);
 }
+// Distance to the image along an axis: n on the low face, -n on the high one, 0 inside.
+__device__ __forceinline__ int image_of(int x, int n) { return x == 0 ? n : (x == n - 1 ? -n : 0); }
 template <class F>
-__device__ __forceinline__ void at_images(int n, int x, int y, int z, F f) {
-    const int ox = x == 0 ? n : (x == n - 1 ? -n : 0), oy = y == 0 ? n : (y == n - 1 ? -n : 0),
-              oz = z == 0 ? n : (z == n - 1 ? -n : 0);
+__device__ __forceinline__ void at_images(int n, size_t v, int ox, int oy, int oz, F f) {   // v: the voxel's index
 #pragma unroll 1
-    for (int k = 1; k < 8; ++k) {
-        if (((k & 1) && !ox) || ((k & 2) && !oy) || ((k & 4) && !oz)) continue;
-        f(voxel(n, x + (k & 1 ? ox : 0), y + (k & 2 ? oy : 0), z + (k & 4 ? oz : 0)));
-    }
+    for (int m = (ox ? 1 : 0) | (oy ? 2 : 0) | (oz ? 4 : 0), k = m; k; k = (k - 1) & m)   // the subsets of its faces
+        f(v + (ptrdiff_t)(k & 1 ? ox : 0) + (ptrdiff_t)(n + 2) * ((k & 2 ? oy : 0) + (ptrdiff_t)(n + 2) * (k & 4 ? oz : 0)));
 }
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
@@ -402,8 +400,10 @@ __global__ void __launch_bounds__(32 * TZ, TZ == 8 ? 2 : 4)
                     const __nv_bfloat162 b2z = __floats2bfloat162_rn(so[3 * e + 2], 0.0f);
                     const uint4 u = make_uint4(*reinterpret_cast<const uint32_t*>(&b01), *reinterpret_cast<const uint32_t*>(&b2z), 0u, 0u);
                     const int x = cx + e % TX, y = cy + e / TX, z = cz + tz;
-                    reinterpret_cast<uint4*>(a.out)[voxel(n, x, y, z)] = u;
-                    at_images(n, x, y, z, [&](size_t i) { reinterpret_cast<uint4*>(a.out)[i] = u; });
+                    const size_t v = voxel(n, x, y, z);
+                    reinterpret_cast<uint4*>(a.out)[v] = u;
+                    at_images(n, v, image_of(x, n), image_of(y, n), image_of(z, n),
+                              [&](size_t i) { reinterpret_cast<uint4*>(a.out)[i] = u; });
                 }
             }
             __syncwarp();   // the outputs have been read before the next tile's are written
@@ -606,15 +606,20 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t lbo, uint32_
 __device__ __forceinline__ void tc_stage(uint32_t sbase, const __nv_bfloat16* __restrict__ in, int n, int t, bool in8) {
     const int txn = n / 128, tyn = n / TC_TY;
     const int x0 = (t % txn) * 128, y0 = ((t / txn) % tyn) * TC_TY, z0 = (t / (txn * tyn)) * TC_TZ;
-#pragma unroll 1
-    for (int row = 0; row < TC_HY * TC_HZ; ++row) {
-        const int hy = row % TC_HY, hz = row / TC_HY;
-        const __nv_bfloat16* src = in + (((size_t)(z0 + hz) * (n + 2) + y0 + hy) * (n + 2) + x0) * (in8 ? 8 : C);
-        for (int j = threadIdx.x; j < (in8 ? 1 : 2) * TC_HX; j += 128) {
-            const int hx = in8 ? j : j >> 1, k = in8 ? 0 : j & 1;
-            cp_async16(sbase + k * TC_PLANE + (row * TC_HX + hx) * 16,
-                       in8 ? src + hx * 8 : src + hx * C + half_slot(hx, k) * 8);
-        }
+    // thread t copies the 16-byte pieces t, t + 128, ... of each of the 16 rows: the same place in every row
+    const int vb = in8 ? 16 : 32, pieces = in8 ? TC_HX : 2 * TC_HX;
+    const size_t ys = (size_t)(n + 2) * vb, zs = ys * (n + 2);
+    const char* base = reinterpret_cast<const char*>(in) + (size_t)z0 * zs + (size_t)y0 * ys + (size_t)x0 * vb;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int j = threadIdx.x + 128 * i;
+        if (j >= pieces) break;
+        const int hx = in8 ? j : j >> 1, k = in8 ? 0 : j & 1;
+        const char* src = base + (size_t)hx * vb + (in8 ? 0 : half_slot(hx, k) * 16);
+        const uint32_t dst = sbase + k * TC_PLANE + hx * 16;
+#pragma unroll
+        for (int row = 0; row < TC_HY * TC_HZ; ++row)
+            cp_async16(dst + row * (TC_HX * 16), src + (row / TC_HY) * zs + (row % TC_HY) * ys);
     }
     asm volatile("cp.async.commit_group;\n" ::);
 }
@@ -741,7 +746,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a, bool in8) {
                     op[half_slot(lane + 1, 1)] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
                 };
                 put(vs);
-                at_images(n, vx, vy, vz, put);
+                at_images(n, vs, image_of(vx, n), image_of(vy, n), image_of(vz, n), put);
             } else {   // EPI_OUT: channels 0..2
                 float dzv[3];
 #pragma unroll
@@ -760,7 +765,8 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a, bool in8) {
                     const __nv_bfloat162 b2z = __floats2bfloat162_rn(dzv[2], 0.0f);
                     const uint4 u = make_uint4(*reinterpret_cast<const uint32_t*>(&b01), *reinterpret_cast<const uint32_t*>(&b2z), 0u, 0u);
                     reinterpret_cast<uint4*>(a.out)[vs] = u;
-                    at_images(n, vx, vy, vz, [&](size_t i) { reinterpret_cast<uint4*>(a.out)[i] = u; });
+                    at_images(n, vs, image_of(vx, n), image_of(vy, n), image_of(vz, n),
+                              [&](size_t i) { reinterpret_cast<uint4*>(a.out)[i] = u; });
                 }
             }
         }
