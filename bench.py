@@ -45,13 +45,13 @@ EXTRA = {"deposit": ("particle", 16), "gather": ("cell", 12)}
 STEP_PHASES = ("sort", "deposit", "fft_fwd", "poisson", "fft_inv", "fft_inv_x", "gather")
 # Single-kernel phases, and the DRAM bytes (read + write) ncu measured for each kernel at
 # 256^3 particles / 512^3 mesh (per launch, MB), scaled to other sizes with N_m = 2 N_p by the
-# cell count: force z pass 536.8 + 1077.0, inverse x 1610.7 + 1561.6, force y inverse
-# 1071.0 + 1609.0, gather 2494.7 + 454.1, deposit 1243.8 + 792.8.
-DRAM_512 = {"poisson": 1613.8e6, "fft_inv_x": 3172.3e6, "fft_inv": 2680.0e6, "gather": 2948.8e6,
+# cell count: force z pass 539.5 + 1078.0, inverse x 1610.7 + 1561.6, force y inverse
+# 1071.0 + 1608.0, gather 2494.7 + 454.1, deposit 1243.8 + 792.8.
+DRAM_512 = {"poisson": 1617.5e6, "fft_inv_x": 3172.3e6, "fft_inv": 2679.0e6, "gather": 2948.8e6,
             "deposit": 2036.6e6}
 # Phases that run another kernel at 1024^3 than the one measured at 512^3 (the force z pass there
-# is another paired-lane kernel): their DRAM bytes per launch measured at 1024^3 (4561 + 8599 MB).
-DRAM_1024 = {"poisson": 13160.0e6}
+# is another paired-lane kernel): their DRAM bytes per launch measured at 1024^3 (4552 + 8600 MB).
+DRAM_1024 = {"poisson": 13152.0e6}
 
 
 def roofline(phase_ms, phase_n, np_, nm, hbm):

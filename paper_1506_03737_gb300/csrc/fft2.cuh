@@ -64,9 +64,10 @@ struct Tw2 {
 };
 // The same with the powers too, each rounded once: w[k][j] = w^(k j), k < 8, j < JN. A chain repeats the rounding of w1[j] in
 // every power, and whatever it takes from a root's modulus it takes from each line alike, so that it stays in the mean of
-// a P(k) bin. For the lengths that would otherwise get their roots from the full table (32, 48 and 80 points, which
-// the Stockham engine transformed): power lost per line 6.9e-8, 4.0e-8 and 3.9e-8 by chains, 3.8e-8, 3.7e-8 and
-// nothing by this table (2.8e-8, 1.8e-8 and nothing there).
+// a P(k) bin. For the lengths whose other engine takes its roots from the full table (32, 48 and 80 points): rms error of a
+// transform 9.2e-8, 9.8e-8 and 1.22e-7 by chains, 7.3e-8, 7.9e-8 and 8.7e-8 by this table, power of a line off by
+// -7.9e-8, -5.9e-8 and -3.0e-8, now -3.8e-8, -3.7e-8 and 0.8e-8 (emulated on the CPU against FP64), in the same time. At 64, 160 and 192
+// points it would gain as much but costs 0.4 to 1% on their meshes (spectrum of 64^3 cells 64.1 -> 66.5 us): chains there.
 template <int JN>
 struct Tw8 {
     static_assert(JN == 16 || JN == 32, "");
@@ -236,10 +237,10 @@ __global__ void __launch_bounds__(K2<L>::T) k2_fy(float2* __restrict__ data, siz
 // (fire and forget; shared-memory FP64 atomics are retry loops on which the lanes of a warp collide), over 16
 // copies of the bins. What bounded the binning was the search for the next bin, which the lanes of a warp reach
 // at different modes (BinWalk), and a square root and a division per mode. At 64^3, 128^3, 512^3 and 1024^3 with
-// 32 to 100 bins the pass took 17, 42, 717 and 5171 us with them, then 9, 16, 290 and 1978 us (512^3
-// with its tiles moved by boxes, k2_power_box: 228). Counting the modes apart, over 1/48 of the grid, took
+// 32 to 100 bins the pass took 17, 42, 717 and 5171 us with them, 8, 16, 298 and 2109 us now (512^3
+// with its tiles moved by boxes, k2_power_box: 235). Counting the modes apart, over 1/48 of the grid, took
 // 460 us at 1024^3: the loops were too few and too long. Every pair of modes is divided by its own window: a factor
-// per column times a table per z is 4 us less at 512^3 (1722 of 1726 for the call), but their few roundings
+// per column times a table per z is faster (512^3 227 us, 1024^3 1998), but their few roundings
 // stay in a bin's mean (P(k) off by 1.60, 1.77 and 2.37e-7 at 128^3, 192^3 and 384^3 instead of 1.51, 1.62 and 2.33e-7).
 // |n| is summed in units of the fundamental, which is applied to the sums in FP64.
 template <int L, int C, int T>

@@ -628,7 +628,8 @@ __global__ void __launch_bounds__(FyBox<L>::T, FyBox<L>::MINB)
 // P(k) z pass of the blocked layout at 256, 384 and 512 points: 4-column tiles by boxes, stages as in the passes above
 // (the radix-32 ones on pairs), |X|^2 into shared memory, power_bin_tile. The next tile arrives during stage B and
 // the binning, which bounds the pass (one search and one flush per run, three reductions in L2 each). Against
-// k2_fz: 49 -> 46, 115 -> 112 and 287 -> 228 us at 256, 384 and 512 points (100 bins). Not at 320 (68 -> 69), and not at
+// k2_fz: 49 -> 46, 115 -> 112 and 287 -> 228 us at 256, 384 and 512 points (100 bins; before every mode had its own window,
+// with which it takes 235 at 512). Not at 320 (68 -> 69), and not at
 // 1024: its stages need 256 threads, and runs of 8 modes then double the reductions (1.98 -> 3.11 ms; binning by
 // half of the threads 2.07; the same at 512 points 259 us).
 template <int L>
